@@ -1397,11 +1397,14 @@ extern "C" int mueller_rhs_planewave(mueller_ctx* c, const double* dirs, const d
   if (!c || !dirs || !pols || !rhs_dev || (nrhs < 1 || nrhs > 65535)) return fail(MUELLER_EINVAL, "invalid rhs arguments");
   cudaStream_t s = (cudaStream_t)stream;
   DevBuf tmp;
-  double *dd, *dp;
+  double *dd, *dp, *scratch;
+  const int nth = n_theta_for(c->S);
   std::vector<double> vd(dirs, dirs + 3 * nrhs), vp(pols, pols + 3 * nrhs);
   CK(tmp.upload(&dd, vd, s)); CK(tmp.upload(&dp, vp, s));
   FieldGeom g{c->geo[0], c->geo[1], c->geo[2], c->geo[3], c->geo[4], c->S.N};
-  launch_rhs_planewave(g, c->S.M, c->S.k0, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, n_theta_for(c->S),
+  if (tmp.alloc(&scratch, rhs_planewave_scratch_doubles(c->S.M, nrhs, nth)) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "wave table");
+  launch_rhs_planewave(g, c->S.M, c->S.k0.x, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, nth, scratch,
                        (cd*)rhs_dev, s);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
@@ -1499,12 +1502,15 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
   const int nth = std::max(nth_base, std::min(8192, (int)std::ceil(40.0 * S.rmax / dmin_all)));
   cudaStream_t s = (cudaStream_t)stream;
   DevBuf tmp;
-  cd *cur, *xs;
-  double *X, *dgr, *dgz, *dgrp, *dgzp, *dgw, *dLm;
+  cd *cur, *xs, *part;
+  double *pts, *X, *dgr, *dgz, *dgrp, *dgzp, *dgw, *dLm;
   int* dn0;
   std::vector<double> vx(targets, targets + 3 * ntargets);
   const long long nvec = (long long)(2 * S.M + 1) * nrhs;
-  if (tmp.alloc(&cur, (size_t)nrhs * nsub * nth * 4) != cudaSuccess ||
+  const long long nring = (long long)nsub * nth;
+  if (tmp.alloc(&cur, (size_t)near_field_group(nring, nrhs) * nring * 6) != cudaSuccess ||
+      tmp.alloc(&pts, (size_t)nring * 4) != cudaSuccess ||
+      tmp.alloc(&part, near_field_part(nring, ntargets, nrhs)) != cudaSuccess ||
       tmp.alloc(&xs, (size_t)nvec * 4 * nsub) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "evaluation buffers");
   CK(tmp.upload(&X, vx, s));
@@ -1513,7 +1519,7 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
   CK(tmp.upload(&dn0, node0, s));
   launch_interp_currents((const cd*)x_dev, 4 * S.N, nsub, dn0, dLm, nvec, xs, s);
   FieldGeom g{dgr, dgz, dgrp, dgzp, dgw, nsub};
-  launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, (cd*)out_dev, s);
+  launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, pts, part, (cd*)out_dev, s);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return MUELLER_OK;
@@ -1546,12 +1552,13 @@ extern "C" int mueller_far_field_grid(mueller_ctx* c, const mueller_c128* x_dev,
   cudaStream_t s = (cudaStream_t)stream;
   const int M = c->S.M, nth = n_theta_for(c->S);
   DevBuf tmp;
-  cd *coef, *F;
-  if (tmp.alloc(&coef, (size_t)n_polar * c->S.N * (2 * M + 3)) != cudaSuccess ||
+  double* coef;
+  cd* F;
+  if (tmp.alloc(&coef, far_field_grid_coef_doubles(c->S.N, M, n_polar)) != cudaSuccess ||
       tmp.alloc(&F, (size_t)nrhs * n_polar * (2 * M + 1) * 3) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "far-field grid buffers");
   FieldGeom g{c->geo[0], c->geo[1], c->geo[2], c->geo[3], c->geo[4], c->S.N};
-  launch_far_field_grid(g, M, c->S.k0, c->S.omega, c->S.eps0, (const cd*)x_dev, nrhs, n_polar, n_azim, nth, coef, F,
+  launch_far_field_grid(g, M, c->S.k0.x, c->S.omega, c->S.eps0, (const cd*)x_dev, nrhs, n_polar, n_azim, nth, coef, F,
                         (cd*)E_dev, s);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
