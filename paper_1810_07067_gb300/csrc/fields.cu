@@ -605,12 +605,11 @@ __global__ void __launch_bounds__(256) ffgrid_coef_kernel(FieldGeom g, int M, do
 // X_0 = z' J1 (and the same of M), J_rho = (U_+ + U_-)/2, J_phi = (U_+ - U_-)/(2i),
 // J_z = U_0; the real and imaginary parts of the phase are summed apart (A, B),
 // so the two mirrored angles are A + iB and A - iB: 4 multiply-adds per term
-// for both.  FP64 pipe (24 multiply-adds per node, mode, angle pair and side,
-// the 22 flops per angle it replaces plus a sincos each); the whole grid, N = 512,
-// M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex coefficients per
-// angle, the phase formed per mode and side).  One CTA per (mode, 16 polar angles, WT right-hand sides); a
-// thread owns one (angle, side) and every JS-th node; the nodes pass through
-// shared memory FFM_JC at a time.
+// for both.  FP64 pipe: 24 multiply-adds per node, mode, angle pair and side; the
+// whole grid, N = 512, M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex
+// coefficients per angle and the phase formed per mode and side).  One CTA per
+// (mode, 16 polar angles, WT right-hand sides); a thread owns one (angle, side)
+// and every JS-th node; the nodes pass through shared memory FFM_JC at a time.
 #define FFM_PT 16
 #define FFM_JC 16
 template <int WT>

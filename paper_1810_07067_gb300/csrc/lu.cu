@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include "smem.cuh"
 #include "lu.cuh"
+#include "lu_oz.cuh"
 
 std::mutex& lu_capture_mutex() {
   static std::mutex m;
@@ -33,13 +34,21 @@ namespace cg = cooperative_groups;
 // Pivot measure: |a|^2 in FP64 for complex128; |Re a| + |Im a| in FP32 for
 // complex64 (LAPACK's complex pivot measure; GB300's FP64 pipe is too slow to
 // sit on the panel's critical path).  Largest measure, lowest row on ties.
+// The FP64 measure is compared as an integer (the bits of a non-negative double
+// keep its order; 0 = no candidate, NaN is never one): the comparisons of the
+// search would otherwise queue on the FP64 pipe.
 template <class T> struct Pivot;
 template <> struct Pivot<cd> {
-  using V = double;
-  __device__ static V measure(cd a) { return norm2(a); }
+  using V = unsigned long long;
+  static constexpr V NONE = 0, ZERO = 1;
+  __device__ static V measure(cd a) {
+    const V b = (V)__double_as_longlong(norm2(a));
+    return b > 0x7FF0000000000000ull ? NONE : b + 1;
+  }
 };
 template <> struct Pivot<cf> {
   using V = float;
+  static constexpr V NONE = -1.f, ZERO = 0.f;
   __device__ static V measure(cf a) { return fabsf(a.x) + fabsf(a.y); }
 };
 
@@ -66,7 +75,7 @@ __global__ void __launch_bounds__(1024) panel_kernel(const LuMat* __restrict__ m
   for (int jj = 0; jj < nbk; ++jj) {
     const int c = k0 + jj;
     T* col = M + (size_t)c * n;
-    V best = V(-1);
+    V best = Pivot<T>::NONE;
     int bi = n;
     for (int r = c + tid; r < n; r += NT) argmax_merge(best, bi, Pivot<T>::measure(col[r]), r);
     for (int o = 16; o > 0; o >>= 1) {
@@ -77,7 +86,7 @@ __global__ void __launch_bounds__(1024) panel_kernel(const LuMat* __restrict__ m
     if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
     __syncthreads();
     if (wid == 0) {
-      best = (lane < (NT >> 5)) ? red_v[lane] : V(-1);
+      best = (lane < (NT >> 5)) ? red_v[lane] : Pivot<T>::NONE;
       bi = (lane < (NT >> 5)) ? red_i[lane] : n;
       for (int o = 16; o > 0; o >>= 1) {
         V v2 = __shfl_xor_sync(0xffffffffu, best, o);
@@ -85,9 +94,9 @@ __global__ void __launch_bounds__(1024) panel_kernel(const LuMat* __restrict__ m
         argmax_merge(best, bi, v2, i2);
       }
       if (lane == 0) {
-        s_p = (best > V(0)) ? bi : -1;
-        pv[c] = (best > V(0)) ? bi : c;
-        if (best <= V(0) && info[0] == 0) info[0] = c + 1;
+        s_p = (best > Pivot<T>::ZERO) ? bi : -1;
+        pv[c] = (best > Pivot<T>::ZERO) ? bi : c;
+        if (best <= Pivot<T>::ZERO && info[0] == 0) info[0] = c + 1;
       }
     }
     __syncthreads();
@@ -155,6 +164,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
   __shared__ V cand_v[2][8];
   __shared__ int cand_i[2][8];
   __shared__ T cand_row[2][8][LU_NB];   // each CTA's candidate row of the panel
+  __shared__ T cand_inv[2][8];          // and the reciprocal of its candidate
   __shared__ T top_row[2][LU_NB];       // row c (CTA 0 owns every row c of the panel)
   __shared__ V red_v[PANEL_THREADS / 32];
   __shared__ int red_i[PANEL_THREADS / 32];
@@ -162,6 +172,9 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int row0 = k0 + q * R;
   const int nr = max(0, min(R, n - row0));  // rows owned by this CTA
+  int Rt = 32;                              // threads along the rows: a power of two of at least R rows
+  while (Rt < R && Rt < PANEL_THREADS) Rt *= 2;
+  const int ng = PANEL_THREADS / Rt, jg = tid / Rt;
   for (int t = tid; t < nbk * nr; t += PANEL_THREADS) {
     int r = t % nr, j = t / nr;
     a[j * R + r] = M[(size_t)(k0 + j) * n + row0 + r];
@@ -170,7 +183,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
   for (int jj = 0; jj < nbk; ++jj) {
     const int c = k0 + jj, buf = jj & 1;
     const T* aj = a + jj * R;
-    V best = V(-1);
+    V best = Pivot<T>::NONE;
     int bi = n;
     for (int r = max(0, c - row0) + tid; r < nr; r += PANEL_THREADS)
       argmax_merge(best, bi, Pivot<T>::measure(aj[r]), row0 + r);
@@ -182,7 +195,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
     if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
     __syncthreads();
     if (wid == 0) {
-      best = (lane < PANEL_THREADS / 32) ? red_v[lane] : V(-1);
+      best = (lane < PANEL_THREADS / 32) ? red_v[lane] : Pivot<T>::NONE;
       bi = (lane < PANEL_THREADS / 32) ? red_i[lane] : n;
       for (int o = 16; o > 0; o >>= 1) {
         V v2 = __shfl_xor_sync(0xffffffffu, best, o);
@@ -196,15 +209,19 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
       if (lane == 0) s_bi = bi;
     }
     __syncthreads();
+    if (wid == 0 && lane < C) {  // one warp's division, beside the exchange of the rows
+      const int b = s_bi;
+      cl.map_shared_rank(cand_inv[buf], lane)[q] = b < n ? cone<T>() / aj[b - row0] : czero<T>();
+    }
     // the candidate row (and, from CTA 0, row c) into every CTA
     const int cb = s_bi;
-    if (tid < nbk * C) {
-      const int j = tid % nbk, u = tid / nbk;
+    for (int e = tid - 32; e >= 0 && e < nbk * C; e += PANEL_THREADS - 32) {
+      const int j = e % nbk, u = e / nbk;
       if (cb < n) cl.map_shared_rank(cand_row[buf][q], u)[j] = a[j * R + cb - row0];
       if (q == 0) cl.map_shared_rank(top_row[buf], u)[j] = a[j * R + c - row0];
     }
     cl.sync();
-    best = V(-1);
+    best = Pivot<T>::NONE;
     bi = n;
     int win = -1;
     for (int u = 0; u < C; ++u) {
@@ -212,7 +229,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
       const int i2 = cand_i[buf][u];
       if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; win = u; }
     }
-    const int p = (best > V(0)) ? bi : -1;
+    const int p = (best > Pivot<T>::ZERO) ? bi : -1;
     if (q == 0 && tid == 0) {
       pv[c] = (p >= 0) ? p : c;
       if (p < 0 && info[0] == 0) info[0] = c + 1;
@@ -225,12 +242,15 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
         if (q == 0) a[tid * R + c - row0] = prow[tid];                       // the pivot row to c
       }
       __syncthreads();
-      const T inv = cone<T>() / prow[jj];
-      for (int r = max(0, c + 1 - row0) + tid; r < nr; r += PANEL_THREADS) {
-        T l = a[jj * R + r] * inv;
-        a[jj * R + r] = l;
-        for (int j = jj + 1; j < nbk; ++j) a[j * R + r] = a[j * R + r] - l * prow[j];
+      const T inv = cand_inv[buf][win];
+      // PANEL_THREADS / Rt threads share a row's columns when a CTA owns few rows
+      for (int r = max(0, c + 1 - row0) + tid % Rt; r < nr; r += Rt) {
+        const T l = a[jj * R + r] * inv;
+        for (int j = jj + 1 + jg; j < nbk; j += ng) a[j * R + r] = a[j * R + r] - l * prow[j];
       }
+      __syncthreads();
+      if (jg == 0)
+        for (int r = max(0, c + 1 - row0) + tid % Rt; r < nr; r += Rt) a[jj * R + r] = a[jj * R + r] * inv;
     }
     __syncthreads();
   }
@@ -241,15 +261,28 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
   cl.sync();  // no CTA leaves while a peer could still address its shared memory
 }
 
+static int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
+    cudaGetLastError();
+    sms = 1;
+  }
+  return sms;
+}
+
 // Cluster size: the smallest of 1, 2, 4, 8 whose row slices of the largest
-// matrix (rows = its n - k0) fit PANEL_SMEM_MAX; smaller matrices of a ragged
-// batch own fewer rows of the same slices.  Returns false (nothing launched)
+// matrix (rows = its n - k0) fit PANEL_SMEM_MAX, then doubled while that leaves
+// one CTA per SM and 64 rows per CTA (the rank-1 updates are bound by the FP64
+// pipe of the SMs a matrix has); smaller matrices of a ragged batch own fewer
+// rows of the same slices.  Returns false (nothing launched)
 // when none fits or no such cluster can be resident; the caller then uses
 // panel_kernel.
 template <class T>
 static bool launch_panel_cluster(const LuMat* mats, int rows, int k0, int batch, cudaStream_t s) {
   int C = 1;
   while (C < 8 && (size_t)LU_NB * ((rows + C - 1) / C) * sizeof(T) > PANEL_SMEM_MAX) C *= 2;
+  while (C < 8 && 2 * C * batch <= sm_count() && rows >= 128 * C) C *= 2;
   const int R = (rows + C - 1) / C;
   const size_t smem = (size_t)LU_NB * R * sizeof(T);
   if (smem > PANEL_SMEM_MAX) return false;
@@ -992,16 +1025,6 @@ __global__ void __launch_bounds__(192, 1) gemm_update_tc_kernel(const LuMat* __r
 }
 
 // ---------------------------------------------------------------- driver
-static int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
-    cudaGetLastError();
-    sms = 1;
-  }
-  return sms;
-}
-
 // R3 of outer block K0 for the matrices 0..active-1 (those with n > K0 + LU_OB);
 // rest = nmax - K0 - LU_OB is the largest trailing size.
 template <int TN>
@@ -1143,25 +1166,56 @@ int lu_tile_table(int* rest_hi, int* count_hi, int* tile, float* ms, int cap) {
   return k;
 }
 
+// Complex128 workspace: the matrices (largest first) are factored in groups whose
+// luz_matrix_bytes fit the pool; without a pool that holds the largest matrix
+// the updates run on the FP64 pipe.
+size_t lu_z_pool_bytes(const int* n, int count, size_t most) {
+  size_t need = 0, one = 0;
+  for (int b = 0; b < count; ++b) {
+    const size_t w = luz_matrix_bytes(n[b]);
+    need += w;
+    one = std::max(one, w);
+  }
+  return std::max(one, std::min(need, most));
+}
+
 // Right-looking blocked LU of every matrix of the table, largest first: at
 // step k0 the launches cover the matrices with n > k0 (a prefix of the sorted
 // table), each kernel reading its matrix, size and pivots from the table.
+// Complex128 with a pool and complex64 work on two levels (LU_NB panels in
+// LU_OB blocks, products on the tensor cores); complex128 without a pool
+// updates the trailing matrix after every panel on the FP64 pipe.  The choice
+// changes rounding, so it is one for all matrices of a call.
 template <class T>
 static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s, LuTiming* tm, int* tc_err, int tile,
-                                  bool graph) {
+                                  bool graph, const LuPool& pool) {
   if (count <= 0) return cudaSuccess;
   std::vector<LuMat> it(items, items + count);
   std::stable_sort(it.begin(), it.end(), [](const LuMat& a, const LuMat& b) { return a.n > b.n; });
-  const int nmax = it[0].n;
-  LuMat* d = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d, sizeof(LuMat) * count, s);
-  if (e != cudaSuccess) return e;
-  cudaMemcpyAsync(d, it.data(), sizeof(LuMat) * count, cudaMemcpyHostToDevice, s);
-  lu_info_zero_kernel<<<(count + 255) / 256, 256, 0, s>>>(d, count);
   constexpr bool c64 = std::is_same<T, cf>::value;
+  std::vector<int> groups = {0};  // first matrix of every group
+  const bool two_level = c64 || (pool.p && luz_matrix_bytes(it[0].n) <= pool.bytes);
+  if (!c64 && two_level) {
+    size_t o = 0;
+    for (int b = 0; b < count; ++b) {
+      const size_t w = luz_matrix_bytes(it[b].n);
+      if (o + w > pool.bytes) {
+        groups.push_back(b);
+        o = 0;
+      }
+      it[b].ws = (unsigned char*)pool.p + o;
+      o += w;
+    }
+  }
+  groups.push_back(count);
+  LuMat* dall = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&dall, sizeof(LuMat) * count, s);
+  if (e != cudaSuccess) return e;
+  cudaMemcpyAsync(dall, it.data(), sizeof(LuMat) * count, cudaMemcpyHostToDevice, s);
+  lu_info_zero_kernel<<<(count + 255) / 256, 256, 0, s>>>(dall, count);
   if constexpr (c64) {
     tc_set_attributes();
-    if (tile == 0) autotune_tiles(nmax, count, s);
+    if (tile == 0) autotune_tiles(it[0].n, count, s);
   }
   cudaStream_t ls = s, cs = nullptr;
   // while this thread captures, no other thread of the library frees device
@@ -1184,7 +1238,6 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
   std::vector<cudaEvent_t> ev;
   int launches = 1, gemm_launches = 0, tn_steps[3] = {0, 0, 0};
   double gemm_flops = 0.0, gemm_bytes = 0.0;
-  int active = count;
   auto timed_launch = [&](auto&& launch) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (timed) {
@@ -1197,89 +1250,100 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
       ev.push_back(e0); ev.push_back(e1);
     }
   };
-  // one LU_NB panel at column k0: factor, interchange, rows of U right of it
-  // (mode 0: all columns; mode 1: within the LU_OB block starting at K0)
-  auto panel_step = [&](int k0, int K0, int mode) -> int {
-    while (active > 0 && it[active - 1].n <= k0) --active;
-    const int nbk = std::min(LU_NB, nmax - k0);
-    bool done = false;
-    if constexpr (c64) done = launch_panel_reg(d, nmax - k0, k0, active, ls);
-    if (!done && !launch_panel_cluster<T>(d, nmax - k0, k0, active, ls)) panel_kernel<T><<<active, 1024, 0, ls>>>(d, k0);
-    ++launches;
-    const int hi = mode == 1 ? std::min(K0 + LU_OB, nmax) : nmax;
-    if (hi - nbk > 0) {
-      swap_kernel<T><<<dim3((hi - nbk + SWAP_COLS - 1) / SWAP_COLS, active), 256, 0, ls>>>(d, k0, K0, mode);
-      ++launches;
-    }
-    const int rest = hi - k0 - nbk;
-    if (rest > 0) {
-      trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
-      ++launches;
-    }
-    return rest;
-  };
-  if constexpr (c64) {
-    // two-level: LU_NB panels inside LU_OB blocks, one rank-LU_OB tensor-core update per block
-    for (int K0 = 0; K0 < nmax; K0 += LU_OB) {
-      for (int p = 0; p < LU_OB_CHUNKS; ++p) {
-        const int k0 = K0 + p * LU_NB;
-        if (k0 >= nmax) break;
-        const int bcols = panel_step(k0, K0, 1);                    // R1: block columns right of the panel
-        if (bcols <= 0) continue;
-        const int rows = nmax - k0 - LU_NB;
-        strip_update_kernel<T><<<dim3((rows + GT - 1) / GT, (bcols + GT - 1) / GT, active), 256, 0, ls>>>(
-            d, K0, k0, 1);
-        ++launches;
-      }
-      const int rest = nmax - K0 - LU_OB;                           // columns right of the block
-      if (rest <= 0) continue;
-      int a3 = active;                                               // the matrices that have them
-      while (a3 > 0 && it[a3 - 1].n <= K0 + LU_OB) --a3;
-      if (a3 <= 0) continue;
-      for (int p = 0; p < LU_OB_CHUNKS; ++p) {                      // the block's interchanges, in order
-        swap_kernel<T><<<dim3((rest + SWAP_COLS - 1) / SWAP_COLS, a3), 256, 0, ls>>>(d, K0 + p * LU_NB, K0, 2);
-        ++launches;
-      }
-      for (int p = 0; p < LU_OB_CHUNKS; ++p) {                      // rows of U right of the block; R2
-        const int k0 = K0 + p * LU_NB;
-        trsm_kernel<T><<<dim3((rest + 127) / 128, a3), 128, 0, ls>>>(d, k0, K0, 2);
-        ++launches;
-        const int brows = LU_OB - (p + 1) * LU_NB;
-        if (brows > 0) {
-          strip_update_kernel<T><<<dim3((brows + GT - 1) / GT, (rest + GT - 1) / GT, a3), 256, 0, ls>>>(
-              d, K0, k0, 2);
-          ++launches;
-        }
-      }
-      // R3
-      const int tn = tile ? tile : tuned_tile(rest, a3);
-      timed_launch([&] { tc_update(tn, d, K0, rest, a3, tc_err, ls); });
-      ++tn_steps[tn == 32 ? 0 : tn == 64 ? 1 : 2];
-      launches += 2;
-      for (int b = 0; b < a3; ++b) {
-        const double rb = (double)(it[b].n - K0 - LU_OB);
+  for (size_t gi = 0; gi + 1 < groups.size(); ++gi) {
+    const LuMat* d = dall + groups[gi];
+    const LuMat* g = it.data() + groups[gi];
+    int active = groups[gi + 1] - groups[gi];
+    const int nmax = g[0].n;
+    auto count_update = [&](int k, int K) {  // trailing update of K columns at column k
+      for (int b = 0; b < active; ++b) {
+        const double rb = (double)(g[b].n - k - K);
         if (rb > 0) {
-          gemm_flops += 8.0 * rb * rb * LU_OB;
+          gemm_flops += 8.0 * rb * rb * K;
           gemm_bytes += 2.0 * sizeof(T) * rb * rb;   // the trailing matrix read and written once
         }
       }
       ++gemm_launches;
-    }
-  } else {
-    for (int k0 = 0; k0 < nmax; k0 += LU_NB) {
-      const int rest = panel_step(k0, 0, 0);
-      if (rest <= 0) continue;
-      const int t = (rest + GT - 1) / GT;
-      timed_launch([&] { gemm_update_kernel<T><<<dim3(t, t, active), 256, 0, ls>>>(d, k0); });
+    };
+    // one LU_NB panel at column k0: factor, interchange, rows of U right of it
+    // (mode 0: all columns; mode 1: within the LU_OB block starting at K0)
+    auto panel_step = [&](int k0, int K0, int mode) -> int {
+      while (active > 0 && g[active - 1].n <= k0) --active;
+      const int nbk = std::min(LU_NB, nmax - k0);
+      bool done = false;
+      if constexpr (c64) done = launch_panel_reg(d, nmax - k0, k0, active, ls);
+      if (!done && !launch_panel_cluster<T>(d, nmax - k0, k0, active, ls))
+        panel_kernel<T><<<active, 1024, 0, ls>>>(d, k0);
       ++launches;
-      for (int b = 0; b < active; ++b) {
-        const double rb = (double)(it[b].n - k0 - LU_NB);
-        if (rb > 0) {
-          gemm_flops += 8.0 * rb * rb * LU_NB;
-          gemm_bytes += 2.0 * sizeof(T) * rb * rb;
-        }
+      const int hi = mode == 1 ? std::min(K0 + LU_OB, nmax) : nmax;
+      if (hi - nbk > 0) {
+        swap_kernel<T><<<dim3((hi - nbk + SWAP_COLS - 1) / SWAP_COLS, active), 256, 0, ls>>>(d, k0, K0, mode);
+        ++launches;
       }
-      ++gemm_launches;
+      const int rest = hi - k0 - nbk;
+      if (rest > 0) {
+        if (!c64 && two_level) luz_panel_rows(d, K0, k0, rest, active, ls);
+        else trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
+        ++launches;
+      }
+      return rest;
+    };
+    if (two_level) {
+      // LU_NB panels inside LU_OB blocks, one rank-LU_OB tensor-core update per block
+      for (int K0 = 0; K0 < nmax; K0 += LU_OB) {
+        for (int p = 0; p < LU_OB_CHUNKS; ++p) {
+          const int k0 = K0 + p * LU_NB;
+          if (k0 >= nmax) break;
+          const int bcols = panel_step(k0, K0, 1);                    // R1: block columns right of the panel
+          if (bcols <= 0) continue;
+          const int rows = nmax - k0 - LU_NB;
+          if constexpr (c64) {
+            strip_update_kernel<T><<<dim3((rows + GT - 1) / GT, (bcols + GT - 1) / GT, active), 256, 0, ls>>>(
+                d, K0, k0, 1);
+            ++launches;
+          } else {
+            launches += luz_panel_update(d, K0, k0, nmax, active, tc_err, ls);
+          }
+        }
+        const int rest = nmax - K0 - LU_OB;                           // columns right of the block
+        if (rest <= 0) continue;
+        while (active > 0 && g[active - 1].n <= K0 + LU_OB) --active;  // the matrices that have them
+        if (active <= 0) continue;
+        for (int p = 0; p < LU_OB_CHUNKS; ++p) {                      // the block's interchanges, in order
+          swap_kernel<T><<<dim3((rest + SWAP_COLS - 1) / SWAP_COLS, active), 256, 0, ls>>>(d, K0 + p * LU_NB, K0, 2);
+          ++launches;
+        }
+        if constexpr (c64) {
+          for (int p = 0; p < LU_OB_CHUNKS; ++p) {                    // rows of U right of the block; R2
+            const int k0 = K0 + p * LU_NB;
+            trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, 2);
+            ++launches;
+            const int brows = LU_OB - (p + 1) * LU_NB;
+            if (brows > 0) {
+              strip_update_kernel<T><<<dim3((brows + GT - 1) / GT, (rest + GT - 1) / GT, active), 256, 0, ls>>>(
+                  d, K0, k0, 2);
+              ++launches;
+            }
+          }
+          // R3
+          const int tn = tile ? tile : tuned_tile(rest, active);
+          timed_launch([&] { tc_update(tn, d, K0, rest, active, tc_err, ls); });
+          ++tn_steps[tn == 32 ? 0 : tn == 64 ? 1 : 2];
+          launches += 2;
+        } else {
+          timed_launch([&] { launches += luz_block_update(d, K0, nmax, active, tc_err, ls); });
+        }
+        count_update(K0, LU_OB);
+      }
+    } else if constexpr (!c64) {
+      for (int k0 = 0; k0 < nmax; k0 += LU_NB) {
+        const int rest = panel_step(k0, 0, 0);
+        if (rest <= 0) continue;
+        const int t = (rest + GT - 1) / GT;
+        timed_launch([&] { gemm_update_kernel<T><<<dim3(t, t, active), 256, 0, ls>>>(d, k0); });
+        ++launches;
+        count_update(k0, LU_NB);
+      }
     }
   }
   if (graph) {
@@ -1294,11 +1358,11 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) {  // nothing of the capture ran: factor with direct launches instead
       cudaGetLastError();
-      cudaFreeAsync(d, s);
-      return lu_factor_impl<T>(items, count, s, tm, tc_err, tile, false);
+      cudaFreeAsync(dall, s);
+      return lu_factor_impl<T>(items, count, s, tm, tc_err, tile, false, pool);
     }
   }
-  cudaFreeAsync(d, s);
+  cudaFreeAsync(dall, s);
   if (tm) {
     tm->launches += launches;
     tm->gemm_flops += gemm_flops;
@@ -1318,15 +1382,16 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
 }
 
 cudaError_t lu_factor_many(const LuMat* items, int count, bool c64, cudaStream_t s, LuTiming* tm, int* tc_err,
-                           int tile, bool graph) {
-  return c64 ? lu_factor_impl<cf>(items, count, s, tm, tc_err, tile, graph)
-             : lu_factor_impl<cd>(items, count, s, tm, nullptr, 0, graph);
+                           int tile, bool graph, const LuPool& pool) {
+  return c64 ? lu_factor_impl<cf>(items, count, s, tm, tc_err, tile, graph, pool)
+             : lu_factor_impl<cd>(items, count, s, tm, tc_err, 0, graph, pool);
 }
 
-void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* tm) {
+void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* tm, int* tc_err,
+                       const LuPool& pool) {
   std::vector<LuMat> it(batch);
   for (int b = 0; b < batch; ++b) it[b] = LuMat{A + (size_t)b * n * n, piv + (size_t)b * n, info + b, nullptr, n, 0};
-  lu_factor_impl<cd>(it.data(), batch, s, tm, nullptr, 0, false);
+  lu_factor_impl<cd>(it.data(), batch, s, tm, tc_err, 0, false, pool);
 }
 
 void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* tm,
@@ -1335,7 +1400,7 @@ void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStr
   for (int b = 0; b < batch; ++b)
     it[b] = LuMat{A + (size_t)b * n * n, piv + (size_t)b * n, info + b,
                   (__nv_bfloat16*)ws + tcu_ws_matrix_elems(n) * b, n, 0};
-  lu_factor_impl<cf>(it.data(), batch, s, tm, tc_err, tile, false);
+  lu_factor_impl<cf>(it.data(), batch, s, tm, tc_err, tile, false, LuPool{});
 }
 
 // ---------------------------------------------------------------- solves

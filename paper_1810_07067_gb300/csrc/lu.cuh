@@ -17,7 +17,18 @@ struct LuTiming {
   int graph = 0;             // 1: the steps ran as one captured CUDA graph
   int tile_steps[3] = {0, 0, 0};  // complex64: steps whose update used column tiles of 32, 64, 128
 };
-void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* t = nullptr);
+// Device workspace of the complex128 factorization (256-byte aligned); lu_z_pool_bytes
+// bytes hold all matrices of the call up to `most` bytes, and at least the
+// largest.  An empty pool, or one too small for the largest matrix, is allowed:
+// the updates then run on the FP64 pipe.
+struct LuPool {
+  void* p = nullptr;
+  size_t bytes = 0;
+};
+size_t lu_z_pool_bytes(const int* n, int count, size_t most);
+// tc_err (device int, may be null) is set if a bounded wait gives up.
+void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* t, int* tc_err,
+                       const LuPool& pool);
 // The same factorization in complex64 (mixed-precision path).
 // The trailing updates run on tensor cores (tcgen05, split-BF16); ws is a
 // device workspace of lu_c64_workspace_bytes(n, batch) bytes (256-byte
@@ -28,9 +39,9 @@ void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStr
                            void* ws, int tile = 0);
 
 // One matrix of a (possibly ragged) batched factorization: A is n x n
-// column-major (complex128 or complex64), piv [n], info [1]; ws (complex64
-// only) is its own lu_c64_workspace_bytes(n, 1)-byte workspace, 16-byte
-// aligned.
+// column-major (complex128 or complex64), piv [n], info [1]; ws is its own
+// lu_c64_workspace_bytes(n, 1)-byte workspace, 16-byte aligned, for complex64
+// (complex128: assigned from the call's pool).
 struct LuMat {
   void* A;
   int* piv;
@@ -44,7 +55,7 @@ struct LuMat {
 // captured into a CUDA graph and launched once on s.  Returns the first CUDA
 // error (cudaSuccess when every launch was issued).
 cudaError_t lu_factor_many(const LuMat* items, int count, bool c64, cudaStream_t s, LuTiming* t, int* tc_err,
-                           int tile, bool graph);
+                           int tile, bool graph, const LuPool& pool);
 // The autotuner's decisions so far: per entry the upper end of its trailing-size
 // bucket, of its matrix-count bucket, the tile chosen and the measured ms per
 // matrix of tiles 32, 64, 128 (ms[3k..3k+2]); returns the number of entries.

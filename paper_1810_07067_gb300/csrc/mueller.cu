@@ -839,6 +839,12 @@ static size_t support_tc_scratch_bytes(int N, int nphi, int M) {
          ozaki_real_b_elems(Ms, nkt) * 2 + (size_t)N * NEAR_SLOTS * 4 + 64;
 }
 
+// Scratch of one body's assembly (spectra, digit rows and products at n_phi = 512).
+static size_t assembly_scratch_bytes(int N, int M) {
+  return (size_t)N * NEAR_SLOTS * NFAM * (size_t)(M + 2) * sizeof(cd) +
+         std::max(support_tc_scratch_bytes(N, 512, M), far_tc_scratch_bytes(N, 512, M));
+}
+
 // Support spectra: on the tensor cores (sampling, digit rows, one real product
 // per chunk of pairs, spectra) when the half grid fits one exact product
 // (n_phi / 2 + 1 <= OZR_KMAX samples), else the warp-per-pair kernel.
@@ -1138,6 +1144,22 @@ static int build_finish(mueller_ctx* c, const LuTiming& lt, double ms_lu, int wa
   return MUELLER_OK;
 }
 
+// Workspace of a complex128 factorization: what all matrices need, up to `most`
+// bytes, else what the largest needs, else none (the FP64 pipe).
+static LuPool lu_z_pool(DevBuf& buf, const std::vector<int>& n, size_t most) {
+  for (size_t cap : {most, (size_t)0}) {
+    LuPool pool;
+    pool.bytes = lu_z_pool_bytes(n.data(), (int)n.size(), cap);
+    unsigned char* p = nullptr;
+    if (buf.alloc(&p, pool.bytes) == cudaSuccess) {
+      pool.p = p;
+      return pool;
+    }
+    cudaGetLastError();
+  }
+  return LuPool{};
+}
+
 // The (mode) matrices of one body as LU table entries; ws_base: the body's
 // complex64 workspace (lu_c64_workspace_bytes(n, M + 1) bytes) or null.
 static void lu_items_of(mueller_ctx* c, unsigned char* ws_base, std::vector<LuMat>& items) {
@@ -1178,7 +1200,9 @@ extern "C" int mueller_build(const mueller_curve* curve, const mueller_media* me
     }
     lu_factor_batched_c64(c->A32, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, ws, c->lu_tile);
   } else {
-    lu_factor_batched(c->A, (int)n, M + 1, c->piv, c->info, s, &lt);
+    const std::vector<int> ns(M + 1, (int)n);
+    const LuPool pool = lu_z_pool(wsb, ns, assembly_scratch_bytes(c->S.N, M));
+    lu_factor_batched(c->A, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, pool);
   }
   cudaEventRecord(e2, s);
   cudaError_t err = cudaStreamSynchronize(s);
@@ -1224,13 +1248,23 @@ extern "C" int mueller_build_many(int count, const mueller_curve* curves, const 
       return drop(fail(MUELLER_ENOMEM, "tensor-core LU workspace"));
     lu_items_of(cs[i], ws, items);
   }
+  LuPool pool;
+  if (!mixed) {
+    std::vector<int> ns;
+    size_t most = 0;  // the wave's estimate (mueller_build_many_bytes) holds one body's assembly scratch
+    for (int i = 0; i < count; ++i) {
+      ns.insert(ns.end(), M[i] + 1, cs[i]->S.n);
+      most = std::max(most, assembly_scratch_bytes(cs[i]->S.N, M[i]));
+    }
+    pool = lu_z_pool(wsb, ns, most);
+  }
   // one table entry per (body, mode); a body's timeout flag is shared by the wave
   LuTiming lt;
   cudaEvent_t e1, e2;
   cudaEventCreate(&e1); cudaEventCreate(&e2);
   cudaEventRecord(e1, s);
   cudaError_t err = lu_factor_many(items.data(), (int)items.size(), mixed, s, &lt, cs[0]->tc_err,
-                                   opts->lu_tile, true);
+                                   opts->lu_tile, true, pool);
   cudaEventRecord(e2, s);
   cudaError_t err2 = cudaStreamSynchronize(s);
   float b = 0;
@@ -1616,9 +1650,18 @@ extern "C" int mueller_modal_kernels(const double* pairs_host, long long npairs,
 extern "C" int mueller_lu_batched(mueller_c128* A_dev, int n, int batch, int* piv_dev, int* info_dev, void* stream) {
   g_err.clear();
   if (!A_dev || !piv_dev || !info_dev || n < 1 || batch < 1) return fail(MUELLER_EINVAL, "invalid LU arguments");
-  lu_factor_batched((cd*)A_dev, n, batch, piv_dev, info_dev, (cudaStream_t)stream);
+  cudaStream_t s = (cudaStream_t)stream;
+  DevBuf tmp;
+  int* err = nullptr;
+  if (tmp.alloc(&err, 1) != cudaSuccess) return fail(MUELLER_ENOMEM, "LU status word");
+  CK(cudaMemsetAsync(err, 0, sizeof(int), s));
+  const LuPool pool = lu_z_pool(tmp, std::vector<int>(batch, n), (size_t)4 << 30);
+  lu_factor_batched((cd*)A_dev, n, batch, piv_dev, info_dev, s, nullptr, err, pool);
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize((cudaStream_t)stream));
+  int herr = 0;
+  CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (herr) return fail(MUELLER_ETIMEOUT, "a device-side wait of the tensor-core LU update timed out");
   return MUELLER_OK;
 }
 
@@ -1650,8 +1693,7 @@ extern "C" size_t mueller_build_bytes(int N, int M, int precision, size_t* resid
   const size_t A32 = precision != 0 ? modes * n * n * sizeof(cf) : 0;
   const size_t sl = precision == 1 ? ozaki_matrix_slices_elems((int)npad, (int)modes) * 2 + modes * npad * 8 : 0;
   const size_t small = modes * n * 4 + modes * 16 + (size_t)N * 64;
-  const size_t scratch = (size_t)N * NEAR_SLOTS * NFAM * (size_t)(M + 2) * sizeof(cd) +
-                        std::max(support_tc_scratch_bytes(N, 512, M), far_tc_scratch_bytes(N, 512, M));
+  const size_t scratch = assembly_scratch_bytes(N, M);  // also bounds the FP64 LU's workspace (lu_z_pool)
   if (resident) *resident = (precision == 1 ? 0 : A) + A32 + sl + small;
   return A + A32 + sl + small + scratch;
 }

@@ -104,6 +104,23 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Four groups of 8 consecutive 32-bit TMEM columns of this warp's 32 lanes ->
+// registers, one wait for all (in the same statement: the values exist only
+// after it).
+__device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3, float (&v)[4][8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=&f"(v[0][0]), "=&f"(v[0][1]), "=&f"(v[0][2]), "=&f"(v[0][3]), "=&f"(v[0][4]), "=&f"(v[0][5]), "=&f"(v[0][6]), "=&f"(v[0][7]),
+        "=&f"(v[1][0]), "=&f"(v[1][1]), "=&f"(v[1][2]), "=&f"(v[1][3]), "=&f"(v[1][4]), "=&f"(v[1][5]), "=&f"(v[1][6]), "=&f"(v[1][7]),
+        "=&f"(v[2][0]), "=&f"(v[2][1]), "=&f"(v[2][2]), "=&f"(v[2][3]), "=&f"(v[2][4]), "=&f"(v[2][5]), "=&f"(v[2][6]), "=&f"(v[2][7]),
+        "=&f"(v[3][0]), "=&f"(v[3][1]), "=&f"(v[3][2]), "=&f"(v[3][3]), "=&f"(v[3][4]), "=&f"(v[3][5]), "=&f"(v[3][6]), "=&f"(v[3][7])
+      : "r"(t0), "r"(t1), "r"(t2), "r"(t3));
+}
+
 // 16 consecutive 32-bit TMEM columns of this warp's 32 lanes -> registers.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
