@@ -93,3 +93,28 @@ __host__ __device__ __forceinline__ void digits28(long long F, int* d) {
   d[0] = hi;
 }
 
+// V 2^E rounded to nearest even, in integer arithmetic (a 64-bit conversion
+// would take the FP64 pipe).
+__host__ __device__ __forceinline__ double fixed_to_double(long long V, int E) {
+  const unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
+  if (u == 0) return 0.0;
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)u);
+#else
+  const int lz = __builtin_clzll(u);
+#endif
+  const unsigned long long t = u << lz;
+  unsigned long long m = t >> 11;
+  const unsigned r = (unsigned)t & 0x7FFu;
+  m += (r > 0x400u || (r == 0x400u && (m & 1ull))) ? 1ull : 0ull;
+  const int ex = 1023 + 63 - lz + E;  // exponent field; m carries the hidden bit
+  if (ex < 1 || ex > 2045) return ldexp((double)V, E);
+  const unsigned long long b = (((unsigned long long)(ex - 1) << 52) + m) | (V < 0 ? 0x8000000000000000ull : 0ull);
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double d;
+  memcpy(&d, &b, sizeof d);
+  return d;
+#endif
+}

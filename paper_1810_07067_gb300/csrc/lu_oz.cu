@@ -105,22 +105,6 @@ __device__ __forceinline__ int z_grade(unsigned high) {
   return (x == 0 || x >= 0x7FF) ? 0 : x - 1023;
 }
 
-// V 2^E rounded to nearest even, on the integer pipe.
-__device__ __forceinline__ double z_to_double(long long V, int E) {
-  const unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
-  if (E >= Z_NAN / 2) return __longlong_as_double(0x7FF8000000000000ll);
-  if (u == 0) return 0.0;
-  const int lz = __clzll((long long)u);
-  const unsigned long long t = u << lz;
-  unsigned long long m = t >> 11;
-  const unsigned r = (unsigned)t & 0x7FFu;
-  m += (r > 0x400u || (r == 0x400u && (m & 1ull))) ? 1ull : 0ull;
-  const int ex = 1023 + 63 - lz + E;  // exponent field; m carries the hidden bit
-  if (ex < 1 || ex > 2045) return ldexp((double)V, E);
-  const unsigned long long b = ((unsigned long long)(ex - 1) << 52) + m;
-  return __longlong_as_double((long long)(V < 0 ? b | 0x8000000000000000ull : b));
-}
-
 // ---------------------------------------------------------------- slicing
 // Grading exponents sE[k] of the K rows k0.. : from the columns [c0, c1) of the
 // matrix, or from maxima already formed (dmax).  All threads.
@@ -452,7 +436,8 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
           const long long lo = (long long)(__float2int_rn(v[0][c]) * 128 + __float2int_rn(v[1][c])) * 16384 +
                                (__float2int_rn(v[2][c]) * 128 + __float2int_rn(v[3][c]));
           const long long V = hi[h][c] * 524288 + ((lo + 256) >> 9);
-          const double d = z_to_double(V, Er + w.colE[jt + c]);
+          const int E = Er + w.colE[jt + c];
+          const double d = E >= Z_NAN / 2 ? nan("") : fixed_to_double(V, E);
           if (h == 0) cv[c].x -= d;
           else cv[c].y -= d;
         }

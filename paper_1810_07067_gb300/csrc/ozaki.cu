@@ -11,7 +11,10 @@
 // part is below 2^-68 of |a||y| per term).  Tensor memory holds one FP32
 // accumulator per level, [Re | Im] side by side (8 x 2 jt columns, jt the job
 // tile of 16 or 32 right-hand-side columns); every 256 values of k they are
-// drained into FP64 registers.  The complex product takes two MMAs per digit
+// drained: the levels joined in 64-bit integers, converted on the integer pipe and
+// added in FP64 once per value (a conversion and a multiply-add per level on the
+// FP64 pipe took longer than the products: N = 512, M = 64, 192 vectors per mode,
+// 24.7 -> 15.0 ms a residual).  The complex product takes two MMAs per digit
 // pair: the B operand stacks the digits of Re y over those of Im y (2 jt
 // rows), so Re a [Re y | Im y] + Im a [-Im y | Re y] lands in [Re | Im] of the
 // accumulator; the y slices are stored as [-Im, Re, Im] per digit, and the
@@ -191,7 +194,8 @@ static_assert(OzShape<16>::NACC * OzShape<16>::SET_COLS <= 512 && OzShape<OZ_JT>
               "accumulator sets exceed tensor memory");
 static_assert(OzShape<OZ_JT>::SMEM <= 227 * 1024, "stages exceed shared memory");
 
-// CTA per (row tile, mode, job tile of JT columns).  Every wait is bounded:
+// CTA per (job tile of JT columns, row tile, mode): the job tiles of a row tile run
+// together and share its digits in L2.  Every wait is bounded:
 // a role that gives up sets the CTA's failure flag (and *err), the others
 // stop at their next wait, and before the CTA exits the copy thread lets its
 // copies in flight land and the MMA thread waits for its MMAs.
@@ -208,7 +212,7 @@ __global__ void __launch_bounds__(192, 1)
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail;
   volatile int* fail = &s_fail;
-  const int rt = blockIdx.x, m = blockIdx.y, jt = blockIdx.z;
+  const int jt = blockIdx.x, rt = blockIdx.y, m = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nrt = npad / OZ_RT, nkt = npad / OZ_KT;
   const int nchunk = (nkt + OZ_CHUNK - 1) / OZ_CHUNK;
@@ -293,19 +297,26 @@ __global__ void __launch_bounds__(192, 1)
       if (!tc::mbar_wait(&tfull[set], (c / NACC) & 1)) { *fail = 1; break; }
       tc::fence_after();
       const uint32_t tw = tmem + (uint32_t)set * S::SET_COLS + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-      for (int l = 0; l < OZ_S; ++l) {
-        const double sc = ldexp(1.0, -7 * (l + 2));
+      // the chunk's levels joined in integers (units of 2^-55, below 2^63), one FP64
+      // addition per value
 #pragma unroll
-        for (int h = 0; h < 2 * JT; h += 32) {  // 32 columns per load: [Re | Im] of JT = 16, half of it for JT = 32
-          float v[32];
-          tc::tmem_ld32(tw + (uint32_t)(l * 2 * JT + h), v);
+      for (int h = 0; h < 2 * JT; h += 8) {
+        float v[4][8];
+        tc::tmem_ld8x4(tw + h, tw + 2 * JT + h, tw + 4 * JT + h, tw + 6 * JT + h, v);
+        long long hi[8];
 #pragma unroll
-          for (int u = 0; u < 32; ++u) {
-            const int col = h + u;
-            if (col < JT) zre[col] = fma(sc, (double)v[u], zre[col]);
-            else zim[col - JT] = fma(sc, (double)v[u], zim[col - JT]);
-          }
+        for (int u = 0; u < 8; ++u)
+          hi[u] = (long long)(__float2int_rn(v[0][u]) * 128 + __float2int_rn(v[1][u])) * 16384 +
+                  (__float2int_rn(v[2][u]) * 128 + __float2int_rn(v[3][u]));
+        tc::tmem_ld8x4(tw + 8 * JT + h, tw + 10 * JT + h, tw + 12 * JT + h, tw + 14 * JT + h, v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const long long lo = (long long)(__float2int_rn(v[0][u]) * 128 + __float2int_rn(v[1][u])) * 16384 +
+                               (__float2int_rn(v[2][u]) * 128 + __float2int_rn(v[3][u]));
+          const double d = fixed_to_double(hi[u] * 1048576 + ((lo + 128) >> 8), -55);
+          const int col = h + u;
+          if (col < JT) zre[col] += d;
+          else zim[col - JT] += d;
         }
       }
       tc::fence_before();
@@ -356,7 +367,7 @@ static void oz_residual_launch(const __nv_bfloat16* Asl, const double* rowscale,
                                const double* colscale, int* err, cudaStream_t s) {
   using S = OzShape<JT>;
   cudaFuncSetAttribute(oz_residual_kernel<JT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
-  oz_residual_kernel<JT><<<dim3(npad / OZ_RT, M + 1, njt), S::THREADS, S::SMEM, s>>>(
+  oz_residual_kernel<JT><<<dim3(njt, npad / OZ_RT, M + 1), S::THREADS, S::SMEM, s>>>(
       Asl, rowscale, Ysl, colscale, n, npad, M, nrhs, njt, bw, r, rnorm, err);
 }
 
