@@ -1402,325 +1402,3 @@ void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStr
                   (__nv_bfloat16*)ws + tcu_ws_matrix_elems(n) * b, n, 0};
   lu_factor_impl<cf>(it.data(), batch, s, tm, tc_err, tile, false, LuPool{});
 }
-
-// ---------------------------------------------------------------- solves
-// Blocked forward/back substitution.  One CTA per (factor m, group of SG
-// right-hand sides); a job is (rhs index, sign) with sign - meaning mode -m.
-// The solution vectors are formed in place in x (each job owns its slot).
-// Per block of SB rows: the SB x SB diagonal triangle is solved in shared
-// memory, then the rows below (above, for U) are updated with the block column
-// of the factor, which is read once per CTA.
-#define SB 64
-#define SG 8
-__device__ __forceinline__ void job_of(int m, int M, int nrhs, int job, int* q, int* ridx, bool* neg) {
-  *ridx = job % nrhs;
-  *neg = job >= nrhs;
-  *q = *neg ? (M - m) : (M + m);
-}
-
-template <class T> __device__ __forceinline__ T conv(cd a);
-template <> __device__ __forceinline__ cd conv<cd>(cd a) { return a; }
-template <> __device__ __forceinline__ cf conv<cf>(cd a) { return to_cf(a); }
-__device__ __forceinline__ cd to_cd(cd a) { return a; }
-
-// TF: factor type (cd, or cf for the mixed path's correction solves, which
-// then run in FP32 arithmetic on FP64 storage).  PHYS: right-hand sides and
-// solutions in physical unknowns (scaled by the sqrt weights here); otherwise
-// both are already in the weighted space.
-//
-// Schedule of one pass (forward shown; the backward pass mirrors it): with
-// block i solved (its x in Xs[i & 1]), threads 0..63 update the rows of block
-// i+1 with block i's factor column, then warp 0 solves block i+1's diagonal
-// triangle in registers (rows lane and lane + 32, broadcast by shuffles),
-// while the other threads load the diagonal block i+2 into shared memory and
-// update every row beyond block i+1 (a streaming product, eight factor
-// columns in flight per thread): the triangle is off the critical path.
-template <int SGT> struct SolveShape { static constexpr int NT = SGT <= 4 ? 512 : 256; };
-
-template <class T> __device__ __forceinline__ T shfl_c(T v, int src) {
-  T r;
-  r.x = __shfl_sync(0xffffffffu, v.x, src);
-  r.y = __shfl_sync(0xffffffffu, v.y, src);
-  return r;
-}
-
-// Warp 0: the diagonal triangle of the block at rows kb.. (bs rows) for all
-// G jobs, JC at a time (2 under the 64-register cap of 1024-thread CTAs);
-// unit lower (FWD) or upper with its diagonal.  The solution goes to Xo
-// (shared, for the block's column product) and to X.
-template <class TF, int SGT, bool FWD, int JC = (SolveShape<SGT>::NT >= 1024 ? 2 : 4)>
-__device__ __forceinline__ void warp_triangle(const TF (*Lb)[SB + 1], TF (*Xo)[SGT], cd* const* X, int kb, int bs,
-                                              int G, int lane) {
-  for (int g0 = 0; g0 < G; g0 += JC) {
-    TF xv[2][JC];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int r = lane + 32 * s;
-#pragma unroll
-      for (int gg = 0; gg < JC; ++gg)
-        xv[s][gg] = (r < bs && g0 + gg < G) ? conv<TF>(X[g0 + gg][kb + r]) : czero<TF>();
-    }
-    if (FWD) {
-      for (int c = 0; c < bs - 1; ++c) {
-        const int owner = c & 31;
-        TF xc[JC];
-#pragma unroll
-        for (int gg = 0; gg < JC; ++gg) xc[gg] = shfl_c(c < 32 ? xv[0][gg] : xv[1][gg], owner);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int r = lane + 32 * s;
-          if (r > c && r < bs) {
-            const TF l = Lb[r][c];
-#pragma unroll
-            for (int gg = 0; gg < JC; ++gg) xv[s][gg] = xv[s][gg] - l * xc[gg];
-          }
-        }
-      }
-    } else {
-      for (int c = bs - 1; c >= 0; --c) {
-        const int owner = c & 31, slot = c >> 5;
-        const TF d = Lb[c][c];
-        TF xc[JC];
-#pragma unroll
-        for (int gg = 0; gg < JC; ++gg) xc[gg] = shfl_c(slot ? xv[1][gg] : xv[0][gg], owner) / d;
-        if (lane == owner) {
-#pragma unroll
-          for (int gg = 0; gg < JC; ++gg) {
-            if (slot) xv[1][gg] = xc[gg];
-            else xv[0][gg] = xc[gg];
-          }
-        }
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int r = lane + 32 * s;
-          if (r < c) {
-            const TF u = Lb[r][c];
-#pragma unroll
-            for (int gg = 0; gg < JC; ++gg) xv[s][gg] = xv[s][gg] - u * xc[gg];
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int r = lane + 32 * s;
-#pragma unroll
-      for (int gg = 0; gg < JC; ++gg)
-        if (r < bs && g0 + gg < G) {
-          Xo[r][g0 + gg] = xv[s][gg];
-          X[g0 + gg][kb + r] = to_cd(xv[s][gg]);
-        }
-    }
-  }
-}
-
-// x_r -= sum_c F[r, kb + c] x_c over the bs columns of one block (x_c in Xb).
-template <class TF, int SGT>
-__device__ __forceinline__ void block_row_update(const TF* __restrict__ F, int n, int r, int kb, int bs,
-                                                 const TF (*Xb)[SGT], cd* const* X, int G) {
-  TF acc[SGT];
-#pragma unroll
-  for (int g = 0; g < SGT; ++g) acc[g] = czero<TF>();
-#pragma unroll 8
-  for (int c = 0; c < bs; ++c) {
-    const TF l = F[(size_t)(kb + c) * n + r];
-#pragma unroll
-    for (int g = 0; g < SGT; ++g) acc[g] = fma(l, Xb[c][g], acc[g]);
-  }
-#pragma unroll
-  for (int g = 0; g < SGT; ++g)
-    if (g < G) X[g][r] = X[g][r] - to_cd(acc[g]);
-}
-
-// The same for rows r and r + 1 (r even, both below the matrix's end): one
-// 16-byte load per factor column feeds both rows (more bytes in flight per
-// thread on this bandwidth-bound product).
-template <int SGT>
-__device__ __forceinline__ void block_row_update2(const cf* __restrict__ F, int n, int r, int kb, int bs,
-                                                  const cf (*Xb)[SGT], cd* const* X, int G) {
-  cf acc0[SGT], acc1[SGT];
-#pragma unroll
-  for (int g = 0; g < SGT; ++g) { acc0[g] = czero<cf>(); acc1[g] = czero<cf>(); }
-#pragma unroll 8
-  for (int c = 0; c < bs; ++c) {
-    const float4 v = __ldg((const float4*)(F + (size_t)(kb + c) * n + r));
-    const cf l0 = CF(v.x, v.y), l1 = CF(v.z, v.w);
-#pragma unroll
-    for (int g = 0; g < SGT; ++g) {
-      const cf xc = Xb[c][g];
-      acc0[g] = fma(l0, xc, acc0[g]);
-      acc1[g] = fma(l1, xc, acc1[g]);
-    }
-  }
-#pragma unroll
-  for (int g = 0; g < SGT; ++g)
-    if (g < G) {
-      X[g][r] = X[g][r] - to_cd(acc0[g]);
-      X[g][r + 1] = X[g][r + 1] - to_cd(acc1[g]);
-    }
-}
-
-// Rows [r0, r1) of the block's column product by the threads t0.. of a
-// stride: pairs of rows with 16-byte loads for complex64 factors (n even).
-template <class TF, int SGT>
-__device__ __forceinline__ void rows_update(const TF* __restrict__ F, int n, int r0, int r1, int kb, int bs,
-                                           const TF (*Xb)[SGT], cd* const* X, int G, int t0, int stride) {
-  if constexpr (std::is_same<TF, cf>::value) {
-    if ((n & 1) == 0 && (r0 & 1) == 0) {
-      for (int r = r0 + 2 * t0; r < r1; r += 2 * stride) {
-        if (r + 1 < r1) block_row_update2<SGT>(F, n, r, kb, bs, Xb, X, G);
-        else block_row_update<TF, SGT>(F, n, r, kb, bs, Xb, X, G);
-      }
-      return;
-    }
-  }
-  for (int r = r0 + t0; r < r1; r += stride) block_row_update<TF, SGT>(F, n, r, kb, bs, Xb, X, G);
-}
-
-template <class TF, int SGT>
-__host__ __device__ constexpr size_t solve_smem_fixed() {
-  return 2 * (size_t)SB * (SB + 1) * sizeof(TF) + 2 * (size_t)SB * SGT * sizeof(TF);
-}
-
-template <class TF, bool PHYS, int SGT>
-__global__ void __launch_bounds__(SolveShape<SGT>::NT) solve_blocked_kernel(
-    const TF* __restrict__ LU, const int* __restrict__ piv, int n, int M, const double* __restrict__ sw,
-    const cd* __restrict__ rhs, cd* __restrict__ x, int nrhs) {
-  extern __shared__ __align__(16) unsigned char sraw[];
-  TF (*Ls)[SB][SB + 1] = (TF (*)[SB][SB + 1])sraw;                                   // [2] diagonal blocks
-  TF (*Xs)[SB][SGT] = (TF (*)[SB][SGT])(sraw + 2 * (size_t)SB * (SB + 1) * sizeof(TF));  // [2] block solutions
-  int* perm = (int*)(sraw + solve_smem_fixed<TF, SGT>());  // [n] composed interchanges, then pv_s [n]
-  const int m = blockIdx.x;
-  const int job0 = blockIdx.y * SGT;
-  const int njobs_all = (m == 0) ? nrhs : 2 * nrhs;
-  if (job0 >= njobs_all) return;
-  const int G = min(SGT, njobs_all - job0);
-  const TF* L = LU + (size_t)m * n * n;
-  const int* pv = piv + (size_t)m * n;
-  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
-  cd* X[SGT];
-  for (int g = 0; g < SGT; ++g) {
-    int q, ri; bool neg;
-    job_of(m, M, nrhs, job0 + (g < G ? g : 0), &q, &ri, &neg);
-    X[g] = x + ((size_t)q * nrhs + ri) * n;
-  }
-  // row interchanges (LAPACK order) composed into perm: (P b)[r] = b[perm[r]]
-  int* pv_s = perm + n;  // the pivots staged in shared memory for the serial composition
-  for (int r = tid; r < n; r += T) { perm[r] = r; pv_s[r] = pv[r]; }
-  __syncthreads();
-  if (tid == 0) {
-    for (int k = 0; k < n; ++k) {
-      int p = pv_s[k];
-      if (p != k) { int t = perm[k]; perm[k] = perm[p]; perm[p] = t; }
-    }
-  }
-  __syncthreads();
-  // permuted, scaled (sqrt weights per node) and reflected right-hand sides
-  for (int t = tid; t < G * n; t += T) {
-    int g = t / n, r = t % n;
-    int q, ri; bool neg;
-    job_of(m, M, nrhs, job0 + g, &q, &ri, &neg);
-    int src = perm[r];
-    double sg = (neg && ((src & 3) == 0 || (src & 3) == 3)) ? -1.0 : 1.0;
-    X[g][r] = ((PHYS ? sw[src >> 2] : 1.0) * sg) * rhs[((size_t)q * nrhs + ri) * n + src];
-  }
-  const int nblk = (n + SB - 1) / SB;
-  auto load_diag = [&](int bi, int t0, int step) {
-    const int kb = bi * SB, bs = min(SB, n - kb);
-    TF (*D)[SB + 1] = Ls[bi & 1];
-    for (int t = t0; t < bs * bs; t += step) {
-      const int r = t % bs, c = t / bs;
-      D[r][c] = L[(size_t)(kb + c) * n + kb + r];
-    }
-  };
-  // forward: L unit lower
-  load_diag(0, tid, T);
-  if (nblk > 1) load_diag(1, tid, T);
-  __syncthreads();
-  if (tid < 32) warp_triangle<TF, SGT, true>(Ls[0], Xs[0], X, 0, min(SB, n), G, lane);
-  __syncthreads();
-  for (int i = 0; i < nblk; ++i) {
-    const int kb = i * SB, bs = min(SB, n - kb), b = i & 1;
-    const int kn = kb + SB, bsn = min(SB, n - kn);
-    if (tid < 64) {
-      if (bsn > 0) {
-        if (tid < bsn) block_row_update<TF, SGT>(L, n, kn + tid, kb, bs, Xs[b], X, G);
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (tid < 32) warp_triangle<TF, SGT, true>(Ls[b ^ 1], Xs[b ^ 1], X, kn, bsn, G, lane);
-      }
-    } else {
-      if (i + 2 < nblk) load_diag(i + 2, tid - 64, T - 64);
-      rows_update<TF, SGT>(L, n, kn + SB, n, kb, bs, Xs[b], X, G, tid - 64, T - 64);
-    }
-    __syncthreads();
-  }
-  // backward: U upper, non-unit diagonal
-  const int last = nblk - 1;
-  load_diag(last, tid, T);
-  if (last >= 1) load_diag(last - 1, tid, T);
-  __syncthreads();
-  if (tid < 32) warp_triangle<TF, SGT, false>(Ls[last & 1], Xs[last & 1], X, last * SB, n - last * SB, G, lane);
-  __syncthreads();
-  for (int i = last; i >= 0; --i) {
-    const int kb = i * SB, bs = min(SB, n - kb), b = i & 1;
-    const int kp = kb - SB;  // the block above (full size)
-    if (tid < 64) {
-      if (i >= 1) {
-        block_row_update<TF, SGT>(L, n, kp + tid, kb, bs, Xs[b], X, G);
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (tid < 32) warp_triangle<TF, SGT, false>(Ls[b ^ 1], Xs[b ^ 1], X, kp, SB, G, lane);
-      }
-    } else {
-      if (i - 2 >= 0) load_diag(i - 2, tid - 64, T - 64);
-      rows_update<TF, SGT>(L, n, 0, kp, kb, bs, Xs[b], X, G, tid - 64, T - 64);
-    }
-    __syncthreads();
-  }
-  // back to physical unknowns (and reflection for -m)
-  for (int t = tid; t < G * n; t += T) {
-    int g = t / n, r = t % n;
-    int q, ri; bool neg;
-    job_of(m, M, nrhs, job0 + g, &q, &ri, &neg);
-    double sg = (neg && ((r & 3) == 1 || (r & 3) == 2)) ? -1.0 : 1.0;
-    X[g][r] = (sg / (PHYS ? sw[r >> 2] : 1.0)) * X[g][r];
-  }
-}
-
-// Vectors per CTA: 32 when that still leaves two CTAs per SM (many
-// right-hand sides: every group reads the whole factor, so wider groups read
-// it fewer times), else 8 when that leaves four, else 4 (more CTAs hide the
-// latency of the per-block triangle steps; measured on the cylinder's 65
-// modes x 32 vectors: 4 vectors 53 ms, 8 vectors 63 ms, 2 vectors 75 ms for
-// the three correction solves with residuals, with 256 threads per CTA).
-template <class TF, bool PHYS, int W>
-static void launch_solve_w(const TF* LU, const int* piv, int n, int M, const double* sw, const cd* rhs, cd* x, int nrhs,
-                           int smem_perm, cudaStream_t s) {
-  const int groups = (2 * nrhs + W - 1) / W;
-  const int smem = (int)solve_smem_fixed<TF, W>() + smem_perm;
-  smem_optin(solve_blocked_kernel<TF, PHYS, W>);
-  solve_blocked_kernel<TF, PHYS, W><<<dim3(M + 1, groups), SolveShape<W>::NT, smem, s>>>(LU, piv, n, M, sw, rhs, x,
-                                                                                          nrhs);
-}
-
-template <class TF, bool PHYS>
-static void launch_solve_blocked(const TF* LU, const int* piv, int n, int M, const double* sw, const cd* rhs, cd* x,
-                                 int nrhs, cudaStream_t s) {
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int smem = 2 * n * (int)sizeof(int);
-  const long long modes = M + 1;
-  if (modes * ((2 * nrhs + 31) / 32) >= 2LL * sms) launch_solve_w<TF, PHYS, 32>(LU, piv, n, M, sw, rhs, x, nrhs, smem, s);
-  else if (modes * ((2 * nrhs + SG - 1) / SG) >= 4LL * sms) launch_solve_w<TF, PHYS, SG>(LU, piv, n, M, sw, rhs, x, nrhs, smem, s);
-  else launch_solve_w<TF, PHYS, 4>(LU, piv, n, M, sw, rhs, x, nrhs, smem, s);
-}
-
-void lu_solve_modes(const cd* LU, const int* piv, int n, int M, const double* sw, const cd* rhs, cd* x, int nrhs,
-                    cudaStream_t s) {
-  launch_solve_blocked<cd, true>(LU, piv, n, M, sw, rhs, x, nrhs, s);
-}
-
-void lu_correction_solve_c64(const cf* LU, const int* piv, int n, int M, const cd* r, cd* d, int nrhs,
-                             cudaStream_t s) {
-  launch_solve_blocked<cf, false>(LU, piv, n, M, nullptr, r, d, nrhs, s);
-}

@@ -61,18 +61,26 @@ cudaError_t lu_factor_many(const LuMat* items, int count, bool c64, cudaStream_t
 // matrix of tiles 32, 64, 128 (ms[3k..3k+2]); returns the number of entries.
 int lu_tile_table(int* rest_hi, int* count_hi, int* tile, float* ms, int cap);
 
+// Triangular solves (solve.cu; n a multiple of 64).  scratch: lu_solve_scratch_bytes
+// device bytes, 256-byte aligned, prepared once per factorization and nrhs by
+// lu_solve_prepare (the composed row interchanges); each solve makes
+// lu_solve_launches(n) launches.
+size_t lu_solve_scratch_bytes(int n, int M, int nrhs, bool c64);
+int lu_solve_launches(int n);
+void lu_solve_prepare(const int* piv, int n, int M, void* scratch, cudaStream_t s);
+
 // Solve with factors of modes m = 0..M for right-hand sides of modes -M..M:
 // rhs/x layout [2M+1][nrhs][n] (mode q = m + M); sw[n/4] = sqrt of the L2 weights of the nodes
 // (rows scaled by sw, unknowns by 1/sw inside the factors); negative modes use
 // the reflection A_{-m} = D_r A_m D_c with D_r = (-1,1,1,-1), D_c = (1,-1,-1,1)
 // per node.
-void lu_solve_modes(const cd* LU, const int* piv, int n, int M, const double* sw, const cd* rhs, cd* x, int nrhs,
+void lu_solve_modes(const cd* LU, int n, int M, const double* sw, const cd* rhs, cd* x, int nrhs, void* scratch,
                     cudaStream_t s);
 
 // Mixed path: d = A'^{-1} r with the complex64 factors of modes 0..M in FP32
 // arithmetic, in the L2-weighted space (no sqrt-weight scaling), for all modes
 // -M..M (layout [2M+1][nrhs][n], -m by reflection).
-void lu_correction_solve_c64(const cf* LU, const int* piv, int n, int M, const cd* r, cd* d, int nrhs,
+void lu_correction_solve_c64(const cf* LU, int n, int M, const cd* r, cd* d, int nrhs, void* scratch,
                              cudaStream_t s);
 
 // Held by a thread while it captures the LU's launches into a CUDA graph;

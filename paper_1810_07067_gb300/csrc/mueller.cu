@@ -1310,12 +1310,14 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
   const int ojt = ozaki_job_tile(nrhs), njt = ozaki_job_tiles(nrhs);
   DevBuf tmp;
   cd *bw, *y, *r, *d;
+  unsigned char* sol;  // lu_solve_prepare
   double* norms;  // [3][nvec]: b', y, r
   __nv_bfloat16* Ysl = nullptr;
   double* colscale = nullptr;
   int* derr = nullptr;
   if (tmp.alloc(&bw, (size_t)nvec * n) || tmp.alloc(&y, (size_t)nvec * n) || tmp.alloc(&r, (size_t)nvec * n) ||
       tmp.alloc(&d, (size_t)nvec * n) || tmp.alloc(&norms, (size_t)3 * nvec) ||
+      tmp.alloc(&sol, lu_solve_scratch_bytes(n, M, nrhs, true)) ||
       (tcres && (tmp.alloc(&Ysl, ozaki_vector_slices_elems(c->npad, M + 1, njt, ojt)) ||
                  tmp.alloc(&colscale, (size_t)(M + 1) * njt * ojt) || tmp.alloc(&derr, 1))))
     return fail(MUELLER_ENOMEM, "refinement work vectors");
@@ -1327,9 +1329,10 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
   cudaEventCreate(&e0); cudaEventCreate(&e1);
   cudaEventRecord(e0, s);
   mixed_scale(rhs, bw, c->geo[5], n, nvec, bn, s);
-  lu_correction_solve_c64(c->A32, c->piv, n, M, bw, d, nrhs, s);
+  lu_solve_prepare(c->piv, n, M, sol, s);
+  lu_correction_solve_c64(c->A32, n, M, bw, d, nrhs, sol, s);
   mixed_update(y, d, n, nvec, true, yn, s);
-  int it = 0, launches = 3;
+  int it = 0, launches = 3 + lu_solve_launches(n);
   bool done = false;
   double worst = 0.0;
   std::vector<cudaEvent_t> rev;
@@ -1356,9 +1359,9 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
       worst = std::max(worst, be[v]);
     }
     if (worst <= c->S.refine_tol) { done = true; break; }
-    lu_correction_solve_c64(c->A32, c->piv, n, M, r, d, nrhs, s);
+    lu_correction_solve_c64(c->A32, n, M, r, d, nrhs, sol, s);
     mixed_update(y, d, n, nvec, false, yn, s);
-    launches += 2;
+    launches += 1 + lu_solve_launches(n);
   }
   mixed_unscale(y, x, c->geo[5], n, nvec, s);
   cudaEventRecord(e1, s);
@@ -1403,10 +1406,15 @@ extern "C" int mueller_solve(mueller_ctx* c, const mueller_c128* rhs_dev, int nr
   if ((const void*)rhs_dev == (const void*)x_dev) return fail(MUELLER_EINVAL, "rhs and x must not alias");
   cudaStream_t s = (cudaStream_t)stream;
   if (c->S.precision != 0) return solve_mixed(c, (const cd*)rhs_dev, nrhs, (cd*)x_dev, backward_err, s);
+  DevBuf tmp;
+  unsigned char* sol;
+  if (tmp.alloc(&sol, lu_solve_scratch_bytes(c->S.n, c->S.M, nrhs, false)) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "solve scratch");
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0); cudaEventCreate(&e1);
   cudaEventRecord(e0, s);
-  lu_solve_modes(c->A, c->piv, c->S.n, c->S.M, c->geo[5], (const cd*)rhs_dev, (cd*)x_dev, nrhs, s);
+  lu_solve_prepare(c->piv, c->S.n, c->S.M, sol, s);
+  lu_solve_modes(c->A, c->S.n, c->S.M, c->geo[5], (const cd*)rhs_dev, (cd*)x_dev, nrhs, sol, s);
   cudaEventRecord(e1, s);
   cudaError_t err = cudaEventSynchronize(e1);
   float ms = 0;
@@ -1414,7 +1422,7 @@ extern "C" int mueller_solve(mueller_ctx* c, const mueller_c128* rhs_dev, int nr
   cudaEventDestroy(e0); cudaEventDestroy(e1);
   if (err != cudaSuccess) return fail(MUELLER_ECUDA, cudaGetErrorString(err));
   c->st.ms_solve = ms;
-  c->st.solve_launches = 1;
+  c->st.solve_launches = 1 + lu_solve_launches(c->S.n);
   if (backward_err)
     for (int q = 0; q < (2 * c->S.M + 1) * nrhs; ++q) backward_err[q] = -1.0;  // not computed on the FP64 path
   return MUELLER_OK;
