@@ -125,3 +125,108 @@ __host__ __device__ __forceinline__ void mueller_block_core(const V2* c1, const 
     out[3][0] = HJ_th.a; out[3][1] = HJ_th.b; out[3][2] = ap.aHM * Kth.a; out[3][3] = ap.aHM * Kth.b;
   }
 }
+
+// ---------------------------------------------------------------------------
+// The same block in two steps, for the far-pair assembly: the nine spectra of a
+// mode are first combined, with the target's constants and the media's
+// coefficients, into the 15 families the block's 16 entries are made of, once
+// per pair and mode; the block of mode m then takes sums and differences of the
+// families at m + 1 and m - 1 and their values at m.  About 80 FP64 operations
+// to combine and 100 per block, where the block from the nine spectra takes 370
+// (SIMPLE; each spectrum enters three blocks).
+// With S2 = S_2 - S_4, S3 = S_3 - S_5, D = S_0 - S_1, kg = k0^2 S_0 - k1^2 S_1,
+// gt = D / r^2, rt = S2 / r, zt = S3 / r, T = rt - gt (r, r', z' the target's):
+enum {
+  BK_KG, BK_B, BK_GT, BK_ZT,   // kg, gt + rt, gt, zt
+  BK_U, BK_V, BK_W,            // r'(S_6 + T + kg) + z'(S_7 + zt), r' T + z' zt, r' S_7 + z'(S_8 + kg)
+  BK_E,                        // cEM0 x_0 + cEM1 x_1 of x = S_dz, S_dr, z'(S_g / r + S_dr) - r' S_dz, S_g (4)
+  BK_H = BK_E + 4,             // the same with cHJ
+  BK_N = BK_H + 4
+};
+
+// S[9]: spectra of one mode; out[f * stride], f < BK_N.
+template <bool SIMPLE>
+__host__ __device__ __forceinline__ void mueller_combine(const cd* S, const AsmParams& ap, double irt, double rpt,
+                                                         double zpt, cd* out, int stride) {
+  const cd D = S[0] - S[1];
+  const cd kg = SIMPLE ? ap.k0sq.x * S[0] - ap.k1sq.x * S[1] : ap.k0sq * S[0] - ap.k1sq * S[1];
+  const cd gt = (irt * irt) * D, rt = irt * (S[2] - S[4]), zt = irt * (S[3] - S[5]);
+  const cd T = rt - gt;
+  out[BK_KG * stride] = kg;
+  out[BK_B * stride] = gt + rt;
+  out[BK_GT * stride] = gt;
+  out[BK_ZT * stride] = zt;
+  out[BK_U * stride] = rpt * ((S[6] + T) + kg) + zpt * (S[7] + zt);
+  out[BK_V * stride] = rpt * T + zpt * zt;
+  out[BK_W * stride] = rpt * S[7] + zpt * (S[8] + kg);
+  const double al = zpt * irt;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const cd c0 = h ? ap.cHJ0 : ap.cEM0, c1 = h ? ap.cHJ1 : ap.cEM1;
+    const cd g = SIMPLE ? iy(c0.y, S[0]) + iy(c1.y, S[1]) : c0 * S[0] + c1 * S[1];
+    const cd dr = SIMPLE ? iy(c0.y, S[2]) + iy(c1.y, S[4]) : c0 * S[2] + c1 * S[4];
+    const cd dz = SIMPLE ? iy(c0.y, S[3]) + iy(c1.y, S[5]) : c0 * S[3] + c1 * S[5];
+    cd* o = out + (BK_E + 4 * h) * stride;
+    o[0] = dz;
+    o[stride] = dr;
+    o[2 * stride] = al * g + zpt * dr - rpt * dz;
+    o[3 * stride] = g;
+  }
+}
+
+// |x| with the other sign, without an FP64 operation
+__host__ __device__ __forceinline__ double neg_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
+#else
+  return -x;
+#endif
+}
+__host__ __device__ __forceinline__ cd neg_bits(cd a) { return cd{neg_bits(a.x), neg_bits(a.y)}; }
+
+// The block of mode m from the families F[f * stride + mode] (F at mode 0;
+// modes m + 1 and |m - 1| are read): h0, h1, f2 the pair's weights fac[0] / 2,
+// fac[1] / 2, fac[2] (common factors of the spectra and the block may ride in
+// them), unit: aEJ = 1 and aHM = -1.
+__host__ __device__ __forceinline__ void mueller_block_combined(const cd* F, int stride, int m, const AsmParams& ap,
+                                                                bool unit, double h0, double h1, double f2,
+                                                                double irt, double rpt, double zpt, cd out[4][4]) {
+  const cd* P = F + m + 1;
+  const cd* Q = F + (m >= 1 ? m - 1 : 1);
+  const cd* Z = F + m;
+  auto sum = [&](int f) { return P[f * stride] + Q[f * stride]; };
+  auto dif = [&](int f) { return Q[f * stride] - P[f * stride]; };
+  const double dm = m, m2 = dm * dm, mf2 = dm * f2;
+  {
+    const cd sB = sum(BK_B), dB = dif(BK_B), sg = sum(BK_GT), dg = dif(BK_GT);
+    const cd a = fma(-m2, dg, fma(dm, sB, dif(BK_KG))), b = fma(-m2, sg, fma(dm, dB, sum(BK_KG)));
+    const cd z = Z[BK_ZT * stride];
+    out[0][0] = C(-(h0 * a.y + mf2 * z.y), h0 * a.x + mf2 * z.x);
+    out[0][1] = h1 * b;
+  }
+  {
+    const cd a = fma(-dm, dif(BK_V), sum(BK_U)), b = fma(-dm, sum(BK_V), dif(BK_U));
+    const cd w = Z[BK_W * stride];
+    out[1][0] = C(-(h0 * a.x + f2 * w.x), -(h0 * a.y + f2 * w.y));
+    out[1][1] = C(-h1 * b.y, h1 * b.x);
+  }
+  const double ma = dm * (zpt * irt), mz = (dm * (rpt * irt)) * f2;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {  // E rows with M columns, H rows with J columns
+    const int f = h ? BK_H : BK_E, r = 2 * h, c = 2 - 2 * h;
+    const cd s = sum(f), d = dif(f), zr = Z[(f + 1) * stride], zg = Z[(f + 3) * stride];
+    const cd a = fma(-ma, sum(f + 3), dif(f + 2)), b = fma(-ma, dif(f + 3), sum(f + 2));
+    out[r][c] = C(h0 * s.x - f2 * zr.x, h0 * s.y - f2 * zr.y);
+    out[r][c + 1] = C(h1 * d.y, -h1 * d.x);
+    out[r + 1][c] = C(h0 * a.y + mz * zg.y, -(h0 * a.x + mz * zg.x));
+    out[r + 1][c + 1] = -h1 * b;
+  }
+  const cd k00 = out[0][0], k01 = out[0][1], k10 = out[1][0], k11 = out[1][1];
+  if (unit) {
+    out[2][2] = neg_bits(k00); out[2][3] = neg_bits(k01);
+    out[3][2] = neg_bits(k10); out[3][3] = neg_bits(k11);
+  } else {
+    out[0][0] = ap.aEJ * k00; out[0][1] = ap.aEJ * k01; out[1][0] = ap.aEJ * k10; out[1][1] = ap.aEJ * k11;
+    out[2][2] = ap.aHM * k00; out[2][3] = ap.aHM * k01; out[3][2] = ap.aHM * k10; out[3][3] = ap.aHM * k11;
+  }
+}

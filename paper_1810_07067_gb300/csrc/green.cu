@@ -34,6 +34,7 @@
 #include "block.cuh"
 #include "grid.cuh"
 #include "digits.cuh"
+#include "ozaki.cuh"
 
 __constant__ SeriesTables c_tab;
 
@@ -151,10 +152,143 @@ __device__ __forceinline__ WarpSmem warp_smem(const GreenParams& gp, char* base)
 }
 
 
+// ---------------------------------------------------------------------------
+// One sample of the nine kernels (times 4 pi) at u = rho^2 = d2 + 4 r_t r_s s2,
+// s2 = sin^2(phi / 2): out[f * stride], weighted by w.
+//
+// With the functions of special.cuh (sample_*), per wavenumber
+//   E = c / rho + i k sinc,  E' = (k^2 a / 2) / rho - 1 / (2 rho^3) + i k^3 sig1 / 2,
+// the difference of E'' is (k0^4 eta0 - k1^4 eta1) / rho - g0 / (2 rho^3) + i (k0^5 sig2_0
+// - k1^5 sig2_1) / 4, g0 = -(k0^2 - k1^2) / 4, and a split pair has its band-limited
+// samples q in the place of 1 / rho with the rho^-3 parts rewritten (see the top
+// of the file).  Where both |k| rho >= 2 a pair that is not split takes E, E' and
+// E'' from exp(i k rho) directly; the difference does not cancel there.
+// K0R, K1R: real wavenumbers in real arithmetic.  FP64 pipe: about 180
+// operations a sample for two real wavenumbers (600 with the seven entire functions
+// of each wavenumber and complex products by zero parts): far pairs of the N = 1024,
+// M = 128 body 64 -> 21 ms, its support pairs 26 -> 16.5 ms, the lossy cylinder's
+// (N = 576, M = 64) 36 -> 16 and 13.6 -> 7.4 ms.
+struct PairSample {
+  double d2, rr4, dr0, rs2, zd;  // rr4 = 4 r_t r_s, rs2 = 2 r_s
+  double irt, alpha;             // split pairs
+};
+
+// k^p of a real or complex wavenumber
+template <bool R> __device__ __forceinline__ auto kval(const cd& z) {
+  if constexpr (R) return z.x;
+  else return z;
+}
+// a + i b for real or complex a, b
+__device__ __forceinline__ cd join(double a, double b) { return C(a, b); }
+__device__ __forceinline__ cd join(cd a, cd b) { return C(a.x - b.y, a.y + b.x); }
+__device__ __forceinline__ double fun_fma2(double s, double x, double c) { return fma(s, x, c); }
+__device__ __forceinline__ cd fun_fma2(double s, cd x, cd c) { return fma(s, x, c); }
+__device__ __forceinline__ double dif(double a, double b) { return a - b; }
+__device__ __forceinline__ cd dif(double a, cd b) { return C(a - b.x, -b.y); }
+__device__ __forceinline__ cd dif(cd a, cd b) { return a - b; }
+
+template <bool R>
+__device__ __forceinline__ auto sample_fun(const KPow& kp, double su, double u, double isu) {
+  if constexpr (R) {
+    const double x = kp.k.x * su;
+    if (kp.ak * su < 2.0) return sample_series<double>(c_tab, x * x);
+    double s, c;
+    sincos(x, &s, &c);
+    const double xi = kp.ik.x * isu;
+    return sample_closed<double>(s, c, xi, xi * xi);
+  } else {
+    const cd x = su * kp.k;
+    if (kp.ak * su < 2.0) return sample_series<cd>(c_tab, u * kp.k2);
+    cd s, c;
+    csincos(x, &s, &c);
+    const cd xi = isu * kp.ik;
+    return sample_closed<cd>(s, c, xi, xi * xi);
+  }
+}
+
+// E, E', E'' (times w) from exp(i k rho); isw = w / rho
+template <bool R>
+__device__ __forceinline__ void sample_direct(const KPow& kp, double su, double iu, double isw, cd* E) {
+  const double a1 = 0.5 * iu * isw, a2 = 0.5 * iu * a1;
+  if constexpr (R) {
+    const double x = kp.k.x * su;
+    double s, c;
+    sincos(x, &s, &c);
+    const double p = fma(-x, x, 3.0), x3 = 3.0 * x;
+    E[0] = C(c * isw, s * isw);
+    E[1] = C(a1 * fma(-x, s, -c), a1 * fma(x, c, -s));
+    E[2] = C(a2 * fma(p, c, x3 * s), a2 * fma(p, s, -(x3 * c)));
+  } else {
+    const cd ikr = mul_i(su * kp.k), e = cexpi(su * kp.k);
+    E[0] = isw * e;
+    E[1] = a1 * (e * (ikr - C(1.0)));
+    E[2] = a2 * (e * (ikr * ikr - 3.0 * ikr + C(3.0)));
+  }
+}
+
+template <bool K0R, bool K1R>
+__device__ __forceinline__ void pair_sample(const GreenParams& gp, const PairSample& ps, double s2, double w, bool split,
+                                            double q, cd* __restrict__ out, int stride) {
+  const double u = fma(ps.rr4, s2, ps.d2);
+  const double isu = rsqrt(u);
+  double su = u * isu;
+  su = fma(0.5 * isu, fma(-su, su, u), su);  // sqrt(u)
+  const double rd2 = 2.0 * fma(ps.rs2, s2, ps.dr0), zd2 = 2.0 * ps.zd;
+  if (!split && fmin(gp.kp0.ak, gp.kp1.ak) * su >= 2.0) {
+    const double iu = isu * isu;
+    cd E0[3], E1[3];
+    sample_direct<K0R>(gp.kp0, su, iu, w * isu, E0);
+    sample_direct<K1R>(gp.kp1, su, iu, w * isu, E1);
+    out[0] = E0[0]; out[stride] = E1[0];
+    out[2 * stride] = rd2 * E0[1]; out[3 * stride] = zd2 * E0[1];
+    out[4 * stride] = rd2 * E1[1]; out[5 * stride] = zd2 * E1[1];
+    const cd D1 = E0[1] - E1[1], D2 = E0[2] - E1[2], t1 = D1 + D1;
+    out[6 * stride] = fma(rd2 * rd2, D2, t1);
+    out[7 * stride] = (rd2 * zd2) * D2;
+    out[8 * stride] = fma(zd2 * zd2, D2, t1);
+    return;
+  }
+  const auto f0 = sample_fun<K0R>(gp.kp0, su, u, isu);
+  const auto f1 = sample_fun<K1R>(gp.kp1, su, u, isu);
+  // real-part and imaginary-part functions (complex for a complex wavenumber)
+  const auto G0 = (0.5 * kval<K0R>(gp.kp0.k2)) * f0.a;
+  const auto G1 = (0.5 * kval<K1R>(gp.kp1.k2)) * f1.a;
+  const auto P0 = (0.5 * kval<K0R>(gp.kp0.k3)) * f0.sig1;
+  const auto P1 = (0.5 * kval<K1R>(gp.kp1.k3)) * f1.sig1;
+  const auto eta = dif(kval<K0R>(gp.kp0.k4) * f0.eta, kval<K1R>(gp.kp1.k4) * f1.eta);
+  const auto dPP = dif((0.25 * kval<K0R>(gp.kp0.k5)) * f0.sig2, (0.25 * kval<K1R>(gp.kp1.k5)) * f1.sig2);
+  const auto dG = dif(G0, G1), dP = dif(P0, P1);
+  const auto g0 = kval<K0R && K1R>(gp.gamma0);
+  const double v = w * (split ? q : isu);  // weight of the 1 / rho parts
+  out[0] = join(v * f0.c, w * (kval<K0R>(gp.kp0.k) * f0.sinc));
+  out[stride] = join(v * f1.c, w * (kval<K1R>(gp.kp1.k) * f1.sinc));
+  const double wr = w * rd2, wz = w * zd2, vr = v * rd2, vz = v * zd2;
+  const auto i2 = dP + dP;
+  if (!split) {
+    const double h = 0.5 * isu * isu;  // E' = (G - h) / rho + i P
+    out[2 * stride] = join(vr * fun_add(G0, -h), wr * P0); out[3 * stride] = join(vz * fun_add(G0, -h), wz * P0);
+    out[4 * stride] = join(vr * fun_add(G1, -h), wr * P1); out[5 * stride] = join(vz * fun_add(G1, -h), wz * P1);
+    const auto d2r = eta - h * g0, r2 = dG + dG;
+    out[6 * stride] = join(v * fun_fma2(rd2 * rd2, d2r, r2), w * fun_fma2(rd2 * rd2, dPP, i2));
+    out[7 * stride] = join((vr * zd2) * d2r, (wr * zd2) * dPP);
+    out[8 * stride] = join(v * fun_fma2(zd2 * zd2, d2r, r2), w * fun_fma2(zd2 * zd2, dPP, i2));
+  } else {
+    const double h = 0.5 * ps.irt;
+    out[2 * stride] = join(v * fun_add(rd2 * G0, -h), wr * P0); out[3 * stride] = join(vz * G0, wz * P0);
+    out[4 * stride] = join(v * fun_add(rd2 * G1, -h), wr * P1); out[5 * stride] = join(vz * G1, wz * P1);
+    const auto r2 = dG + dG;
+    const double rda = fma(0.5, rd2, ps.alpha) * ps.irt, zr = ps.zd * ps.irt;
+    out[6 * stride] = join(v * (fun_fma2(rd2 * rd2, eta, r2) - rda * g0), w * fun_fma2(rd2 * rd2, dPP, i2));
+    out[7 * stride] = join(v * ((rd2 * zd2) * eta - zr * g0), (wr * zd2) * dPP);
+    out[8 * stride] = join(v * fun_fma2(zd2 * zd2, eta, r2), w * fun_fma2(zd2 * zd2, dPP, i2));
+  }
+}
+
 // The weighted samples W.smp[f][j] = w_j F_f(phi_j), j = 0..nl/2 (w = 1/2 at
 // both ends), of one pair on its grid g: the first half of warp_pair_spectra,
 // by the threads t = 0..NT-1 of a group whose barrier is sync().
-template <int NT, class Sync>
+// RR: real wavenumbers, 2 both, 1 k0 only, 0 neither, -1 decided at run time.
+template <int NT, int RR = -1, class Sync>
 __device__ __forceinline__ void group_pair_samples(const GreenParams& gp, double rt, double dr0, double zd,
                                                    long long sid, const double* __restrict__ leg, long long n_split,
                                                    const double* __restrict__ cosT, const WarpSmem& W, int t,
@@ -162,7 +296,6 @@ __device__ __forceinline__ void group_pair_samples(const GreenParams& gp, double
   const int Mq = gp.Mq, mask = gp.nphi - 1;
   const int nl = g.nl;  // local grid size; sample j sits at entry j of its tables
   const double* __restrict__ s2L = g.s2L;
-  const int tstride = 1;
   const int H = nl / 2 + 1, Q = nl / 4;  // samples on [0, pi]; fold point
   const double rs = rt - dr0;
   const double d2 = dr0 * dr0 + zd * zd;
@@ -185,76 +318,18 @@ __device__ __forceinline__ void group_pair_samples(const GreenParams& gp, double
     }
     sync();
   }
-  const cd g0 = gp.gamma0;
-  const double kmin = fmin(cabs(gp.kp0.k), cabs(gp.kp1.k));
+  PairSample ps;
+  ps.d2 = d2; ps.rr4 = 4.0 * rt * rs; ps.dr0 = dr0; ps.rs2 = 2.0 * rs; ps.zd = zd;
+  ps.irt = 1.0 / rt; ps.alpha = alpha;
   for (int j = t; j < H; j += NT) {
-    double s2 = s2L[j * tstride];
-    double u = d2 + 4.0 * rt * rs * s2;
-    double su = sqrt(u);
-    double rd = dr0 + 2.0 * rs * s2;
-    cd F[NFAM];
-    if (!split && kmin * su >= 2.0) {
-      // both |k rho| >= 2: the kernels and their u-derivatives directly from
-      // exp(i k rho), 4 pi E = e/rho, 4 pi E' = e (ik rho - 1)/(2 rho^3),
-      // 4 pi E'' = e ((ik rho)^2 - 3 ik rho + 3)/(4 rho^5); the k0 - k1
-      // difference does not cancel at these arguments.
-      double isu = 1.0 / su, iu = isu * isu;
-      cd E0[3], E1[3];
-#pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        cd ikr = mul_i(((w == 0) ? gp.kp0.k : gp.kp1.k) * su);
-        cd e = cexpi(((w == 0) ? gp.kp0.k : gp.kp1.k) * su);
-        cd* E = (w == 0) ? E0 : E1;
-        E[0] = e * isu;
-        E[1] = (0.5 * iu * isu) * (e * (ikr - C(1.0)));
-        E[2] = (0.25 * iu * iu * isu) * (e * (ikr * ikr - 3.0 * ikr + C(3.0)));
-      }
-      F[0] = E0[0]; F[1] = E1[0];
-      F[2] = (2.0 * rd) * E0[1]; F[3] = (2.0 * zd) * E0[1];
-      F[4] = (2.0 * rd) * E1[1]; F[5] = (2.0 * zd) * E1[1];
-      cd D1 = E0[1] - E1[1], D2 = E0[2] - E1[2];
-      F[6] = (4.0 * rd * rd) * D2 + 2.0 * D1;
-      F[7] = (4.0 * rd * zd) * D2;
-      F[8] = (4.0 * zd * zd) * D2 + 2.0 * D1;
-      double wj = (j == 0 || j == H - 1) ? 0.5 : 1.0;
-#pragma unroll
-      for (int f = 0; f < NFAM; ++f) W.smp[f * H + j] = wj * F[f];
-      continue;
-    }
-    Ent e0 = gp.k0_real ? entire_real(c_tab, gp.kp0.k.x, su) : entire(c_tab, gp.kp0, su);
-    Ent e1 = gp.k1_real ? entire_real(c_tab, gp.kp1.k.x, su) : entire(c_tab, gp.kp1, su);
-    cd gam1 = e0.Gam - e1.Gam, gam2 = e0.Gam2 - e1.Gam2, gam1p = e0.Gamp - e1.Gamp;
-    cd dSp = e0.Sp - e1.Sp, dSpp = e0.Spp - e1.Spp;
-    if (!split) {
-      double isu = 1.0 / su, iu3 = isu / u;
-      F[0] = e0.C * isu + mul_i(e0.S);
-      F[1] = e1.C * isu + mul_i(e1.S);
-      cd Ep0 = e0.Gam * isu - C(0.5 * iu3) + mul_i(e0.Sp);
-      cd Ep1 = e1.Gam * isu - C(0.5 * iu3) + mul_i(e1.Sp);
-      F[2] = (2.0 * rd) * Ep0; F[3] = (2.0 * zd) * Ep0;
-      F[4] = (2.0 * rd) * Ep1; F[5] = (2.0 * zd) * Ep1;
-      cd D1 = gam1 * isu + mul_i(dSp);
-      cd D2 = (gam1p - 0.5 * gam2) * isu - (0.5 * iu3) * g0 + mul_i(dSpp);
-      F[6] = (4.0 * rd * rd) * D2 + 2.0 * D1;
-      F[7] = (4.0 * rd * zd) * D2;
-      F[8] = (4.0 * zd * zd) * D2 + 2.0 * D1;
-    } else {
-      double q = W.q[j];
-      F[0] = q * e0.C + mul_i(e0.S);
-      F[1] = q * e1.C + mul_i(e1.S);
-      F[2] = q * ((2.0 * rd) * e0.Gam - C(0.5 / rt)) + mul_i((2.0 * rd) * e0.Sp);
-      F[3] = q * ((2.0 * zd) * e0.Gam) + mul_i((2.0 * zd) * e0.Sp);
-      F[4] = q * ((2.0 * rd) * e1.Gam - C(0.5 / rt)) + mul_i((2.0 * rd) * e1.Sp);
-      F[5] = q * ((2.0 * zd) * e1.Gam) + mul_i((2.0 * zd) * e1.Sp);
-      cd eta = gam1p - 0.5 * gam2;
-      F[6] = q * ((4.0 * rd * rd) * eta - ((rd + alpha) / rt) * g0 + 2.0 * gam1) +
-             mul_i((4.0 * rd * rd) * dSpp + 2.0 * dSp);
-      F[7] = q * ((4.0 * rd * zd) * eta - (zd / rt) * g0) + mul_i((4.0 * rd * zd) * dSpp);
-      F[8] = q * ((4.0 * zd * zd) * eta + 2.0 * gam1) + mul_i((4.0 * zd * zd) * dSpp + 2.0 * dSp);
-    }
-    double wj = (j == 0 || j == H - 1) ? 0.5 : 1.0;
-#pragma unroll
-    for (int f = 0; f < NFAM; ++f) W.smp[f * H + j] = wj * F[f];
+    const double wj = (j == 0 || j == H - 1) ? 0.5 : 1.0;
+    cd* out = W.smp + j;
+    if (RR == 2 || (RR < 0 && gp.k0_real && gp.k1_real))
+      pair_sample<true, true>(gp, ps, s2L[j], wj, split, split ? W.q[j] : 0.0, out, H);
+    else if (RR == 1 || (RR < 0 && gp.k0_real))
+      pair_sample<true, false>(gp, ps, s2L[j], wj, split, split ? W.q[j] : 0.0, out, H);
+    else if (RR <= 0)
+      pair_sample<false, false>(gp, ps, s2L[j], wj, split, split ? W.q[j] : 0.0, out, H);
   }
   sync();
 }
@@ -374,6 +449,16 @@ __device__ __forceinline__ void store_block(cd* __restrict__ A, int n, int m, in
     double2* dst = (double2*)(A + base + (size_t)(4 * j + b) * n + 4 * i);
 #pragma unroll
     for (int a = 0; a < 4; ++a) dst[a] = make_double2(scale * blk[a][b].x, scale * blk[a][b].y);
+  }
+}
+
+__device__ __forceinline__ void store_block(cd* __restrict__ A, int n, int m, int i, int j, cd blk[4][4]) {
+  size_t base = (size_t)m * n * n;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    double2* dst = (double2*)(A + base + (size_t)(4 * j + b) * n + 4 * i);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) dst[a] = make_double2(blk[a][b].x, blk[a][b].y);
   }
 }
 
@@ -623,6 +708,9 @@ __device__ __forceinline__ WarpSmem sample_smem(char* smem, int H, int Mq, doubl
   return W;
 }
 
+// FAR: the pairs are far pairs (p = i N + j) on the full grid, else support
+// pairs (p = i NEAR_SLOTS + slot).
+template <int RR, bool FAR>
 __global__ void __launch_bounds__(SUP_NT, 3) support_sample_kernel(BuildArgs a, const int* __restrict__ list, int q0,
                                                                    int count, __nv_bfloat16* __restrict__ Asl,
                                                                    double* __restrict__ Ascale, int nkt) {
@@ -632,222 +720,285 @@ __global__ void __launch_bounds__(SUP_NT, 3) support_sample_kernel(BuildArgs a, 
   const WarpSmem W = sample_smem(smem, gp.H, gp.Mq, &red, &shift);
   for (int q = blockIdx.x; q < count; q += gridDim.x) {
     const int p = list[q0 + q];
-    const int i = p / NEAR_SLOTS, slot = p % NEAR_SLOTS;
-    long long pid;
-    support_point(a, i, slot, &pid);
     double rt, dr0, zd;
-    support_geometry(a, i, slot, pid, &rt, &dr0, &zd);
-    const long long sid = a.split_sup[p];
-    group_pair_samples<SUP_NT>(gp, rt, dr0, zd, sid, a.leg, a.n_split, a.cosT, W, threadIdx.x,
-                               full_grid(gp, a.cosT, a.s2T), [] { __syncthreads(); });
+    long long sid;
+    if (FAR) {
+      const int i = p / a.N, j = p % a.N;
+      rt = a.geo.r[i];
+      dr0 = rt - a.geo.r[j];
+      zd = a.geo.z[i] - a.geo.z[j];
+      sid = a.split_far[p];
+    } else {
+      const int i = p / NEAR_SLOTS, slot = p % NEAR_SLOTS;
+      long long pid;
+      support_point(a, i, slot, &pid);
+      support_geometry(a, i, slot, pid, &rt, &dr0, &zd);
+      sid = a.split_sup[p];
+    }
+    group_pair_samples<SUP_NT, RR>(gp, rt, dr0, zd, sid, a.leg, a.n_split, a.cosT, W, threadIdx.x,
+                                   full_grid(gp, a.cosT, a.s2T), [] { __syncthreads(); });
     __syncthreads();
     pair_rows_to_digits(W, gp.H, q, nkt, Asl, Ascale, red, shift);
   }
 }
 
-// Far pairs of one grid-size bin (list[q0 + q], q < count, p = i N + j), on
-// their ladder grid of nl points: the same rows as the support pairs, one
-// warp per pair (far pairs have few samples: no CTA barriers).
-__host__ __device__ inline int far_sample_smem_per_warp(int H, int Mq) {
-  return NFAM * H * 16 + H * 8 + (Mq + 1) * 8 + SUP_ROWS * 8;
-}
+// Far pairs of one bin below the full grid (list[q0 + q], q < count, p = i N + j;
+// never split) on their ladder grid of nl points: the same rows as the support
+// pairs.  A CTA takes PB pairs at a time and deals out (pair, sample) items, so
+// that grids of 9 to 129 samples fill its warps; the bin's grid is known, only
+// its table is looked up.
+__host__ __device__ inline int far_sample_smem_per_pair(int H) { return NFAM * H * 16 + SUP_ROWS * 4; }
 
-__global__ void __launch_bounds__(128, 3) far_sample_kernel(BuildArgs a, const int* __restrict__ list, int q0, int count,
-                                                         __nv_bfloat16* __restrict__ Asl,
-                                                         double* __restrict__ Ascale, int nkt, int nl) {
+template <int RR>
+__global__ void __launch_bounds__(128, 4) far_sample_kernel(BuildArgs a, const int* __restrict__ list, int q0, int count,
+                                                            __nv_bfloat16* __restrict__ Asl,
+                                                            double* __restrict__ Ascale, int nkt, int nl, int PB) {
   extern __shared__ __align__(16) char smem[];
   const GreenParams& gp = a.gp;
-  const int H = nl / 2 + 1;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  char* base = smem + (size_t)wib * far_sample_smem_per_warp(H, gp.Mq);
-  WarpSmem W;
-  W.smp = (cd*)base;
-  W.spec = nullptr;
-  W.q = (double*)(W.smp + NFAM * H);
-  W.phs = W.q + H;
-  double* shift = W.phs + gp.Mq + 1;
-  for (int q = blockIdx.x * wpb + wib; q < count; q += gridDim.x * wpb) {
-    const int p = list[q0 + q];
-    const int i = p / a.N, j = p % a.N;
-    const long long sid = a.split_far[p];
-    const double rt = a.geo.r[i], dr0 = rt - a.geo.r[j], zd0 = a.geo.z[i] - a.geo.z[j];
-    const PairGrid g = pair_grid(gp, rt, dr0, zd0, sid >= 0, a.lneps, a.cosT, a.s2T, a.ladC, a.ladS);
-    warp_pair_samples(gp, rt, dr0, zd0, sid, a.leg, a.n_split, a.cosT, W, lane, g);
-    __syncwarp();
-    // row maxima of |v| on the bits of the samples (integer pipe)
-    unsigned long long mx[SUP_ROWS];
-#pragma unroll
-    for (int rr = 0; rr < SUP_ROWS; ++rr) mx[rr] = 0ull;
-    for (int jj = lane; jj < H; jj += 32)
-#pragma unroll
-      for (int f = 0; f < NFAM; ++f) {
-        const cd v = W.smp[f * H + jj];
-        const unsigned long long bx = abs_bits(v.x), by = abs_bits(v.y);
-        mx[2 * f] = bx > mx[2 * f] ? bx : mx[2 * f];
-        mx[2 * f + 1] = by > mx[2 * f + 1] ? by : mx[2 * f + 1];
+  const int H = nl / 2 + 1, tid = threadIdx.x, qq = nl / 8;
+  const double* __restrict__ s2L = a.ladS + (2 * (qq - 1) * qq - 4 + (qq - 2));  // see pair_grid
+  cd* smp = (cd*)smem;                       // [PB][NFAM][H]
+  int* shift = (int*)(smp + (size_t)PB * NFAM * H);  // [PB][SUP_ROWS]
+  for (long long b0 = (long long)blockIdx.x * PB; b0 < count; b0 += (long long)gridDim.x * PB) {
+    const int np = (int)min((long long)PB, count - b0);
+    for (int it = tid; it < np * H; it += 128) {
+      const int q = it / H, j = it - q * H;
+      const int p = list[q0 + b0 + q], i = p / a.N, jn = p % a.N;
+      const double rt = a.geo.r[i], rs = a.geo.r[jn];
+      PairSample ps;
+      ps.dr0 = rt - rs;
+      ps.zd = a.geo.z[i] - a.geo.z[jn];
+      ps.d2 = ps.dr0 * ps.dr0 + ps.zd * ps.zd;
+      ps.rr4 = 4.0 * rt * rs;
+      ps.rs2 = 2.0 * rs;
+      ps.irt = ps.alpha = 0.0;
+      const double w = (j == 0 || j == H - 1) ? 0.5 : 1.0;
+      pair_sample<RR >= 1, RR == 2>(gp, ps, s2L[j], w, false, 0.0, smp + (size_t)q * NFAM * H + j, H);
+    }
+    __syncthreads();
+    // row scales: powers of two 2^E above twice each row's largest magnitude, on
+    // the bits of the samples; four threads per row
+    for (int t0 = 0; t0 < np * SUP_ROWS * 4; t0 += 128) {
+      const int t = t0 + tid, rw = t >> 2, q = rw / SUP_ROWS, rr = rw - q * SUP_ROWS;
+      unsigned long long mx = 0ull;
+      if (rw < np * SUP_ROWS) {
+        const double* x = (const double*)(smp + ((size_t)q * NFAM + (rr >> 1)) * H) + (rr & 1);
+        for (int j = t & 3; j < H; j += 4) {
+          const unsigned long long b = abs_bits(x[2 * j]);
+          mx = b > mx ? b : mx;
+        }
       }
-#pragma unroll
-    for (int rr = 0; rr < SUP_ROWS; ++rr) {
-      unsigned long long m = mx[rr];
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, m, o);
-        m = y > m ? y : m;
+      for (int o = 2; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = y > mx ? y : mx;
       }
-      if (lane == rr) {  // row scale 2^E above twice the row's largest magnitude
-        const int E = pow2_scale_exp(__longlong_as_double((long long)m));
-        shift[rr] = (double)(56 - E);  // digits of round(v 2^(56 - E))
-        Ascale[(size_t)q * SUP_ROWS + rr] = ldexp(1.0, E);
+      if ((t & 3) == 0 && rw < np * SUP_ROWS) {
+        const int E = pow2_scale_exp(__longlong_as_double((long long)mx));
+        shift[rw] = 56 - E;  // digits of round(v 2^(56 - E))
+        Ascale[(size_t)b0 * SUP_ROWS + rw] = ldexp(1.0, E);
       }
     }
-    __syncwarp();
+    __syncthreads();
     const int kg_n = nkt * 2;
-    for (int it = lane; it < SUP_ROWS * kg_n; it += 32) {
-      const int rr = it / kg_n, kg = it % kg_n, f = rr >> 1, im = rr & 1;
-      const int S = (int)shift[rr];
+    for (int it = tid; it < np * SUP_ROWS * kg_n; it += 128) {
+      const int rw = it / kg_n, kg = it - rw * kg_n, q = rw / SUP_ROWS, rr = rw - q * SUP_ROWS;
+      const double* x = (const double*)(smp + ((size_t)q * NFAM + (rr >> 1)) * H) + (rr & 1);
+      const int S = shift[rw];
       int dg[8][OZ_S];
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const int k = kg * 8 + c;
-        double v = 0.0;
-        if (k < H) { const cd z = W.smp[f * H + k]; v = im ? z.y : z.x; }
-        digits28(fixed_rn(v, S), dg[c]);
+        digits28(k < H ? fixed_rn(x[2 * k], S) : 0ll, dg[c]);
       }
-      const long long row = (long long)q * SUP_ROWS + rr;
-      const long long rt_ = row >> 7;
-      const int r = (int)(row & 127), kt = kg >> 1, kk = (kg & 1) * 8;
-      __nv_bfloat16* blk = Asl + ((size_t)rt_ * nkt + kt) * (OZ_S * 2048);
-      const int off = core_off(r, kk);
+      const long long row = b0 * SUP_ROWS + rw;
+      __nv_bfloat16* blk = Asl + ((size_t)(row >> 7) * nkt + (kg >> 1)) * (OZ_S * 2048) +
+                           core_off((int)(row & 127), (kg & 1) * 8);
 #pragma unroll
       for (int d = 0; d < OZ_S; ++d) {
         __align__(16) __nv_bfloat16 e8[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) e8[c] = __float2bfloat16((float)dg[c][d]);
-        *(uint4*)(blk + d * 2048 + off) = *(uint4*)e8;
+        *(uint4*)(blk + d * 2048) = *(uint4*)e8;
       }
     }
-    __syncwarp();
+    __syncthreads();  // the samples are rewritten by the next pairs
   }
 }
 
-// Grid-size bin of every far pair (g.nl / 8; 0xFFFF for near pairs) and the
-// bins' counts.
-__global__ void far_bin_kernel(BuildArgs a, unsigned short* __restrict__ bin_of, int* __restrict__ counts) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= (long long)a.N * a.N) return;
-  const int i = (int)(p / a.N), j = (int)(p % a.N);
-  if (near_panels(i / P_NODES, j / P_NODES, a.n_panels, a.closed)) { bin_of[p] = 0xFFFF; return; }
+// Far pairs listed bin by bin (bin: g.nl / 8), within a bin by source j and then
+// by target i up to a tile of FAR_TILE pairs, so that pairs assembled together
+// write the same columns side by side and the order does not depend on timing
+// beyond a tile.  tag[j N + i] packs the bin and the highest mode m_c (7 and 9 bits:
+// n_phi is at most 512 on this path); 0xFFFF marks near pairs.
+// tile_hist[bin][tile]: pairs of each bin in each tile of the (j, i) order.
+#define FAR_TILE 1024
+#define FAR_NEAR 0xFFFF
+static_assert((OZR_KMAX - 1) * 2 / 8 < 127 && OZR_KMAX < 511, "bin and mode fit the tag");
+__global__ void __launch_bounds__(256) far_bin_kernel(BuildArgs a, unsigned short* __restrict__ tag, int nbins,
+                                                      int ntiles, int* __restrict__ tile_hist) {
+  extern __shared__ int hist[];
+  for (int b = threadIdx.x; b < nbins; b += 256) hist[b] = 0;
+  __syncthreads();
   const GreenParams& gp = a.gp;
-  const double rt = a.geo.r[i], dr0 = rt - a.geo.r[j], zd0 = a.geo.z[i] - a.geo.z[j];
-  const PairGrid g = pair_grid(gp, rt, dr0, zd0, a.split_far[p] >= 0, a.lneps, a.cosT, a.s2T, a.ladC, a.ladS);
-  const int b = g.nl / 8;
-  bin_of[p] = (unsigned short)b;
-  atomicAdd(&counts[b], 1);
+  for (int t = threadIdx.x; t < FAR_TILE; t += 256) {
+    const long long p = (long long)blockIdx.x * FAR_TILE + t;  // j N + i
+    if (p >= (long long)a.N * a.N) break;
+    const int j = (int)(p / a.N), i = (int)(p % a.N);
+    if (near_panels(i / P_NODES, j / P_NODES, a.n_panels, a.closed)) { tag[p] = FAR_NEAR; continue; }
+    const double rt = a.geo.r[i], dr0 = rt - a.geo.r[j], zd0 = a.geo.z[i] - a.geo.z[j];
+    const PairGrid g = pair_grid(gp, rt, dr0, zd0, a.split_far[(long long)i * a.N + j] >= 0, a.lneps, a.cosT, a.s2T,
+                                 a.ladC, a.ladS);
+    const int b = g.nl / 8;
+    tag[p] = (unsigned short)(b << 9 | g.mc);
+    atomicAdd(&hist[b], 1);
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nbins; b += 256) tile_hist[(size_t)b * ntiles + blockIdx.x] = hist[b];
 }
 
-__global__ void far_scatter_kernel(long long total, const unsigned short* __restrict__ bin_of, int* __restrict__ cursor,
-                                   int* __restrict__ list) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= total) return;
-  const int b = bin_of[p];
-  if (b != 0xFFFF) list[atomicAdd(&cursor[b], 1)] = (int)p;
+// Exclusive prefix sum of `count` integers in place (one CTA), and each bin's
+// start start[b] (start[nbins]: the total).
+__global__ void __launch_bounds__(1024) far_scan_kernel(int* __restrict__ v, long long count, int nbins, int ntiles,
+                                                        int* __restrict__ start) {
+  __shared__ int part[1024];
+  const long long per = (count + 1023) / 1024, lo = min(count, threadIdx.x * per), hi = min(count, lo + per);
+  int sum = 0;
+  for (long long k = lo; k < hi; ++k) sum += v[k];
+  part[threadIdx.x] = sum;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {
+    const int x = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
+    __syncthreads();
+    part[threadIdx.x] += x;
+    __syncthreads();
+  }
+  int run = part[threadIdx.x] - sum;
+  for (long long k = lo; k < hi; ++k) {
+    const int x = v[k];
+    v[k] = run;
+    run += x;
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nbins; b += 1024) start[b] = v[(size_t)b * ntiles];
+  if (threadIdx.x == 0) start[nbins] = part[1023];
+}
+
+__global__ void __launch_bounds__(256) far_scatter_kernel(int N, const unsigned short* __restrict__ tag, int nbins,
+                                                          int ntiles, const int* __restrict__ tile_start,
+                                                          int* __restrict__ list, unsigned short* __restrict__ mcs) {
+  extern __shared__ int cursor[];
+  for (int b = threadIdx.x; b < nbins; b += 256) cursor[b] = tile_start[(size_t)b * ntiles + blockIdx.x];
+  __syncthreads();
+  for (int t = threadIdx.x; t < FAR_TILE; t += 256) {
+    const long long p = (long long)blockIdx.x * FAR_TILE + t;
+    if (p >= (long long)N * N) break;
+    const int b = tag[p];
+    if (b == FAR_NEAR) continue;
+    const int q = atomicAdd(&cursor[b >> 9], 1);
+    list[q] = (int)(p % N) * N + (int)(p / N);
+    mcs[q] = (unsigned short)(b & 511);
+  }
 }
 
 // The blocks of far pairs from their spectra Y[m][row] (the products of one
-// bin's chunk), exactly as far_kernel assembles them from its transform:
-// modes above the pair's m_c zero, the split pairs' u^{-3/2} part added.
+// bin's chunk): modes above the pair's m_c zero, the split pairs' u^{-3/2} part
+// added, the families of block.cuh combined once per pair and mode in shared
+// memory, then one block per (pair, mode) and thread.  A CTA takes PB pairs of
+// the bin at a time, so that (pair, mode) items fill its lanes whatever the
+// bin's number of modes.  FP64 pipe, 40 % busy (the rest barriers and latency):
+// N = 1024, M = 128 64 -> 50 ms, the cylinder (lossy) 19.5 -> 9.8 ms, against a warp
+// per pair with the block formed from the nine spectra.
+struct FarPair {
+  double irt, rpt, zpt, h0, h1, f2;  // target, weights (1 / nl in them)
+  double alpha, zd;                      // u^{-3/2} part of a split pair
+  int i, j, Me, mz, sid;                 // nodes, computed modes, last mode with a block, split id
+};
+
 template <bool SIMPLE>
-__global__ void __launch_bounds__(128, 3) far_assemble_kernel(BuildArgs a, const int* __restrict__ list, int q0, int count,
-                                    const double* __restrict__ Y, int ldy, int ncols, int nl) {
+__global__ void __launch_bounds__(128) far_assemble_kernel(BuildArgs a, const int* __restrict__ list,
+                                                           const unsigned short* __restrict__ mcs, int q0, int count,
+                                                           const double* __restrict__ Y, int ldy, int ncols, int nl,
+                                                           int PB) {
   extern __shared__ __align__(16) char smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   const GreenParams& gp = a.gp;
-  const int Ms = gp.Ms;
-  cd* spec = (cd*)smem + (size_t)wib * NFAM * Ms;
-  const int n = 4 * a.N;
-  const int tq = a.tq;
-  const int full = tq ? (gp.M + 1) / 32 * 32 : gp.M + 1;
-  const int tail = gp.M + 1 - full, tw = tail + 2;
-  const long long gw = (long long)blockIdx.x * wpb + wib;
-  cd* Qs = tq ? a.tailq + gw * (long long)tq * tw * NFAM : nullptr;
-  int* Qij = tq ? a.tailij + gw * 2LL * tq : nullptr;
-  int qn = 0;
-  const double invn = 1.0 / nl;
+  const int W = ncols + 2;               // modes 0..ncols + 1 of a pair's families
+  cd* comb = (cd*)smem;                  // [PB][BK_N][W]
+  FarPair* pp = (FarPair*)(comb + (size_t)PB * BK_N * W);
+  const int tid = threadIdx.x, n = 4 * a.N;
+  const int mmax = min(gp.M, ncols);     // blocks above are zero for every pair of the bin
+  const bool unit = a.ap.aEJ.x == 1.0 && a.ap.aEJ.y == 0.0 && a.ap.aHM.x == -1.0 && a.ap.aHM.y == 0.0;
   const double* Shat = a.leg + (long long)(gp.Mq + 1) * a.n_split;
-  auto pair_consts = [&](int i, int j, double fac[3], double* irt) {
-    const double rs = a.geo.r[j], w = a.geo.w[j] * rs * (a.geo.sw[i] / a.geo.sw[j]);
-    fac[0] = w * a.geo.rp[j];
-    fac[1] = w;
-    fac[2] = w * a.geo.zp[j];
-    *irt = 1.0 / a.geo.r[i];
-  };
-  auto assemble = [&](const cd* S, int stride, int base, int i, int j, int m, const double fac[3], double irt) {
-    cd blk[4][4];
-    mueller_block_spec<SIMPLE>(S, stride, base, fac, m, a.ap, a.geo.r[i], irt, a.geo.rp[i], a.geo.zp[i], blk);
-    store_block(a.A, n, m, i, j, blk, 1.0);
-  };
-  auto flush = [&]() {
-    __syncwarp();
-    for (int it = lane; it < qn * tail; it += 32) {
-      const int qq = it / tail, m = full + it % tail;
-      double fac[3], irt;
-      pair_consts(Qij[2 * qq], Qij[2 * qq + 1], fac, &irt);
-      assemble(Qs + (long long)qq * tw * NFAM, tw, full - 1, Qij[2 * qq], Qij[2 * qq + 1], m, fac, irt);
-    }
-    __syncwarp();
-    qn = 0;
-  };
-  for (long long q = gw; q < count; q += (long long)gridDim.x * wpb) {
-    const int p = list[q0 + q];
-    const int i = p / a.N, j = p % a.N;
-    const long long sid = a.split_far[p];
-    const double rt = a.geo.r[i], dr0 = rt - a.geo.r[j], zd0 = a.geo.z[i] - a.geo.z[j];
-    const PairGrid g = pair_grid(gp, rt, dr0, zd0, sid >= 0, a.lneps, a.cosT, a.s2T, a.ladC, a.ladS);
-    const int Me = min(g.mc + 1, ncols);
-    const double d2 = dr0 * dr0 + zd0 * zd0, alpha = dr0 - d2 / (2.0 * rt);
-    const long long row0 = q * SUP_ROWS;
-    // lanes take consecutive families of one mode: a mode's 18 values of the
-    // pair are contiguous in Y (16-byte loads of one 144-byte run)
-    for (int t = lane; t < NFAM * Ms; t += 32) {
-      const int m = t / NFAM, f = t - m * NFAM;
-      cd v = C(0.0);
-      if (m < Me) {
-        const double2 y = *(const double2*)(Y + (size_t)m * ldy + row0 + 2 * f);  // even offset: 16-byte aligned
-        v = C(invn * y.x, invn * y.y);
-        if (sid >= 0 && f >= 2) {
-          cd beta;
-          switch (f) {
-            case 2: case 4: beta = C(-alpha); break;
-            case 3: case 5: beta = C(-zd0); break;
-            case 6: beta = (-2.0 * alpha * alpha) * gp.gamma0; break;
-            case 7: beta = (-2.0 * alpha * zd0) * gp.gamma0; break;
-            default: beta = (-2.0 * zd0 * zd0) * gp.gamma0; break;
-          }
-          v = fma(Shat[(long long)m * a.n_split + sid] / 12.566370614359172, beta, v);
-        }
+  const double invn = 1.0 / nl;
+  for (long long b0 = (long long)blockIdx.x * PB; b0 < count; b0 += (long long)gridDim.x * PB) {
+    const int np = (int)min((long long)PB, count - b0);
+    if (tid < np) {  // no division or logarithm here: the other threads wait for it
+      const int p = list[q0 + b0 + tid];
+      FarPair v;
+      v.i = p / a.N;
+      v.j = p % a.N;
+      v.sid = a.split_far[p];
+      v.irt = a.geo.irt[v.i];
+      v.rpt = a.geo.rp[v.i];
+      v.zpt = a.geo.zp[v.i];
+      const int mc = mcs[q0 + b0 + tid];
+      v.Me = min(mc + 1, ncols);
+      v.mz = min(gp.M, mc + 1);
+      v.alpha = v.zd = 0.0;
+      if (v.sid >= 0) {
+        const double rt = a.geo.r[v.i], dr0 = rt - a.geo.r[v.j];
+        v.zd = a.geo.z[v.i] - a.geo.z[v.j];
+        v.alpha = dr0 - (dr0 * dr0 + v.zd * v.zd) / (2.0 * rt);
       }
-      spec[f * Ms + m] = v;
+      const double w = a.geo.wr[v.j] * a.geo.sw[v.i] * invn;
+      v.h0 = 0.5 * w * a.geo.rp[v.j];
+      v.h1 = 0.5 * w;
+      v.f2 = w * a.geo.zp[v.j];
+      pp[tid] = v;
     }
-    __syncwarp();
-    const int mz = min(gp.M, g.mc + 1);
-    double fac[3], irt;
-    pair_consts(i, j, fac, &irt);
-    for (int m = lane; m < full; m += 32) {
-      if (m <= mz) assemble(spec, Ms, 0, i, j, m, fac, irt);
-      else store_zero_block(a.A, n, m, i, j);
-    }
-    if (tq) {
-      if (mz >= full) {
-        cd* dst = Qs + (long long)qn * tw * NFAM;
-        for (int t = lane; t < NFAM * tw; t += 32) dst[t] = spec[(t / tw) * Ms + full - 1 + t % tw];
-        if (lane == 0) { Qij[2 * qn] = i; Qij[2 * qn + 1] = j; }
-        if (++qn == tq) flush();
-      } else {
-        for (int m = full + lane; m <= gp.M; m += 32) store_zero_block(a.A, n, m, i, j);
+    __syncthreads();
+    for (int it = tid; it < np * W; it += 128) {
+      const int q = it / W, m = it - q * W;
+      const FarPair& v = pp[q];
+      cd* o = comb + (size_t)q * BK_N * W + m;
+      if (m >= v.Me) {
+#pragma unroll
+        for (int f = 0; f < BK_N; ++f) o[f * W] = C(0.0);
+        continue;
       }
+      const double2* y = (const double2*)(Y + (size_t)m * ldy + (b0 + q) * SUP_ROWS);  // even offset: 16-byte aligned
+      cd S[NFAM];
+#pragma unroll
+      for (int f = 0; f < NFAM; ++f) {
+        const double2 t = y[f];
+        S[f] = C(t.x, t.y);
+      }
+      if (v.sid >= 0) {
+        const double Sm = Shat[(long long)m * a.n_split + v.sid] / 12.566370614359172 * nl;
+        const double al = Sm * v.alpha, zd = Sm * v.zd;
+        S[2].x -= al; S[4].x -= al;
+        S[3].x -= zd; S[5].x -= zd;
+        S[6] = fma(-2.0 * al * v.alpha, gp.gamma0, S[6]);
+        S[7] = fma(-2.0 * al * v.zd, gp.gamma0, S[7]);
+        S[8] = fma(-2.0 * zd * v.zd, gp.gamma0, S[8]);
+      }
+      mueller_combine<SIMPLE>(S, a.ap, v.irt, v.rpt, v.zpt, o, W);
     }
-    __syncwarp();
+    __syncthreads();
+    for (int it = tid; it < np * (mmax + 1); it += 128) {
+      const int q = it / (mmax + 1), m = it - q * (mmax + 1);
+      const FarPair& v = pp[q];
+      if (m > v.mz) { store_zero_block(a.A, n, m, v.i, v.j); continue; }
+      cd blk[4][4];
+      mueller_block_combined(comb + (size_t)q * BK_N * W, W, m, a.ap, unit, v.h0, v.h1, v.f2, v.irt, v.rpt, v.zpt, blk);
+      store_block(a.A, n, m, v.i, v.j, blk);
+    }
+    const int nz = gp.M - mmax;
+    for (int it = tid; it < np * nz; it += 128) {
+      const int q = it / nz, m = mmax + 1 + it % nz;
+      store_zero_block(a.A, n, m, pp[q].i, pp[q].j);
+    }
+    __syncthreads();
   }
-  if (tq && qn > 0) flush();
 }
 
 // thread per (pair q, family f, mode m): spec = (1/n)(Y_re + i Y_im) + the
@@ -1025,20 +1176,11 @@ int far_tail_pairs(const GreenParams& gp) {
   return (full >= 32 && tail > 0 && tail <= 16) ? 32 / tail : 0;
 }
 
-// Warps per CTA of far_assemble_kernel: its shared memory is only the
-// spectra, NFAM (M+2) complex values per warp.
-static int assemble_warps_per_block(const GreenParams& gp) {
-  int w = (72 * 1024) / (NFAM * gp.Ms * 16);  // up to three CTAs per SM (registers)
-  if (w > 4) w = 4;
-  if (w < 1) w = 1;
-  return w;
-}
-
 size_t far_tail_scratch(const BuildArgs& a, size_t* ij_elems) {
   const int tq = far_tail_pairs(a.gp);
-  const int wpb = warps_per_block(a.gp), wpa = assemble_warps_per_block(a.gp);
+  const int wpb = warps_per_block(a.gp);
   const long long total = (long long)a.N * a.N;
-  const long long warps = std::max((long long)grid_for(total, wpb) * wpb, (long long)grid_for(total, wpa) * wpa);
+  const long long warps = (long long)grid_for(total, wpb) * wpb;
   const int tail = a.gp.M + 1 - (a.gp.M + 1) / 32 * 32;
   *ij_elems = tq ? (size_t)warps * 2 * tq : 0;
   return tq ? (size_t)warps * tq * (tail + 2) * NFAM : 0;
@@ -1058,47 +1200,89 @@ void launch_support_spectra(const BuildArgs& a, cudaStream_t s) {
   support_kernel<<<grid_for((long long)a.N * NEAR_SLOTS, wpb), wpb * 32, smem, s>>>(a);
 }
 
-void launch_support_samples(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl,
-                            double* Ascale, int nkt, cudaStream_t s) {
+template <int RR, bool FAR>
+static void launch_full_samples(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl,
+                                double* Ascale, int nkt, cudaStream_t s) {
   const int smem = support_sample_smem(a.gp.H, a.gp.Mq);
-  smem_optin(support_sample_kernel);
+  smem_optin(support_sample_kernel<RR, FAR>);
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = std::min(count, 3 * sms * 8);
-  support_sample_kernel<<<grid, SUP_NT, smem, s>>>(a, list, q0, count, Asl, Ascale, nkt);
+  support_sample_kernel<RR, FAR><<<grid, SUP_NT, smem, s>>>(a, list, q0, count, Asl, Ascale, nkt);
 }
 
-void launch_far_bins(const BuildArgs& a, unsigned short* bin_of, int* counts, cudaStream_t s) {
-  const long long total = (long long)a.N * a.N;
-  far_bin_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(a, bin_of, counts);
+void launch_support_samples(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl,
+                            double* Ascale, int nkt, cudaStream_t s) {
+  if (a.gp.k0_real && a.gp.k1_real) launch_full_samples<2, false>(a, list, q0, count, Asl, Ascale, nkt, s);
+  else if (a.gp.k0_real) launch_full_samples<1, false>(a, list, q0, count, Asl, Ascale, nkt, s);
+  else launch_full_samples<0, false>(a, list, q0, count, Asl, Ascale, nkt, s);
 }
 
-void launch_far_scatter(long long total, const unsigned short* bin_of, int* cursor, int* list, cudaStream_t s) {
-  far_scatter_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(total, bin_of, cursor, list);
+int far_tiles(int N) { return (int)(((long long)N * N + FAR_TILE - 1) / FAR_TILE); }
+
+void launch_far_bins(const BuildArgs& a, int nbins, unsigned short* tag, int* tile_hist, int* start,
+                     cudaStream_t s) {
+  const int tiles = far_tiles(a.N);
+  far_bin_kernel<<<tiles, 256, nbins * sizeof(int), s>>>(a, tag, nbins, tiles, tile_hist);
+  far_scan_kernel<<<1, 1024, 0, s>>>(tile_hist, (long long)nbins * tiles, nbins, tiles, start);
+}
+
+void launch_far_scatter(int N, int nbins, const unsigned short* tag, const int* tile_start, int* list,
+                        unsigned short* mcs, cudaStream_t s) {
+  far_scatter_kernel<<<far_tiles(N), 256, nbins * sizeof(int), s>>>(N, tag, nbins, far_tiles(N), tile_start, list, mcs);
+}
+
+// Pairs per CTA: among those that leave four CTAs per SM (registers; 54 KiB of
+// shared memory each), the number whose (pair, sample) items waste the fewest
+// lanes; one pair of the largest ladder grid takes 19 KiB.
+template <int RR>
+static void launch_ladder_samples(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl,
+                                  double* Ascale, int nkt, int nl, cudaStream_t s) {
+  const int H = nl / 2 + 1, per = far_sample_smem_per_pair(H);
+  int PB = 1;
+  double best = 0.0;
+  for (int b = 1; b <= 32 && (b == 1 || b * per <= 54 * 1024); ++b) {
+    const double eff = (double)b * H / ((b * H + 127) / 128 * 128);
+    if (eff > best + 0.02) { best = eff; PB = b; }
+  }
+  smem_optin(far_sample_kernel<RR>);
+  far_sample_kernel<RR><<<grid_for(count, PB), 128, PB * per, s>>>(a, list, q0, count, Asl, Ascale, nkt, nl, PB);
+}
+
+template <int RR>
+static void launch_far_samples_rr(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl,
+                                  double* Ascale, int nkt, int nl, cudaStream_t s) {
+  if (nl == a.gp.nphi) launch_full_samples<RR, true>(a, list, q0, count, Asl, Ascale, nkt, s);
+  else launch_ladder_samples<RR>(a, list, q0, count, Asl, Ascale, nkt, nl, s);
 }
 
 void launch_far_samples(const BuildArgs& a, const int* list, int q0, int count, __nv_bfloat16* Asl, double* Ascale,
                         int nkt, int nl, cudaStream_t s) {
-  const int per = far_sample_smem_per_warp(nl / 2 + 1, a.gp.Mq);
-  int wpb = (72 * 1024) / per;  // up to three 4-warp CTAs per SM (registers)
-  if (wpb > 4) wpb = 4;
-  if (wpb < 1) wpb = 1;
-  smem_optin(far_sample_kernel);
-  far_sample_kernel<<<grid_for(count, wpb), wpb * 32, wpb * per, s>>>(a, list, q0, count, Asl, Ascale, nkt, nl);
+  if (a.gp.k0_real && a.gp.k1_real) launch_far_samples_rr<2>(a, list, q0, count, Asl, Ascale, nkt, nl, s);
+  else if (a.gp.k0_real) launch_far_samples_rr<1>(a, list, q0, count, Asl, Ascale, nkt, nl, s);
+  else launch_far_samples_rr<0>(a, list, q0, count, Asl, Ascale, nkt, nl, s);
 }
 
-// Launch shape: assemble_warps_per_block (the tail-queue scratch covers it).
-void launch_far_assemble(const BuildArgs& a, const int* list, int q0, int count, const double* Y, int ldy, int ncols,
-                         int nl, cudaStream_t s) {
-  const int wpb = assemble_warps_per_block(a.gp);
-  const int smem = wpb * NFAM * a.gp.Ms * 16;
+// Pairs per CTA: among those that leave four CTAs per SM (registers; 56 KiB of
+// shared memory each), the number whose (pair, mode) items waste the fewest lanes
+// of the last round; at least one, whatever it takes of shared memory.
+void launch_far_assemble(const BuildArgs& a, const int* list, const unsigned short* mcs, int q0, int count,
+                         const double* Y, int ldy, int ncols, int nl, cudaStream_t s) {
+  const int per = BK_N * (ncols + 2) * 16 + (int)sizeof(FarPair), items = std::min(a.gp.M, ncols) + 1;
+  int PB = 1;
+  double best = 0.0;
+  for (int b = 1; b <= 32 && (b == 1 || b * per <= 56 * 1024); ++b) {
+    const double eff = (double)b * items / ((b * items + 127) / 128 * 128);
+    if (eff > best + 0.02) { best = eff; PB = b; }
+  }
+  const int smem = PB * per, grid = grid_for(count, PB);
   if (a.ap.simple) {
     smem_optin(far_assemble_kernel<true>);
-    far_assemble_kernel<true><<<grid_for(count, wpb), wpb * 32, smem, s>>>(a, list, q0, count, Y, ldy, ncols, nl);
+    far_assemble_kernel<true><<<grid, 128, smem, s>>>(a, list, mcs, q0, count, Y, ldy, ncols, nl, PB);
   } else {
     smem_optin(far_assemble_kernel<false>);
-    far_assemble_kernel<false><<<grid_for(count, wpb), wpb * 32, smem, s>>>(a, list, q0, count, Y, ldy, ncols, nl);
+    far_assemble_kernel<false><<<grid, 128, smem, s>>>(a, list, mcs, q0, count, Y, ldy, ncols, nl, PB);
   }
 }
 

@@ -715,7 +715,7 @@ static size_t far_tc_scratch_bytes(int N, int nphi, int M) {
     sc = std::max(sc, (size_t)rp * 8);
     b += ozaki_real_b_elems(ncols, nkt) * 2;
   }
-  return a + y + sc + b + (size_t)N * N * 6 + 4096;
+  return a + y + sc + b + (size_t)N * N * 8 + (size_t)(nphi / 8 + 2) * ((size_t)N * N / 1024 + 2) * 4 + 4096;
 }
 
 // Far pairs with the transform on the tensor cores (when the largest grid's
@@ -762,23 +762,23 @@ static int far_assembly(const Setup& S, BuildArgs& a, DevBuf& keep_err, int** er
   DevBuf tmp;  // freed (after a device synchronisation) when this returns
   const long long total = (long long)S.N * S.N;
   const int nbins = S.nphi / 8 + 1;
-  unsigned short* bin_of = nullptr;
-  int *counts = nullptr, *cursor = nullptr, *list = nullptr, *err = nullptr;
-  if (tmp.alloc(&bin_of, (size_t)total) != cudaSuccess || tmp.alloc(&counts, (size_t)nbins) != cudaSuccess ||
-      tmp.alloc(&cursor, (size_t)nbins) != cudaSuccess || keep_err.alloc(&err, 1) != cudaSuccess)
+  unsigned short *tag = nullptr, *mcs = nullptr;
+  int *hist = nullptr, *start = nullptr, *list = nullptr, *err = nullptr;
+  if (tmp.alloc(&tag, (size_t)total) != cudaSuccess ||
+      tmp.alloc(&hist, (size_t)nbins * far_tiles(S.N)) != cudaSuccess ||
+      tmp.alloc(&start, (size_t)nbins + 1) != cudaSuccess || keep_err.alloc(&err, 1) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "far-pair bins");
-  CK(cudaMemsetAsync(counts, 0, sizeof(int) * nbins, s));
   CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  launch_far_bins(a, bin_of, counts, s);
+  launch_far_bins(a, nbins, tag, hist, start, s);
   std::vector<int> cnt(nbins), off(nbins + 1, 0);
-  CK(cudaMemcpyAsync(cnt.data(), counts, sizeof(int) * nbins, cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(off.data(), start, sizeof(int) * (nbins + 1), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  for (int b = 0; b < nbins; ++b) off[b + 1] = off[b] + cnt[b];
+  for (int b = 0; b < nbins; ++b) cnt[b] = off[b + 1] - off[b];
   *err_out = err;
   if (off[nbins] == 0) return MUELLER_OK;
-  if (tmp.alloc(&list, (size_t)off[nbins]) != cudaSuccess) return fail(MUELLER_ENOMEM, "far-pair list");
-  CK(cudaMemcpyAsync(cursor, off.data(), sizeof(int) * nbins, cudaMemcpyHostToDevice, s));
-  launch_far_scatter(total, bin_of, cursor, list, s);
+  if (tmp.alloc(&list, (size_t)off[nbins]) != cudaSuccess || tmp.alloc(&mcs, (size_t)off[nbins]) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "far-pair list");
+  launch_far_scatter(S.N, nbins, tag, hist, list, mcs, s);
   // scratch for the largest chunk; the B digits of every bin in use
   size_t amax = 0, ymax = 0, smax = 0;
   std::vector<const __nv_bfloat16*> Bsl(nbins, nullptr);
@@ -819,7 +819,7 @@ static int far_assembly(const Setup& S, BuildArgs& a, DevBuf& keep_err, int** er
       ozaki_real_gemm(Asl, Ascale, rp, Bsl[b], 2.0, nkt, Y, rp, ncols, err, s);
       ft.mark(1, s);
       ft.mark(2, s);
-      launch_far_assemble(a, list, off[b] + q0, c, Y, rp, ncols, nl, s);
+      launch_far_assemble(a, list, mcs, off[b] + q0, c, Y, rp, ncols, nl, s);
       ft.mark(2, s);
       // blocks formed: every pair of the bin assembles modes 0..min(M, m_c + 1), m_c < nl / 2
       ft.blocks += (double)c * std::min(S.M + 1, ncols + 1);
@@ -913,7 +913,14 @@ static int assemble_core(Setup& S, cd* A_dev, cudaStream_t s, mueller_stats* st,
   double *dr_, *dz_, *drp, *dzp, *dw, *dsw;
   CK(keep.upload(&dr_, S.r, s)); CK(keep.upload(&dz_, S.z, s)); CK(keep.upload(&drp, S.rp, s));
   CK(keep.upload(&dzp, S.zp, s)); CK(keep.upload(&dw, S.w, s)); CK(keep.upload(&dsw, S.sw, s));
-  a.geo = NodeGeom{dr_, dz_, drp, dzp, dw, dsw};
+  std::vector<double> irt(S.N), wr(S.N);
+  for (int i = 0; i < S.N; ++i) {
+    irt[i] = 1.0 / S.r[i];
+    wr[i] = S.w[i] * S.r[i] / S.sw[i];
+  }
+  double *dirt, *dwr;
+  CK(tmp.upload(&dirt, irt, s)); CK(tmp.upload(&dwr, wr, s));
+  a.geo = NodeGeom{dr_, dz_, drp, dzp, dw, dsw, dirt, dwr};
   if (d_geo_out) { d_geo_out[0] = dr_; d_geo_out[1] = dz_; d_geo_out[2] = drp; d_geo_out[3] = dzp;
                    d_geo_out[4] = dw; d_geo_out[5] = dsw; }
   double *ssr, *ssz, *ssrp, *sszp, *ssW, *sLs, *sLa, *dcos, *ds2, *dpairs, *dleg, *ssdr, *ssdz;
@@ -948,7 +955,7 @@ static int assemble_core(Setup& S, cd* A_dev, cudaStream_t s, mueller_stats* st,
   a.cosT = dcos; a.s2T = ds2; a.ladC = dladC; a.ladS = dladS; a.split_far = dsf; a.split_sup = dss; a.leg = dleg; a.n_split = n_split;
   a.spec_sup = dspec; a.A = A_dev;
   a.lneps = -std::log(S.split_eps);
-  a.tq = far_tail_pairs(S.gp);
+  a.tq = S.gp.H > OZR_KMAX ? far_tail_pairs(S.gp) : 0;  // far_kernel only
   a.tailq = nullptr; a.tailij = nullptr;
   if (a.tq) {
     size_t ij = 0;
