@@ -623,6 +623,171 @@ __device__ __forceinline__ void support_geometry(const BuildArgs& a, int i, int 
   else { *dr0 = *rt - a.sup.r[pid]; *zd = a.geo.z[i] - a.sup.z[pid]; }
 }
 
+// ---------------------------------------------------------------------------
+// Geometry and tables of a build, formed on the device (on the host they took
+// 2 to 4 ms per body: thread starts, N^2 flags uploaded, one copy per table).
+
+// cosines and sin^2 of every grid: blockIdx.y = 0 the full grid, q the ladder grid of 8 q points
+__global__ void tables_kernel(int nphi, int qmax, double* __restrict__ tab) {
+  const int q = blockIdx.y, t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = q ? 8 * q : nphi;
+  if (q == 1 || t >= n) return;  // the ladder starts at 16 points
+  double *c = tab, *s2 = tab + nphi;
+  if (q) {
+    double* lad = tab + nphi + nphi / 2 + 1;
+    c = lad + (4 * (q - 1) * q - 8);
+    s2 = lad + ladder_cos_doubles(qmax) + (2 * (q - 1) * q - 4 + (q - 2));
+  }
+  c[t] = cospi(2.0 * t / n);
+  if (t <= n / 2) {
+    const double v = sinpi((double)t / n);
+    s2[t] = v * v;
+  }
+}
+
+// one thread per support point: geometry from the panel's degree-15 interpolants
+__global__ void __launch_bounds__(128) support_points_kernel(BuildArgs a, const double* __restrict__ ndr,
+                                                             const double* __restrict__ ndz,
+                                                             const double* __restrict__ wt_self,
+                                                             const double* __restrict__ wt_adj,
+                                                             double* __restrict__ sup) {
+  const int t = blockIdx.x * 128 + threadIdx.x, Q = blockIdx.y;
+  if (t >= PTS_PER_PANEL) return;
+  const size_t npts = (size_t)a.n_panels * PTS_PER_PANEL, id = (size_t)Q * PTS_PER_PANEL + t;
+  const bool own = t < P_NODES * SELF_PTS;
+  const double* L = nullptr;
+  double wt = 0.0;
+  if (own) {
+    L = a.sup.Lself + (size_t)t * P_NODES;
+    wt = wt_self[t];
+  } else {
+    const int e = (t - P_NODES * SELF_PTS) / ADJ_PTS, s = (t - P_NODES * SELF_PTS) % ADJ_PTS;
+    const int rule = a.sup.adj_rule[2 * Q + e];
+    if (rule >= 0 && s < a.sup.adj_n[2 * Q + e]) {
+      const size_t k = (size_t)(rule * 2 + e) * ADJ_PTS + s;
+      L = a.sup.Ladj + k * P_NODES;
+      wt = wt_adj[k];
+    }
+  }
+  double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (L) {  // else no neighbour at this end, or beyond the rule's points
+    const double *r = a.geo.r + Q * P_NODES, *z = a.geo.z + Q * P_NODES;
+    const double *dr = ndr + Q * P_NODES, *dz = ndz + Q * P_NODES;
+    double vr = 0.0, vz = 0.0, vdr = 0.0, vdz = 0.0, ddr = 0.0, ddz = 0.0;
+    const int tgt = own ? t / SELF_PTS : -1;
+    for (int k = 0; k < P_NODES; ++k) {
+      vr += L[k] * r[k]; vz += L[k] * z[k]; vdr += L[k] * dr[k]; vdz += L[k] * dz[k];
+      if (own && k != tgt) {  // x_t - x_s = -sum_{k != t} L_k(tau_s) (x_k - x_t)
+        ddr -= L[k] * (r[k] - r[tgt]);
+        ddz -= L[k] * (z[k] - z[tgt]);
+      }
+    }
+    const double sp = hypot(vdr, vdz);
+    v[0] = vr; v[1] = vz; v[2] = vdr / sp; v[3] = vdz / sp; v[4] = wt * sp; v[5] = ddr; v[6] = ddz;
+  }
+#pragma unroll
+  for (int f = 0; f < 7; ++f) sup[f * npts + id] = v[f];
+}
+
+// One warp per target: COUNT the split pairs of its row, or number and list them
+// in order of source and slot from the rows' prefix sums.
+template <bool COUNT>
+__global__ void __launch_bounds__(128) split_rows_kernel(BuildArgs a, double cthr, int* __restrict__ row,
+                                                         int* __restrict__ split_far, int* __restrict__ split_sup,
+                                                         double* __restrict__ pairs, int* __restrict__ sup_list) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= a.N) return;
+  const double rt = a.geo.r[i], zt = a.geo.z[i];
+  int nf = COUNT ? 0 : row[i], ns = COUNT ? 0 : row[a.N + i], nv = COUNT ? 0 : row[2 * a.N + i];
+  const unsigned below = (1u << lane) - 1u;
+  auto put = [&](int id, double dr, double dz) {
+    double* v = pairs + 4 * (size_t)id;
+    v[0] = rt; v[1] = zt; v[2] = dr; v[3] = dz;
+  };
+  for (int j0 = 0; j0 < a.N; j0 += 32) {  // N is a multiple of 16
+    const int j = j0 + lane;
+    const bool far = j < a.N && !near_panels(i / P_NODES, j / P_NODES, a.n_panels, a.closed);
+    const double dr = far ? rt - a.geo.r[j] : 0.0, dz = far ? zt - a.geo.z[j] : 0.0;
+    const bool sp = far && split_pair(rt, dr, dz, cthr);
+    const unsigned b = __ballot_sync(0xffffffffu, sp);
+    if (!COUNT && j < a.N) {
+      const int id = nf + __popc(b & below);
+      split_far[(size_t)i * a.N + j] = sp ? id : -1;
+      if (sp) put(id, dr, dz);
+    }
+    nf += __popc(b);
+  }
+  for (int s0 = 0; s0 < NEAR_SLOTS; s0 += 32) {  // a multiple of 32
+    const int slot = s0 + lane;
+    long long pid = 0;
+    const bool ok = support_point(a, i, slot, &pid);
+    double r, dr = 0.0, dz = 0.0;
+    if (ok) support_geometry(a, i, slot, pid, &r, &dr, &dz);
+    const bool sp = ok && split_pair(rt, dr, dz, cthr);
+    const unsigned b = __ballot_sync(0xffffffffu, sp), v = __ballot_sync(0xffffffffu, ok);
+    if (!COUNT) {
+      const int id = ns + __popc(b & below);
+      split_sup[(size_t)i * NEAR_SLOTS + slot] = sp ? id : -1;
+      if (sp) put(id, dr, dz);
+      if (ok) sup_list[nv + __popc(v & below)] = i * NEAR_SLOTS + slot;
+    }
+    ns += __popc(b);
+    nv += __popc(v);
+  }
+  if (COUNT && lane == 0) { row[i] = nf; row[a.N + i] = ns; row[2 * a.N + i] = nv; }
+}
+
+// Exclusive prefix sum of `count` integers in place (one CTA of 1024); returns the total.
+__device__ int block_scan(int* __restrict__ v, long long count, int* part) {
+  const long long per = (count + 1023) / 1024, lo = min(count, threadIdx.x * per), hi = min(count, lo + per);
+  int sum = 0;
+  for (long long k = lo; k < hi; ++k) sum += v[k];
+  __syncthreads();
+  part[threadIdx.x] = sum;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {
+    const int x = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
+    __syncthreads();
+    part[threadIdx.x] += x;
+    __syncthreads();
+  }
+  int run = part[threadIdx.x] - sum;
+  for (long long k = lo; k < hi; ++k) {
+    const int x = v[k];
+    v[k] = run;
+    run += x;
+  }
+  __syncthreads();
+  return part[1023];
+}
+
+__global__ void __launch_bounds__(1024) split_scan_kernel(int* __restrict__ row, int N, int* __restrict__ counts) {
+  __shared__ int part[1024];
+  const int split = block_scan(row, 2LL * N, part);
+  const int pts = block_scan(row + 2 * N, N, part);
+  if (threadIdx.x == 0) { counts[0] = split; counts[1] = pts; }
+}
+
+void launch_tables(const GreenParams& gp, double* tab, cudaStream_t s) {
+  tables_kernel<<<dim3((gp.nphi + 127) / 128, gp.qmax >= 2 ? gp.qmax + 1 : 1), 128, 0, s>>>(gp.nphi, gp.qmax, tab);
+}
+
+void launch_support_points(const BuildArgs& a, const double* dr, const double* dz, const double* wt_self,
+                           const double* wt_adj, double* sup, cudaStream_t s) {
+  support_points_kernel<<<dim3((PTS_PER_PANEL + 127) / 128, a.n_panels), 128, 0, s>>>(a, dr, dz, wt_self, wt_adj, sup);
+}
+
+void launch_split_count(const BuildArgs& a, double cthr, int* row, int* counts, cudaStream_t s) {
+  split_rows_kernel<true><<<(a.N + 3) / 4, 128, 0, s>>>(a, cthr, row, nullptr, nullptr, nullptr, nullptr);
+  split_scan_kernel<<<1, 1024, 0, s>>>(row, a.N, counts);
+}
+
+void launch_split_list(const BuildArgs& a, double cthr, const int* row, int* split_far, int* split_sup,
+                       double* pairs, int* sup_list, cudaStream_t s) {
+  split_rows_kernel<false><<<(a.N + 3) / 4, 128, 0, s>>>(a, cthr, const_cast<int*>(row), split_far, split_sup, pairs,
+                                                         sup_list);
+}
+
 // CTA of SUP_NT threads per support pair of the chunk: list[q0 + q], q < count.
 // Shared: the samples [NFAM][H], q [H], the Legendre coefficients [Mq + 1].
 #define SUP_NT 128
@@ -856,31 +1021,13 @@ __global__ void __launch_bounds__(256) far_bin_kernel(BuildArgs a, unsigned shor
   for (int b = threadIdx.x; b < nbins; b += 256) tile_hist[(size_t)b * ntiles + blockIdx.x] = hist[b];
 }
 
-// Exclusive prefix sum of `count` integers in place (one CTA), and each bin's
-// start start[b] (start[nbins]: the total).
+// Prefix sums of the tiles' counts and each bin's start (start[nbins]: the total).
 __global__ void __launch_bounds__(1024) far_scan_kernel(int* __restrict__ v, long long count, int nbins, int ntiles,
                                                         int* __restrict__ start) {
   __shared__ int part[1024];
-  const long long per = (count + 1023) / 1024, lo = min(count, threadIdx.x * per), hi = min(count, lo + per);
-  int sum = 0;
-  for (long long k = lo; k < hi; ++k) sum += v[k];
-  part[threadIdx.x] = sum;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int x = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
-    __syncthreads();
-    part[threadIdx.x] += x;
-    __syncthreads();
-  }
-  int run = part[threadIdx.x] - sum;
-  for (long long k = lo; k < hi; ++k) {
-    const int x = v[k];
-    v[k] = run;
-    run += x;
-  }
-  __syncthreads();
+  const int total = block_scan(v, count, part);
   for (int b = threadIdx.x; b < nbins; b += 1024) start[b] = v[(size_t)b * ntiles];
-  if (threadIdx.x == 0) start[nbins] = part[1023];
+  if (threadIdx.x == 0) start[nbins] = total;
 }
 
 __global__ void __launch_bounds__(256) far_scatter_kernel(int N, const unsigned short* __restrict__ tag, int nbins,

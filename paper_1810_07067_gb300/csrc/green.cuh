@@ -92,7 +92,33 @@ HD int green_smem_bytes(const GreenParams& gp) {
 __host__ __device__ void legendre_one(double rt, double dr, double dz, long long p, long long n, int Mq, int Ms,
                                       double* leg, const double* rinv, int nr);
 
+// Whether the pair (target r_t, displacement dr, dz) is split (mueller.cu, SplitTest).
+HD bool split_pair(double rt, double dr, double dz, double cthr) {
+  const double d2 = dr * dr + dz * dz, B = 2.0 * rt * (rt - dr);
+  return d2 < cthr * B;
+}
+
 // host-side launchers (green.cu)
+// doubles of the grid ladder's cosine tables, and of them with the sin^2 tables
+HD size_t ladder_cos_doubles(int qmax) { return qmax < 2 ? 0 : (size_t)4 * qmax * (qmax + 1) - 8; }
+HD size_t ladder_doubles(int qmax) {
+  return qmax < 2 ? 0 : ladder_cos_doubles(qmax) + (size_t)2 * qmax * (qmax + 1) - 4 + (qmax - 1);
+}
+// tab: cos(2 pi t / n_phi), sin^2(pi j / n_phi), then the ladder's cosines and sin^2
+// (the order and offsets of pair_grid)
+void launch_tables(const GreenParams& gp, double* tab, cudaStream_t s);
+// support points (r, z, r', z', weight, and the own panel's displacements, each
+// [n_panels * PTS_PER_PANEL], in that order in sup) from the nodes and the rules
+void launch_support_points(const BuildArgs& a, const double* dr, const double* dz, const double* wt_self,
+                           const double* wt_adj, double* sup, cudaStream_t s);
+// split far and support pairs and valid support points per row, then their
+// exclusive prefix sums (row[3N]: far splits, support splits after all far ones,
+// support points); counts: split pairs, support points
+void launch_split_count(const BuildArgs& a, double cthr, int* row, int* counts, cudaStream_t s);
+// ids of the split pairs (-1: not split), their (r_t, z_t, dr, dz), and the
+// support pairs listed by target and slot
+void launch_split_list(const BuildArgs& a, double cthr, const int* row, int* split_far, int* split_sup,
+                       double* pairs, int* sup_list, cudaStream_t s);
 void launch_legendre(const double* pairs, long long n_split, int Mq, int Ms, double* leg, cudaStream_t s);
 int far_tail_pairs(const GreenParams& gp);
 // elements of BuildArgs::tailq (return) and tailij (*ij_elems) for the launch of launch_far_assembly

@@ -1188,7 +1188,7 @@ size_t lu_z_pool_bytes(const int* n, int count, size_t most) {
 // changes rounding, so it is one for all matrices of a call.
 template <class T>
 static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s, LuTiming* tm, int* tc_err, int tile,
-                                  bool graph, const LuPool& pool) {
+                                  bool graph, const LuPool& pool, LuMat* dall) {
   if (count <= 0) return cudaSuccess;
   std::vector<LuMat> it(items, items + count);
   std::stable_sort(it.begin(), it.end(), [](const LuMat& a, const LuMat& b) { return a.n > b.n; });
@@ -1208,9 +1208,7 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
     }
   }
   groups.push_back(count);
-  LuMat* dall = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&dall, sizeof(LuMat) * count, s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   cudaMemcpyAsync(dall, it.data(), sizeof(LuMat) * count, cudaMemcpyHostToDevice, s);
   lu_info_zero_kernel<<<(count + 255) / 256, 256, 0, s>>>(dall, count);
   if constexpr (c64) {
@@ -1358,11 +1356,9 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) {  // nothing of the capture ran: factor with direct launches instead
       cudaGetLastError();
-      cudaFreeAsync(dall, s);
-      return lu_factor_impl<T>(items, count, s, tm, tc_err, tile, false, pool);
+      return lu_factor_impl<T>(items, count, s, tm, tc_err, tile, false, pool, dall);
     }
   }
-  cudaFreeAsync(dall, s);
   if (tm) {
     tm->launches += launches;
     tm->gemm_flops += gemm_flops;
@@ -1382,23 +1378,23 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
 }
 
 cudaError_t lu_factor_many(const LuMat* items, int count, bool c64, cudaStream_t s, LuTiming* tm, int* tc_err,
-                           int tile, bool graph, const LuPool& pool) {
-  return c64 ? lu_factor_impl<cf>(items, count, s, tm, tc_err, tile, graph, pool)
-             : lu_factor_impl<cd>(items, count, s, tm, tc_err, 0, graph, pool);
+                           int tile, bool graph, const LuPool& pool, LuMat* table) {
+  return c64 ? lu_factor_impl<cf>(items, count, s, tm, tc_err, tile, graph, pool, table)
+             : lu_factor_impl<cd>(items, count, s, tm, tc_err, 0, graph, pool, table);
 }
 
 void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* tm, int* tc_err,
-                       const LuPool& pool) {
+                       const LuPool& pool, LuMat* table) {
   std::vector<LuMat> it(batch);
   for (int b = 0; b < batch; ++b) it[b] = LuMat{A + (size_t)b * n * n, piv + (size_t)b * n, info + b, nullptr, n, 0};
-  lu_factor_impl<cd>(it.data(), batch, s, tm, tc_err, 0, false, pool);
+  lu_factor_impl<cd>(it.data(), batch, s, tm, tc_err, 0, false, pool, table);
 }
 
 void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* tm,
-                           int* tc_err, void* ws, int tile) {
+                           int* tc_err, void* ws, LuMat* table, int tile) {
   std::vector<LuMat> it(batch);
   for (int b = 0; b < batch; ++b)
     it[b] = LuMat{A + (size_t)b * n * n, piv + (size_t)b * n, info + b,
                   (__nv_bfloat16*)ws + tcu_ws_matrix_elems(n) * b, n, 0};
-  lu_factor_impl<cf>(it.data(), batch, s, tm, tc_err, tile, false, LuPool{});
+  lu_factor_impl<cf>(it.data(), batch, s, tm, tc_err, tile, false, LuPool{}, table);
 }

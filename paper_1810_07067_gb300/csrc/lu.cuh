@@ -27,8 +27,10 @@ struct LuPool {
 };
 size_t lu_z_pool_bytes(const int* n, int count, size_t most);
 // tc_err (device int, may be null) is set if a bounded wait gives up.
+// table: device room for the call's matrix table (batch entries).
+struct LuMat;
 void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* t, int* tc_err,
-                       const LuPool& pool);
+                       const LuPool& pool, LuMat* table);
 // The same factorization in complex64 (mixed-precision path).
 // The trailing updates run on tensor cores (tcgen05, split-BF16); ws is a
 // device workspace of lu_c64_workspace_bytes(n, batch) bytes (256-byte
@@ -36,7 +38,7 @@ void lu_factor_batched(cd* A, int n, int batch, int* piv, int* info, cudaStream_
 // tile: column tile of the update (32, 64 or 128), 0 = autotuned per step.
 size_t lu_c64_workspace_bytes(int n, int batch);
 void lu_factor_batched_c64(cf* A, int n, int batch, int* piv, int* info, cudaStream_t s, LuTiming* t, int* tc_err,
-                           void* ws, int tile = 0);
+                           void* ws, LuMat* table, int tile = 0);
 
 // One matrix of a (possibly ragged) batched factorization: A is n x n
 // column-major (complex128 or complex64), piv [n], info [1]; ws is its own
@@ -55,7 +57,7 @@ struct LuMat {
 // captured into a CUDA graph and launched once on s.  Returns the first CUDA
 // error (cudaSuccess when every launch was issued).
 cudaError_t lu_factor_many(const LuMat* items, int count, bool c64, cudaStream_t s, LuTiming* t, int* tc_err,
-                           int tile, bool graph, const LuPool& pool);
+                           int tile, bool graph, const LuPool& pool, LuMat* table);
 // The autotuner's decisions so far: per entry the upper end of its trailing-size
 // bucket, of its matrix-count bucket, the tile chosen and the measured ms per
 // matrix of tiles 32, 64, 128 (ms[3k..3k+2]); returns the number of entries.

@@ -8,9 +8,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <list>
 #include <map>
 #include <mutex>
-#include <thread>
 #include <tuple>
 #include <vector>
 
@@ -72,6 +72,9 @@ struct Rules {
   std::vector<double> self_u, self_w;   // reference self rule on [0, 1]
   std::vector<double> adj_u, adj_w;     // reference adjacent rule on [0, 1] at corners (graded composite)
   std::vector<double> adjs_u, adjs_w;   // reference adjacent rule on [0, 1] at smooth junctions
+  // interpolation rows and weights of the support points (eq. eq_nyslike2): own
+  // panel [target][SELF_PTS], neighbours [rule][end][ADJ_PTS]; L rows of 16, end rows
+  std::vector<double> Lself, Ladj, wt_self, wt_adj, Lm1, Lp1;
 };
 
 // Reference rule on [0, 1] graded toward 0: intervals [4^-(j+1), 4^-j] and
@@ -89,6 +92,8 @@ static void graded_rule(int levels, int ng, std::vector<double>& u, std::vector<
   }
 }
 
+static void lagrange_row(const Rules& R, double t, double* L);
+
 static Rules make_rules() {
   Rules R;
   gauss_legendre(P_NODES, R.x16, R.w16);
@@ -100,6 +105,37 @@ static Rules make_rules() {
   graded_rule(5, 16, R.adj_u, R.adj_w);
   R.adjs_u.assign(MUELLER_ADJ_U, MUELLER_ADJ_U + MUELLER_ADJ_SMOOTH);
   R.adjs_w.assign(MUELLER_ADJ_W, MUELLER_ADJ_W + MUELLER_ADJ_SMOOTH);
+  const int ns = (int)R.self_u.size();
+  R.Lself.assign((size_t)P_NODES * SELF_PTS * P_NODES, 0.0);
+  R.wt_self.assign((size_t)P_NODES * SELF_PTS, 0.0);
+  for (int a = 0; a < P_NODES; ++a) {
+    const double ti = R.x16[a], Lm = ti + 1.0, Lp = 1.0 - ti;
+    for (int s = 0; s < ns; ++s) {
+      const int k0 = a * SELF_PTS + s, k1 = k0 + ns;
+      R.wt_self[k0] = Lm * R.self_w[s];
+      R.wt_self[k1] = Lp * R.self_w[s];
+      lagrange_row(R, ti - Lm * R.self_u[s], &R.Lself[(size_t)k0 * P_NODES]);
+      lagrange_row(R, ti + Lp * R.self_u[s], &R.Lself[(size_t)k1 * P_NODES]);
+    }
+  }
+  // neighbouring panels: per rule (0 smooth junction, 1 corner) and panel end
+  // (0: tau = -1, 1: tau = +1), points tau = -1 + 2u or 1 - 2u
+  R.Ladj.assign((size_t)4 * ADJ_PTS * P_NODES, 0.0);
+  R.wt_adj.assign((size_t)4 * ADJ_PTS, 0.0);
+  for (int rule = 0; rule < 2; ++rule) {
+    const std::vector<double>& u = rule ? R.adj_u : R.adjs_u;
+    const std::vector<double>& w = rule ? R.adj_w : R.adjs_w;
+    for (int e = 0; e < 2; ++e)
+      for (size_t s = 0; s < u.size(); ++s) {
+        const size_t k = (size_t)(rule * 2 + e) * ADJ_PTS + s;
+        R.wt_adj[k] = 2.0 * w[s];
+        lagrange_row(R, e == 0 ? -1.0 + 2.0 * u[s] : 1.0 - 2.0 * u[s], &R.Ladj[k * P_NODES]);
+      }
+  }
+  R.Lm1.resize(P_NODES);
+  R.Lp1.resize(P_NODES);
+  lagrange_row(R, -1.0, R.Lm1.data());
+  lagrange_row(R, 1.0, R.Lp1.data());
   return R;
 }
 
@@ -131,13 +167,9 @@ struct Setup {
   int refine_max_iter = 10;
   cd k0{}, k1{}, eps0{}, mu0{}, eps1{}, mu1{};
   std::vector<double> r, z, rp, zp, w, sw;                  // nodes
-  std::vector<double> sr, sz, srp, szp, sW;                 // support points
-  std::vector<double> sdr, sdz;                             // own-panel: target - point
-  std::vector<double> Lself, Ladj;
+  std::vector<double> dr, dz;                               // tangents with respect to tau
   std::vector<int> adj_rule, adj_n;    // [nP][2]: rule (0 smooth, 1 corner) and point count of each panel end
-  std::vector<int> split_far, split_sup;
-  std::vector<double> split_pairs;                          // [n_split][4]
-  long long n_far = 0, n_sup = 0;
+  long long n_far = 0;
   GreenParams gp{};
   AsmParams ap{};
   cd sE{}, sH{};
@@ -185,25 +217,8 @@ struct SplitTest {
     const double sh = std::sinh(0.5 * (-std::log(eps) / span));
     cthr = 2.0 * sh * sh;
   }
-  bool operator()(double rt, double dr, double dz) const {
-    const double d2 = dr * dr + dz * dz, B = 2.0 * rt * (rt - dr);
-    return d2 < cthr * B;
-  }
+  bool operator()(double rt, double dr, double dz) const { return split_pair(rt, dr, dz, cthr); }
 };
-
-// Runs body(lo, hi) over [0, count) in contiguous chunks on up to 16 host threads.
-template <class F>
-static void parallel_chunks(int count, const F& body) {
-  const int hw = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-  const int nt = std::max(1, std::min(hw, count / 4));
-  if (nt == 1) { body(0, count); return; }
-  std::vector<std::thread> th;
-  for (int t = 0; t < nt; ++t) {
-    const int lo = (int)((long long)count * t / nt), hi = (int)((long long)count * (t + 1) / nt);
-    th.emplace_back([&body, lo, hi] { body(lo, hi); });
-  }
-  for (auto& x : th) x.join();
-}
 
 static int setup_inputs(const mueller_curve* cv, const mueller_media* md, int M, const mueller_options* op,
                         Setup& S) {
@@ -234,6 +249,7 @@ static int setup_inputs(const mueller_curve* cv, const mueller_media* md, int M,
   S.k1 = md->omega * csqrt_im_nonneg(S.eps1 * S.mu1);
   const int N = S.N;
   S.r.assign(cv->r, cv->r + N); S.z.assign(cv->z, cv->z + N);
+  S.dr.assign(cv->dr, cv->dr + N); S.dz.assign(cv->dz, cv->dz + N);
   S.rp.resize(N); S.zp.resize(N); S.w.resize(N); S.sw.resize(N);
   double area = 0.0;
   S.rmax = 0.0;
@@ -278,47 +294,16 @@ static int setup_inputs(const mueller_curve* cv, const mueller_media* md, int M,
   return MUELLER_OK;
 }
 
-// Support points and interpolation tables (eq. eq_nyslike2).
-static void setup_support(const mueller_curve* cv, Setup& S) {
+// Rules of the panel ends: junction j joins panel j's end +1 and panel j+1's end
+// -1 (the last one wraps for closed curves), a corner when the two end
+// tangents, from the panels' degree-15 interpolants of (dr, dz), differ by more
+// than 10 degrees.  The support points themselves and the split of the pairs
+// are formed on the device (launch_support_points, launch_split_count).
+static void setup_support(Setup& S) {
   const Rules& R = rules();
-  const int ns = (int)R.self_u.size();
-  S.Lself.assign((size_t)P_NODES * SELF_PTS * P_NODES, 0.0);
-  std::vector<double> tau_self((size_t)P_NODES * SELF_PTS), wt_self((size_t)P_NODES * SELF_PTS);
-  for (int a = 0; a < P_NODES; ++a) {
-    double ti = R.x16[a], Lm = ti + 1.0, Lp = 1.0 - ti;
-    for (int s = 0; s < ns; ++s) {
-      tau_self[a * SELF_PTS + s] = ti - Lm * R.self_u[s];
-      wt_self[a * SELF_PTS + s] = Lm * R.self_w[s];
-      tau_self[a * SELF_PTS + ns + s] = ti + Lp * R.self_u[s];
-      wt_self[a * SELF_PTS + ns + s] = Lp * R.self_w[s];
-    }
-    for (int s = 0; s < SELF_PTS; ++s)
-      lagrange_row(R, tau_self[a * SELF_PTS + s], &S.Lself[((size_t)a * SELF_PTS + s) * P_NODES]);
-  }
-  // neighbouring panels: per rule (0 smooth junction, 1 corner) and panel end
-  // (0: tau = -1, 1: tau = +1), points tau = -1 + 2u or 1 - 2u
-  std::vector<double> tau_adj(4 * ADJ_PTS, 0.0), wt_adj(4 * ADJ_PTS, 0.0);
-  S.Ladj.assign((size_t)4 * ADJ_PTS * P_NODES, 0.0);
-  for (int rule = 0; rule < 2; ++rule) {
-    const std::vector<double>& u = rule ? R.adj_u : R.adjs_u;
-    const std::vector<double>& w = rule ? R.adj_w : R.adjs_w;
-    for (int e = 0; e < 2; ++e)
-      for (size_t s = 0; s < u.size(); ++s) {
-        const size_t k = (size_t)(rule * 2 + e) * ADJ_PTS + s;
-        tau_adj[k] = e == 0 ? -1.0 + 2.0 * u[s] : 1.0 - 2.0 * u[s];
-        wt_adj[k] = 2.0 * w[s];
-        lagrange_row(R, tau_adj[k], &S.Ladj[k * P_NODES]);
-      }
-  }
-  // junction j joins panel j's end +1 and panel j+1's end -1 (the last one
-  // wraps for closed curves): a corner when the two end tangents, from the
-  // panels' degree-15 interpolants of (dr, dz), differ by more than 10 degrees
-  std::vector<double> Lm1(P_NODES), Lp1(P_NODES);
-  lagrange_row(R, -1.0, Lm1.data());
-  lagrange_row(R, 1.0, Lp1.data());
   auto tangent = [&](int Q, const std::vector<double>& L, double* t) {
     t[0] = t[1] = 0.0;
-    for (int k = 0; k < P_NODES; ++k) { t[0] += L[k] * cv->dr[Q * P_NODES + k]; t[1] += L[k] * cv->dz[Q * P_NODES + k]; }
+    for (int k = 0; k < P_NODES; ++k) { t[0] += L[k] * S.dr[Q * P_NODES + k]; t[1] += L[k] * S.dz[Q * P_NODES + k]; }
   };
   const int wrap = S.closed && S.nP > 2;
   S.adj_rule.assign((size_t)2 * S.nP, -1);
@@ -326,198 +311,102 @@ static void setup_support(const mueller_curve* cv, Setup& S) {
   for (int j = 0; j < S.nP - 1 + wrap; ++j) {
     const int A = j, B = (j + 1) % S.nP;
     double ta[2], tb[2];
-    tangent(A, Lp1, ta);
-    tangent(B, Lm1, tb);
+    tangent(A, R.Lp1, ta);
+    tangent(B, R.Lm1, tb);
     const double c = (ta[0] * tb[0] + ta[1] * tb[1]) / (std::hypot(ta[0], ta[1]) * std::hypot(tb[0], tb[1]));
     const int rule = c < 0.98480775301220806 ? 1 : 0;  // cos 10 degrees
     const int n = rule ? (int)R.adj_u.size() : (int)R.adjs_u.size();
     S.adj_rule[2 * A + 1] = rule; S.adj_n[2 * A + 1] = n;
     S.adj_rule[2 * B + 0] = rule; S.adj_n[2 * B + 0] = n;
   }
-  const size_t npts = (size_t)S.nP * PTS_PER_PANEL;
-  S.sr.resize(npts); S.sz.resize(npts); S.srp.resize(npts); S.szp.resize(npts); S.sW.resize(npts);
-  S.sdr.assign(npts, 0.0); S.sdz.assign(npts, 0.0);
-  parallel_chunks(S.nP, [&](int q_lo, int q_hi) {
-  for (int Q = q_lo; Q < q_hi; ++Q) {
-    const double* r = cv->r + Q * P_NODES;
-    const double* z = cv->z + Q * P_NODES;
-    const double* dr = cv->dr + Q * P_NODES;
-    const double* dz = cv->dz + Q * P_NODES;
-    for (int t = 0; t < PTS_PER_PANEL; ++t) {
-      const double* L;
-      double wt;
-      if (t < P_NODES * SELF_PTS) { L = &S.Lself[(size_t)t * P_NODES]; wt = wt_self[t]; }
-      else {
-        const int e = (t - P_NODES * SELF_PTS) / ADJ_PTS, s = (t - P_NODES * SELF_PTS) % ADJ_PTS;
-        const int rule = S.adj_rule[2 * Q + e];
-        if (rule < 0 || s >= S.adj_n[2 * Q + e]) {  // no neighbour at this end, or beyond the rule's points
-          const size_t id = (size_t)Q * PTS_PER_PANEL + t;
-          S.sr[id] = S.sz[id] = S.srp[id] = S.szp[id] = S.sW[id] = 0.0;
-          continue;
-        }
-        const size_t k = (size_t)(rule * 2 + e) * ADJ_PTS + s;
-        L = &S.Ladj[k * P_NODES]; wt = wt_adj[k];
-      }
-      double vr = 0, vz = 0, vdr = 0, vdz = 0;
-      for (int k = 0; k < P_NODES; ++k) {
-        vr += L[k] * r[k]; vz += L[k] * z[k]; vdr += L[k] * dr[k]; vdz += L[k] * dz[k];
-      }
-      double sp = std::hypot(vdr, vdz);
-      size_t id = (size_t)Q * PTS_PER_PANEL + t;
-      S.sr[id] = vr; S.sz[id] = vz; S.srp[id] = vdr / sp; S.szp[id] = vdz / sp; S.sW[id] = wt * sp;
-      if (t < P_NODES * SELF_PTS) {
-        // own-panel point of target a: x_t - x_s = -sum_{k != a} L_k(tau_s) (x_k - x_a)
-        int a = t / SELF_PTS;
-        double ddr = 0.0, ddz = 0.0;
-        for (int k = 0; k < P_NODES; ++k) {
-          if (k == a) continue;
-          ddr -= L[k] * (r[k] - r[a]);
-          ddz -= L[k] * (z[k] - z[a]);
-        }
-        S.sdr[id] = ddr; S.sdz[id] = ddz;
-      }
-    }
-  }
-  });
-}
-
-static bool near_panels_h(int Pi, int Pj, int nP, int closed) {
-  int d = Pi - Pj;
-  if (d >= -1 && d <= 1) return true;
-  if (closed && nP > 2 && (d == nP - 1 || d == -(nP - 1))) return true;
-  return false;
-}
-
-static long long support_pid(const Setup& S, int i, int slot) {
-  int P = i / P_NODES, loc = i % P_NODES;
-  if (slot < SELF_PTS) return (long long)P * PTS_PER_PANEL + loc * SELF_PTS + slot;
-  if (slot < SELF_PTS + ADJ_PTS) {
-    int Q = P - 1;
-    if (Q < 0) { if (!S.closed) return -1; Q = S.nP - 1; }
-    if (slot - SELF_PTS >= S.adj_n[2 * Q + 1]) return -1;  // beyond the rule of Q's end +1
-    return (long long)Q * PTS_PER_PANEL + P_NODES * SELF_PTS + ADJ_PTS + (slot - SELF_PTS);
-  }
-  int Q = P + 1;
-  if (Q >= S.nP) { if (!S.closed) return -1; Q = 0; }
-  if (slot - SELF_PTS - ADJ_PTS >= S.adj_n[2 * Q + 0]) return -1;  // beyond the rule of Q's end -1
-  return (long long)Q * PTS_PER_PANEL + P_NODES * SELF_PTS + (slot - SELF_PTS - ADJ_PTS);
-}
-
-// Split pairs get ids in a fixed order: far pairs (i, j) row-major, then
-// support pairs (i, slot) row-major.  Rows are classified on host threads
-// (flags and per-row counts), then numbered from the prefix sums.
-static void setup_pairs(Setup& S) {
-  const int N = S.N;
-  const SplitTest split(S.nphi, S.M, S.split_eps);
-  S.split_far.assign((size_t)N * N, -1);
-  S.split_sup.assign((size_t)N * NEAR_SLOTS, -1);
-  std::vector<long long> cnt_far(N + 1, 0), cnt_sup(N + 1, 0), nfar(N, 0), nsup(N, 0);
-  auto sup_disp = [&](int i, int slot, long long pid, double* dr, double* dz) {
-    if (slot < SELF_PTS) { *dr = S.sdr[pid]; *dz = S.sdz[pid]; }
-    else { *dr = S.r[i] - S.sr[pid]; *dz = S.z[i] - S.sz[pid]; }
-  };
-  parallel_chunks(N, [&](int lo, int hi) {
-    for (int i = lo; i < hi; ++i) {
-      long long cf = 0, cs = 0;
-      for (int j = 0; j < N; ++j) {
-        if (near_panels_h(i / P_NODES, j / P_NODES, S.nP, S.closed)) continue;
-        ++nfar[i];
-        if (split(S.r[i], S.r[i] - S.r[j], S.z[i] - S.z[j])) { S.split_far[(size_t)i * N + j] = 0; ++cf; }
-      }
-      for (int slot = 0; slot < NEAR_SLOTS; ++slot) {
-        long long pid = support_pid(S, i, slot);
-        if (pid < 0) continue;
-        ++nsup[i];
-        double dr, dz;
-        sup_disp(i, slot, pid, &dr, &dz);
-        if (split(S.r[i], dr, dz)) { S.split_sup[(size_t)i * NEAR_SLOTS + slot] = 0; ++cs; }
-      }
-      cnt_far[i + 1] = cf;
-      cnt_sup[i + 1] = cs;
-    }
-  });
-  for (int i = 0; i < N; ++i) cnt_far[i + 1] += cnt_far[i];
-  cnt_sup[0] = cnt_far[N];
-  for (int i = 0; i < N; ++i) cnt_sup[i + 1] += cnt_sup[i];
-  S.n_far = 0; S.n_sup = 0;
-  for (int i = 0; i < N; ++i) { S.n_far += nfar[i]; S.n_sup += nsup[i]; }
-  S.split_pairs.assign((size_t)cnt_sup[N] * 4, 0.0);
-  parallel_chunks(N, [&](int lo, int hi) {
-    for (int i = lo; i < hi; ++i) {
-      long long id = cnt_far[i];
-      for (int j = 0; j < N; ++j) {
-        int& f = S.split_far[(size_t)i * N + j];
-        if (f < 0) continue;
-        f = (int)id;
-        const double v[4] = {S.r[i], S.z[i], S.r[i] - S.r[j], S.z[i] - S.z[j]};
-        std::copy(v, v + 4, &S.split_pairs[(size_t)id * 4]);
-        ++id;
-      }
-      id = cnt_sup[i];
-      for (int slot = 0; slot < NEAR_SLOTS; ++slot) {
-        int& f = S.split_sup[(size_t)i * NEAR_SLOTS + slot];
-        if (f < 0) continue;
-        f = (int)id;
-        double dr, dz;
-        sup_disp(i, slot, support_pid(S, i, slot), &dr, &dz);
-        const double v[4] = {S.r[i], S.z[i], dr, dz};
-        std::copy(v, v + 4, &S.split_pairs[(size_t)id * 4]);
-        ++id;
-      }
-    }
-  });
+  long long near = 0;  // near panels of all panels: itself and its neighbours
+  for (int P = 0; P < S.nP; ++P) near += 1 + (P > 0 || wrap) + (P + 1 < S.nP || wrap);
+  S.n_far = (long long)S.N * S.N - near * P_NODES * P_NODES;
 }
 
 // ---------------------------------------------------------------- device staging
-// Process-wide cache of freed device blocks.  Builds allocate and free
-// buffers of several GB (matrices, complex64 copies, residual slices, spectra
-// scratch), and mapping or unmapping one costs milliseconds; released blocks
-// of at least 64 MiB are kept, per device, up to a cap (32 GiB by default,
-// mueller_cache_limit) and handed out again for a request of the same size
-// (rounded up to 2 MiB).  Releasing synchronizes the device first, as
-// cudaFree does, so no kernel still uses a block when it is reused.  When an
-// allocation fails the cache is emptied and the allocation retried.
+// Process-wide cache of freed device blocks, per device.  A build, a solve or a
+// field evaluation takes tens of buffers, and a cudaMalloc, a cudaFree or the
+// mapping of several GB costs tens of microseconds to milliseconds each (the
+// N = 64 sphere: 1.5 of 7.5 ms); released blocks are handed out again for
+// requests of the same rounded size.  Blocks of at least 64 MiB are rounded up to
+// 2 MiB and kept up to a cap (32 GiB by default, mueller_cache_limit); smaller ones
+// are rounded up to a quarter of their power of two and kept up to 256 MiB (none
+// when the cap is 0); beyond its cap a kind gives up what was released longest ago.  Releasing synchronizes the device first, once per group of
+// buffers, as cudaFree does for each, so no kernel of any stream still uses a
+// block when it is reused.  When an allocation fails the cache is emptied and the
+// allocation retried; mueller_cache_trim empties it too.
 namespace devcache {
-constexpr size_t kMinBlock = (size_t)64 << 20, kRound = (size_t)2 << 20;
+constexpr size_t kMinBlock = (size_t)64 << 20, kRound = (size_t)2 << 20, kSmallCap = (size_t)256 << 20;
+struct Block {
+  int dev;
+  size_t bytes;
+  void* p;
+};
+// big (0) and small (1) blocks, least recently released first
 std::mutex mu;
-std::multimap<std::pair<int, size_t>, void*> blocks;  // (device, bytes) -> block
-size_t cached = 0, cap = (size_t)32 << 30;
+std::list<Block> blocks[2];
+size_t held[2] = {0, 0}, cap = (size_t)32 << 30;
 
-inline size_t rounded(size_t b) { return (b + kRound - 1) / kRound * kRound; }
+inline size_t rounded(size_t b) {
+  if (b >= kMinBlock) return (b + kRound - 1) / kRound * kRound;
+  if (b <= 512) return 512;
+  size_t q = 128;  // a quarter of the largest power of two up to b
+  while (q * 8 <= b) q *= 2;
+  return (b + q - 1) / q * q;
+}
 
-void trim() {
-  std::lock_guard<std::mutex> capture(lu_capture_mutex());
-  std::lock_guard<std::mutex> lk(mu);
+// Takes blocks off the front until at most `most` bytes of the kind are held (mu held).
+void take_over(int kind, size_t most, std::vector<Block>& out) {
+  while (held[kind] > most) {
+    out.push_back(blocks[kind].front());
+    held[kind] -= out.back().bytes;
+    blocks[kind].pop_front();
+  }
+}
+
+void free_blocks(const std::vector<Block>& v) {
   int cur = 0;
   cudaGetDevice(&cur);
-  for (auto& e : blocks) {
-    cudaSetDevice(e.first.first);
-    cudaFree(e.second);
+  for (const Block& b : v) {
+    if (b.dev != cur) cudaSetDevice(b.dev);
+    cudaFree(b.p);
+    if (b.dev != cur) cudaSetDevice(cur);
   }
-  cudaSetDevice(cur);
-  blocks.clear();
-  cached = 0;
 }
+
+void shrink(size_t most_big, size_t most_small) {
+  std::lock_guard<std::mutex> capture(lu_capture_mutex());
+  std::vector<Block> out;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    take_over(0, most_big, out);
+    take_over(1, most_small, out);
+  }
+  free_blocks(out);
+}
+
+void trim() { shrink(0, 0); }
 
 size_t bytes_held() {
   std::lock_guard<std::mutex> lk(mu);
-  return cached;
+  return held[0] + held[1];
 }
 
 cudaError_t alloc(void** p, size_t bytes) {
-  const bool big = bytes >= kMinBlock;
-  const size_t req = big ? rounded(bytes) : bytes;
-  if (big) {
-    int dev = 0;
-    cudaGetDevice(&dev);
+  const size_t req = rounded(bytes);
+  const int kind = req >= kMinBlock ? 0 : 1;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  {
     std::lock_guard<std::mutex> lk(mu);
-    auto it = blocks.find({dev, req});
-    if (it != blocks.end()) {
-      *p = it->second;
-      blocks.erase(it);
-      cached -= req;
-      return cudaSuccess;
-    }
+    for (auto it = blocks[kind].rbegin(); it != blocks[kind].rend(); ++it)
+      if (it->bytes == req && it->dev == dev) {
+        *p = it->p;
+        held[kind] -= req;
+        blocks[kind].erase(std::next(it).base());
+        return cudaSuccess;
+      }
   }
   cudaError_t e = cudaMalloc(p, req);
   if (e != cudaSuccess && bytes_held() > 0) {
@@ -528,22 +417,27 @@ cudaError_t alloc(void** p, size_t bytes) {
   return e;
 }
 
-void release(void* p, size_t bytes) {
-  if (!p) return;
+// Gives back buffers (pointer, requested bytes) of the current device; blocks
+// beyond the caps leave, the least recently released first.
+void release(const std::pair<void*, size_t>* bufs, size_t count) {
+  if (count == 0) return;
   std::lock_guard<std::mutex> capture(lu_capture_mutex());
-  if (bytes >= kMinBlock) {
-    const size_t req = rounded(bytes);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceSynchronize();
+  int dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceSynchronize();
+  std::vector<Block> out;
+  {
     std::lock_guard<std::mutex> lk(mu);
-    if (cached + req <= cap) {
-      blocks.insert({{dev, req}, p});
-      cached += req;
-      return;
+    for (size_t k = 0; k < count; ++k) {
+      const size_t req = rounded(bufs[k].second);
+      const int kind = req >= kMinBlock ? 0 : 1;
+      blocks[kind].push_back(Block{dev, req, bufs[k].first});
+      held[kind] += req;
     }
+    take_over(0, cap, out);
+    take_over(1, cap > 0 ? kSmallCap : 0, out);
   }
-  cudaFree(p);
+  free_blocks(out);
 }
 }  // namespace devcache
 
@@ -556,7 +450,7 @@ extern "C" size_t mueller_cache_limit(size_t bytes) {
     old = devcache::cap;
     devcache::cap = bytes;
   }
-  if (devcache::bytes_held() > bytes) devcache::trim();
+  devcache::shrink(bytes, bytes > 0 ? devcache::kSmallCap : 0);
   return old;
 }
 
@@ -564,7 +458,7 @@ extern "C" size_t mueller_cache_bytes(void) { return devcache::bytes_held(); }
 
 struct DevBuf {
   std::vector<std::pair<void*, size_t>> ptrs;
-  ~DevBuf() { for (auto& e : ptrs) devcache::release(e.first, e.second); }
+  ~DevBuf() { devcache::release(ptrs.data(), ptrs.size()); }
   template <class T>
   cudaError_t alloc(T** p, size_t count) {
     const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
@@ -580,7 +474,7 @@ struct DevBuf {
   void release(void* p) {  // give one buffer back before the others
     for (size_t k = 0; k < ptrs.size(); ++k)
       if (ptrs[k].first == p) {
-        devcache::release(p, ptrs[k].second);
+        devcache::release(&ptrs[k], 1);
         ptrs.erase(ptrs.begin() + k);
         return;
       }
@@ -848,33 +742,20 @@ static size_t assembly_scratch_bytes(int N, int M) {
 // Support spectra: on the tensor cores (sampling, digit rows, one real product
 // per chunk of pairs, spectra) when the half grid fits one exact product
 // (n_phi / 2 + 1 <= OZR_KMAX samples), else the warp-per-pair kernel.
-static int support_spectra(const Setup& S, BuildArgs& a, DevBuf& tmp, int** err_out, cudaStream_t s) {
+static int support_spectra(const Setup& S, BuildArgs& a, const int* dlist, int total, DevBuf& tmp, int** err_out,
+                           cudaStream_t s) {
   const int H = S.gp.H, Ms = S.gp.Ms;
   if (H > OZR_KMAX) {
     launch_support_spectra(a, s);
     return MUELLER_OK;
   }
-  std::vector<int> list;
-  list.reserve((size_t)S.N * (SELF_PTS + 2 * 32));
-  for (int i = 0; i < S.N; ++i) {
-    const int P = i / P_NODES;
-    for (int slot = 0; slot < NEAR_SLOTS; ++slot) {
-      if (support_pid(S, i, slot) < 0) continue;
-      // the device skips the wrap-around neighbour of a closed curve of one or two panels
-      if (slot >= SELF_PTS && S.closed && S.nP <= 2 &&
-          ((slot < SELF_PTS + ADJ_PTS && P == 0) || (slot >= SELF_PTS + ADJ_PTS && P == S.nP - 1)))
-        continue;
-      list.push_back(i * NEAR_SLOTS + slot);
-    }
-  }
-  if (list.empty()) return MUELLER_OK;
   const int nkt = (H + 15) / 16;
   const int rows_pad = (SUP_TC_CHUNK * 2 * NFAM + 127) / 128 * 128;
-  int* dlist = nullptr;
+  if (total == 0) return MUELLER_OK;
   __nv_bfloat16* Asl = nullptr;
   double *Ascale = nullptr, *Y = nullptr;
   int* err = nullptr;
-  if (tmp.upload(&dlist, list, s) != cudaSuccess || tmp.alloc(&Asl, ozaki_real_a_elems(rows_pad, nkt)) != cudaSuccess ||
+  if (tmp.alloc(&Asl, ozaki_real_a_elems(rows_pad, nkt)) != cudaSuccess ||
       tmp.alloc(&Ascale, (size_t)rows_pad) != cudaSuccess || tmp.alloc(&Y, (size_t)Ms * rows_pad) != cudaSuccess ||
       tmp.alloc(&err, 1) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "support transform scratch");
@@ -885,7 +766,6 @@ static int support_spectra(const Setup& S, BuildArgs& a, DevBuf& tmp, int** err_
     if (rc != MUELLER_OK) return rc;
   }
   CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  const int total = (int)list.size();
   for (int q0 = 0; q0 < total; q0 += SUP_TC_CHUNK) {
     const int cnt = std::min(SUP_TC_CHUNK, total - q0);
     const int rows = cnt * 2 * NFAM, rp = (rows + 127) / 128 * 128;
@@ -923,36 +803,45 @@ static int assemble_core(Setup& S, cd* A_dev, cudaStream_t s, mueller_stats* st,
   a.geo = NodeGeom{dr_, dz_, drp, dzp, dw, dsw, dirt, dwr};
   if (d_geo_out) { d_geo_out[0] = dr_; d_geo_out[1] = dz_; d_geo_out[2] = drp; d_geo_out[3] = dzp;
                    d_geo_out[4] = dw; d_geo_out[5] = dsw; }
-  double *ssr, *ssz, *ssrp, *sszp, *ssW, *sLs, *sLa, *dcos, *ds2, *dpairs, *dleg, *ssdr, *ssdz;
-  int *dsf, *dss;
-  CK(tmp.upload(&ssr, S.sr, s)); CK(tmp.upload(&ssz, S.sz, s)); CK(tmp.upload(&ssrp, S.srp, s));
-  CK(tmp.upload(&sszp, S.szp, s)); CK(tmp.upload(&ssW, S.sW, s));
-  CK(tmp.upload(&ssdr, S.sdr, s)); CK(tmp.upload(&ssdz, S.sdz, s));
-  CK(tmp.upload(&sLs, S.Lself, s)); CK(tmp.upload(&sLa, S.Ladj, s));
-  int *dadj_rule, *dadj_n;
+  const Rules& R = rules();
+  // tables by size: support points, grid ladder, full grid
+  const size_t npts = (size_t)S.nP * PTS_PER_PANEL, nlad = ladder_doubles(S.gp.qmax);
+  double *ddr, *ddz, *sLs, *sLa, *dws, *dwa, *dsup, *dtab, *dpairs = nullptr, *dleg;
+  int *dsf, *dss, *dadj_rule, *dadj_n, *drow, *dcounts;
+  CK(tmp.upload(&ddr, S.dr, s)); CK(tmp.upload(&ddz, S.dz, s));
+  CK(tmp.upload(&sLs, R.Lself, s)); CK(tmp.upload(&sLa, R.Ladj, s));
+  CK(tmp.upload(&dws, R.wt_self, s)); CK(tmp.upload(&dwa, R.wt_adj, s));
   CK(tmp.upload(&dadj_rule, S.adj_rule, s)); CK(tmp.upload(&dadj_n, S.adj_n, s));
-  CK(tmp.upload(&dcos, cos_table(S.nphi), s)); CK(tmp.upload(&ds2, s2_table(S.nphi), s));
-  double *dladC = nullptr, *dladS = nullptr;
-  if (S.gp.qmax >= 2) {
-    std::vector<double> lc, ls;
-    for (int q = 2; q <= S.gp.qmax; ++q) {
-      const std::vector<double> c = cos_table(8 * q), t = s2_table(8 * q);
-      lc.insert(lc.end(), c.begin(), c.end());
-      ls.insert(ls.end(), t.begin(), t.end());
-    }
-    CK(tmp.upload(&dladC, lc, s)); CK(tmp.upload(&dladS, ls, s));
-  }
-  CK(tmp.upload(&dsf, S.split_far, s)); CK(tmp.upload(&dss, S.split_sup, s));
-  CK(tmp.upload(&dpairs, S.split_pairs, s));
-  const long long n_split = (long long)S.split_pairs.size() / 4;
+  if (tmp.alloc(&dsup, 7 * npts) != cudaSuccess ||
+      tmp.alloc(&dtab, (size_t)S.nphi + S.nphi / 2 + 1 + nlad) != cudaSuccess ||
+      tmp.alloc(&dsf, (size_t)S.N * S.N) != cudaSuccess || tmp.alloc(&dss, (size_t)S.N * NEAR_SLOTS) != cudaSuccess ||
+      tmp.alloc(&drow, (size_t)3 * S.N) != cudaSuccess || tmp.alloc(&dcounts, 2) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "assembly tables");
+  a.sup = SupportTable{dsup, dsup + npts, dsup + 2 * npts, dsup + 3 * npts, dsup + 4 * npts, dsup + 5 * npts,
+                       dsup + 6 * npts, sLs, sLa, dadj_rule, dadj_n};
+  a.cosT = dtab; a.s2T = dtab + S.nphi;
+  double* lad = dtab + S.nphi + S.nphi / 2 + 1;
+  a.ladC = lad; a.ladS = lad + ladder_cos_doubles(S.gp.qmax);
+  a.split_far = dsf; a.split_sup = dss;
+  launch_tables(S.gp, dtab, s);
+  launch_support_points(a, ddr, ddz, dws, dwa, dsup, s);
+  // split pairs: ids in row order, far pairs first; counts: split pairs, support points
+  const double cthr = SplitTest(S.nphi, S.M, S.split_eps).cthr;
+  int counts[2] = {0, 0};
+  launch_split_count(a, cthr, drow, dcounts, s);
+  CK(cudaMemcpyAsync(counts, dcounts, sizeof(counts), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  const long long n_split = counts[0];
+  int* dsup_list;
   const int Ms = S.gp.Ms, Mq = S.gp.Mq;
-  if (tmp.alloc(&dleg, (size_t)(Mq + 1 + Ms) * n_split) != cudaSuccess)
+  if (tmp.alloc(&dpairs, (size_t)4 * n_split) != cudaSuccess || tmp.alloc(&dsup_list, (size_t)counts[1]) != cudaSuccess ||
+      tmp.alloc(&dleg, (size_t)(Mq + 1 + Ms) * n_split) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "Legendre scratch");
+  launch_split_list(a, cthr, drow, dsf, dss, dpairs, dsup_list, s);
   cd* dspec;
   if (tmp.alloc(&dspec, (size_t)S.N * NEAR_SLOTS * NFAM * Ms) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "support spectra scratch");
-  a.sup = SupportTable{ssr, ssz, ssrp, sszp, ssW, ssdr, ssdz, sLs, sLa, dadj_rule, dadj_n};
-  a.cosT = dcos; a.s2T = ds2; a.ladC = dladC; a.ladS = dladS; a.split_far = dsf; a.split_sup = dss; a.leg = dleg; a.n_split = n_split;
+  a.leg = dleg; a.n_split = n_split;
   a.spec_sup = dspec; a.A = A_dev;
   a.lneps = -std::log(S.split_eps);
   a.tq = S.gp.H > OZR_KMAX ? far_tail_pairs(S.gp) : 0;  // far_kernel only
@@ -979,7 +868,7 @@ static int assemble_core(Setup& S, cd* A_dev, cudaStream_t s, mueller_stats* st,
   T.mark();
   int* sup_err = nullptr;
   {
-    const int rc = support_spectra(S, a, tmp, &sup_err, s);
+    const int rc = support_spectra(S, a, dsup_list, counts[1], tmp, &sup_err, s);
     if (rc != MUELLER_OK) return rc;
   }
   T.mark();
@@ -997,7 +886,7 @@ static int assemble_core(Setup& S, cd* A_dev, cudaStream_t s, mueller_stats* st,
   if (st) ft.finish(st);
   if (st) {
     st->ms_legendre = T.ms(0, 1); st->ms_far = T.ms(1, 2); st->ms_support = T.ms(2, 3); st->ms_near = T.ms(3, 4);
-    st->n_phi_used = S.nphi; st->n_split_pairs = n_split; st->n_far_pairs = S.n_far; st->n_support_pairs = S.n_sup;
+    st->n_phi_used = S.nphi; st->n_split_pairs = n_split; st->n_far_pairs = S.n_far; st->n_support_pairs = counts[1];
   }
   return MUELLER_OK;
 }
@@ -1064,8 +953,7 @@ static int build_prepare(const mueller_curve* curve, const mueller_media* media,
   c->rec_r.assign(curve->r, curve->r + c->S.N); c->rec_z.assign(curve->z, curve->z + c->S.N);
   c->rec_dr.assign(curve->dr, curve->dr + c->S.N); c->rec_dz.assign(curve->dz, curve->dz + c->S.N);
   c->rec_media = *media; c->rec_opts = *opts;
-  setup_support(curve, c->S);
-  setup_pairs(c->S);
+  setup_support(c->S);
   const size_t n = c->S.n;
   const bool mixed = c->S.precision != 0;
   const bool slices = c->S.precision == 1;
@@ -1198,6 +1086,12 @@ extern "C" int mueller_build(const mueller_curve* curve, const mueller_media* me
   cudaEvent_t e1, e2;
   cudaEventCreate(&e1); cudaEventCreate(&e2);
   cudaEventRecord(e1, s);
+  LuMat* tab = nullptr;
+  if (wsb.alloc(&tab, (size_t)M + 1) != cudaSuccess) {
+    cudaEventDestroy(e1); cudaEventDestroy(e2);
+    delete c;
+    return fail(MUELLER_ENOMEM, "LU table");
+  }
   if (mixed) {
     unsigned char* ws = nullptr;
     if (wsb.alloc(&ws, lu_c64_workspace_bytes((int)n, M + 1)) != cudaSuccess) {
@@ -1205,11 +1099,11 @@ extern "C" int mueller_build(const mueller_curve* curve, const mueller_media* me
       delete c;
       return fail(MUELLER_ENOMEM, "tensor-core LU workspace");
     }
-    lu_factor_batched_c64(c->A32, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, ws, c->lu_tile);
+    lu_factor_batched_c64(c->A32, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, ws, tab, c->lu_tile);
   } else {
     const std::vector<int> ns(M + 1, (int)n);
     const LuPool pool = lu_z_pool(wsb, ns, assembly_scratch_bytes(c->S.N, M));
-    lu_factor_batched(c->A, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, pool);
+    lu_factor_batched(c->A, (int)n, M + 1, c->piv, c->info, s, &lt, c->tc_err, pool, tab);
   }
   cudaEventRecord(e2, s);
   cudaError_t err = cudaStreamSynchronize(s);
@@ -1267,11 +1161,13 @@ extern "C" int mueller_build_many(int count, const mueller_curve* curves, const 
   }
   // one table entry per (body, mode); a body's timeout flag is shared by the wave
   LuTiming lt;
+  LuMat* tab = nullptr;
+  if (wsb.alloc(&tab, items.size()) != cudaSuccess) return drop(fail(MUELLER_ENOMEM, "LU table"));
   cudaEvent_t e1, e2;
   cudaEventCreate(&e1); cudaEventCreate(&e2);
   cudaEventRecord(e1, s);
   cudaError_t err = lu_factor_many(items.data(), (int)items.size(), mixed, s, &lt, cs[0]->tc_err,
-                                   opts->lu_tile, true, pool);
+                                   opts->lu_tile, true, pool, tab);
   cudaEventRecord(e2, s);
   cudaError_t err2 = cudaStreamSynchronize(s);
   float b = 0;
@@ -1303,8 +1199,7 @@ extern "C" int mueller_assemble(const mueller_curve* curve, const mueller_media*
   Setup S;
   int rc = setup_inputs(curve, media, M, opts, S);
   if (rc) return rc;
-  setup_support(curve, S);
-  setup_pairs(S);
+  setup_support(S);
   DevBuf keep;
   return assemble_core(S, (cd*)A_dev, (cudaStream_t)stream, nullptr, keep, nullptr);
 }
@@ -1668,10 +1563,12 @@ extern "C" int mueller_lu_batched(mueller_c128* A_dev, int n, int batch, int* pi
   cudaStream_t s = (cudaStream_t)stream;
   DevBuf tmp;
   int* err = nullptr;
-  if (tmp.alloc(&err, 1) != cudaSuccess) return fail(MUELLER_ENOMEM, "LU status word");
+  LuMat* tab = nullptr;
+  if (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&tab, (size_t)batch) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "LU status word and table");
   CK(cudaMemsetAsync(err, 0, sizeof(int), s));
   const LuPool pool = lu_z_pool(tmp, std::vector<int>(batch, n), (size_t)4 << 30);
-  lu_factor_batched((cd*)A_dev, n, batch, piv_dev, info_dev, s, nullptr, err, pool);
+  lu_factor_batched((cd*)A_dev, n, batch, piv_dev, info_dev, s, nullptr, err, pool, tab);
   CK(cudaGetLastError());
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1688,10 +1585,12 @@ extern "C" int mueller_lu_batched_c64(mueller_c64* A_dev, int n, int batch, int*
   DevBuf tmp;
   int* err = nullptr;
   unsigned char* ws = nullptr;
-  if (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&ws, lu_c64_workspace_bytes(n, batch)) != cudaSuccess)
+  LuMat* tab = nullptr;
+  if (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&tab, (size_t)batch) != cudaSuccess ||
+      tmp.alloc(&ws, lu_c64_workspace_bytes(n, batch)) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "tensor-core LU workspace");
   CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  lu_factor_batched_c64((cf*)A_dev, n, batch, piv_dev, info_dev, s, nullptr, err, ws);
+  lu_factor_batched_c64((cf*)A_dev, n, batch, piv_dev, info_dev, s, nullptr, err, ws, tab);
   CK(cudaGetLastError());
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
