@@ -45,62 +45,91 @@ void upload_series_tables(const SeriesTables& t) { cudaMemcpyToSymbol(c_tab, &t,
 // pairs: [n][4] = (r_t, z_t, r_t - r_s, z_t - z_s); leg: [(Mq+1)+Ms][n] index-major:
 // rows 0..Mq hold P^_n = P_n / sqrt(B), rows Mq+1.. hold S^_m = S_m / B^{3/2}.
 // rinv[k] = 1 / (2k + 1) for k < nr (shared memory): the recurrences divide by
-// odd integers at every step, and FP64 division costs several dependent
-// operations, so the quotients are multiplications by the table's entries.
+// odd integers at every step.
+//
+// With c = chi - 1 and E_m = 2 D_m = 2 (P_{m-1} - P_m) the recurrence (2m+1) P_{m+1} = 4 m
+// chi P_m - (2m-1) P_{m-1} keeps the O(1) differences accurate when chi -> 1:
+//   up:   P_m = P_{m-1} - E_m / 2,  E_{m+1} = w - (w + E_m) / (2m + 1), w = E_m - 4 c P_m
+//   down: P_m = P_{m+1} + E_{m+1} / 2,  E_m = w + (w + E_{m+1}) / (2m - 1), w = E_{m+1} + 4 c P_m
+// four FP64 operations a step, on one serial chain per pair: the kernel is bound
+// by that chain when the pairs are few and by the FP64 pipe when they are many.
+// Downward (Miller) the start is arbitrary and its error, like every rounding on
+// the way, falls by zeta^2 a step: the steps from m* = M_q + 19.6 / l (l =
+// ln(1/zeta)) to M_q + 11.5 / l run in FP32, whose rounding of 6e-8 is below
+// 1e-17 at M_q; then FP64 to mode 0 for the normalisation P_0, and once more from
+// M_q with the normalised values, stored as they come. (One FP64 pass from m* with
+// a division a step and unscaled values rescaled in memory took 250 us for the
+// 64-node sphere; modal_kernels of 64 pairs as a whole fell from 311 to 157 us and
+// the sphere from 4.29 to 4.11 ms with this form.)
 __host__ __device__ void legendre_one(double rt, double dr, double dz, long long p, long long n, int Mq, int Ms,
                                       double* __restrict__ leg, const double* rinv, int nr) {
   auto inv_odd = [&](int k) { return k < nr ? rinv[k] : 1.0 / (2.0 * k + 1.0); };  // 1 / (2k + 1)
-  double rs = rt - dr;
-  double d2 = dr * dr + dz * dz, B = 2.0 * rt * rs;
-  double c = d2 / B, cp1 = 2.0 + c;          // chi - 1, chi + 1
-  double kp2 = c / cp1;
-  double K = ellipk_c(sqrt(kp2));
-  double E = ellipe_c(kp2);
-  double P0 = 4.0 * K / sqrt(cp1);
-  double lz = log1p(c + sqrt(c * cp1));      // -ln(zeta)
-  // Work with P_m and the differences D_m = P_{m-1} - P_m: the recurrence
-  // (2m+1) P_{m+1} = 4 m chi P_m - (2m-1) P_{m-1} becomes
-  // D_{m+1} = ((2m-1) D_m - 4 m c P_m) / (2m+1), P_{m+1} = P_m - D_{m+1},
-  // which keeps the O(1) differences accurate when chi -> 1.
-  double* Pv = leg;                                // rows 0..Mq: P_m, later P^_m
-  double* Sv = leg + (long long)(Mq + 1) * n;      // rows 0..Ms-1: D_m, later S^_m
+  const double rs = rt - dr;
+  const double d2 = dr * dr + dz * dz, B = 2.0 * rt * rs;
+  const double c = d2 / B, cp1 = 2.0 + c, c4 = 4.0 * c;  // chi - 1, chi + 1
+  double K, E;
+  ellipke(sqrt(c / cp1), &K, &E);
+  const double scp1 = sqrt(cp1), isB = 1.0 / sqrt(B), isB3 = isB * isB * isB;
+  const double P0 = 4.0 * K / scp1;
+  const double lz = log1p(c + sqrt(c) * scp1);  // -ln(zeta)
+  double* Pv = leg;                                // rows 0..Mq: P^_m
+  double* Sv = leg + (long long)(Mq + 1) * n;      // rows 0..Ms-1: S^_m
+  // S_m = (1 - 2m)(chi P_m - P_{m-1})/(chi^2 - 1) = (2m - 1)(D_m - c P_m)/(c (c + 2)), of P^ = P isB
+  const double sfac = 0.5 * isB * isB / (c * cp1), c2 = 2.0 * c;
+  Sv[p] = 4.0 * E / (c * scp1) * isB3;
   const double LN32 = 3.4657359027997265;
   if (2.0 * Mq * lz <= LN32) {
-    double P = P0, D = 4.0 * sqrt(cp1) * E - c * P0;  // P_0, D_1
+    double P = P0 * isB, e = 2.0 * (4.0 * scp1 * E - c * P0) * isB;  // P^_0, E_1
+    double k = 1.0;                                                 // 2m - 1
     Pv[p] = P;
     for (int m = 1; m <= Mq; ++m) {
-      if (m < Ms) Sv[(long long)m * n + p] = D;
-      double Pn = P - D;                              // P_m
-      Pv[(long long)m * n + p] = Pn;
-      D = ((2.0 * m - 1.0) * D - 4.0 * m * c * Pn) * inv_odd(m);  // D_{m+1}
-      P = Pn;
+      P = fma(-0.5, e, P);
+      Pv[(long long)m * n + p] = P;
+      if (m < Ms) {
+        Sv[(long long)m * n + p] = k * sfac * fma(-c2, P, e);
+        k += 2.0;
+      }
+      const double w = fma(-c4, P, e);
+      e = fma(-inv_odd(m), w + e, w);
     }
   } else {
-    // Miller: P~_{m*+1} = 0, P~_{m*} = 1, recurring down in (P, D).
-    int mstar = Mq + (int)ceil(19.6 / lz) + 2;
-    double Pn = 0.0, Dn = 1.0;
-    for (int m = mstar; m >= 0; --m) {
-      double Pm = Pn + Dn;
-      if (m <= Mq) Pv[(long long)m * n + p] = Pm;
-      if (m >= 1) {
-        double Dm = ((2.0 * m + 1.0) * Dn + 4.0 * m * c * Pm) * inv_odd(m - 1);
-        if (m < Ms) Sv[(long long)m * n + p] = Dm;
-        Pn = Pm; Dn = Dm;
+    // P~_{m*+1} = 0, E~_{m*+1} = 2, down to M_q
+    const int mstar = Mq + (int)ceil(19.6 / lz) + 2, m32 = Mq + (int)ceil(11.5 / lz) + 2;
+    float Pf = 0.f, ef = 2.f;
+    const float c4f = (float)c4;
+    for (int m = mstar; m > m32; --m) {
+      Pf = fmaf(0.5f, ef, Pf);
+      const float w = fmaf(c4f, Pf, ef);
+      ef = fmaf((float)inv_odd(m - 1), w + ef, w);
+    }
+    double P = (double)Pf, e = (double)ef;
+    int m = mstar > m32 ? m32 : mstar;
+    for (; m > Mq; --m) {
+      P = fma(0.5, e, P);
+      const double w = fma(c4, P, e);
+      e = fma(inv_odd(m - 1), w + e, w);
+    }
+    const double Pq = P, eq = e;  // P_{Mq+1}, E_{Mq+1}
+    for (; m >= 1; --m) {
+      P = fma(0.5, e, P);
+      const double w = fma(c4, P, e);
+      e = fma(inv_odd(m - 1), w + e, w);
+    }
+    const double scale = P0 * isB / fma(0.5, e, P);  // P_0
+    P = Pq * scale;
+    e = eq * scale;
+    double k = 2.0 * Ms - 3.0;  // 2m - 1
+    for (m = Mq; m >= 0; --m) {
+      P = fma(0.5, e, P);
+      Pv[(long long)m * n + p] = P;
+      const double w = fma(c4, P, e);
+      e = m >= 1 ? fma(inv_odd(m - 1), w + e, w) : 0.0;
+      if (m >= 1 && m < Ms) {
+        Sv[(long long)m * n + p] = k * sfac * fma(-c2, P, e);
+        k -= 2.0;
       }
     }
-    double scale = P0 / Pv[p];
-    for (int m = 0; m <= Mq; ++m) Pv[(long long)m * n + p] *= scale;
-    for (int m = 1; m < Ms; ++m) Sv[(long long)m * n + p] *= scale;
   }
-  // S_m = (1 - 2m)(chi P_m - P_{m-1})/(chi^2 - 1) = (2m - 1)(D_m - c P_m)/(c (c + 2))
-  double isB = 1.0 / sqrt(B), isB3 = isB * isB * isB;
-  Sv[p] = 4.0 * E / (c * sqrt(cp1)) * isB3;
-  const double sfac = isB3 / (c * cp1);
-  for (int m = 1; m < Ms; ++m) {
-    double D = Sv[(long long)m * n + p], P = Pv[(long long)m * n + p];
-    Sv[(long long)m * n + p] = (2.0 * m - 1.0) * (D - c * P) * sfac;
-  }
-  for (int m = 0; m <= Mq; ++m) Pv[(long long)m * n + p] *= isB;
 }
 
 // Entries of the reciprocal table: the largest index either recurrence reaches
