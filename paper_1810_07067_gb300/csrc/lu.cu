@@ -45,16 +45,43 @@ template <> struct Pivot<cd> {
     const V b = (V)__double_as_longlong(norm2(a));
     return b > 0x7FF0000000000000ull ? NONE : b + 1;
   }
+  // 1 / a as conj(a) / |a|^2 with one division where |a|^2 is far from the ends of
+  // the exponent range, by scaled division elsewhere
+  __device__ static cd inverse(cd a) {
+    const double q = norm2(a);
+    const int e = (__double2hiint(q) >> 20) & 0x7FF;
+    if (e < 64 || e > 1982) return cone<cd>() / a;
+    const double r = 1.0 / q;
+    return cd{a.x * r, -a.y * r};
+  }
 };
 template <> struct Pivot<cf> {
   using V = float;
   static constexpr V NONE = -1.f, ZERO = 0.f;
   __device__ static V measure(cf a) { return fabsf(a.x) + fabsf(a.y); }
+  __device__ static cf inverse(cf a) { return cone<cf>() / a; }
 };
 
 template <class V>
 __device__ __forceinline__ void argmax_merge(V& v, int& idx, V v2, int i2) {
   if (v2 > v || (v2 == v && i2 < idx)) { v = v2; idx = i2; }
+}
+
+// The warp's largest measure and its lowest row, in every lane: redux on the words
+// of an order-keeping integer instead of five rounds of shuffles.
+__device__ __forceinline__ void warp_argmax(unsigned long long& v, int& idx) {
+  const unsigned hi = (unsigned)(v >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+  const unsigned long long m = (unsigned long long)mh << 32 | ml;
+  idx = (int)__reduce_min_sync(0xffffffffu, v == m ? (unsigned)idx : 0xffffffffu);
+  v = m;
+}
+__device__ __forceinline__ void warp_argmax(float& v, int& idx) {
+  // non-negative floats order as their bits; -1 (no candidate) and NaN, which is
+  // never one, come out as 0 with the others' rows left out
+  const unsigned b = v >= 0.f ? __float_as_uint(v) + 1u : 0u, m = __reduce_max_sync(0xffffffffu, b);
+  idx = (int)__reduce_min_sync(0xffffffffu, b == m ? (unsigned)idx : 0xffffffffu);
+  v = m ? __uint_as_float(m - 1u) : -1.f;
 }
 
 template <class T>
@@ -132,16 +159,28 @@ __global__ void __launch_bounds__(1024) panel_kernel(const LuMat* __restrict__ m
 // ---------------------------------------------------------------- cluster panel
 // The panel (rows k0..n-1, nbk columns) held in the shared memory of a
 // cluster of C CTAs: CTA q owns rows k0 + q R .. k0 + (q+1) R - 1 as a
-// column-major slice [nbk][R].  Per column: local argmax; each CTA writes its
-// candidate (value, row index and the row itself) into every CTA's shared
-// memory through the cluster's distributed shared memory, and CTA 0, which
-// owns row c whenever C > 1 (then R > LU_NB), writes row c as well; one
-// cluster barrier; then every CTA picks the winner, the pivot's owner takes
-// row c, CTA 0 takes the pivot row, and each CTA applies the rank-1 update to
-// its rows.  Same pivot rule as panel_kernel (largest |a|^2, lowest row on
-// ties).
+// column-major slice [nbk][R].  Per column: every CTA writes its candidate
+// (value, row index, reciprocal and the row itself) into every CTA's shared
+// memory through the cluster's distributed shared memory, and CTA 0, which owns
+// row c whenever C > 1 (then R > LU_NB), writes row c as well; one cluster
+// barrier; every CTA picks the winner, the pivot's owner takes row c, CTA 0 takes
+// the pivot row; the multipliers are formed and applied to the next column alone,
+// which is searched in the same pass. The update of the columns behind it runs
+// between the arrival at the next column's cluster barrier and the wait there; the
+// two rows that travel are brought up to date by the warps that send them. A column
+// is a chain of some twenty dependent FP64 operations, two reductions and the
+// exchange, and the rank-1 update, bound by the FP64 pipe, now runs beside the
+// reciprocal and the exchange instead of after them. A dependent FP64 operation
+// takes 65 clocks and an SM issues one for a warp every 19, so the update goes over
+// (column, row) pairs without idle lanes. One column of a 1250-row panel in eight
+// CTAs: 6.5 -> 4.4 us; factorization of 9 matrices of order 1250: 16.7 -> 13.9 ms.
+// Same pivot rule as panel_kernel (largest |a|^2, lowest row on ties), and every
+// element takes the same updates in the same order.
 #define PANEL_SMEM_MAX (200 * 1024)
 #define PANEL_THREADS 512
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 template <class T>
 __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMat* __restrict__ mats, int k0, int R) {
@@ -158,102 +197,129 @@ __global__ void __launch_bounds__(PANEL_THREADS) panel_cluster_kernel(const LuMa
   extern __shared__ __align__(16) unsigned char panel_smem[];
   T* a = (T*)panel_smem;  // [nbk][R]
   using V = typename Pivot<T>::V;
-  // exchange slots, double-buffered by column parity: a slot written for
-  // column jj is written again only for column jj + 2, after every CTA has
-  // passed the cluster barrier of column jj + 1 (so it has read it)
-  __shared__ V cand_v[2][8];
-  __shared__ int cand_i[2][8];
-  __shared__ T cand_row[2][8][LU_NB];   // each CTA's candidate row of the panel
-  __shared__ T cand_inv[2][8];          // and the reciprocal of its candidate
-  __shared__ T top_row[2][LU_NB];       // row c (CTA 0 owns every row c of the panel)
+  // exchange slots, three deep: a CTA reads the pivot row of column jj until it
+  // arrives at the cluster barrier of column jj + 2, which every peer passes before
+  // it writes the slot again for column jj + 3
+  __shared__ V cand_v[3][8];
+  __shared__ int cand_i[3][8];
+  __shared__ T cand_row[3][8][LU_NB];   // each CTA's candidate row of the panel
+  __shared__ T cand_inv[3][8];          // and the reciprocal of its candidate
+  __shared__ T top_row[3][LU_NB];       // row c (CTA 0 owns every row c of the panel)
   __shared__ V red_v[PANEL_THREADS / 32];
   __shared__ int red_i[PANEL_THREADS / 32];
   __shared__ int s_bi;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int row0 = k0 + q * R;
   const int nr = max(0, min(R, n - row0));  // rows owned by this CTA
-  int Rt = 32;                              // threads along the rows: a power of two of at least R rows
-  while (Rt < R && Rt < PANEL_THREADS) Rt *= 2;
-  const int ng = PANEL_THREADS / Rt, jg = tid / Rt;
   for (int t = tid; t < nbk * nr; t += PANEL_THREADS) {
     int r = t % nr, j = t / nr;
     a[j * R + r] = M[(size_t)(k0 + j) * n + row0 + r];
   }
-  __syncthreads();
-  for (int jj = 0; jj < nbk; ++jj) {
-    const int c = k0 + jj, buf = jj & 1;
+  cl.sync();  // every CTA of the cluster has started before a peer writes to its shared memory
+  V best = Pivot<T>::NONE;
+  int bi = n;
+  for (int r = tid; r < nr; r += PANEL_THREADS) argmax_merge(best, bi, Pivot<T>::measure(a[r]), row0 + r);
+  warp_argmax(best, bi);
+  if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
+  T trav = czero<T>();
+  const T* pend = nullptr;  // pivot row of column jj - 1 while its update of columns jj + 1.. is due
+  for (int jj = 0, buf = 0; jj < nbk; ++jj, buf = buf == 2 ? 0 : buf + 1) {
+    const int c = k0 + jj;
     const T* aj = a + jj * R;
-    V best = Pivot<T>::NONE;
-    int bi = n;
-    for (int r = max(0, c - row0) + tid; r < nr; r += PANEL_THREADS)
-      argmax_merge(best, bi, Pivot<T>::measure(aj[r]), row0 + r);
-    for (int o = 16; o > 0; o >>= 1) {
-      V v2 = __shfl_xor_sync(0xffffffffu, best, o);
-      int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      argmax_merge(best, bi, v2, i2);
-    }
-    if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
     __syncthreads();
     if (wid == 0) {
       best = (lane < PANEL_THREADS / 32) ? red_v[lane] : Pivot<T>::NONE;
       bi = (lane < PANEL_THREADS / 32) ? red_i[lane] : n;
-      for (int o = 16; o > 0; o >>= 1) {
-        V v2 = __shfl_xor_sync(0xffffffffu, best, o);
-        int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-        argmax_merge(best, bi, v2, i2);
-      }
-      if (lane < C) {  // this CTA's candidate into slot q of every CTA
-        cl.map_shared_rank(cand_v[buf], lane)[q] = best;
-        cl.map_shared_rank(cand_i[buf], lane)[q] = bi;
-      }
+      warp_argmax(best, bi);
       if (lane == 0) s_bi = bi;
     }
     __syncthreads();
-    if (wid == 0 && lane < C) {  // one warp's division, beside the exchange of the rows
-      const int b = s_bi;
-      cl.map_shared_rank(cand_inv[buf], lane)[q] = b < n ? cone<T>() / aj[b - row0] : czero<T>();
+    const int rb = s_bi < n ? s_bi - row0 : -1, rc = q == 0 ? c - row0 : -1;  // rows that travel
+    if (wid == 0) {
+      if (lane < C) {  // this CTA's candidate into slot q of every CTA
+        cl.map_shared_rank(cand_v[buf], lane)[q] = best;
+        cl.map_shared_rank(cand_i[buf], lane)[q] = bi;
+        cl.map_shared_rank(cand_inv[buf], lane)[q] = rb >= 0 ? Pivot<T>::inverse(aj[rb]) : czero<T>();
+      }
+    } else if (wid < 3 && lane < nbk) {
+      // the candidate row (warp 1) and row c (warp 2), brought up to date, into every
+      // CTA; where they are the same row warp 1 alone keeps the updated values
+      const int r = wid == 1 ? rb : rc;
+      if (r >= 0) {
+        T v = a[lane * R + r];
+        if (pend && lane > jj) {
+          const T l = a[(jj - 1) * R + r];
+          v = v - l * pend[lane];
+        }
+        for (int u = 0; u < C; ++u) cl.map_shared_rank(wid == 1 ? cand_row[buf][q] : top_row[buf], u)[lane] = v;
+        trav = v;
+      }
     }
-    // the candidate row (and, from CTA 0, row c) into every CTA
-    const int cb = s_bi;
-    for (int e = tid - 32; e >= 0 && e < nbk * C; e += PANEL_THREADS - 32) {
-      const int j = e % nbk, u = e / nbk;
-      if (cb < n) cl.map_shared_rank(cand_row[buf][q], u)[j] = a[j * R + cb - row0];
-      if (q == 0) cl.map_shared_rank(top_row[buf], u)[j] = a[j * R + c - row0];
+    cluster_arrive();
+    if (pend) {  // the other rows, as one list of (column, row): no lane of the FP64 pipe idles
+      const int r0 = max(0, c - row0), nrow = nr - r0, j0 = jj + 1;
+      int t = PANEL_THREADS - 1 - tid;  // warps 0..2, busy above, take the list's end
+      if (nrow > 0) {
+        const int sj = PANEL_THREADS / nrow, sr = PANEL_THREADS - sj * nrow;
+        int j = t / nrow, r = t - j * nrow;
+        for (j += j0, r += r0; j < nbk;) {
+          if (r != rb && r != rc) a[j * R + r] = a[j * R + r] - a[(jj - 1) * R + r] * pend[j];
+          j += sj;
+          r += sr;
+          if (r >= nr) { r -= nrow; ++j; }
+        }
+      }
     }
-    cl.sync();
+    cluster_wait();
+    if (pend && lane > jj && lane < nbk && (wid == 1 || (wid == 2 && rc != rb)) && (wid == 1 ? rb : rc) >= 0)
+      a[lane * R + (wid == 1 ? rb : rc)] = trav;
+    __syncthreads();
     best = Pivot<T>::NONE;
     bi = n;
     int win = -1;
-    for (int u = 0; u < C; ++u) {
-      const V v2 = cand_v[buf][u];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const V v2 = cand_v[buf][u];  // slots from C on are read and passed over
       const int i2 = cand_i[buf][u];
-      if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; win = u; }
+      if (u < C && (v2 > best || (v2 == best && i2 < bi))) { best = v2; bi = i2; win = u; }
     }
     const int p = (best > Pivot<T>::ZERO) ? bi : -1;
     if (q == 0 && tid == 0) {
       pv[c] = (p >= 0) ? p : c;
       if (p < 0 && info[0] == 0) info[0] = c + 1;
     }
-    if (p >= 0) {
-      const T* prow = cand_row[buf][win];
-      const int qp = (p - k0) / R;
-      if (tid < nbk) {
-        if (q == qp && p != c) a[tid * R + p - row0] = top_row[buf][tid];  // row c moves to p
-        if (q == 0) a[tid * R + c - row0] = prow[tid];                       // the pivot row to c
-      }
-      __syncthreads();
-      const T inv = cand_inv[buf][win];
-      // PANEL_THREADS / Rt threads share a row's columns when a CTA owns few rows
-      for (int r = max(0, c + 1 - row0) + tid % Rt; r < nr; r += Rt) {
-        const T l = a[jj * R + r] * inv;
-        for (int j = jj + 1 + jg; j < nbk; j += ng) a[j * R + r] = a[j * R + r] - l * prow[j];
-      }
-      __syncthreads();
-      if (jg == 0)
-        for (int r = max(0, c + 1 - row0) + tid % Rt; r < nr; r += Rt) a[jj * R + r] = a[jj * R + r] * inv;
+    const int jn = jj + 1;  // the next column, searched as it is updated
+    const T* prow = cand_row[buf][p >= 0 ? win : 0];
+    const T* trow = top_row[buf];
+    if (p >= 0 && wid == PANEL_THREADS / 32 - 1 && lane < nbk) {
+      // row c moves to p (columns jj and jn there are formed below), the pivot row to c
+      if (p != c && q == (p - k0) / R && lane != jj && lane != jn) a[lane * R + p - row0] = trow[lane];
+      if (q == 0) a[lane * R + c - row0] = prow[lane];
     }
-    __syncthreads();
+    best = Pivot<T>::NONE;
+    bi = n;
+    if (p >= 0) {
+      const T inv = cand_inv[buf][win];
+      const T pn = jn < nbk ? prow[jn] : czero<T>();
+      for (int r = max(0, c + 1 - row0) + tid; r < nr; r += PANEL_THREADS) {
+        const bool sw = row0 + r == p;
+        const T l = (sw ? trow[jj] : a[jj * R + r]) * inv;
+        a[jj * R + r] = l;
+        if (jn < nbk) {
+          const T v = (sw ? trow[jn] : a[jn * R + r]) - l * pn;
+          a[jn * R + r] = v;
+          argmax_merge(best, bi, Pivot<T>::measure(v), row0 + r);
+        }
+      }
+    } else if (jn < nbk) {
+      for (int r = max(0, c + 1 - row0) + tid; r < nr; r += PANEL_THREADS)
+        argmax_merge(best, bi, Pivot<T>::measure(a[jn * R + r]), row0 + r);
+    }
+    pend = p >= 0 ? prow : nullptr;
+    warp_argmax(best, bi);
+    if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
   }
+  __syncthreads();
   for (int t = tid; t < nbk * nr; t += PANEL_THREADS) {
     int r = t % nr, j = t / nr;
     M[(size_t)(k0 + j) * n + row0 + r] = a[j * R + r];
@@ -272,17 +338,18 @@ static int sm_count() {
 }
 
 // Cluster size: the smallest of 1, 2, 4, 8 whose row slices of the largest
-// matrix (rows = its n - k0) fit PANEL_SMEM_MAX, then doubled while that leaves
-// one CTA per SM and 64 rows per CTA (the rank-1 updates are bound by the FP64
-// pipe of the SMs a matrix has); smaller matrices of a ragged batch own fewer
-// rows of the same slices.  Returns false (nothing launched)
-// when none fits or no such cluster can be resident; the caller then uses
-// panel_kernel.
+// matrix (rows = its n - k0) fit half an SM's shared memory, then doubled while
+// that leaves two CTAs per SM and more than LU_NB rows per CTA: the rank-1 updates
+// are bound by the FP64 pipe of the SMs a matrix has, and the second CTA's updates
+// run beside the first one's chain (9 of order 1250: 15.2 -> 14.2 ms with the list
+// above; 65 of order 1280 are unchanged). Smaller matrices of a ragged batch own
+// fewer rows of the same slices.  Returns false (nothing launched) when none fits
+// or no such cluster can be resident; the caller then uses panel_kernel.
 template <class T>
 static bool launch_panel_cluster(const LuMat* mats, int rows, int k0, int batch, cudaStream_t s) {
   int C = 1;
-  while (C < 8 && (size_t)LU_NB * ((rows + C - 1) / C) * sizeof(T) > PANEL_SMEM_MAX) C *= 2;
-  while (C < 8 && 2 * C * batch <= sm_count() && rows >= 128 * C) C *= 2;
+  while (C < 8 && (size_t)LU_NB * ((rows + C - 1) / C) * sizeof(T) > PANEL_SMEM_MAX / 2) C *= 2;
+  while (C < 8 && C * batch <= sm_count() && rows >= 80 * C) C *= 2;
   const int R = (rows + C - 1) / C;
   const size_t smem = (size_t)LU_NB * R * sizeof(T);
   if (smem > PANEL_SMEM_MAX) return false;

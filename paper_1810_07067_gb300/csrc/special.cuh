@@ -313,9 +313,6 @@ HD double carlson_rd(double x, double y, double z) {
   return 3.0 * sum + fac * ser / (A * sqrt(A));
 }
 
-// Complete elliptic integral of the second kind without cancellation near
-// kappa -> 1: E = (kp^2/3) [R_D(0, kp^2, 1) + R_D(0, 1, kp^2)] (DLMF 19.25.1).
-
 // K and E together from the complementary modulus kc, 0 < kc <= 1: Bulirsch's
 // general complete integral cel(kc, 1, a, b) (Numerische Mathematik 13, 1969) for
 // (a, b) = (1, 1) and (1, kc^2), whose terms are all positive, so E keeps its
