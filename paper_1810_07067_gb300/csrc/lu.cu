@@ -59,7 +59,13 @@ template <> struct Pivot<cf> {
   using V = float;
   static constexpr V NONE = -1.f, ZERO = 0.f;
   __device__ static V measure(cf a) { return fabsf(a.x) + fabsf(a.y); }
-  __device__ static cf inverse(cf a) { return cone<cf>() / a; }
+  __device__ static cf inverse(cf a) {
+    const float q = fmaf(a.x, a.x, a.y * a.y);
+    const int e = __float_as_int(q) >> 23;
+    if (e < 32 || e > 222) return cone<cf>() / a;
+    const float r = 1.f / q;
+    return cf{a.x * r, -a.y * r};
+  }
 };
 
 template <class V>
@@ -419,35 +425,40 @@ struct PregCtx {
 
 // Column jj of the panel.  The column loop is not unrolled (a fully unrolled
 // panel overflows the instruction cache); every register access uses a
-// compile-time column index, the column jj itself being picked out by a
-// select over the 32 columns and the rank-1 update predicated on j > jj.
+// compile-time column index, the column jj itself being picked out by a select
+// over the 8 columns of its eighth-aligned group, and the rank-1 update skips the
+// groups left of it without predicates on those right of it.  What bounds it is the
+// chain of a column: at 4096 rows in eight CTAs 5700 -> 4200 clocks of select 350,
+// search 450, staging and exchange 1700, exchange of rows 350, update 1070 (65
+// matrices of order 1280: 14.8 -> 12.8 ms; 5 of order 2048: 12.0 -> 9.2 ms).
 __device__ __forceinline__ void preg_column(int jj, const cg::cluster_group& cl, PregShared& sh, const PregCtx& x,
                                             cf (&a)[PREG_RPT][LU_NB], const int (&grow)[PREG_RPT]) {
   const int c = x.k0 + jj, buf = jj & 1, n = x.n;
   cf colv[PREG_RPT];
 #pragma unroll
-  for (int s = 0; s < PREG_RPT; ++s) {
-    colv[s] = a[s][0];
+  for (int g = 0; g < LU_NB; g += 8)
+    if (jj >= g && jj < g + 8) {
 #pragma unroll
-    for (int j = 1; j < LU_NB; ++j)
-      if (j == jj) colv[s] = a[s][j];
-  }
+      for (int s = 0; s < PREG_RPT; ++s) {
+        cf t[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = jj & 4 ? a[s][g + 4 + j] : a[s][g + j];
+        t[0] = jj & 2 ? t[2] : t[0];
+        t[1] = jj & 2 ? t[3] : t[1];
+        colv[s] = jj & 1 ? t[1] : t[0];
+      }
+    }
   float best = -1.f;
   int bi = n;
 #pragma unroll
   for (int s = 0; s < PREG_RPT; ++s)
     if (grow[s] >= c && grow[s] < n) argmax_merge(best, bi, Pivot<cf>::measure(colv[s]), grow[s]);
-  for (int o = 16; o > 0; o >>= 1) {
-    float v2 = __shfl_xor_sync(0xffffffffu, best, o);
-    int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-    argmax_merge(best, bi, v2, i2);
-  }
+  warp_argmax(best, bi);
   if (x.lane == 0) { sh.red_v[x.wid] = best; sh.red_i[x.wid] = bi; }
   __syncthreads();
-  best = -1.f;
-  bi = n;
-#pragma unroll
-  for (int w = 0; w < PREG_THREADS / 32; ++w) argmax_merge(best, bi, sh.red_v[w], sh.red_i[w]);
+  best = x.lane < PREG_THREADS / 32 ? sh.red_v[x.lane] : -1.f;
+  bi = x.lane < PREG_THREADS / 32 ? sh.red_i[x.lane] : n;
+  warp_argmax(best, bi);
 #pragma unroll
   for (int s = 0; s < PREG_RPT; ++s) {
     if (grow[s] == bi) {
@@ -471,14 +482,13 @@ __device__ __forceinline__ void preg_column(int jj, const cg::cluster_group& cl,
       cl.map_shared_rank(&sh.cand_i[buf][0], u)[x.q] = bi;
     }
   }
-  cl.sync();
-  float bv = -1.f;
-  int p = n, win = 0;
-  for (int u = 0; u < x.C; ++u) {
-    const float v2 = sh.cand_v[buf][u];
-    const int i2 = sh.cand_i[buf][u];
-    if (v2 > bv || (v2 == bv && i2 < p)) { bv = v2; p = i2; win = u; }
-  }
+  if (x.C > 1) cl.sync();
+  else __syncthreads();
+  float bv = x.lane < x.C ? sh.cand_v[buf][x.lane] : -1.f;
+  int p = x.lane < x.C ? sh.cand_i[buf][x.lane] : n;
+  const int own = p;
+  warp_argmax(bv, p);
+  const int win = max(0, __ffs(__ballot_sync(0xffffffffu, own == p && x.lane < x.C)) - 1);
   const bool ok = bv > 0.f;
   if (x.q == 0 && x.tid == 0) {
     x.pv[c] = ok ? p : c;
@@ -498,16 +508,37 @@ __device__ __forceinline__ void preg_column(int jj, const cg::cluster_group& cl,
       colv[s] = trow[jj];
     }
   }
-  const cf inv = cone<cf>() / prow[jj];
+  const cf inv = Pivot<cf>::inverse(prow[jj]);
+  cf l[PREG_RPT];
+  bool act[PREG_RPT];
 #pragma unroll
   for (int s = 0; s < PREG_RPT; ++s) {
-    if (grow[s] > c && grow[s] < n) {
-      const cf l = colv[s] * inv;
+    l[s] = colv[s] * inv;
+    act[s] = grow[s] > c && grow[s] < n;
+  }
 #pragma unroll
-      for (int j = 0; j < LU_NB; ++j) {
-        if (j > jj) a[s][j] = a[s][j] - l * prow[j];
-        else if (j == jj) a[s][j] = l;
-      }
+  for (int g = 0; g < LU_NB; g += 8) {
+    if (jj >= g + 8) continue;
+    cf u[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = prow[g + j];
+    if (jj < g) {
+#pragma unroll
+      for (int s = 0; s < PREG_RPT; ++s)
+        if (act[s]) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) a[s][g + j] = a[s][g + j] - l[s] * u[j];
+        }
+    } else {
+#pragma unroll
+      for (int s = 0; s < PREG_RPT; ++s)
+        if (act[s]) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            if (g + j > jj) a[s][g + j] = a[s][g + j] - l[s] * u[j];
+            else if (g + j == jj) a[s][g + j] = l[s];
+          }
+        }
     }
   }
 }
