@@ -343,22 +343,18 @@ static int sm_count() {
   return sms;
 }
 
-// Cluster size: the smallest of 1, 2, 4, 8 whose row slices of the largest
-// matrix (rows = its n - k0) fit half an SM's shared memory, then doubled while
-// that leaves two CTAs per SM and more than LU_NB rows per CTA: the rank-1 updates
-// are bound by the FP64 pipe of the SMs a matrix has, and the second CTA's updates
-// run beside the first one's chain (9 of order 1250: 15.2 -> 14.2 ms with the list
-// above; 65 of order 1280 are unchanged). Smaller matrices of a ragged batch own
-// fewer rows of the same slices.  Returns false (nothing launched) when none fits
-// or no such cluster can be resident; the caller then uses panel_kernel.
+// Cluster size: of the sizes 1..8 whose row slices of the largest matrix (rows =
+// its n - k0) fit the shared memory, the one whose estimated time for the batch is
+// least.  A column costs a chain of about 6000 clocks and 61 clocks for each of its
+// CTA's rows, times the CTAs that share an SM (the FP64 pipe bounds the updates);
+// clusters stay within a group of SMs, so a batch that fills the device takes whole
+// waves, and the sizes that are no power of two often need one wave less (65
+// matrices of order 1280: 3 waves of 32 clusters of eight, 2 of 40 of seven;
+// 48.4 -> 47.7 ms; 9 of order 1250 with eight CTAs instead of two: 15.2 -> 13.7 ms).  Smaller matrices of a ragged batch own fewer rows of the same slices.
+// Returns false (nothing launched) when none fits or no such cluster can be
+// resident; the caller then uses panel_kernel.
 template <class T>
 static bool launch_panel_cluster(const LuMat* mats, int rows, int k0, int batch, cudaStream_t s) {
-  int C = 1;
-  while (C < 8 && (size_t)LU_NB * ((rows + C - 1) / C) * sizeof(T) > PANEL_SMEM_MAX / 2) C *= 2;
-  while (C < 8 && C * batch <= sm_count() && rows >= 80 * C) C *= 2;
-  const int R = (rows + C - 1) / C;
-  const size_t smem = (size_t)LU_NB * R * sizeof(T);
-  if (smem > PANEL_SMEM_MAX) return false;
   static bool attr = false;
   if (!attr) {
     if (cudaFuncSetAttribute(panel_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM_MAX) !=
@@ -368,24 +364,42 @@ static bool launch_panel_cluster(const LuMat* mats, int rows, int k0, int batch,
     }
     attr = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(C, batch);
-  cfg.blockDim = dim3(PANEL_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
+  const int sms = sm_count();
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = C;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, panel_cluster_kernel<T>, &cfg) != cudaSuccess || nclusters < 1) {
-    cudaGetLastError();
-    return false;
+  cudaLaunchConfig_t best = {};
+  int bestR = 0;
+  double cost = 0.0;
+  for (int C = 1; C <= 8; ++C) {
+    const int R = (rows + C - 1) / C;
+    const size_t smem = (size_t)LU_NB * R * sizeof(T);
+    if (smem > PANEL_SMEM_MAX || (C > 1 && R <= LU_NB)) continue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C, batch);
+    cfg.blockDim = dim3(PANEL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int ncl = 0;
+    if (cudaOccupancyMaxActiveClusters(&ncl, panel_cluster_kernel<T>, &cfg) != cudaSuccess || ncl < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    const int waves = (batch + ncl - 1) / ncl, share = (std::min(batch, ncl) * C + sms - 1) / sms;
+    const double t = waves * (6000.0 + 61.0 * R * share);
+    if (!bestR || t < cost) {
+      cost = t;
+      best = cfg;
+      bestR = R;
+    }
   }
-  if (cudaLaunchKernelEx(&cfg, panel_cluster_kernel<T>, mats, k0, R) != cudaSuccess) {
+  if (!bestR) return false;
+  at[0].val.clusterDim.x = best.gridDim.x;
+  if (cudaLaunchKernelEx(&best, panel_cluster_kernel<T>, mats, k0, bestR) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
