@@ -22,6 +22,7 @@ std::mutex& lu_capture_mutex() {
   static std::mutex m;
   return m;
 }
+#include "split3.cuh"
 #include "tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -441,7 +442,7 @@ struct PregCtx {
 // panel overflows the instruction cache); every register access uses a
 // compile-time column index, the column jj itself being picked out by a select
 // over the 8 columns of its eighth-aligned group, and the rank-1 update skips the
-// groups left of it without predicates on those right of it.  What bounds it is the
+// groups left of it and has no predicates right of it.  What bounds it is the
 // chain of a column: at 4096 rows in eight CTAs 5700 -> 4200 clocks of select 350,
 // search 450, staging and exchange 1700, exchange of rows 350, update 1070 (65
 // matrices of order 1280: 14.8 -> 12.8 ms; 5 of order 2048: 12.0 -> 9.2 ms).
@@ -884,14 +885,6 @@ template <int TN> struct TcuShape {
 
 __device__ __forceinline__ int tcu_off(int r, int k) {  // 4 core matrices along k
   return ((r >> 3) * (LU_NB / 8) + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7);
-}
-
-__device__ __forceinline__ void split3(float x, __nv_bfloat16* p) {
-  __nv_bfloat16 h = __float2bfloat16_rn(x);
-  float r1 = x - __bfloat162float(h);
-  __nv_bfloat16 m = __float2bfloat16_rn(r1);
-  float r2 = r1 - __bfloat162float(m);
-  p[0] = h; p[1] = m; p[2] = __float2bfloat16_rn(r2);
 }
 
 // Workspace of one matrix: the L block column (rows K0+LU_OB.., LU_OB

@@ -80,9 +80,10 @@ void lu_solve_modes(const cd* LU, int n, int M, const double* sw, const cd* rhs,
                     cudaStream_t s);
 
 // Mixed path: d = A'^{-1} r with the complex64 factors of modes 0..M in FP32
-// arithmetic, in the L2-weighted space (no sqrt-weight scaling), for all modes
-// -M..M (layout [2M+1][nrhs][n], -m by reflection).
-void lu_correction_solve_c64(const cf* LU, int n, int M, const cd* r, cd* d, int nrhs, void* scratch,
+// precision, in the L2-weighted space (no sqrt-weight scaling), for all modes
+// -M..M (layout [2M+1][nrhs][n], -m by reflection; 16-byte aligned).  err (device
+// int) is set if a bounded wait gives up.
+void lu_correction_solve_c64(const cf* LU, int n, int M, const cd* r, cd* d, int nrhs, void* scratch, int* err,
                              cudaStream_t s);
 
 // Held by a thread while it captures the LU's launches into a CUDA graph;

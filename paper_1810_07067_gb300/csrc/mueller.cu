@@ -1220,10 +1220,10 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
   if (tmp.alloc(&bw, (size_t)nvec * n) || tmp.alloc(&y, (size_t)nvec * n) || tmp.alloc(&r, (size_t)nvec * n) ||
       tmp.alloc(&d, (size_t)nvec * n) || tmp.alloc(&norms, (size_t)3 * nvec) ||
       tmp.alloc(&sol, lu_solve_scratch_bytes(n, M, nrhs, true)) ||
-      (tcres && (tmp.alloc(&Ysl, ozaki_vector_slices_elems(c->npad, M + 1, njt, ojt)) ||
-                 tmp.alloc(&colscale, (size_t)(M + 1) * njt * ojt) || tmp.alloc(&derr, 1))))
+      tmp.alloc(&derr, 1) || (tcres && (tmp.alloc(&Ysl, ozaki_vector_slices_elems(c->npad, M + 1, njt, ojt)) ||
+                                        tmp.alloc(&colscale, (size_t)(M + 1) * njt * ojt))))
     return fail(MUELLER_ENOMEM, "refinement work vectors");
-  if (derr) CK(cudaMemsetAsync(derr, 0, sizeof(int), s));
+  CK(cudaMemsetAsync(derr, 0, sizeof(int), s));
   double *bn = norms, *yn = norms + nvec, *rn = norms + 2 * nvec;
   std::vector<double> hA(M + 1), hn((size_t)3 * nvec), be((size_t)nvec, 0.0);
   CK(cudaMemcpyAsync(hA.data(), c->normA, sizeof(double) * (M + 1), cudaMemcpyDeviceToHost, s));
@@ -1232,7 +1232,7 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
   cudaEventRecord(e0, s);
   mixed_scale(rhs, bw, c->geo[5], n, nvec, bn, s);
   lu_solve_prepare(c->piv, n, M, sol, s);
-  lu_correction_solve_c64(c->A32, n, M, bw, d, nrhs, sol, s);
+  lu_correction_solve_c64(c->A32, n, M, bw, d, nrhs, sol, derr, s);
   mixed_update(y, d, n, nvec, true, yn, s);
   int it = 0, launches = 3 + lu_solve_launches(n);
   bool done = false;
@@ -1261,7 +1261,7 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
       worst = std::max(worst, be[v]);
     }
     if (worst <= c->S.refine_tol) { done = true; break; }
-    lu_correction_solve_c64(c->A32, n, M, r, d, nrhs, sol, s);
+    lu_correction_solve_c64(c->A32, n, M, r, d, nrhs, sol, derr, s);
     mixed_update(y, d, n, nvec, false, yn, s);
     launches += 1 + lu_solve_launches(n);
   }
@@ -1289,13 +1289,11 @@ static int solve_mixed(mueller_ctx* c, const cd* rhs, int nrhs, cd* x, double* b
                             ojt * njt * (M + 1);
   c->st.backward_err_max = worst;
   if (backward_err) std::copy(be.begin(), be.end(), backward_err);
-  if (derr) {
-    int h = 0;
-    inject_status(derr, "residual_timeout", s);
-    cudaMemcpyAsync(&h, derr, sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    if (h) return fail(MUELLER_ETIMEOUT, "a device-side wait of the tensor-core residual timed out");
-  }
+  int h = 0;
+  if (tcres) inject_status(derr, "residual_timeout", s);
+  cudaMemcpyAsync(&h, derr, sizeof(int), cudaMemcpyDeviceToHost, s);
+  cudaStreamSynchronize(s);
+  if (h) return fail(MUELLER_ETIMEOUT, "a device-side wait of the tensor-core residual or solve timed out");
   if (!done) return fail(MUELLER_ENOCONV, "refinement stopped at refine_max_iter");
   return MUELLER_OK;
 }
