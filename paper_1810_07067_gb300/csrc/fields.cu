@@ -2,6 +2,7 @@
 #include <algorithm>
 #include "smem.cuh"
 #include "fields.cuh"
+#include "fields_oz.cuh"
 
 // One CTA per (node, wave): samples of the tangential traces on the node's
 // ring at n_theta azimuths, then their Fourier coefficients for m = -M..M.
@@ -607,7 +608,8 @@ __global__ void __launch_bounds__(256) ffgrid_coef_kernel(FieldGeom g, int M, do
 // so the two mirrored angles are A + iB and A - iB: 4 multiply-adds per term
 // for both.  FP64 pipe: 24 multiply-adds per node, mode, angle pair and side; the
 // whole grid, N = 512, M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex
-// coefficients per angle and the phase formed per mode and side).  One CTA per
+// coefficients per angle and the phase formed per mode and side; 1.65 ms with the
+// sums on the tensor cores, which take all but small grids).  One CTA per
 // (mode, 16 polar angles, WT right-hand sides); a thread owns one (angle, side)
 // and every JS-th node; the nodes pass through shared memory FFM_JC at a time.
 #define FFM_PT 16
@@ -686,38 +688,7 @@ __global__ void __launch_bounds__(128) ffgrid_mode_kernel(FieldGeom g, int M, do
   }
   const int p = p0 + pl, w = w0 + wl;
   if (js != 0 || p >= P2 || w >= nrhs) return;
-  double sth, cth;
-  sincospi((p + 0.5) / n_polar, &sth, &cth);
-  const double inv4pi = 1.0 / (4.0 * 3.141592653589793);
-  const cd pre = -C(k0 * k0) / (C(0.0, omega) * eps0);
-  const cd ik = C(0.0, k0);
-  for (int mir = 0; mir < 2; ++mir) {
-    const int pm = mir ? n_polar - 1 - p : p;
-    if (mir && pm == p) break;
-    const double c = mir ? -cth : cth;
-    cd t[6];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      cd U[3];
-#pragma unroll
-      for (int u = 0; u < 3; ++u) {
-        const cd iB = mul_i(B[3 * h + u]);
-        cd v = mir ? A[3 * h + u] - iB : A[3 * h + u] + iB;
-        U[u] = (mi[u] & 1) ? -mul_i(v) : v;  // c_m = -i b_m for odd m
-      }
-      t[3 * h] = 0.5 * (U[0] + U[2]);
-      t[3 * h + 1] = -mul_i(0.5 * (U[0] - U[2]));
-      t[3 * h + 2] = U[1];
-    }
-    const double xh[3] = {sth, 0.0, c};
-    const cd xJ = xh[0] * t[0] + xh[2] * t[2];
-    cd cr[3];
-    cr[0] = xh[1] * t[5] - xh[2] * t[4];
-    cr[1] = xh[2] * t[3] - xh[0] * t[5];
-    cr[2] = xh[0] * t[4] - xh[1] * t[3];
-    cd* dst = F + (((size_t)w * n_polar + pm) * (2 * M + 1) + q) * 3;
-    for (int a = 0; a < 3; ++a) dst[a] = inv4pi * (pre * (t[a] - xh[a] * xJ) + ik * cr[a]);
-  }
+  ffgrid_vector(A, B, m, M, k0, omega, eps0, p, n_polar, F + (size_t)w * n_polar * (2 * M + 1) * 3);
 }
 
 // E[w][p][s][3] (Cartesian) = R_z(phi_s) sum_m e^{i m phi_s} F_m: one CTA per
@@ -779,21 +750,34 @@ static void launch_ffgrid_mode(const FieldGeom& g, int M, double k0, double omeg
       g, M, k0, omega, eps0, n_polar, P2, coef, phase, x, nrhs, F);
 }
 
+// Sums of fewer multiply-adds than this stay on the FP64 pipe (one launch; the
+// tensor-core form takes four and cuts both operands into digits): N = 128, M = 32,
+// 60 angles, one side (6e6) 0.14 ms there and 0.18 ms on the tensor cores; N = 256,
+// 90 angles, one side (2e7) 0.26 ms in both, eight sides 0.60 and 0.30 ms; N = 512,
+// M = 64, 180 angles, one side (1.4e8) 1.17 and 0.89 ms, eight sides 3.34 and 1.29 ms.
+#define FFO_MIN 2e7
+size_t far_field_grid_work_bytes(int N, int M, int n_polar, int nrhs) {
+  const double fma = 24.0 * ((n_polar + 1) / 2) * N * (2.0 * M + 1.0) * nrhs;
+  return fma >= FFO_MIN ? ffgrid_oz_bytes(N, M, n_polar, nrhs) : 0;
+}
+
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar) {
   return (size_t)((n_polar + 1) / 2) * N * (M + 4);  // M + 2 coefficients and the complex phase
 }
 
 void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                           int n_polar, int n_azim, int n_alpha, double* coef, cd* F, cd* E, cudaStream_t s) {
+                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
+                           cudaStream_t s) {
   const int P2 = (n_polar + 1) / 2, Q = n_alpha / 4 + 1;
   double2* phase = (double2*)coef;                 // 16-byte aligned at the block's start
   double* b = coef + 2 * (size_t)P2 * g.N;
   const int smem1 = (n_alpha + 2 * FFC_R * Q) * (int)sizeof(double);
   smem_optin(ffgrid_coef_kernel);
   ffgrid_coef_kernel<<<dim3(P2, (g.N + FFC_R - 1) / FFC_R), 256, smem1, s>>>(g, M, k0, n_polar, n_alpha, b, phase);
-  // right-hand sides per CTA: the smallest of 1, 2, 4, 8 that holds them (the
-  // angles' coefficients are read once per group)
-  if (nrhs <= 1) launch_ffgrid_mode<1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  // without the workspace on the FP64 pipe; right-hand sides per CTA: the smallest
+  // of 1, 2, 4, 8 that holds them (the angles' coefficients are read once per group)
+  if (work) launch_ffgrid_products(g, M, k0, omega, eps0, x, nrhs, n_polar, b, phase, work, F, err, s);
+  else if (nrhs <= 1) launch_ffgrid_mode<1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else if (nrhs <= 2) launch_ffgrid_mode<2>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else if (nrhs <= 4) launch_ffgrid_mode<4>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else launch_ffgrid_mode<8>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);

@@ -34,10 +34,14 @@ void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const d
 
 // Far field on the grid theta_p = (p + 1/2) pi / n_polar, phi_s = 2 pi s / n_azim:
 // E[rhs][p][s][3] (k0 real, n_alpha a multiple of 4); work buffers coef of
-// far_field_grid_coef_doubles values, F [rhs][n_polar][2M+1][3].
+// far_field_grid_coef_doubles values, F [rhs][n_polar][2M+1][3], and work of
+// far_field_grid_work_bytes (256-byte aligned; null: the sums run on the FP64
+// pipe); err (device int) is set if a bounded wait gives up.
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar);
+size_t far_field_grid_work_bytes(int N, int M, int n_polar, int nrhs);
 void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                           int n_polar, int n_azim, int n_alpha, double* coef, cd* F, cd* E, cudaStream_t s);
+                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
+                           cudaStream_t s);
 
 // Currents x[v][n] at the nodes -> xs[v][4 nsub] at refined nodes (rows Lm[nsub][16]
 // of the panel interpolants, node0 = first node of each sub-node's panel).

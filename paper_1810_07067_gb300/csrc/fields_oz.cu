@@ -1,0 +1,373 @@
+// Far field on a grid: sums over the nodes on BF16 tensor cores with FP64 accuracy.
+//
+// Mode m at the polar angles p needs, for the currents X_u (u = 0, 1, 2) of every
+// right-hand side, sum_j b_a(p, j) {cos, sin}(p, j) X_u(j) with a = |m + 1|, |m|,
+// |m - 1| (ffgrid_mode_kernel forms them on the FP64 pipe). Grouped by a these are
+// M + 2 real products: the rows (angle, cos or sin), the columns (u, sign of the
+// shifted mode, right-hand side, J or M, Re or Im), the nodes along k. Both operands
+// are cut into 8 exact digits of 7 bits (a scale per row and per column), the digit
+// products accumulate exactly in tensor memory 256 nodes at a time, the 8 levels
+// are joined in 64-bit integers and the chunks added in FP64: rounding below that
+// of FP64 sums of the same terms.
+//
+// FP64 multiply-adds bound the other form (24 per node, mode, angle pair and side);
+// here what is left is integer work and the bytes of the digits. N = 512, M = 64,
+// 8 sides, 180 polar angles: 2.55 -> 0.48 ms.
+#include <algorithm>
+#include "digits.cuh"
+#include "fields_oz.cuh"
+#include "ozaki.cuh"
+#include "smem.cuh"
+#include "tc.cuh"
+
+namespace {
+
+#define FFO_ATILE (OZ_RT * OZ_KT)
+#define FFO_ABLOCK (OZ_S * FFO_ATILE)       // bf16 elements per (row tile, k-tile)
+#define FFO_NT 32                           // columns of a tile
+#define FFO_BTILE (FFO_NT * OZ_KT)
+#define FFO_BBLOCK (OZ_S * FFO_BTILE)       // per (column tile, k-tile)
+#define FFO_STAGE ((FFO_ABLOCK + FFO_BBLOCK) * 2)
+#define FFO_NST 4
+#define FFO_SET (OZ_S * FFO_NT)             // tensor-memory columns of one accumulator set
+#define FFO_BYTES ((size_t)512 << 20)       // digits of either operand held at a time
+
+// exponent field of the largest |v| seen -> E with |v| / 2^E < 1/2; all zero: 2^E = 2^-1020
+__device__ __forceinline__ int scale_exp(unsigned ex) { return (int)max(ex, 1u) - 1021; }
+__device__ __forceinline__ unsigned exp_field(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7FFu; }
+// 2^E; a column with an infinity or NaN gets NaN, which its products then are
+__device__ __forceinline__ double scale_of(unsigned ex) {
+  return ex == 0x7FFu ? __longlong_as_double(0x7FF8000000000000ll) : ldexp(1.0, scale_exp(ex));
+}
+// digits of 8 consecutive k of one row: one 16-byte core-matrix row per digit
+__device__ __forceinline__ void put_digits(__nv_bfloat16* dst, int stride, const double* v, int E) {
+  __align__(16) __nv_bfloat16 pc[OZ_S][8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    int d[OZ_S];
+    digits28(fixed_rn(v[c], 56 - E), d);
+#pragma unroll
+    for (int q = 0; q < OZ_S; ++q) pc[q][c] = __float2bfloat16_rn((float)d[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < OZ_S; ++q) *(uint4*)(dst + (size_t)q * stride) = *(const uint4*)pc[q];
+}
+
+// Rows 2 pp + t (t = 0 cos, 1 sin) of index a for the angles p0 + pp: one CTA per (pp, a).
+__global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int P2, int p0, int nrt, const double* __restrict__ coef,
+                                                      const double2* __restrict__ phase, __nv_bfloat16* __restrict__ Asl,
+                                                      double* __restrict__ rscale) {
+  __shared__ unsigned red[2][2];
+  const int pp = blockIdx.x, a = blockIdx.y, tid = threadIdx.x, nkt = N / OZ_KT;
+  const double* b = coef + ((size_t)a * P2 + p0 + pp) * N;
+  const double2* ph = phase + (size_t)(p0 + pp) * N;
+  unsigned ex[2] = {0u, 0u};
+  for (int j = tid; j < N; j += 64) {
+    ex[0] = max(ex[0], exp_field(b[j] * ph[j].x));
+    ex[1] = max(ex[1], exp_field(b[j] * ph[j].y));
+  }
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    ex[t] = __reduce_max_sync(0xffffffffu, ex[t]);
+    if ((tid & 31) == 0) red[t][tid >> 5] = ex[t];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    ex[t] = max(red[t][0], red[t][1]);
+    if (tid == 0) rscale[(size_t)a * nrt * OZ_RT + 2 * pp + t] = scale_of(ex[t]);
+  }
+  for (int j = 8 * tid; j < N; j += 8 * 64) {  // N is a multiple of 16
+    double v[2][8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const double2 f = ph[j + c];
+      v[0][c] = b[j + c] * f.x;
+      v[1][c] = b[j + c] * f.y;
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int r = 2 * pp + t, rt = r / OZ_RT, rr = r % OZ_RT;
+      put_digits(Asl + (((size_t)a * nrt + rt) * nkt + j / OZ_KT) * FFO_ABLOCK + core_off(rr, j % OZ_KT), FFO_ATILE, v[t],
+                 scale_exp(ex[t]));
+    }
+  }
+}
+
+// Columns of mode q and right-hand side w0 + w: X_0 = r' J1 + i J2, X_1 = z' J1,
+// X_2 = r' J1 - i J2 (and of M), for a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w).
+__global__ void __launch_bounds__(64) ffo_cols_kernel(FieldGeom g, int M, const cd* __restrict__ x, int nrhs, int w0,
+                                                      int nw, int nct, __nv_bfloat16* __restrict__ Bsl,
+                                                      double* __restrict__ cscale) {
+  __shared__ unsigned red[6][2];
+  const int q = blockIdx.x, w = blockIdx.y, m = q - M, N = g.N, nkt = N / OZ_KT, tid = threadIdx.x;
+  const cd* xv = x + ((size_t)q * nrhs + w0 + w) * 4 * N;
+  auto value = [&](int j, int h, int u) {
+    const cd v1 = xv[4 * j + 2 * h];
+    if (u == 1) return g.zp[j] * v1;
+    const cd r1 = g.rp[j] * v1, v2 = mul_i(xv[4 * j + 2 * h + 1]);
+    return u == 0 ? r1 + v2 : r1 - v2;
+  };
+  unsigned ex[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) ex[c] = 0u;
+  for (int j = tid; j < N; j += 64)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const cd v = value(j, c / 3, c % 3);
+      ex[c] = max(ex[c], max(exp_field(v.x), exp_field(v.y)));
+    }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    ex[c] = __reduce_max_sync(0xffffffffu, ex[c]);
+    if ((tid & 31) == 0) red[c][tid >> 5] = ex[c];
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int c = 0; c < 6; ++c) {
+    const int h = c / 3, u = c % 3, s = m + 1 - u, a = abs(s);
+    const unsigned e = max(red[c][0], red[c][1]);
+    const int col = ((u * 2 + (s < 0)) * nw + w) * 4 + 2 * h, ct = col / FFO_NT, cc = col % FFO_NT;
+    if (tid == 0) {
+      cscale[((size_t)a * nct) * FFO_NT + col] = scale_of(e);
+      cscale[((size_t)a * nct) * FFO_NT + col + 1] = scale_of(e);
+    }
+    __nv_bfloat16* base = Bsl + ((size_t)a * nct + ct) * nkt * FFO_BBLOCK;
+    for (int j = 8 * tid; j < N; j += 8 * 64) {
+      double re[8], im[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const cd v = value(j + i, h, u);
+        re[i] = v.x;
+        im[i] = v.y;
+      }
+      __nv_bfloat16* d = base + (size_t)(j / OZ_KT) * FFO_BBLOCK;
+      put_digits(d + core_off(cc, j % OZ_KT), FFO_BTILE, re, scale_exp(e));
+      put_digits(d + core_off(cc + 1, j % OZ_KT), FFO_BTILE, im, scale_exp(e));
+    }
+  }
+}
+
+// Y[a][column][row] = sum over the nodes.  Persistent: CTA b takes the tiles b, b +
+// gridDim.x, ... (column tile fastest, then row tile, then a), in chunks of
+// OZ_CHUNK k-tiles: warps 0-3 drain a chunk's 8 levels into FP64 sums while the next
+// chunk's products run in the other accumulator set; warp 4 copies, warp 5 issues.
+// Every wait is bounded; a role that gives up sets the failure flag and *err.
+__global__ void __launch_bounds__(192, 1)
+    ffo_gemm_kernel(const __nv_bfloat16* __restrict__ Asl, const double* __restrict__ rscale,
+                    const __nv_bfloat16* __restrict__ Bsl, const double* __restrict__ cscale, int nkt, int nrt, int nct,
+                    long long ntiles, double* __restrict__ Y, int* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  uint64_t* full = (uint64_t*)(smem + FFO_NST * FFO_STAGE);
+  uint64_t *empty = full + FFO_NST, *tfull = empty + FFO_NST, *tempty = tfull + 2, *mdone = tempty + 2;
+  uint32_t* tbase = (uint32_t*)(mdone + 1);
+  volatile int* fail = (volatile int*)(tbase + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nch = (nkt + OZ_CHUNK - 1) / OZ_CHUNK;
+  if (warp == 0) tc::tmem_alloc(tbase, 512);
+  if (tid == 32) {
+    *fail = 0;
+    for (int b = 0; b < FFO_NST; ++b) { tc::mbar_init(&full[b], 1); tc::mbar_init(&empty[b], 1); }
+    for (int b = 0; b < 2; ++b) { tc::mbar_init(&tfull[b], 1); tc::mbar_init(&tempty[b], 4); }
+    tc::mbar_init(mdone, 1);
+    tc::mbar_fence_init();
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = *tbase;
+  int issued = 0;
+  if (warp == 4) {
+    if (lane == 0) {
+      int q = 0;
+      for (long long t = blockIdx.x; t < ntiles && !*fail; t += gridDim.x) {
+        const long long ar = t / nct, a = ar / nrt;
+        const __nv_bfloat16* Ab = Asl + (size_t)ar * nkt * FFO_ABLOCK;
+        const __nv_bfloat16* Bb = Bsl + ((size_t)a * nct + t % nct) * nkt * FFO_BBLOCK;
+        for (int kt = 0; kt < nkt; ++kt, ++q) {
+          const int st = q % FFO_NST;
+          if (q >= FFO_NST && !tc::mbar_wait(&empty[st], ((q / FFO_NST) - 1) & 1)) { *fail = 1; break; }
+          unsigned char* base = smem + (size_t)st * FFO_STAGE;
+          tc::mbar_expect_tx(&full[st], FFO_STAGE);
+          tc::bulk_g2s(base, Ab + (size_t)kt * FFO_ABLOCK, FFO_ABLOCK * 2, &full[st]);
+          tc::bulk_g2s(base + FFO_ABLOCK * 2, Bb + (size_t)kt * FFO_BBLOCK, FFO_BBLOCK * 2, &full[st]);
+          issued = q + 1;
+        }
+      }
+    }
+  } else if (warp == 5) {
+    if (lane == 0) {
+      const uint32_t idesc = tc::idesc_bf16_f32(OZ_RT, FFO_NT, false);
+      int q = 0, k = 0;
+      for (long long t = blockIdx.x; t < ntiles && !*fail; t += gridDim.x) {
+        for (int kt = 0; kt < nkt && !*fail; ++k) {
+          const int set = k & 1, kt1 = min(nkt, kt + OZ_CHUNK);
+          if (k >= 2 && !tc::mbar_wait(&tempty[set], ((k >> 1) - 1) & 1)) { *fail = 1; break; }
+          tc::fence_after();
+          const uint32_t acc0 = tmem + (uint32_t)(set * FFO_SET);
+          for (bool first = true; kt < kt1; ++kt, ++q, first = false) {
+            const int st = q % FFO_NST;
+            if (!tc::mbar_wait(&full[st], (q / FFO_NST) & 1)) { *fail = 1; break; }
+            tc::fence_after();
+            unsigned char* base = smem + (size_t)st * FFO_STAGE;
+            const uint64_t a0 = tc::desc_noswizzle(tc::smem_u32(base), 128, 256);
+            const uint64_t b0 = tc::desc_noswizzle(tc::smem_u32(base + FFO_ABLOCK * 2), 128, 256);
+#pragma unroll
+            for (int s = 0; s < OZ_S; ++s) {
+#pragma unroll
+              for (int u = 0; u < OZ_S - s; ++u)
+                tc::mma_bf16(acc0 + (uint32_t)((s + u) * FFO_NT), a0 + (uint64_t)(s * (FFO_ATILE * 2 / 16)),
+                             b0 + (uint64_t)(u * (FFO_BTILE * 2 / 16)), idesc, (first && s == 0) ? 0u : 1u);  // (0, u) opens level u
+            }
+            tc::commit(&empty[st]);
+          }
+          if (*fail) break;
+          tc::commit(&tfull[set]);
+        }
+      }
+      tc::commit(mdone);  // arrives once every MMA issued above has completed
+      if (!tc::mbar_wait(mdone, 0)) *fail = 1;
+    }
+  } else {
+    int k = 0;
+    bool ok = true;
+    for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      double acc[FFO_NT];
+#pragma unroll
+      for (int c = 0; c < FFO_NT; ++c) acc[c] = 0.0;
+      for (int ch = 0; ch < nch; ++ch, ++k) {
+        const int set = k & 1;
+        if (!tc::mbar_wait(&tfull[set], (k >> 1) & 1)) { *fail = 1; ok = false; break; }
+        tc::fence_after();
+        const uint32_t tw = tmem + (uint32_t)(set * FFO_SET) + ((uint32_t)(warp * 32) << 16);
+        // levels joined in units of 2^-55 (below 2^63), one FP64 addition per value
+#pragma unroll
+        for (int h = 0; h < FFO_NT; h += 8) {
+          float v[4][8];
+          tc::tmem_ld8x4(tw + h, tw + FFO_NT + h, tw + 2 * FFO_NT + h, tw + 3 * FFO_NT + h, v);
+          long long hi[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            hi[u] = (long long)(__float2int_rn(v[0][u]) * 128 + __float2int_rn(v[1][u])) * 16384 +
+                    (__float2int_rn(v[2][u]) * 128 + __float2int_rn(v[3][u]));
+          tc::tmem_ld8x4(tw + 4 * FFO_NT + h, tw + 5 * FFO_NT + h, tw + 6 * FFO_NT + h, tw + 7 * FFO_NT + h, v);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const long long lo = (long long)(__float2int_rn(v[0][u]) * 128 + __float2int_rn(v[1][u])) * 16384 +
+                                 (__float2int_rn(v[2][u]) * 128 + __float2int_rn(v[3][u]));
+            acc[h + u] += fixed_to_double(hi[u] * 1048576 + ((lo + 128) >> 8), -55);
+          }
+        }
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&tempty[set]);
+      }
+      if (!ok) break;
+      const long long ar = t / nct, a = ar / nrt;
+      const int r = warp * 32 + lane;
+      const double rs = rscale[ar * OZ_RT + r];
+      const double* cs = cscale + ((size_t)a * nct + t % nct) * FFO_NT;
+      double* y = Y + ((size_t)a * nct + t % nct) * FFO_NT * nrt * OZ_RT + (ar % nrt) * OZ_RT + r;
+#pragma unroll
+      for (int c = 0; c < FFO_NT; ++c) y[(size_t)c * nrt * OZ_RT] = acc[c] * rs * cs[c];
+    }
+  }
+  __syncthreads();
+  if (*fail) {
+    if (tid == 0) atomicExch(err, 1);
+    if (warp == 4 && lane == 0) {
+      // the copies still in flight land before the CTA exits (bounded)
+      for (int st = 0; st < FFO_NST; ++st) {
+        const int last = issued - 1 - ((issued - 1 - st) % FFO_NST + FFO_NST) % FFO_NST;  // newest k-tile issued into st
+        if (last >= 0) tc::mbar_wait(&full[st], (last / FFO_NST) & 1, 1 << 20);
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// One thread per (angle, mode, right-hand side).
+__global__ void __launch_bounds__(128) ffo_vector_kernel(int M, double k0, double omega, cd eps0, int n_polar, int P2,
+                                                         int p0, int np, int nrt, int nct, int w0, int nw,
+                                                         const double* __restrict__ Y, cd* __restrict__ F) {
+  const int pp = blockIdx.x * 128 + threadIdx.x, q = blockIdx.y, m = q - M;
+  if (pp >= np) return;
+  for (int w = blockIdx.z; w < nw; w += gridDim.z) {
+    cd A[6], B[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int h = c / 3, u = c % 3, s = m + 1 - u;
+      const int col = ((u * 2 + (s < 0)) * nw + w) * 4 + 2 * h;
+      const double* y = Y + (((size_t)abs(s) * nct) * FFO_NT + col) * nrt * OZ_RT + 2 * pp;
+      const double2 re = *(const double2*)y, im = *(const double2*)(y + (size_t)nrt * OZ_RT);
+      A[c] = C(re.x, im.x);
+      B[c] = C(re.y, im.y);
+    }
+    ffgrid_vector(A, B, m, M, k0, omega, eps0, p0 + pp, n_polar, F + (size_t)(w0 + w) * n_polar * (2 * M + 1) * 3);
+  }
+}
+
+// Angles and right-hand sides of a pass: as many as keep either operand's digits
+// within FFO_BYTES, at least one row tile of angles and one side.
+struct FfoPlan {
+  int P2, na, nkt, np, nw, nrt, nct;  // np angles and nw sides of a full pass
+  size_t a, r, b, c, y;               // bytes of the parts
+};
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+FfoPlan ffo_plan(int N, int M, int n_polar, int nrhs) {
+  FfoPlan f{};
+  f.P2 = (n_polar + 1) / 2;
+  f.na = M + 2;
+  f.nkt = N / OZ_KT;
+  const size_t ta = (size_t)f.na * f.nkt * FFO_ABLOCK * 2, tb = (size_t)f.na * f.nkt * FFO_BBLOCK * 2;
+  f.nrt = (int)std::max<size_t>(1, std::min<size_t>((2 * f.P2 + OZ_RT - 1) / OZ_RT, FFO_BYTES / ta));
+  f.np = std::min(f.P2, f.nrt * OZ_RT / 2);
+  f.nw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / tb * FFO_NT / 24));
+  f.nct = (24 * f.nw + FFO_NT - 1) / FFO_NT;
+  f.a = up256(f.nrt * ta);
+  f.r = up256((size_t)f.na * f.nrt * OZ_RT * 8);
+  f.b = up256(f.nct * tb);
+  f.c = up256((size_t)f.na * f.nct * FFO_NT * 8);
+  f.y = up256((size_t)f.na * f.nct * FFO_NT * f.nrt * OZ_RT * 8);
+  return f;
+}
+
+}  // namespace
+
+size_t ffgrid_oz_bytes(int N, int M, int n_polar, int nrhs) {
+  const FfoPlan f = ffo_plan(N, M, n_polar, nrhs);
+  return f.a + f.r + f.b + f.c + f.y;
+}
+
+void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
+                            int n_polar, const double* coef, const double2* phase, void* work, cd* F, int* err,
+                            cudaStream_t s) {
+  const FfoPlan f = ffo_plan(g.N, M, n_polar, nrhs);
+  char* p = (char*)work;
+  auto* Asl = (__nv_bfloat16*)p;
+  auto* rscale = (double*)(p += f.a);
+  auto* Bsl = (__nv_bfloat16*)(p += f.r);
+  auto* cscale = (double*)(p += f.b);
+  auto* Y = (double*)(p += f.c);
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int smem = FFO_NST * FFO_STAGE + 256;
+  smem_optin(ffo_gemm_kernel);
+  for (int p0 = 0; p0 < f.P2; p0 += f.np) {
+    const int np = std::min(f.np, f.P2 - p0), nrt = (2 * np + OZ_RT - 1) / OZ_RT;
+    ffo_rows_kernel<<<dim3(np, f.na), 64, 0, s>>>(g.N, f.P2, p0, nrt, coef, phase, Asl, rscale);
+    for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
+      const int nw = std::min(f.nw, nrhs - w0), nct = (24 * nw + FFO_NT - 1) / FFO_NT;
+      ffo_cols_kernel<<<dim3(2 * M + 1, nw), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
+      const long long ntiles = (long long)f.na * nrt * nct;
+      ffo_gemm_kernel<<<(int)std::min<long long>(ntiles, sms), 192, smem, s>>>(Asl, rscale, Bsl, cscale, f.nkt, nrt, nct,
+                                                                              ntiles, Y, err);
+      ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
+          M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
+    }
+  }
+}

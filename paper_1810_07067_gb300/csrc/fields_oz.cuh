@@ -1,0 +1,53 @@
+// Far field on a grid: the product of ring integrals and currents on the tensor
+// cores (fields_oz.cu), and the far-field vector both forms of that product end in.
+#pragma once
+#include <cuda_bf16.h>
+#include "cplx.cuh"
+#include "fields.cuh"
+
+// F of mode m (index q) at polar angle p and, when it is another one, at its mirror
+// n_polar - 1 - p, from the sums A (cosine of the phase) and B (sine): u = 0, 1, 2
+// of J1/J2 and then of M1/M2 (see ffgrid_mode_kernel); dst is F[w].
+__device__ __forceinline__ void ffgrid_vector(const cd* A, const cd* B, int m, int M, double k0, double omega, cd eps0,
+                                              int p, int n_polar, cd* dst) {
+  const int mi[3] = {abs(m + 1), abs(m), abs(m - 1)};
+  double sth, cth;
+  sincospi((p + 0.5) / n_polar, &sth, &cth);
+  const double inv4pi = 1.0 / (4.0 * 3.141592653589793);
+  const cd pre = -C(k0 * k0) / (C(0.0, omega) * eps0);
+  const cd ik = C(0.0, k0);
+  for (int mir = 0; mir < 2; ++mir) {
+    const int pm = mir ? n_polar - 1 - p : p;
+    if (mir && pm == p) break;
+    const double c = mir ? -cth : cth;
+    cd t[6];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      cd U[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const cd iB = mul_i(B[3 * h + u]);
+        cd v = mir ? A[3 * h + u] - iB : A[3 * h + u] + iB;
+        U[u] = (mi[u] & 1) ? -mul_i(v) : v;  // c_m = -i b_m for odd m
+      }
+      t[3 * h] = 0.5 * (U[0] + U[2]);
+      t[3 * h + 1] = -mul_i(0.5 * (U[0] - U[2]));
+      t[3 * h + 2] = U[1];
+    }
+    const double xh[3] = {sth, 0.0, c};
+    const cd xJ = xh[0] * t[0] + xh[2] * t[2];
+    cd cr[3];
+    cr[0] = xh[1] * t[5] - xh[2] * t[4];
+    cr[1] = xh[2] * t[3] - xh[0] * t[5];
+    cr[2] = xh[0] * t[4] - xh[1] * t[3];
+    cd* o = dst + ((size_t)pm * (2 * M + 1) + (m + M)) * 3;
+    for (int a = 0; a < 3; ++a) o[a] = inv4pi * (pre * (t[a] - xh[a] * xJ) + ik * cr[a]);
+  }
+}
+
+// Workspace of launch_ffgrid_products in bytes (256-byte aligned), and the products
+// themselves into F; err (device int) is set if a bounded wait gives up.
+size_t ffgrid_oz_bytes(int N, int M, int n_polar, int nrhs);
+void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
+                            int n_polar, const double* coef, const double2* phase, void* work, cd* F, int* err,
+                            cudaStream_t s);
