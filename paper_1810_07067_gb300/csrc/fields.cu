@@ -608,8 +608,8 @@ __global__ void __launch_bounds__(256) ffgrid_coef_kernel(FieldGeom g, int M, do
 // so the two mirrored angles are A + iB and A - iB: 4 multiply-adds per term
 // for both.  FP64 pipe: 24 multiply-adds per node, mode, angle pair and side; the
 // whole grid, N = 512, M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex
-// coefficients per angle and the phase formed per mode and side; 1.65 ms with the
-// sums on the tensor cores, which take all but small grids).  One CTA per
+// coefficients per angle and the phase formed per mode and side; 0.94 ms on the
+// tensor cores, which take all but small grids).  One CTA per
 // (mode, 16 polar angles, WT right-hand sides); a thread owns one (angle, side)
 // and every JS-th node; the nodes pass through shared memory FFM_JC at a time.
 #define FFM_PT 16
@@ -750,15 +750,16 @@ static void launch_ffgrid_mode(const FieldGeom& g, int M, double k0, double omeg
       g, M, k0, omega, eps0, n_polar, P2, coef, phase, x, nrhs, F);
 }
 
-// Sums of fewer multiply-adds than this stay on the FP64 pipe (one launch; the
-// tensor-core form takes four and cuts both operands into digits): N = 128, M = 32,
+// Sums of fewer multiply-adds than this stay on the FP64 pipe (three launches; the
+// tensor-core form takes a dozen and cuts every operand into digits): N = 128, M = 32,
 // 60 angles, one side (6e6) 0.14 ms there and 0.18 ms on the tensor cores; N = 256,
-// 90 angles, one side (2e7) 0.26 ms in both, eight sides 0.60 and 0.30 ms; N = 512,
-// M = 64, 180 angles, one side (1.4e8) 1.17 and 0.89 ms, eight sides 3.34 and 1.29 ms.
+// M = 64, 90 angles, one side (4e7) 0.37 and 0.29 ms; M = 32, eight sides 0.60 and
+// 0.31 ms; N = 512, M = 64, 180 angles, one side (1.4e8) 1.17 and 0.55 ms, eight sides
+// 3.34 and 0.86 ms.
 #define FFO_MIN 2e7
-size_t far_field_grid_work_bytes(int N, int M, int n_polar, int nrhs) {
+size_t far_field_grid_work_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
   const double fma = 24.0 * ((n_polar + 1) / 2) * N * (2.0 * M + 1.0) * nrhs;
-  return fma >= FFO_MIN ? ffgrid_oz_bytes(N, M, n_polar, nrhs) : 0;
+  return fma >= FFO_MIN ? ffgrid_oz_bytes(N, M, n_polar, n_azim, n_alpha, nrhs) : 0;
 }
 
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar) {
@@ -768,16 +769,19 @@ size_t far_field_grid_coef_doubles(int N, int M, int n_polar) {
 void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
                            int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
                            cudaStream_t s) {
+  if (work) {
+    launch_ffgrid_products(g, M, k0, omega, eps0, x, nrhs, n_polar, n_azim, n_alpha, work, F, E, err, s);
+    return;
+  }
   const int P2 = (n_polar + 1) / 2, Q = n_alpha / 4 + 1;
   double2* phase = (double2*)coef;                 // 16-byte aligned at the block's start
   double* b = coef + 2 * (size_t)P2 * g.N;
   const int smem1 = (n_alpha + 2 * FFC_R * Q) * (int)sizeof(double);
   smem_optin(ffgrid_coef_kernel);
   ffgrid_coef_kernel<<<dim3(P2, (g.N + FFC_R - 1) / FFC_R), 256, smem1, s>>>(g, M, k0, n_polar, n_alpha, b, phase);
-  // without the workspace on the FP64 pipe; right-hand sides per CTA: the smallest
-  // of 1, 2, 4, 8 that holds them (the angles' coefficients are read once per group)
-  if (work) launch_ffgrid_products(g, M, k0, omega, eps0, x, nrhs, n_polar, b, phase, work, F, err, s);
-  else if (nrhs <= 1) launch_ffgrid_mode<1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  // right-hand sides per CTA: the smallest of 1, 2, 4, 8 that holds them (the
+  // angles' coefficients are read once per group)
+  if (nrhs <= 1) launch_ffgrid_mode<1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else if (nrhs <= 2) launch_ffgrid_mode<2>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else if (nrhs <= 4) launch_ffgrid_mode<4>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   else launch_ffgrid_mode<8>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);

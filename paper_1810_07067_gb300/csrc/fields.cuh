@@ -33,12 +33,12 @@ void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const d
                        cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, cd* out, cudaStream_t s);
 
 // Far field on the grid theta_p = (p + 1/2) pi / n_polar, phi_s = 2 pi s / n_azim:
-// E[rhs][p][s][3] (k0 real, n_alpha a multiple of 4); work buffers coef of
-// far_field_grid_coef_doubles values, F [rhs][n_polar][2M+1][3], and work of
-// far_field_grid_work_bytes (256-byte aligned; null: the sums run on the FP64
-// pipe); err (device int) is set if a bounded wait gives up.
+// E[rhs][p][s][3] (k0 real, n_alpha a multiple of 4); F [rhs][n_polar][2M+1][3] and
+// either work of far_field_grid_work_bytes (256-byte aligned; err, a device int, is
+// set if a bounded wait gives up) or coef of far_field_grid_coef_doubles values (work
+// null: FP64 pipe).
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar);
-size_t far_field_grid_work_bytes(int N, int M, int n_polar, int nrhs);
+size_t far_field_grid_work_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs);
 void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
                            int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
                            cudaStream_t s);

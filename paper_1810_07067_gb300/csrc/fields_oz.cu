@@ -10,10 +10,16 @@
 // are joined in 64-bit integers and the chunks added in FP64: rounding below that
 // of FP64 sums of the same terms.
 //
-// FP64 multiply-adds bound the other form (24 per node, mode, angle pair and side);
-// here what is left is integer work and the bytes of the digits. N = 512, M = 64,
-// 8 sides, 180 polar angles: 2.55 -> 0.48 ms.
+// The ring integrals b_a before and the sums over the modes after are contractions
+// with cosine tables and go the same way.
+//
+// FP64 multiply-adds bound the other form (24 per node, mode, angle pair and side in
+// the sums over the nodes); here what is left is the samples' sincos, integer work
+// and the bytes of the digits. N = 512, M = 64, 8 sides, 180 x 360 directions: ring
+// integrals 0.64 -> 0.22 ms, sums over the nodes 2.55 -> 0.48 ms, azimuths 0.47 ->
+// 0.15 ms.
 #include <algorithm>
+#include <cmath>
 #include "digits.cuh"
 #include "fields_oz.cuh"
 #include "ozaki.cuh"
@@ -54,12 +60,13 @@ __device__ __forceinline__ void put_digits(__nv_bfloat16* dst, int stride, const
 }
 
 // Rows 2 pp + t (t = 0 cos, 1 sin) of index a for the angles p0 + pp: one CTA per (pp, a).
-__global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int P2, int p0, int nrt, const double* __restrict__ coef,
-                                                      const double2* __restrict__ phase, __nv_bfloat16* __restrict__ Asl,
-                                                      double* __restrict__ rscale) {
+// coef: b_a of row pp N + j at [a & 1][a / 2][row], ldc rows to a column, ncc columns.
+__global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int nrt, const double* __restrict__ coef, int ncc,
+                                                      size_t ldc, const double2* __restrict__ phase,
+                                                      __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
   __shared__ unsigned red[2][2];
   const int pp = blockIdx.x, a = blockIdx.y, tid = threadIdx.x, nkt = N / OZ_KT;
-  const double* b = coef + ((size_t)a * P2 + p0 + pp) * N;
+  const double* b = coef + ((size_t)(a & 1) * ncc + (a >> 1)) * ldc + (size_t)pp * N;
   const double2* ph = phase + (size_t)(p0 + pp) * N;
   unsigned ex[2] = {0u, 0u};
   for (int j = tid; j < N; j += 64) {
@@ -148,15 +155,16 @@ __global__ void __launch_bounds__(64) ffo_cols_kernel(FieldGeom g, int M, const 
   }
 }
 
-// Y[a][column][row] = sum over the nodes.  Persistent: CTA b takes the tiles b, b +
+// Y[a][column][row] = sum over k of index a's rows and columns, times sc and the
+// scales given.  Persistent: CTA b takes the tiles b, b +
 // gridDim.x, ... (column tile fastest, then row tile, then a), in chunks of
 // OZ_CHUNK k-tiles: warps 0-3 drain a chunk's 8 levels into FP64 sums while the next
 // chunk's products run in the other accumulator set; warp 4 copies, warp 5 issues.
 // Every wait is bounded; a role that gives up sets the failure flag and *err.
 __global__ void __launch_bounds__(192, 1)
-    ffo_gemm_kernel(const __nv_bfloat16* __restrict__ Asl, const double* __restrict__ rscale,
-                    const __nv_bfloat16* __restrict__ Bsl, const double* __restrict__ cscale, int nkt, int nrt, int nct,
-                    long long ntiles, double* __restrict__ Y, int* __restrict__ err) {
+    digit_gemm_kernel(const __nv_bfloat16* __restrict__ Asl, const double* __restrict__ rscale,
+                    const __nv_bfloat16* __restrict__ Bsl, const double* __restrict__ cscale, double sc, int nkt, int nrt,
+                    int nct, long long ntiles, double* __restrict__ Y, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full = (uint64_t*)(smem + FFO_NST * FFO_STAGE);
   uint64_t *empty = full + FFO_NST, *tfull = empty + FFO_NST, *tempty = tfull + 2, *mdone = tempty + 2;
@@ -265,11 +273,11 @@ __global__ void __launch_bounds__(192, 1)
       if (!ok) break;
       const long long ar = t / nct, a = ar / nrt;
       const int r = warp * 32 + lane;
-      const double rs = rscale[ar * OZ_RT + r];
-      const double* cs = cscale + ((size_t)a * nct + t % nct) * FFO_NT;
+      const double rs = rscale ? rscale[ar * OZ_RT + r] * sc : sc;
+      const double* cs = cscale ? cscale + ((size_t)a * nct + t % nct) * FFO_NT : nullptr;
       double* y = Y + ((size_t)a * nct + t % nct) * FFO_NT * nrt * OZ_RT + (ar % nrt) * OZ_RT + r;
 #pragma unroll
-      for (int c = 0; c < FFO_NT; ++c) y[(size_t)c * nrt * OZ_RT] = acc[c] * rs * cs[c];
+      for (int c = 0; c < FFO_NT; ++c) y[(size_t)c * nrt * OZ_RT] = cs ? acc[c] * rs * cs[c] : acc[c] * rs;
     }
   }
   __syncthreads();
@@ -310,64 +318,273 @@ __global__ void __launch_bounds__(128) ffo_vector_kernel(int M, double k0, doubl
   }
 }
 
-// Angles and right-hand sides of a pass: as many as keep either operand's digits
+// ---------------------------------------------------------------------------
+// Ring integrals b_m(a) = sum_t weight_t {cos, sin}(a cos theta_t) cos(m theta_t) over the
+// Q = n / 4 + 1 samples of ring_even_coef, for many arguments a: two real products
+// (even and odd m) of the samples' digits with one table of weighted cosines.
+
+// Digits of the table, column c of parity par for m = 2 c + par <= M + 1, and
+// cost[t] = cos theta_t.  One CTA per (column, parity).
+__global__ void __launch_bounds__(32) ring_table_kernel(int M, int n, int nkt, int nct, int E,
+                                                        __nv_bfloat16* __restrict__ Bsl, double* __restrict__ cost) {
+  const int c = blockIdx.x, par = blockIdx.y, m = 2 * c + par, Q = n / 4 + 1;
+  if (c == 0 && par == 0)
+    for (int t = threadIdx.x; t < nkt * OZ_KT; t += 32) cost[t] = t < Q ? cospi(2.0 * t / n) : 0.0;
+  if (m > M + 1) return;
+  __nv_bfloat16* base = Bsl + ((size_t)par * nct + c / FFO_NT) * nkt * FFO_BBLOCK;
+  for (int t0 = 8 * threadIdx.x; t0 < nkt * OZ_KT; t0 += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = t0 + i;
+      v[i] = t < Q ? (t == 0 || t == Q - 1 ? 2.0 : 4.0) / n * cospi(2.0 * (int)((long long)m * t % n) / n) : 0.0;
+    }
+    put_digits(base + (size_t)(t0 / OZ_KT) * FFO_BBLOCK + core_off(c % FFO_NT, t0 % OZ_KT), FFO_BTILE, v, E);
+  }
+}
+
+// Digits of the samples of 128 rows and 8 consecutive t: row = k N + i has the
+// argument scale[k] r_i (scale[k] = k0 d_rho of wave k) or, without scale, (r_i
+// sin theta_p) k0 of the polar angle p = p0 + k.
+__global__ void __launch_bounds__(128) ring_samples_kernel(const double* __restrict__ r, int N, int nrows,
+                                                           const double2* __restrict__ scale, double k0, int p0,
+                                                           int n_polar, const double* __restrict__ cost, int nkt, int nrt,
+                                                           __nv_bfloat16* __restrict__ Asl) {
+  const int row = blockIdx.x * 128 + threadIdx.x, t0 = 8 * blockIdx.y;
+  if (row >= nrows) return;
+  const int k = row / N, i = row - k * N;
+  double arg;
+  if (scale) arg = scale[k].x * r[i];
+  else {
+    double sth, cth;
+    sincospi((p0 + k + 0.5) / n_polar, &sth, &cth);
+    arg = r[i] * sth * k0;
+  }
+  double v[2][8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) sincos(arg * cost[t0 + c], &v[1][c], &v[0][c]);
+  const size_t o = ((size_t)blockIdx.x * nkt + t0 / OZ_KT) * FFO_ABLOCK + core_off(threadIdx.x, t0 % OZ_KT);
+#pragma unroll
+  for (int par = 0; par < 2; ++par) put_digits(Asl + (size_t)par * nrt * nkt * FFO_ABLOCK + o, FFO_ATILE, v[par], 1);
+}
+
+// Phases 2 pi w_j r_j e^{-i k0 z_j cos theta_p} of the angles 0..P2 - 1.
+__global__ void __launch_bounds__(128) ffo_phase_kernel(FieldGeom g, double k0, int n_polar, double2* __restrict__ phase) {
+  const int p = blockIdx.x, j = blockIdx.y * 128 + threadIdx.x;
+  if (j >= g.N) return;
+  double s, c;
+  sincos(k0 * (g.z[j] * cospi((p + 0.5) / n_polar)), &s, &c);
+  const double wr = 6.283185307179586 * g.w[j] * g.r[j];
+  phase[(size_t)p * g.N + j] = make_double2(wr * c, -wr * s);
+}
+
+// ---------------------------------------------------------------------------
+// Azimuths of the grid: rows (rhs, polar angle, component, Re or Im) of F_m + F_-m
+// (index 0, with cos m phi_s) and i (F_m - F_-m) (index 1, with sin), the modes along k.
+
+// One CTA per (polar angle, rhs): its 6 rows of both indices.
+__global__ void __launch_bounds__(128) synth_rows_kernel(int M, int n_polar, const cd* __restrict__ F, int nkt, int nrt,
+                                                         __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
+  extern __shared__ __align__(16) double sv[];  // [12][nkt 16]
+  __shared__ unsigned ex[12];
+  const int K = nkt * OZ_KT, wp = blockIdx.y * n_polar + blockIdx.x, tid = threadIdx.x;
+  const cd* src = F + (size_t)wp * (2 * M + 1) * 3;
+  if (tid < 12) ex[tid] = 0u;
+  __syncthreads();
+  const int a = tid % 3;
+  unsigned mx[4] = {0u, 0u, 0u, 0u};
+  for (int m = tid / 3; m < K && tid < 126; m += 42) {
+    cd sm = C(0.0), dm = C(0.0);
+    if (m <= M) {
+      const cd u = src[(M + m) * 3 + a], v = src[(M - m) * 3 + a];
+      sm = m ? u + v : u;
+      dm = mul_i(u - v);
+    }
+    const double v[4] = {sm.x, sm.y, dm.x, dm.y};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sv[((c >> 1) * 6 + 2 * a + (c & 1)) * K + m] = v[c];
+      mx[c] = max(mx[c], exp_field(v[c]));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) atomicMax(&ex[(c >> 1) * 6 + 2 * a + (c & 1)], mx[c]);
+  __syncthreads();
+  for (int it = tid; it < 12 * (K / 8); it += 128) {
+    const int row = it % 12, k = (it / 12) * 8, b = row / 6;
+    const long long r = 6ll * wp + row % 6;
+    put_digits(Asl + (((size_t)b * nrt + r / OZ_RT) * nkt + k / OZ_KT) * FFO_ABLOCK + core_off((int)(r % OZ_RT), k % OZ_KT),
+               FFO_ATILE, sv + row * K + k, scale_exp(ex[row]));
+  }
+  if (tid < 12) rscale[(size_t)(tid / 6) * nrt * OZ_RT + 6ll * wp + tid % 6] = scale_of(ex[tid]);
+}
+
+// cos and sin of m phi_s, column s = 0..n_azim / 2.  One CTA per (column, index).
+__global__ void __launch_bounds__(32) synth_table_kernel(int M, int n, int nkt, int nct, __nv_bfloat16* __restrict__ Bsl) {
+  const int s = blockIdx.x, b = blockIdx.y;
+  __nv_bfloat16* base = Bsl + ((size_t)b * nct + s / FFO_NT) * nkt * FFO_BBLOCK;
+  for (int m0 = 8 * threadIdx.x; m0 < nkt * OZ_KT; m0 += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int m = m0 + i;
+      const double x = 2.0 * (int)((long long)m * s % n) / n;
+      v[i] = m > M ? 0.0 : b ? sinpi(x) : cospi(x);
+    }
+    put_digits(base + (size_t)(m0 / OZ_KT) * FFO_BBLOCK + core_off(s % FFO_NT, m0 % OZ_KT), FFO_BTILE, v, 1);
+  }
+}
+
+// Both azimuths s and n - s of a sum, turned into Cartesian components.
+__global__ void __launch_bounds__(128) synth_join_kernel(int n_polar, int n_azim, const double* __restrict__ Y, size_t ldy,
+                                                         int nct, cd* __restrict__ E) {
+  const int s = blockIdx.y * 128 + threadIdx.x, wp = blockIdx.z * n_polar + blockIdx.x;
+  if (s > n_azim / 2) return;
+  cd a[3], b[3];
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    const double2 x = *(const double2*)(Y + (size_t)s * ldy + 6ll * wp + 2 * u);
+    const double2 y = *(const double2*)(Y + ((size_t)nct * FFO_NT + s) * ldy + 6ll * wp + 2 * u);
+    a[u] = C(x.x, x.y);
+    b[u] = C(y.x, y.y);
+  }
+  for (int mir = 0; mir < 2; ++mir) {
+    const int sm = mir ? n_azim - s : s;
+    if (mir && (s == 0 || sm == s)) break;
+    double sn, cs;
+    sincospi(2.0 * sm / n_azim, &sn, &cs);
+    const cd v0 = mir ? a[0] - b[0] : a[0] + b[0], v1 = mir ? a[1] - b[1] : a[1] + b[1];
+    cd* dst = E + ((size_t)wp * n_azim + sm) * 3;
+    dst[0] = cs * v0 - sn * v1;
+    dst[1] = sn * v0 + cs * v1;
+    dst[2] = mir ? a[2] - b[2] : a[2] + b[2];
+  }
+}
+
+void digit_gemm(const __nv_bfloat16* Asl, const double* rscale, const __nv_bfloat16* Bsl, const double* cscale, double sc,
+                int nkt, int nrt, int nct, int na, double* Y, int* err, cudaStream_t s) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  smem_optin(digit_gemm_kernel);
+  const long long ntiles = (long long)na * nrt * nct;
+  digit_gemm_kernel<<<(int)std::min<long long>(ntiles, sms), 192, FFO_NST * FFO_STAGE + 256, s>>>(
+      Asl, rscale, Bsl, cscale, sc, nkt, nrt, nct, ntiles, Y, err);
+}
+
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+size_t tiles(size_t v, size_t t) { return (v + t - 1) / t; }
+
+// Ring integrals of rows k N + i, k < count.
+struct RingPlan {
+  int nkt, nct, E;
+  size_t a_row_tile, b, cost, y_row_tile;  // bytes, per 128 rows (a, y) or in all
+};
+RingPlan ring_plan(int M, int n) {
+  RingPlan f{};
+  f.nkt = (int)tiles(n / 4 + 1, OZ_KT);
+  f.nct = (int)tiles(M / 2 + 1 + (M & 1), FFO_NT);  // m = 0, 2, ... (1, 3, ...) up to M + 1
+  int e = 0;
+  frexp(4.0 / n, &e);
+  f.E = e + 1;
+  f.a_row_tile = (size_t)2 * f.nkt * FFO_ABLOCK * 2;
+  f.b = up256((size_t)2 * f.nct * f.nkt * FFO_BBLOCK * 2);
+  f.cost = up256((size_t)f.nkt * OZ_KT * 8);
+  f.y_row_tile = (size_t)2 * f.nct * FFO_NT * OZ_RT * 8;
+  return f;
+}
+void ring_table(const RingPlan& f, int M, int n, __nv_bfloat16* Bsl, double* cost, cudaStream_t s) {
+  ring_table_kernel<<<dim3(f.nct * FFO_NT, 2), 32, 0, s>>>(M, n, f.nkt, f.nct, f.E, Bsl, cost);
+}
+void ring_integrals(const RingPlan& f, const FieldGeom& g, int count, const double2* scale, double k0, int p0, int n_polar,
+                    __nv_bfloat16* Asl, const __nv_bfloat16* Bsl, const double* cost, double* Y, int* err, cudaStream_t s) {
+  const int nrows = count * g.N, nrt = (int)tiles(nrows, OZ_RT);
+  ring_samples_kernel<<<dim3(nrt, 2 * f.nkt), 128, 0, s>>>(g.r, g.N, nrows, scale, k0, p0, n_polar, cost, f.nkt, nrt, Asl);
+  digit_gemm(Asl, nullptr, Bsl, nullptr, ldexp(1.0, 1 + f.E), f.nkt, nrt, f.nct, 2, Y, err, s);
+}
+
+// Angles and right-hand sides of a pass: as many as keep any operand's digits
 // within FFO_BYTES, at least one row tile of angles and one side.
 struct FfoPlan {
   int P2, na, nkt, np, nw, nrt, nct;  // np angles and nw sides of a full pass
-  size_t a, r, b, c, y;               // bytes of the parts
+  RingPlan ring;
+  int snkt, snct, snw;                // azimuths: k-tiles, column tiles, sides of a pass
+  size_t phase, a, r, b, c, y, tb, cost, coef;  // bytes of the parts
 };
-size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
-FfoPlan ffo_plan(int N, int M, int n_polar, int nrhs) {
+FfoPlan ffo_plan(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
   FfoPlan f{};
   f.P2 = (n_polar + 1) / 2;
   f.na = M + 2;
   f.nkt = N / OZ_KT;
+  f.ring = ring_plan(M, n_alpha);
   const size_t ta = (size_t)f.na * f.nkt * FFO_ABLOCK * 2, tb = (size_t)f.na * f.nkt * FFO_BBLOCK * 2;
-  f.nrt = (int)std::max<size_t>(1, std::min<size_t>((2 * f.P2 + OZ_RT - 1) / OZ_RT, FFO_BYTES / ta));
+  const size_t tr = f.ring.a_row_tile * tiles((size_t)OZ_RT / 2 * N, OZ_RT);  // samples of one row tile of angles
+  f.nrt = (int)std::max<size_t>(1, std::min<size_t>(tiles(2 * f.P2, OZ_RT), FFO_BYTES / std::max(ta, tr)));
   f.np = std::min(f.P2, f.nrt * OZ_RT / 2);
-  f.nw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / tb * FFO_NT / 24));
-  f.nct = (24 * f.nw + FFO_NT - 1) / FFO_NT;
-  f.a = up256(f.nrt * ta);
-  f.r = up256((size_t)f.na * f.nrt * OZ_RT * 8);
-  f.b = up256(f.nct * tb);
+  const size_t ty = (size_t)f.na * FFO_NT * f.nrt * OZ_RT * 8;  // sums of a column tile
+  f.nw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / std::max(tb, ty) * FFO_NT / 24));
+  f.nct = (int)tiles(24 * f.nw, FFO_NT);
+  f.snkt = (int)tiles(M + 1, OZ_KT);
+  f.snct = (int)tiles(n_azim / 2 + 1, FFO_NT);
+  const size_t sa = (size_t)2 * f.snkt * FFO_ABLOCK * 2 * tiles((size_t)6 * n_polar, OZ_RT);  // one side's rows, about
+  const size_t sy = (size_t)2 * f.snct * FFO_NT * 6 * n_polar * 8;
+  f.snw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / std::max(sa, sy)));
+  const size_t srt = tiles((size_t)6 * f.snw * n_polar, OZ_RT), rrt = tiles((size_t)f.np * N, OZ_RT);
+  f.phase = up256((size_t)f.P2 * N * 16);
+  f.a = up256(std::max({f.nrt * ta, rrt * f.ring.a_row_tile, srt * 2 * f.snkt * FFO_ABLOCK * 2}));
+  f.r = up256(std::max((size_t)f.na * f.nrt, 2 * srt) * OZ_RT * 8);
+  f.b = up256(std::max(f.nct * tb, (size_t)2 * f.snct * f.snkt * FFO_BBLOCK * 2));
   f.c = up256((size_t)f.na * f.nct * FFO_NT * 8);
-  f.y = up256((size_t)f.na * f.nct * FFO_NT * f.nrt * OZ_RT * 8);
+  f.y = up256(std::max((size_t)f.na * f.nct * FFO_NT * f.nrt, (size_t)2 * f.snct * FFO_NT * srt) * OZ_RT * 8);
+  f.tb = f.ring.b;
+  f.cost = f.ring.cost;
+  f.coef = up256(rrt * f.ring.y_row_tile);
   return f;
 }
 
 }  // namespace
 
-size_t ffgrid_oz_bytes(int N, int M, int n_polar, int nrhs) {
-  const FfoPlan f = ffo_plan(N, M, n_polar, nrhs);
-  return f.a + f.r + f.b + f.c + f.y;
+size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
+  const FfoPlan f = ffo_plan(N, M, n_polar, n_azim, n_alpha, nrhs);
+  return f.phase + f.a + f.r + f.b + f.c + f.y + f.tb + f.cost + f.coef;
 }
 
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                            int n_polar, const double* coef, const double2* phase, void* work, cd* F, int* err,
-                            cudaStream_t s) {
-  const FfoPlan f = ffo_plan(g.N, M, n_polar, nrhs);
+                            int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s) {
+  const FfoPlan f = ffo_plan(g.N, M, n_polar, n_azim, n_alpha, nrhs);
   char* p = (char*)work;
-  auto* Asl = (__nv_bfloat16*)p;
+  auto* phase = (double2*)p;
+  auto* Asl = (__nv_bfloat16*)(p += f.phase);
   auto* rscale = (double*)(p += f.a);
   auto* Bsl = (__nv_bfloat16*)(p += f.r);
   auto* cscale = (double*)(p += f.b);
   auto* Y = (double*)(p += f.c);
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int smem = FFO_NST * FFO_STAGE + 256;
-  smem_optin(ffo_gemm_kernel);
+  auto* Tsl = (__nv_bfloat16*)(p += f.y);
+  auto* cost = (double*)(p += f.tb);
+  auto* coef = (double*)(p += f.cost);
+  ffo_phase_kernel<<<dim3(f.P2, (g.N + 127) / 128), 128, 0, s>>>(g, k0, n_polar, phase);
+  ring_table(f.ring, M, n_alpha, Tsl, cost, s);
   for (int p0 = 0; p0 < f.P2; p0 += f.np) {
-    const int np = std::min(f.np, f.P2 - p0), nrt = (2 * np + OZ_RT - 1) / OZ_RT;
-    ffo_rows_kernel<<<dim3(np, f.na), 64, 0, s>>>(g.N, f.P2, p0, nrt, coef, phase, Asl, rscale);
+    const int np = std::min(f.np, f.P2 - p0), nrt = (int)tiles(2 * np, OZ_RT);
+    ring_integrals(f.ring, g, np, nullptr, k0, p0, n_polar, Asl, Tsl, cost, coef, err, s);
+    ffo_rows_kernel<<<dim3(np, f.na), 64, 0, s>>>(g.N, p0, nrt, coef, f.ring.nct * FFO_NT,
+                                                 tiles((size_t)np * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
     for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
-      const int nw = std::min(f.nw, nrhs - w0), nct = (24 * nw + FFO_NT - 1) / FFO_NT;
+      const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles(24 * nw, FFO_NT);
       ffo_cols_kernel<<<dim3(2 * M + 1, nw), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
-      const long long ntiles = (long long)f.na * nrt * nct;
-      ffo_gemm_kernel<<<(int)std::min<long long>(ntiles, sms), 192, smem, s>>>(Asl, rscale, Bsl, cscale, f.nkt, nrt, nct,
-                                                                              ntiles, Y, err);
+      digit_gemm(Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
       ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
           M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
     }
+  }
+  synth_table_kernel<<<dim3(n_azim / 2 + 1, 2), 32, 0, s>>>(M, n_azim, f.snkt, f.snct, Bsl);
+  smem_optin(synth_rows_kernel);
+  for (int w0 = 0; w0 < nrhs; w0 += f.snw) {
+    const int nw = std::min(f.snw, nrhs - w0), nrt = (int)tiles((size_t)6 * nw * n_polar, OZ_RT);
+    synth_rows_kernel<<<dim3(n_polar, nw), 128, 12 * f.snkt * OZ_KT * 8, s>>>(
+        M, n_polar, F + (size_t)w0 * n_polar * (2 * M + 1) * 3, f.snkt, nrt, Asl, rscale);
+    digit_gemm(Asl, rscale, Bsl, nullptr, 2.0, f.snkt, nrt, f.snct, 2, Y, err, s);
+    synth_join_kernel<<<dim3(n_polar, (n_azim / 2 + 128) / 128, nw), 128, 0, s>>>(
+        n_polar, n_azim, Y, (size_t)nrt * OZ_RT, f.snct, E + (size_t)w0 * n_polar * n_azim * 3);
   }
 }

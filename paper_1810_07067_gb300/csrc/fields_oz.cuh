@@ -45,9 +45,9 @@ __device__ __forceinline__ void ffgrid_vector(const cd* A, const cd* B, int m, i
   }
 }
 
-// Workspace of launch_ffgrid_products in bytes (256-byte aligned), and the products
-// themselves into F; err (device int) is set if a bounded wait gives up.
-size_t ffgrid_oz_bytes(int N, int M, int n_polar, int nrhs);
+// Workspace of launch_ffgrid_products in bytes (256-byte aligned), and the whole grid
+// by products on the tensor cores: ring integrals, sums over the nodes (into F), sums
+// over the modes (into E); err (device int) is set if a bounded wait gives up.
+size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs);
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                            int n_polar, const double* coef, const double2* phase, void* work, cd* F, int* err,
-                            cudaStream_t s);
+                            int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s);

@@ -1494,19 +1494,20 @@ extern "C" int mueller_far_field_grid(mueller_ctx* c, const mueller_c128* x_dev,
   cudaStream_t s = (cudaStream_t)stream;
   const int M = c->S.M, nth = n_theta_for(c->S);
   DevBuf tmp;
-  double* coef;
+  double* coef = nullptr;
   cd* F;
-  if (tmp.alloc(&coef, far_field_grid_coef_doubles(c->S.N, M, n_polar)) != cudaSuccess ||
-      tmp.alloc(&F, (size_t)nrhs * n_polar * (2 * M + 1) * 3) != cudaSuccess)
+  if (tmp.alloc(&F, (size_t)nrhs * n_polar * (2 * M + 1) * 3) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "far-field grid buffers");
   FieldGeom g{c->geo[0], c->geo[1], c->geo[2], c->geo[3], c->geo[4], c->S.N};
-  unsigned char* work = nullptr;  // without it the sums run on the FP64 pipe
+  unsigned char* work = nullptr;  // without it everything runs on the FP64 pipe
   int* err = nullptr;
-  const size_t bytes = far_field_grid_work_bytes(c->S.N, M, n_polar, nrhs);
+  const size_t bytes = far_field_grid_work_bytes(c->S.N, M, n_polar, n_azim, nth, nrhs);
   if (bytes && (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&work, bytes) != cudaSuccess)) {
     cudaGetLastError();
     work = nullptr;
   }
+  if (!work && tmp.alloc(&coef, far_field_grid_coef_doubles(c->S.N, M, n_polar)) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "far-field grid buffers");
   if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
   launch_far_field_grid(g, M, c->S.k0.x, c->S.omega, c->S.eps0, (const cd*)x_dev, nrhs, n_polar, n_azim, nth, coef,
                         work, F, (cd*)E_dev, err, s);
