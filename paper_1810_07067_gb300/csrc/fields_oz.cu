@@ -503,6 +503,51 @@ void ring_integrals(const RingPlan& f, const FieldGeom& g, int count, const doub
   digit_gemm(Asl, nullptr, Bsl, nullptr, ldexp(1.0, 1 + f.E), f.nkt, nrt, f.nct, 2, Y, err, s);
 }
 
+// Modal data of plane waves from the ring integrals (the formulas of rhs_kernel): rows
+// w N + i of coef, one thread per (node, wave) and a run of qc modes.  FP64 pipe: 39
+// operations per mode and node for both traces of E and of H (N = 512, M = 64, 96
+// waves: 0.59 ms of 0.93 ms).
+template <bool ALIGNED>
+__global__ void __launch_bounds__(128) rhs_rows_kernel(FieldGeom g, int M, const double2* __restrict__ wave,
+                                                       const cd* __restrict__ tab, const double* __restrict__ coef,
+                                                       int ncc, size_t ldc, int w0, int nrhs, int qc,
+                                                       cd* __restrict__ rhs) {
+  const int w = blockIdx.x, i = blockIdx.y * 128 + threadIdx.x, q0 = blockIdx.z * qc, q1 = min(q0 + qc, 2 * M + 1);
+  if (i >= g.N) return;
+  double s, c;
+  sincos(wave[w].y * g.z[i], &s, &c);
+  const cd pz = C(c, s);
+  const double rp = g.rp[i], zp = g.zp[i];
+  const double* row = coef + (size_t)w * g.N + i;
+  auto b = [&](int m) {
+    const int a = abs(m);
+    return row[((size_t)(a & 1) * ncc + (a >> 1)) * ldc];
+  };
+  double bl = b(q0 - M - 1), b0 = b(q0 - M);
+  for (int q = q0; q < q1; ++q) {
+    const double bh = b(q - M + 1);
+    const double rl = rp * bl, rh = rp * bh, z0 = zp * b0;
+    const cd* u = tab + ((size_t)w * (2 * M + 1) + q) * 6;
+    cd* o = rhs + ((size_t)q * nrhs + w0 + w) * (4 * g.N) + 4 * i;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const cd u0 = u[3 * h], u1 = u[3 * h + 1], u2 = u[3 * h + 2];
+      const cd d = C(fma(bl, u0.x, -(bh * u2.x)), fma(bl, u0.y, -(bh * u2.y)));
+      const cd v = C(fma(z0, u1.x, fma(rl, u0.x, rh * u2.x)), fma(z0, u1.y, fma(rl, u0.y, rh * u2.y)));
+      const cd o0 = mul_i(d) * pz, o1 = -(v * pz);
+      if (ALIGNED) {
+        ((double2*)o)[2 * h] = make_double2(o0.x, o0.y);
+        ((double2*)o)[2 * h + 1] = make_double2(o1.x, o1.y);
+      } else {
+        o[2 * h] = o0;
+        o[2 * h + 1] = o1;
+      }
+    }
+    bl = b0;
+    b0 = bh;
+  }
+}
+
 // Angles and right-hand sides of a pass: as many as keep any operand's digits
 // within FFO_BYTES, at least one row tile of angles and one side.
 struct FfoPlan {
@@ -586,5 +631,40 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
     digit_gemm(Asl, rscale, Bsl, nullptr, 2.0, f.snkt, nrt, f.snct, 2, Y, err, s);
     synth_join_kernel<<<dim3(n_polar, (n_azim / 2 + 128) / 128, nw), 128, 0, s>>>(
         n_polar, n_azim, Y, (size_t)nrt * OZ_RT, f.snct, E + (size_t)w0 * n_polar * n_azim * 3);
+  }
+}
+
+// Waves of a pass: as many as keep the samples' digits within FFO_BYTES, at least one.
+static int rhs_oz_waves(const RingPlan& f, int N, int nrhs) {
+  return (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / f.a_row_tile * OZ_RT / N));
+}
+size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs) {
+  const RingPlan f = ring_plan(M, n_theta);
+  const size_t rt = tiles((size_t)rhs_oz_waves(f, N, nrhs) * N, OZ_RT);
+  return up256(rt * f.a_row_tile) + f.b + f.cost + up256(rt * f.y_row_tile);
+}
+void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, int w0, int count, int nrhs,
+                         int n_theta, void* work, cd* rhs, int* err, cudaStream_t s) {
+  const RingPlan f = ring_plan(M, n_theta);
+  const int nw = rhs_oz_waves(f, g.N, nrhs);
+  const size_t rt = tiles((size_t)nw * g.N, OZ_RT);
+  char* p = (char*)work;
+  auto* Asl = (__nv_bfloat16*)p;
+  auto* Tsl = (__nv_bfloat16*)(p += up256(rt * f.a_row_tile));
+  auto* cost = (double*)(p += f.b);
+  auto* coef = (double*)(p += f.cost);
+  ring_table(f, M, n_theta, Tsl, cost, s);
+  for (int v0 = 0; v0 < count; v0 += nw) {
+    const int c = std::min(nw, count - v0), nb = (g.N + 127) / 128;
+    ring_integrals(f, g, c, wave + v0, 0.0, 0, 0, Asl, Tsl, cost, coef, err, s);
+    // runs of modes: some 40000 threads in all, at least four modes each
+    const int runs = std::max(1, std::min((2 * M + 4) / 4, 320 / (nb * c) + 1)), qc = (2 * M + runs) / runs;
+    const dim3 grid(c, nb, (2 * M + qc) / qc);
+    const size_t ldc = tiles((size_t)c * g.N, OZ_RT) * OZ_RT;
+    const cd* t = tab + (size_t)v0 * (2 * M + 1) * 6;
+    if (((size_t)rhs & 15) == 0)
+      rhs_rows_kernel<true><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
+    else
+      rhs_rows_kernel<false><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
   }
 }

@@ -1346,10 +1346,21 @@ extern "C" int mueller_rhs_planewave(mueller_ctx* c, const double* dirs, const d
   FieldGeom g{c->geo[0], c->geo[1], c->geo[2], c->geo[3], c->geo[4], c->S.N};
   if (tmp.alloc(&scratch, rhs_planewave_scratch_doubles(c->S.M, nrhs, nth)) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "wave table");
-  launch_rhs_planewave(g, c->S.M, c->S.k0.x, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, nth, scratch,
-                       (cd*)rhs_dev, s);
+  unsigned char* work = nullptr;  // without it everything runs on the FP64 pipe
+  int* err = nullptr;
+  const size_t bytes = rhs_planewave_work_bytes(c->S.N, c->S.M, nrhs, nth);
+  if (bytes && (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&work, bytes) != cudaSuccess)) {
+    cudaGetLastError();
+    work = nullptr;
+  }
+  if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
+  launch_rhs_planewave(g, c->S.M, c->S.k0.x, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, nth, scratch, work,
+                       (cd*)rhs_dev, err, s);
   CK(cudaGetLastError());
+  int herr = 0;
+  if (work) CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  if (herr) return fail(MUELLER_ETIMEOUT, "a device-side wait of the tensor-core ring integrals timed out");
   return MUELLER_OK;
 }
 
