@@ -796,42 +796,50 @@ __global__ void __launch_bounds__(256) gemm_update_kernel(const LuMat* __restric
 
 // Strip update on the CUDA cores (FP32 arithmetic): C -= L U with
 // L = A[r0..r1, k..k+LU_NB), U = A[k..k+LU_NB, c0..c1); which = 1 gives the
-// block-column strip (rows k+LU_NB..n, columns k+LU_NB..min(K0+LU_OB, n)),
-// which = 2 the block-row strip (rows k+LU_NB..min(K0+LU_OB, n), columns
-// K0+LU_OB..n).  64 x 64 output tiles, 256 threads with 4 x 4 outputs each.
-template <class T>
-__global__ void __launch_bounds__(256) strip_update_kernel(const LuMat* __restrict__ mats, int K0, int k, int which) {
+// block-column strip (rows k+LU_NB..n, columns k+LU_NB..min(K0+LU_OB, n)) in tiles
+// of 128 x 32, which = 2 the block-row strip (rows k+LU_NB..min(K0+LU_OB, n), columns
+// K0+LU_OB..n) in tiles of 32 x 128: the strips are 32, 64 or 96 wide, so neither
+// tile computes padding (64 x 64 tiles did for a quarter of their area; N = 1024, 129
+// modes: 41 -> 30 ms).
+// 256 threads with 4 x 4 outputs each; bound by FP32 multiply-adds and the tiles'
+// loads.
+template <int TR, int TC>
+__global__ void __launch_bounds__(256) strip_update_kernel(const LuMat* __restrict__ mats, int K0, int k) {
+  constexpr bool TALL = TR > TC;
+  constexpr int LX = TR / 4;  // threads along the rows: thread x takes rows x + LX a, columns 4 y + c
   const LuMat mat = mats[blockIdx.z];
   const int n = mat.n;
   if (k + LU_NB >= n) return;
   const int bend = min(K0 + LU_OB, n);
-  const int r0 = k + LU_NB, r1 = which == 1 ? n : bend;
-  const int c0 = which == 1 ? k + LU_NB : K0 + LU_OB, c1 = which == 1 ? bend : n;
-  const int i0 = r0 + blockIdx.x * GT, j0 = c0 + blockIdx.y * GT;
+  const int r0 = k + LU_NB, r1 = TALL ? n : bend;
+  const int c0 = TALL ? k + LU_NB : K0 + LU_OB, c1 = TALL ? bend : n;
+  const int i0 = r0 + blockIdx.x * TR, j0 = c0 + blockIdx.y * TC;
   if (i0 >= r1 || j0 >= c1) return;
-  T* M = (T*)mat.A;
-  __shared__ T As[LU_NB][GT];
-  __shared__ T Bs[LU_NB][GT];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int t = tid; t < LU_NB * GT; t += 256) {
-    const int r = t % GT, kk = t / GT;
-    As[kk][r] = (i0 + r < r1) ? M[(size_t)(k + kk) * n + i0 + r] : czero<T>();
+  cf* M = (cf*)mat.A;
+  __shared__ __align__(16) cf As[LU_NB][TR];
+  __shared__ __align__(16) cf Bs[LU_NB][TC + 2];
+  const int tid = threadIdx.x, tx = tid % LX, ty = tid / LX;
+  for (int t = tid; t < LU_NB * TR; t += 256) {
+    const int r = t % TR, kk = t / TR;
+    As[kk][r] = (i0 + r < r1) ? M[(size_t)(k + kk) * n + i0 + r] : CF(0.f);
+  }
+  for (int t = tid; t < LU_NB * TC; t += 256) {
     const int kb = t % LU_NB, cj = t / LU_NB;
-    Bs[kb][cj] = (j0 + cj < c1) ? M[(size_t)(j0 + cj) * n + k + kb] : czero<T>();
+    Bs[kb][cj] = (j0 + cj < c1) ? M[(size_t)(j0 + cj) * n + k + kb] : CF(0.f);
   }
   __syncthreads();
-  T acc[4][4];
+  cf acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = czero<T>();
+    for (int c = 0; c < 4; ++c) acc[a][c] = CF(0.f);
 #pragma unroll 4
   for (int kk = 0; kk < LU_NB; ++kk) {
-    T av[4], bv[4];
+    cf av[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + 16 * a];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][ty + 16 * c];
+    for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + LX * a];
+    const float4 b0 = *(const float4*)&Bs[kk][4 * ty], b1 = *(const float4*)&Bs[kk][4 * ty + 2];
+    const cf bv[4] = {CF(b0.x, b0.y), CF(b0.z, b0.w), CF(b1.x, b1.y), CF(b1.z, b1.w)};
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -839,16 +847,16 @@ __global__ void __launch_bounds__(256) strip_update_kernel(const LuMat* __restri
   }
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const int gj = j0 + ty + 16 * c;
+    const int gj = j0 + 4 * ty + c;
     if (gj >= c1) continue;
+    cf* d = M + (size_t)gj * n + i0 + tx;
+    cf v[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int gi = i0 + tx + 16 * a;
-      if (gi < r1) {
-        T* d = M + (size_t)gj * n + gi;
-        *d = *d - acc[a][c];
-      }
-    }
+    for (int a = 0; a < 4; ++a)
+      if (i0 + tx + LX * a < r1) v[a] = d[LX * a];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+      if (i0 + tx + LX * a < r1) d[LX * a] = v[a] - acc[a][c];
   }
 }
 
@@ -1401,8 +1409,7 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
           if (bcols <= 0) continue;
           const int rows = nmax - k0 - LU_NB;
           if constexpr (c64) {
-            strip_update_kernel<T><<<dim3((rows + GT - 1) / GT, (bcols + GT - 1) / GT, active), 256, 0, ls>>>(
-                d, K0, k0, 1);
+            strip_update_kernel<128, 32><<<dim3((rows + 127) / 128, (bcols + 31) / 32, active), 256, 0, ls>>>(d, K0, k0);
             ++launches;
           } else {
             launches += luz_panel_update(d, K0, k0, nmax, active, tc_err, ls);
@@ -1423,8 +1430,8 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
             ++launches;
             const int brows = LU_OB - (p + 1) * LU_NB;
             if (brows > 0) {
-              strip_update_kernel<T><<<dim3((brows + GT - 1) / GT, (rest + GT - 1) / GT, active), 256, 0, ls>>>(
-                  d, K0, k0, 2);
+              strip_update_kernel<32, 128><<<dim3((brows + 31) / 32, (rest + 127) / 128, active), 256, 0, ls>>>(
+                  d, K0, k0);
               ++launches;
             }
           }
