@@ -722,6 +722,41 @@ __global__ void trsm_kernel(const LuMat* __restrict__ mats, int k0, int K0, int 
     if (r < nbk) col[r] = x[r];
 }
 
+// The same for complex64, one thread a column: the rows of 128 columns pass through
+// shared memory, a warp to a column, so that they are read and written whole (a
+// thread walking its own column in memory waited for it: N = 1024, 129 modes,
+// 19.1 -> 8.4 ms).
+__global__ void __launch_bounds__(128) trsm_c64_kernel(const LuMat* __restrict__ mats, int k0, int K0, int mode) {
+  const LuMat mat = mats[blockIdx.y];
+  const int n = mat.n;
+  if (k0 + LU_NB >= n) return;  // no columns right of the panel (or the panel is the last)
+  const int c0 = mode == 2 ? K0 + LU_OB : k0 + LU_NB, c1 = mode == 1 ? min(K0 + LU_OB, n) : n;
+  const int j0 = c0 + blockIdx.x * 128, nc = min(128, c1 - j0);
+  if (nc <= 0) return;
+  cf* M = (cf*)mat.A;
+  __shared__ cf L[LU_NB][LU_NB + 1];
+  __shared__ cf X[128][LU_NB + 1];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int c = warp; c < LU_NB; c += 4) L[lane][c] = M[(size_t)(k0 + c) * n + k0 + lane];
+#pragma unroll 8
+  for (int c = warp; c < nc; c += 4) X[c][lane] = M[(size_t)(j0 + c) * n + k0 + lane];
+  __syncthreads();
+  if (tid < nc) {
+    cf x[LU_NB];
+#pragma unroll
+    for (int r = 0; r < LU_NB; ++r) x[r] = X[tid][r];
+#pragma unroll
+    for (int k = 0; k < LU_NB; ++k)
+#pragma unroll
+      for (int r = k + 1; r < LU_NB; ++r) x[r] = x[r] - L[r][k] * x[k];
+#pragma unroll
+    for (int r = 0; r < LU_NB; ++r) X[tid][r] = x[r];
+  }
+  __syncthreads();
+#pragma unroll 8
+  for (int c = warp; c < nc; c += 4) M[(size_t)(j0 + c) * n + k0 + lane] = X[c][lane];
+}
+
 // ---------------------------------------------------------------- trailing update
 // C[i0.., j0..] -= A[i0.., k0..k0+nbk) * A[k0..k0+nbk), j0..], 64x64 tiles,
 // 256 threads, each 4x4 outputs: rows tx + 16a, columns ty + 16b.
@@ -1393,7 +1428,8 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
       }
       const int rest = hi - k0 - nbk;
       if (rest > 0) {
-        if (!c64 && two_level) luz_panel_rows(d, K0, k0, rest, active, ls);
+        if constexpr (c64) trsm_c64_kernel<<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
+        else if (two_level) luz_panel_rows(d, K0, k0, rest, active, ls);
         else trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
         ++launches;
       }
@@ -1426,7 +1462,7 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
         if constexpr (c64) {
           for (int p = 0; p < LU_OB_CHUNKS; ++p) {                    // rows of U right of the block; R2
             const int k0 = K0 + p * LU_NB;
-            trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, 2);
+            trsm_c64_kernel<<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, 2);
             ++launches;
             const int brows = LU_OB - (p + 1) * LU_NB;
             if (brows > 0) {
