@@ -448,8 +448,9 @@ void launch_far_field(const FieldGeom& g, int M, cd k0, double omega, cd eps0, c
 // ring point) pair are formed once for WR right-hand sides, ring points and
 // Cartesian currents come from ring_kernel, and the partial sums of the splits
 // are joined by nearfield_join_kernel.  FP64 pipe; N = 320, M = 32, 2 sides, 100
-// points: 3.0 ms with the rings (8.4 ms with one CTA per point and side, which
-// left a second wave on a third of the SMs and formed the kernels per side).
+// points: 2.7 ms with the rings (8.4 ms with one CTA per point and side, which
+// left a second wave on a third of the SMs and formed the kernels per side; 1.6 ms on
+// the tensor cores, which take all but few pairs).
 template <int WR>
 __global__ void __launch_bounds__(128) nearfield_kernel(long long total, const double4* __restrict__ pts,
                                                         const cd* __restrict__ cur, const double* __restrict__ X,
@@ -548,14 +549,30 @@ size_t near_field_part(long long total, int nt, int nrhs) {
   return (size_t)nt * 12 * std::max(group * near_field_splits(total, nt, group), last * near_field_splits(total, nt, last));
 }
 
+// Fewer (point, ring point) pairs than this stay on the FP64 pipe, whose kernel needs
+// no digits: N = 128, M = 16, 10 points, one side (1.5e5) 0.17 ms there and 0.23 ms on
+// the tensor cores, 50 points (8e5) 0.41 and 0.39 ms; N = 320, M = 32, 100 points (5e6)
+// one side 1.83 and 1.57 ms, two 2.74 and 1.61 ms, eight 10.6 and 2.5 ms.
+#define NF_PAIRS_MIN 7e5
+size_t near_field_work_bytes(long long total, int nt, int nrhs) {
+  const int group = near_field_group(total, nrhs);
+  return (double)total * nt >= NF_PAIRS_MIN ? nearfield_oz_bytes(total, nt, group) : 0;
+}
+
 void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
-                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, cd* out, cudaStream_t s) {
+                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, void* work, cd* out, int* err,
+                       cudaStream_t s) {
   const long long total = (long long)g.N * n_theta;
   const int group = near_field_group(total, nrhs);
   for (int w0 = 0; w0 < nrhs; w0 += group) {
     const int wc = std::min(group, nrhs - w0), splits = near_field_splits(total, nt, wc);
     const long long per = (total + splits - 1) / splits;
     launch_ring<true>(g, M, x, w0, wc, nrhs, n_theta, cur, (double4*)pts, s);
+    if (work) {
+      launch_nearfield_products(total, (const double4*)pts, cur, X_dev, nt, wc, k, cJ, cM, dM, dJ, work,
+                                out + (size_t)w0 * nt * 6, err, s);
+      continue;
+    }
     if (wc == 1)
       nearfield_kernel<1><<<dim3(nt, splits, 1), 128, 0, s>>>(total, (const double4*)pts, cur, X_dev, wc, k, per, part);
     else

@@ -385,8 +385,8 @@ __global__ void __launch_bounds__(128) ffo_phase_kernel(FieldGeom g, double k0, 
 // One CTA per (polar angle, rhs): its 6 rows of both indices.
 __global__ void __launch_bounds__(128) synth_rows_kernel(int M, int n_polar, const cd* __restrict__ F, int nkt, int nrt,
                                                          __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
-  extern __shared__ __align__(16) double sv[];  // [12][nkt 16]
-  __shared__ unsigned ex[12];
+  extern __shared__ __align__(16) double sv[];  // [12][nkt 16], then the rows' largest exponents
+  unsigned* ex = (unsigned*)(sv + 12 * nkt * OZ_KT);
   const int K = nkt * OZ_KT, wp = blockIdx.y * n_polar + blockIdx.x, tid = threadIdx.x;
   const cd* src = F + (size_t)wp * (2 * M + 1) * 3;
   if (tid < 12) ex[tid] = 0u;
@@ -461,12 +461,170 @@ __global__ void __launch_bounds__(128) synth_join_kernel(int n_polar, int n_azim
   }
 }
 
-void digit_gemm(const __nv_bfloat16* Asl, const double* rscale, const __nv_bfloat16* Bsl, const double* cscale, double sc,
-                int nkt, int nrt, int nct, int na, double* Y, int* err, cudaStream_t s) {
+// ---------------------------------------------------------------------------
+// Fields at points: with c1 = G (ik - 1/R), aa = k^2 G + c1/R and bb = -(aa + 2 c1/R)
+// curl curl S V = sum T V, T = aa I + bb h h^T (h = R / |R|), curl S V = sum g x V, g = c1 h:
+// 18 real rows a point (T_xx, T_yy, T_zz, T_xy, T_xz, T_yz, g; Re, Im), the current
+// components as columns (rhs, J or M, component, Re or Im), the ring points along k, cut
+// into indices a of NF_KC points each so that few points still fill the device; the
+// indices' sums are added in FP64. The kernels of a (point, ring point) pair remain
+// FP64 work (about 100 operations) and bound the call, their products with the
+// currents (104 operations per right-hand side in nearfield_kernel) do not: N = 320,
+// M = 32, 2 sides, 100 points 2.74 -> 1.61 ms, of which kernels 0.87 and products 0.34.
+#define NF_KC 512
+#define NF_ROWS 18
+#define NF_LD (NF_KC + 2)
+
+// One CTA per (index, point): the rows of NF_KC ring points through shared memory.
+__global__ void __launch_bounds__(128) nf_rows_kernel(long long total, const double4* __restrict__ pts,
+                                                      const double* __restrict__ X, int p0, cd k, int nrt,
+                                                      __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
+  extern __shared__ __align__(16) double sv[];  // [NF_ROWS][NF_LD], then the rows' largest exponents
+  unsigned* ex = (unsigned*)(sv + NF_ROWS * NF_LD);
+  const int a = blockIdx.x, pp = blockIdx.y, tid = threadIdx.x;
+  const double x0 = X[3 * (p0 + pp)], x1 = X[3 * (p0 + pp) + 1], x2 = X[3 * (p0 + pp) + 2];
+  if (tid < NF_ROWS) ex[tid] = 0u;
+  __syncthreads();
+  unsigned mx[NF_ROWS];
+#pragma unroll
+  for (int t = 0; t < NF_ROWS; ++t) mx[t] = 0u;
+  const bool lossless = k.y == 0.0;
+  const cd k2 = k * k;
+#pragma unroll 1
+  for (int u = 0; u < NF_KC / 128; ++u) {
+    const int col = tid + 128 * u;
+    const long long it = (long long)a * NF_KC + col;
+    cd T[9];
+    if (it < total) {
+      const double4 y = pts[it];
+      const double R0 = x0 - y.x, R1 = x1 - y.y, R2 = x2 - y.z;
+      const double R = sqrt(R0 * R0 + R1 * R1 + R2 * R2), iR = 1.0 / R;
+      const double h0 = R0 * iR, h1 = R1 * iR, h2 = R2 * iR;
+      double sn, cs;
+      sincos(k.x * R, &sn, &cs);
+      double am = y.w * iR;  // 1 / 4 pi with the sums
+      if (!lossless) am *= exp(-(k.y * R));
+      const cd G = C(am * cs, am * sn);
+      const cd c1 = lossless ? C(-(G.x * iR + G.y * k.x), G.x * k.x - G.y * iR) : G * C(-k.y - iR, k.x);
+      const cd w1 = iR * c1;
+      const cd aa = lossless ? fma(k2.x, G, w1) : fma(k2, G, w1);
+      const cd nb = fma(2.0, w1, aa);
+      const cd n0 = h0 * nb, n1 = h1 * nb, n2 = h2 * nb;
+      T[0] = fma(-h0, n0, aa); T[1] = fma(-h1, n1, aa); T[2] = fma(-h2, n2, aa);
+      T[3] = -h0 * n1; T[4] = -h0 * n2; T[5] = -h1 * n2;
+      T[6] = h0 * c1; T[7] = h1 * c1; T[8] = h2 * c1;
+    } else {
+#pragma unroll
+      for (int t = 0; t < 9; ++t) T[t] = C(0.0);
+    }
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      sv[2 * t * NF_LD + col] = T[t].x;
+      sv[(2 * t + 1) * NF_LD + col] = T[t].y;
+      mx[2 * t] = max(mx[2 * t], exp_field(T[t].x));
+      mx[2 * t + 1] = max(mx[2 * t + 1], exp_field(T[t].y));
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < NF_ROWS; ++t) {
+    const unsigned e = __reduce_max_sync(0xffffffffu, mx[t]);
+    if ((tid & 31) == 0) atomicMax(&ex[t], e);
+  }
+  __syncthreads();
+  const int r0 = NF_ROWS * pp;
+  for (int i = tid; i < NF_ROWS * (NF_KC / 8); i += 128) {  // rows fastest: neighbouring core-matrix rows
+    const int t = i % NF_ROWS, c = (i / NF_ROWS) * 8, r = r0 + t;
+    put_digits(Asl + (((size_t)a * nrt + r / OZ_RT) * (NF_KC / OZ_KT) + c / OZ_KT) * FFO_ABLOCK +
+                   core_off(r % OZ_RT, c % OZ_KT),
+               FFO_ATILE, sv + t * NF_LD + c, scale_exp(ex[t]));
+  }
+  if (tid < NF_ROWS) rscale[(size_t)a * nrt * OZ_RT + r0 + tid] = scale_of(ex[tid]);
+}
+
+// Columns of one right-hand side's currents cur[w][it][J 3, M 3].  One CTA per (index, w).
+__global__ void __launch_bounds__(64) nf_cols_kernel(long long total, const cd* __restrict__ cur, int nct,
+                                                     __nv_bfloat16* __restrict__ Bsl, double* __restrict__ cscale) {
+  __shared__ unsigned red[12][2];
+  const int a = blockIdx.x, w = blockIdx.y, tid = threadIdx.x;
+  const long long it0 = (long long)a * NF_KC + 8 * tid;  // total is a multiple of 16
+  const bool in = it0 < total;
+  const cd* src = cur + ((size_t)w * total + it0) * 6;
+  unsigned mx[12];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) mx[c] = 0u;
+  if (in)
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const cd v = src[6 * i + c];
+        mx[2 * c] = max(mx[2 * c], exp_field(v.x));
+        mx[2 * c + 1] = max(mx[2 * c + 1], exp_field(v.y));
+      }
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+    if ((tid & 31) == 0) red[c][tid >> 5] = mx[c];
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int c = 0; c < 12; ++c) {
+    const unsigned e = max(red[c][0], red[c][1]);
+    const int col = 12 * w + c, cc = col % FFO_NT;
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = in ? ((const double*)src)[12 * i + c] : 0.0;
+    put_digits(Bsl + (((size_t)a * nct + col / FFO_NT) * (NF_KC / OZ_KT) + 8 * tid / OZ_KT) * FFO_BBLOCK +
+                   core_off(cc, 8 * tid % OZ_KT),
+               FFO_BTILE, v, scale_exp(e));
+    if (tid == 0) cscale[(size_t)a * nct * FFO_NT + col] = scale_of(e);
+  }
+}
+
+// Ysum[column][row] = the sum of the indices' Y.
+__global__ void __launch_bounds__(128) nf_sum_kernel(int na, long long count, const double* __restrict__ Y,
+                                                     double* __restrict__ Ysum) {
+  const long long e = (long long)blockIdx.x * 128 + threadIdx.x;
+  if (e >= count) return;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int a = 0; a < na; ++a) acc += Y[(size_t)a * count + e];
+  Ysum[e] = acc;
+}
+
+// out[w][p][6]: E = cJ curl curl S J + cM curl S M, H = dM curl curl S M + dJ curl S J.
+__global__ void __launch_bounds__(128) nf_join_kernel(int np, int p0, int nt, int nw, size_t ldy,
+                                                      const double* __restrict__ Ysum, cd cJ, cd cM, cd dM, cd dJ,
+                                                      cd* __restrict__ out) {
+  const long long t = (long long)blockIdx.x * 128 + threadIdx.x;
+  if (t >= (long long)nw * np * 6) return;
+  const int c = (int)(t % 6), pp = (int)(t / 6 % np), w = (int)(t / 6 / np), i = c % 3, j = (i + 1) % 3, l = (i + 2) % 3;
+  const int sym[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
+  // row type r (complex) times component v of current h
+  auto prod = [&](int r, int h, int v) {
+    const double* y = Ysum + (size_t)(12 * w + 6 * h + 2 * v) * ldy + NF_ROWS * pp + 2 * r;
+    return C(y[0] - y[ldy + 1], y[ldy] + y[1]);
+  };
+  const int hc = c < 3 ? 0 : 1, hu = 1 - hc;  // E: curl curl of J, curl of M; H: the other way round
+  const cd cc = (prod(sym[i][i], hc, i) + prod(sym[i][j], hc, j)) + prod(sym[i][l], hc, l);
+  const cd cu = prod(6 + j, hu, l) - prod(6 + l, hu, j);
+  const double inv4pi = 1.0 / (4.0 * 3.141592653589793);
+  out[((size_t)w * nt + p0 + pp) * 6 + c] = inv4pi * (c < 3 ? cJ * cc + cM * cu : dM * cc + dJ * cu);
+}
+
+// The SMs of the device. Kernel limits and queries come before a call's first launch:
+// an attribute call between launches clears the error of a launch that failed.
+int digit_ready() {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   smem_optin(digit_gemm_kernel);
+  smem_optin(synth_rows_kernel);
+  smem_optin(nf_rows_kernel);
+  return sms;
+}
+
+void digit_gemm(int sms, const __nv_bfloat16* Asl, const double* rscale, const __nv_bfloat16* Bsl, const double* cscale,
+                double sc, int nkt, int nrt, int nct, int na, double* Y, int* err, cudaStream_t s) {
   const long long ntiles = (long long)na * nrt * nct;
   digit_gemm_kernel<<<(int)std::min<long long>(ntiles, sms), 192, FFO_NST * FFO_STAGE + 256, s>>>(
       Asl, rscale, Bsl, cscale, sc, nkt, nrt, nct, ntiles, Y, err);
@@ -496,11 +654,11 @@ RingPlan ring_plan(int M, int n) {
 void ring_table(const RingPlan& f, int M, int n, __nv_bfloat16* Bsl, double* cost, cudaStream_t s) {
   ring_table_kernel<<<dim3(f.nct * FFO_NT, 2), 32, 0, s>>>(M, n, f.nkt, f.nct, f.E, Bsl, cost);
 }
-void ring_integrals(const RingPlan& f, const FieldGeom& g, int count, const double2* scale, double k0, int p0, int n_polar,
+void ring_integrals(int sms, const RingPlan& f, const FieldGeom& g, int count, const double2* scale, double k0, int p0, int n_polar,
                     __nv_bfloat16* Asl, const __nv_bfloat16* Bsl, const double* cost, double* Y, int* err, cudaStream_t s) {
   const int nrows = count * g.N, nrt = (int)tiles(nrows, OZ_RT);
   ring_samples_kernel<<<dim3(nrt, 2 * f.nkt), 128, 0, s>>>(g.r, g.N, nrows, scale, k0, p0, n_polar, cost, f.nkt, nrt, Asl);
-  digit_gemm(Asl, nullptr, Bsl, nullptr, ldexp(1.0, 1 + f.E), f.nkt, nrt, f.nct, 2, Y, err, s);
+  digit_gemm(sms, Asl, nullptr, Bsl, nullptr, ldexp(1.0, 1 + f.E), f.nkt, nrt, f.nct, 2, Y, err, s);
 }
 
 // Modal data of plane waves from the ring integrals (the formulas of rhs_kernel): rows
@@ -597,6 +755,7 @@ size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int n
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
                             int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s) {
   const FfoPlan f = ffo_plan(g.N, M, n_polar, n_azim, n_alpha, nrhs);
+  const int sms = digit_ready();
   char* p = (char*)work;
   auto* phase = (double2*)p;
   auto* Asl = (__nv_bfloat16*)(p += f.phase);
@@ -611,24 +770,23 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
   ring_table(f.ring, M, n_alpha, Tsl, cost, s);
   for (int p0 = 0; p0 < f.P2; p0 += f.np) {
     const int np = std::min(f.np, f.P2 - p0), nrt = (int)tiles(2 * np, OZ_RT);
-    ring_integrals(f.ring, g, np, nullptr, k0, p0, n_polar, Asl, Tsl, cost, coef, err, s);
+    ring_integrals(sms, f.ring, g, np, nullptr, k0, p0, n_polar, Asl, Tsl, cost, coef, err, s);
     ffo_rows_kernel<<<dim3(np, f.na), 64, 0, s>>>(g.N, p0, nrt, coef, f.ring.nct * FFO_NT,
                                                  tiles((size_t)np * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
     for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
       const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles(24 * nw, FFO_NT);
       ffo_cols_kernel<<<dim3(2 * M + 1, nw), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
-      digit_gemm(Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
+      digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
       ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
           M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
     }
   }
   synth_table_kernel<<<dim3(n_azim / 2 + 1, 2), 32, 0, s>>>(M, n_azim, f.snkt, f.snct, Bsl);
-  smem_optin(synth_rows_kernel);
   for (int w0 = 0; w0 < nrhs; w0 += f.snw) {
     const int nw = std::min(f.snw, nrhs - w0), nrt = (int)tiles((size_t)6 * nw * n_polar, OZ_RT);
-    synth_rows_kernel<<<dim3(n_polar, nw), 128, 12 * f.snkt * OZ_KT * 8, s>>>(
+    synth_rows_kernel<<<dim3(n_polar, nw), 128, 12 * (f.snkt * OZ_KT * 8 + 4), s>>>(
         M, n_polar, F + (size_t)w0 * n_polar * (2 * M + 1) * 3, f.snkt, nrt, Asl, rscale);
-    digit_gemm(Asl, rscale, Bsl, nullptr, 2.0, f.snkt, nrt, f.snct, 2, Y, err, s);
+    digit_gemm(sms, Asl, rscale, Bsl, nullptr, 2.0, f.snkt, nrt, f.snct, 2, Y, err, s);
     synth_join_kernel<<<dim3(n_polar, (n_azim / 2 + 128) / 128, nw), 128, 0, s>>>(
         n_polar, n_azim, Y, (size_t)nrt * OZ_RT, f.snct, E + (size_t)w0 * n_polar * n_azim * 3);
   }
@@ -646,6 +804,7 @@ size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs) {
 void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, int w0, int count, int nrhs,
                          int n_theta, void* work, cd* rhs, int* err, cudaStream_t s) {
   const RingPlan f = ring_plan(M, n_theta);
+  const int sms = digit_ready();
   const int nw = rhs_oz_waves(f, g.N, nrhs);
   const size_t rt = tiles((size_t)nw * g.N, OZ_RT);
   char* p = (char*)work;
@@ -656,7 +815,7 @@ void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const c
   ring_table(f, M, n_theta, Tsl, cost, s);
   for (int v0 = 0; v0 < count; v0 += nw) {
     const int c = std::min(nw, count - v0), nb = (g.N + 127) / 128;
-    ring_integrals(f, g, c, wave + v0, 0.0, 0, 0, Asl, Tsl, cost, coef, err, s);
+    ring_integrals(sms, f, g, c, wave + v0, 0.0, 0, 0, Asl, Tsl, cost, coef, err, s);
     // runs of modes: some 40000 threads in all, at least four modes each
     const int runs = std::max(1, std::min((2 * M + 4) / 4, 320 / (nb * c) + 1)), qc = (2 * M + runs) / runs;
     const dim3 grid(c, nb, (2 * M + qc) / qc);
@@ -666,5 +825,55 @@ void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const c
       rhs_rows_kernel<true><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
     else
       rhs_rows_kernel<false><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
+  }
+}
+
+// Points of a pass: as many as keep the rows' digits within FFO_BYTES, at least one
+// tile of rows.
+struct NfPlan {
+  int na, np, nrt, nct;
+  size_t a, r, b, c, y, sum;
+};
+static NfPlan nf_plan(long long total, int nt, int nw) {
+  NfPlan f{};
+  f.na = (int)((total + NF_KC - 1) / NF_KC);
+  const size_t tile = (size_t)f.na * (NF_KC / OZ_KT) * FFO_ABLOCK * 2;
+  f.nrt = (int)std::max<size_t>(1, std::min<size_t>(tiles((size_t)NF_ROWS * nt, OZ_RT), FFO_BYTES / tile));
+  f.np = std::min(nt, f.nrt * OZ_RT / NF_ROWS);
+  f.np = (int)tiles(nt, tiles(nt, f.np));  // equal passes
+  f.nrt = (int)tiles((size_t)NF_ROWS * f.np, OZ_RT);
+  f.nct = (int)tiles((size_t)12 * nw, FFO_NT);
+  f.a = up256(f.nrt * tile);
+  f.r = up256((size_t)f.na * f.nrt * OZ_RT * 8);
+  f.b = up256((size_t)f.na * f.nct * (NF_KC / OZ_KT) * FFO_BBLOCK * 2);
+  f.c = up256((size_t)f.na * f.nct * FFO_NT * 8);
+  f.sum = up256((size_t)f.nct * FFO_NT * f.nrt * OZ_RT * 8);
+  f.y = (size_t)f.na * f.sum;
+  return f;
+}
+size_t nearfield_oz_bytes(long long total, int nt, int nw) {
+  const NfPlan f = nf_plan(total, nt, nw);
+  return f.a + f.r + f.b + f.c + f.y + f.sum;
+}
+void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nw, cd k,
+                               cd cJ, cd cM, cd dM, cd dJ, void* work, cd* out, int* err, cudaStream_t s) {
+  const NfPlan f = nf_plan(total, nt, nw);
+  const int sms = digit_ready();
+  char* p = (char*)work;
+  auto* Asl = (__nv_bfloat16*)p;
+  auto* rscale = (double*)(p += f.a);
+  auto* Bsl = (__nv_bfloat16*)(p += f.r);
+  auto* cscale = (double*)(p += f.b);
+  auto* Y = (double*)(p += f.c);
+  auto* Ysum = (double*)(p += f.y);
+  nf_cols_kernel<<<dim3(f.na, nw), 64, 0, s>>>(total, cur, f.nct, Bsl, cscale);
+  for (int p0 = 0; p0 < nt; p0 += f.np) {
+    const int np = std::min(f.np, nt - p0), nrt = (int)tiles((size_t)NF_ROWS * np, OZ_RT);
+    nf_rows_kernel<<<dim3(f.na, np), 128, NF_ROWS * (NF_LD * 8 + 4), s>>>(total, pts, X, p0, k, nrt, Asl, rscale);
+    digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, NF_KC / OZ_KT, nrt, f.nct, f.na, Y, err, s);
+    const long long count = (long long)f.nct * FFO_NT * nrt * OZ_RT, items = (long long)nw * np * 6;
+    nf_sum_kernel<<<(unsigned)((count + 127) / 128), 128, 0, s>>>(f.na, count, Y, Ysum);
+    nf_join_kernel<<<(unsigned)((items + 127) / 128), 128, 0, s>>>(np, p0, nt, nw, (size_t)nrt * OZ_RT, Ysum, cJ, cM, dM,
+                                                                  dJ, out);
   }
 }

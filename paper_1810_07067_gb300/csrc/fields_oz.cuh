@@ -57,3 +57,9 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
 size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs);
 void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, int w0, int count, int nrhs,
                          int n_theta, void* work, cd* rhs, int* err, cudaStream_t s);
+
+// Fields of nw right-hand sides at nt points from their ring points and currents
+// (ring_kernel) into out[w][p][6]; work of nearfield_oz_bytes (256-byte aligned).
+size_t nearfield_oz_bytes(long long total, int nt, int nw);
+void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nw, cd k,
+                               cd cJ, cd cM, cd dM, cd dJ, void* work, cd* out, int* err, cudaStream_t s);

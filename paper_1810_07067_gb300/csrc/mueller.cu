@@ -1455,7 +1455,7 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
   const int nth = std::max(nth_base, std::min(8192, (int)std::ceil(40.0 * S.rmax / dmin_all)));
   cudaStream_t s = (cudaStream_t)stream;
   DevBuf tmp;
-  cd *cur, *xs, *part;
+  cd *cur, *xs, *part = nullptr;
   double *pts, *X, *dgr, *dgz, *dgrp, *dgzp, *dgw, *dLm;
   int* dn0;
   std::vector<double> vx(targets, targets + 3 * ntargets);
@@ -1463,18 +1463,31 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
   const long long nring = (long long)nsub * nth;
   if (tmp.alloc(&cur, (size_t)near_field_group(nring, nrhs) * nring * 6) != cudaSuccess ||
       tmp.alloc(&pts, (size_t)nring * 4) != cudaSuccess ||
-      tmp.alloc(&part, near_field_part(nring, ntargets, nrhs)) != cudaSuccess ||
       tmp.alloc(&xs, (size_t)nvec * 4 * nsub) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "evaluation buffers");
+  unsigned char* work = nullptr;  // without it the sums run on the FP64 pipe
+  int* err = nullptr;
+  const size_t bytes = near_field_work_bytes(nring, ntargets, nrhs);
+  if (bytes && (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&work, bytes) != cudaSuccess)) {
+    cudaGetLastError();
+    work = nullptr;
+  }
+  if (!work && tmp.alloc(&part, near_field_part(nring, ntargets, nrhs)) != cudaSuccess)
+    return fail(MUELLER_ENOMEM, "evaluation buffers");
+  if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
   CK(tmp.upload(&X, vx, s));
   CK(tmp.upload(&dgr, gr, s)); CK(tmp.upload(&dgz, gz, s)); CK(tmp.upload(&dgrp, grp, s));
   CK(tmp.upload(&dgzp, gzp, s)); CK(tmp.upload(&dgw, gw, s)); CK(tmp.upload(&dLm, Lm, s));
   CK(tmp.upload(&dn0, node0, s));
   launch_interp_currents((const cd*)x_dev, 4 * S.N, nsub, dn0, dLm, nvec, xs, s);
   FieldGeom g{dgr, dgz, dgrp, dgzp, dgw, nsub};
-  launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, pts, part, (cd*)out_dev, s);
+  launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, pts, part, work, (cd*)out_dev,
+                    err, s);
   CK(cudaGetLastError());
+  int herr = 0;
+  if (work) CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  if (herr) return fail(MUELLER_ETIMEOUT, "a device-side wait of the tensor-core field evaluation timed out");
   return MUELLER_OK;
 }
 
