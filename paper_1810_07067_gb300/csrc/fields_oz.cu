@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(192, 1)
     }
   } else if (warp == 5) {
     if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16_f32(OZ_RT, FFO_NT, false);
       int q = 0, k = 0;
       for (long long t = blockIdx.x; t < ntiles && !*fail; t += gridDim.x) {
         for (int kt = 0; kt < nkt && !*fail; ++k) {
@@ -221,12 +220,9 @@ __global__ void __launch_bounds__(192, 1)
             const uint64_t a0 = tc::desc_noswizzle(tc::smem_u32(base), 128, 256);
             const uint64_t b0 = tc::desc_noswizzle(tc::smem_u32(base + FFO_ABLOCK * 2), 128, 256);
 #pragma unroll
-            for (int s = 0; s < OZ_S; ++s) {
-#pragma unroll
-              for (int u = 0; u < OZ_S - s; ++u)
-                tc::mma_bf16(acc0 + (uint32_t)((s + u) * FFO_NT), a0 + (uint64_t)(s * (FFO_ATILE * 2 / 16)),
-                             b0 + (uint64_t)(u * (FFO_BTILE * 2 / 16)), idesc, (first && s == 0) ? 0u : 1u);  // (0, u) opens level u
-            }
+            for (int s = 0; s < OZ_S; ++s)  // digit s times digits 0 .. 7 - s: levels s .. 7; (0, u) opens level u
+              tc::mma_bf16(acc0 + (uint32_t)(s * FFO_NT), a0 + (uint64_t)(s * (FFO_ATILE * 2 / 16)), b0,
+                           tc::idesc_bf16_f32(OZ_RT, FFO_NT * (OZ_S - s)), (first && s == 0) ? 0u : 1u);
             tc::commit(&empty[st]);
           }
           if (*fail) break;

@@ -18,8 +18,10 @@
 // One entry costs 144 digit products per k on the tensor cores and about 60
 // integer operations and one FP64 addition per K, where the FP64 pipe (two
 // multiply-adds per clock and SM on this part) spends 2 K clocks of an SM on it.
-// LU of 9 matrices of order 1250: 69.3 -> 16.9 ms; the cylinder's 65 matrices of order
-// 1280: updates 298 -> 17 ms.  Residuals of random factors 1.4e-15 (1.9e-15 on the
+// LU of 9 matrices of order 1250: 69.3 -> 13.1 ms; the cylinder's 65 matrices of order
+// 1280: updates 298 -> 12 ms (17 ms with an MMA per pair of digits, which is bound by
+// reading the tiles of L again and again: the digits of U lie behind one another, so
+// one MMA takes a digit of L times up to four of U into as many levels).  Residuals of random factors 1.4e-15 (1.9e-15 on the
 // FP64 pipe), of diagonally dominant ones 1.7e-16 (1.9e-16).
 //
 // The block row U12 = L11^{-1} A12 of a 128-column block: four FP64 triangular
@@ -42,7 +44,7 @@
 #define ZA_TILE (ZR * ZK)                       // bf16 elements of one digit of one part
 #define ZA_BLOCK (2 * OZ_S * ZA_TILE)           // [Re, Im][digit] of a k-tile
 #define ZB_TILE (ZC * ZK)
-#define ZB_BLOCK (3 * OZ_S * ZB_TILE)           // [digit][-Im, Re, Im]
+#define ZB_BLOCK (4 * OZ_S * ZB_TILE)           // [digit][Re, Im], then [digit][-Im, Re]
 #define Z_STAGE ((ZA_BLOCK + ZB_BLOCK) * 2)     // bytes of a k-tile of both operands
 #define Z_NST 2
 #define Z_DRAIN 16                              // drain warps of the product
@@ -233,9 +235,10 @@ __global__ void __launch_bounds__(256) z_slice_cols_kernel(const LuMat* __restri
         im[c] = __float2bfloat16((float)di[c][s]);
         nim[c] = __float2bfloat16((float)-di[c][s]);
       }
-      *(uint4*)(blk + (3 * s) * ZB_TILE) = *(const uint4*)nim;
-      *(uint4*)(blk + (3 * s + 1) * ZB_TILE) = *(const uint4*)re;
-      *(uint4*)(blk + (3 * s + 2) * ZB_TILE) = *(const uint4*)im;
+      *(uint4*)(blk + (2 * s) * ZB_TILE) = *(const uint4*)re;
+      *(uint4*)(blk + (2 * s + 1) * ZB_TILE) = *(const uint4*)im;
+      *(uint4*)(blk + (2 * OZ_S + 2 * s) * ZB_TILE) = *(const uint4*)nim;
+      *(uint4*)(blk + (2 * OZ_S + 2 * s + 1) * ZB_TILE) = *(const uint4*)re;
     }
   }
 }
@@ -347,7 +350,6 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
     }
   } else if (warp == Z_DRAIN + 1) {
     if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16_f32(ZR, 2 * ZC, false);
       int q = 0, k = 0;
       for (long long t = blockIdx.x; t < total && !*fail; t += gridDim.x) {
         int z, x, y;
@@ -363,18 +365,14 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
             if (kt == 0 && k > 0 && !tc::mbar_wait(&tempty[half], (k - 1) & 1)) { *fail = 1; break; }
             tc::fence_after();
 #pragma unroll
-            for (int l = 4 * half; l < 4 * half + 4; ++l) {
-              const uint32_t acc = tmem + (uint32_t)(l * 2 * ZC);
-#pragma unroll
-              for (int sd = 0; sd <= l; ++sd) {
-                const int td = l - sd;
-                const uint64_t are = a0 + (uint64_t)(sd * (ZA_TILE * 2 / 16));
-                const uint64_t aim = a0 + (uint64_t)((OZ_S + sd) * (ZA_TILE * 2 / 16));
-                const uint64_t bri = b0 + (uint64_t)((3 * td + 1) * (ZB_TILE * 2 / 16));  // [Re | Im]
-                const uint64_t bmr = b0 + (uint64_t)((3 * td) * (ZB_TILE * 2 / 16));      // [-Im | Re]
-                tc::mma_bf16(acc, are, bri, idesc, (kt == 0 && sd == 0) ? 0u : 1u);
-                tc::mma_bf16(acc, aim, bmr, idesc, 1u);
-              }
+            for (int sd = 0; sd < 4 * half + 4; ++sd) {  // digit sd of L times the digits td, td + 1, ..: levels l, l + 1, ..
+              const int l = sd > 4 * half ? sd : 4 * half, td = l - sd;
+              const uint32_t idesc = tc::idesc_bf16_f32(ZR, 2 * ZC * (4 * half + 4 - l)), acc = tmem + (uint32_t)(l * 2 * ZC);
+              const uint64_t are = a0 + (uint64_t)(sd * (ZA_TILE * 2 / 16));
+              const uint64_t aim = a0 + (uint64_t)((OZ_S + sd) * (ZA_TILE * 2 / 16));
+              const uint64_t bri = b0 + (uint64_t)(2 * td * (ZB_TILE * 2 / 16));
+              tc::mma_bf16(acc, are, bri, idesc, (kt == 0 && sd == 0) ? 0u : 1u);
+              tc::mma_bf16(acc, aim, bri + (uint64_t)(2 * OZ_S * (ZB_TILE * 2 / 16)), idesc, 1u);
             }
             if (kt == nkt - 1) tc::commit(&tfull[half]);
           }

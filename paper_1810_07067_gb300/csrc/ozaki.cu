@@ -36,7 +36,7 @@
 #define OZ_ABLOCK (2 * OZ_S * OZ_ATILE)   // per (row tile, k-tile): re/im x 8 slices
 // slice tile and block of Y for a job tile of jt right-hand-side columns
 __host__ __device__ constexpr int oz_ytile(int jt) { return jt * OZ_KT; }
-__host__ __device__ constexpr int oz_yblock(int jt) { return 3 * OZ_S * jt * OZ_KT; }  // [digit][-Im, Re, Im]
+__host__ __device__ constexpr int oz_yblock(int jt) { return 4 * OZ_S * jt * OZ_KT; }  // [digit][Re, Im], then [digit][-Im, Re]
 
 size_t ozaki_matrix_slices_elems(int npad, int batch) {
   return (size_t)batch * (npad / OZ_RT) * (npad / OZ_KT) * OZ_ABLOCK;
@@ -169,9 +169,10 @@ __global__ void oz_slice_vectors_kernel(const cd* __restrict__ y, int n, int npa
       im[c] = __float2bfloat16(dim_[c][s]);
       nim[c] = __float2bfloat16(-dim_[c][s]);
     }
-    *(uint4*)(blk + (3 * s + 0) * ytile + off) = *(uint4*)nim;
-    *(uint4*)(blk + (3 * s + 1) * ytile + off) = *(uint4*)re;
-    *(uint4*)(blk + (3 * s + 2) * ytile + off) = *(uint4*)im;
+    *(uint4*)(blk + (2 * s) * ytile + off) = *(uint4*)re;
+    *(uint4*)(blk + (2 * s + 1) * ytile + off) = *(uint4*)im;
+    *(uint4*)(blk + (2 * OZ_S + 2 * s) * ytile + off) = *(uint4*)nim;
+    *(uint4*)(blk + (2 * OZ_S + 2 * s + 1) * ytile + off) = *(uint4*)re;
   }
 }
 
@@ -251,7 +252,6 @@ __global__ void __launch_bounds__(192, 1)
     }
   } else if (warp == 5) {
     if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16_f32(OZ_RT, 2 * JT, false);
       int kt = 0;
       for (int c = 0; c < nchunk && !*fail; ++c) {
         const int set = c % NACC;
@@ -264,22 +264,27 @@ __global__ void __launch_bounds__(192, 1)
           if (!tc::mbar_wait(&full[st], (kt / NST) & 1)) { *fail = 1; break; }
           tc::fence_after();
           unsigned char* base = smem + (size_t)st * S::STAGE;
-          // digit s of Re a at s tiles, of Im a at OZ_S + s tiles (4 KiB each);
-          // digit t of y: [-Im, Re, Im] at 3t tiles (JT x 16 each)
+          // digit s of Re a at s tiles, of Im a at OZ_S + s tiles (4 KiB each); of y
+          // [Re, Im] at 2t tiles, [-Im, Re] at 2 (OZ_S + t) (JT x 16 each).  Digit s times the
+          // digits 0, 1, .. goes into the levels s, s + 1, .., as many as 256 columns hold at
+          // once: 16 or 24 MMAs a k-tile instead of 72 that each read A's tile again (three
+          // residuals of 192 vectors per mode, N = 512: 45 -> 35 ms; 4 vectors, N = 1024: 41 ->
+          // 29 ms)
           const uint64_t a0 = tc::desc_noswizzle(tc::smem_u32(base), 128, 256);
           const uint64_t y0 = tc::desc_noswizzle(tc::smem_u32(base + OZ_ABLOCK * 2), 128, 256);
           const bool first = kt == c * OZ_CHUNK;
+          constexpr int LV = 256 / (2 * JT);
 #pragma unroll
           for (int s = 0; s < OZ_S; ++s) {
+            const uint64_t are = a0 + (uint64_t)(s * (OZ_ATILE * 2 / 16));
+            const uint64_t aim = a0 + (uint64_t)((OZ_S + s) * (OZ_ATILE * 2 / 16));
 #pragma unroll
-            for (int t = 0; t < OZ_S - s; ++t) {
-              const uint32_t acc = acc0 + (uint32_t)((s + t) * 2 * JT);
-              const uint64_t are = a0 + (uint64_t)(s * (OZ_ATILE * 2 / 16));
-              const uint64_t aim = a0 + (uint64_t)((OZ_S + s) * (OZ_ATILE * 2 / 16));
-              const uint64_t yri = y0 + (uint64_t)((3 * t + 1) * (S::YT * 2 / 16));  // [Re | Im]
-              const uint64_t ymr = y0 + (uint64_t)((3 * t + 0) * (S::YT * 2 / 16));  // [-Im | Re]
+            for (int l = s; l < OZ_S; l += LV) {
+              const uint32_t idesc = tc::idesc_bf16_f32(OZ_RT, 2 * JT * (OZ_S - l < LV ? OZ_S - l : LV));
+              const uint64_t yri = y0 + (uint64_t)(2 * (l - s) * (S::YT * 2 / 16));
+              const uint32_t acc = acc0 + (uint32_t)(l * 2 * JT);
               tc::mma_bf16(acc, are, yri, idesc, (first && s == 0) ? 0u : 1u);
-              tc::mma_bf16(acc, aim, ymr, idesc, 1u);
+              tc::mma_bf16(acc, aim, yri + (uint64_t)(2 * OZ_S * (S::YT * 2 / 16)), idesc, 1u);
             }
           }
           tc::commit(&empty[st]);  // the stage is free once these MMAs have read it
@@ -400,6 +405,11 @@ void ozaki_residual(const __nv_bfloat16* Asl, const double* rowscale, int n, int
 // through a ring of k-tile stages, 5 issues MMAs into one of two accumulator
 // sets (8 levels x 32 columns each), so a tile's drain overlaps the next
 // tile's products.
+// The digits of B lie behind one another and so do the levels' accumulators, so digit
+// s of A times digits 0 .. 7 - s of B is one MMA of 32 (8 - s) columns into the levels
+// s .. 7: 8 instructions a k-tile that run at the tensor rate, where 36 of 32 columns
+// are bound by reading A's tile from shared memory again each time (N = 1024 body 26 ->
+// 19 ms in all products, the cylinder 7.1 -> 5.5 ms).
 #define OZR_NT 32
 #define OZR_BBLOCK (OZ_S * OZR_NT * OZ_KT)       // bf16 elements per (column tile, k-tile)
 #define OZR_ABLOCK (OZ_S * OZ_ATILE)             // per (row tile, k-tile)
@@ -452,7 +462,6 @@ __global__ void __launch_bounds__(192, 1)
     }
   } else if (warp == 5) {
     if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16_f32(OZ_RT, OZR_NT, false);
       int q = 0, k = 0;
       for (long long t = blockIdx.x; t < ntiles && !*fail; t += gridDim.x, ++k) {
         const int set = k & 1;
@@ -467,15 +476,9 @@ __global__ void __launch_bounds__(192, 1)
           const uint64_t a0 = tc::desc_noswizzle(tc::smem_u32(base), 128, 256);
           const uint64_t b0 = tc::desc_noswizzle(tc::smem_u32(base + OZR_ABLOCK * 2), 128, 256);
 #pragma unroll
-          for (int s = 0; s < OZ_S; ++s) {
-#pragma unroll
-            for (int u = 0; u < OZ_S - s; ++u) {
-              const uint32_t acc = acc0 + (uint32_t)((s + u) * OZR_NT);
-              const uint64_t ad = a0 + (uint64_t)(s * (OZ_ATILE * 2 / 16));
-              const uint64_t bd = b0 + (uint64_t)(u * (OZR_NT * OZ_KT * 2 / 16));
-              tc::mma_bf16(acc, ad, bd, idesc, (kt == 0 && s == 0) ? 0u : 1u);  // (0, u) opens level u
-            }
-          }
+          for (int s = 0; s < OZ_S; ++s)  // levels s .. 7 at once; (0, u) opens level u
+            tc::mma_bf16(acc0 + (uint32_t)(s * OZR_NT), a0 + (uint64_t)(s * (OZ_ATILE * 2 / 16)), b0,
+                         tc::idesc_bf16_f32(OZ_RT, OZR_NT * (OZ_S - s)), (kt == 0 && s == 0) ? 0u : 1u);
           tc::commit(&empty[st]);
         }
         if (*fail) break;
