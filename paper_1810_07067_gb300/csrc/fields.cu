@@ -111,7 +111,7 @@ __device__ __forceinline__ double ring_even_coef(const double* smp, int R, int Q
 // the wave alone sits in a table tab[w][q][6]: the factors of b_{m-1}, b_m,
 // b_{m+1} for E and for H.
 // FP64 pipe: N = 512, M = 64, 96 waves: 1.09 ms (7.91 ms with the four sampled
-// traces transformed ring by ring; 0.93 ms with the ring integrals of many waves on
+// traces transformed ring by ring; 0.90 ms with the ring integrals of many waves on
 // the tensor cores).
 
 // double-double helpers (error-free transforms) for the wave's rotation e^{-i m phi_d}:
@@ -267,9 +267,9 @@ size_t rhs_planewave_scratch_doubles(int M, int nrhs, int n_theta) {
 // below 1 KiB x (2M + 1) x 96 bytes whatever the number of waves.
 // Ring integrals of fewer multiply-adds than this stay on the FP64 pipe with the rest
 // of the data (one launch instead of four): N = 512, M = 64: 8 waves (1.3e7) 0.17 ms
-// there and 0.21 ms on the tensor cores, 32 waves (5e7) 0.43 and 0.42 ms, 96 waves
-// (1.6e8) 1.08 and 0.93 ms; N = 128, M = 16, 200 waves (1e7) 0.29 and 0.32 ms.
-#define RHS_FMA_MIN 8e7
+// there and 0.20 ms on the tensor cores, 32 waves (5e7) 0.43 and 0.40 ms, 96 waves
+// (1.6e8) 1.08 and 0.90 ms; N = 128, M = 16, 200 waves (1e7) 0.29 and 0.31 ms.
+#define RHS_FMA_MIN 4e7
 size_t rhs_planewave_work_bytes(int N, int M, int nrhs, int n_theta) {
   const double fma = (double)N * nrhs * (M + 2.0) * (n_theta / 4);
   return fma >= RHS_FMA_MIN ? rhs_oz_bytes(N, M, n_theta, nrhs < RHS_WAVES ? nrhs : RHS_WAVES) : 0;
@@ -290,9 +290,10 @@ void launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd
   const cd hf = C(k0) / (omega * mu0);  // H polarisation (k0 / (omega mu0)) d x e
   for (int w0 = 0; w0 < nrhs; w0 += RHS_WAVES) {
     const int c = nrhs - w0 < RHS_WAVES ? nrhs - w0 : RHS_WAVES;
-    rhs_wave_kernel<<<c, 128, smem_w, s>>>(M, k0, hf, sE, sH, dirs_dev + 3 * (size_t)w0, pols_dev + 3 * (size_t)w0,
-                                           n_theta, tab, wave, cost);
-    if (work) launch_rhs_products(g, M, wave, tab, w0, c, nrhs, n_theta, work, rhs, err, s);
+    const cd one = C(1.0);  // the tensor-core form applies the traces' factors itself
+    rhs_wave_kernel<<<c, 128, smem_w, s>>>(M, k0, work ? one : hf, work ? one : sE, work ? one : sH,
+                                           dirs_dev + 3 * (size_t)w0, pols_dev + 3 * (size_t)w0, n_theta, tab, wave, cost);
+    if (work) launch_rhs_products(g, M, wave, tab, sE, sH * hf, w0, c, nrhs, n_theta, work, rhs, err, s);
     else rhs_kernel<<<dim3(g.N / RHS_R, c), 256, smem, s>>>(g, M, wave, tab, cost, w0, nrhs, n_theta, rhs);
   }
 }

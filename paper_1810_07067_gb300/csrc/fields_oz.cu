@@ -1,4 +1,5 @@
-// Far field on a grid: sums over the nodes on BF16 tensor cores with FP64 accuracy.
+// The contractions of the fields on BF16 tensor cores with FP64 accuracy: the far field
+// on a grid, the ring integrals of plane waves, and the fields at points.
 //
 // Mode m at the polar angles p needs, for the currents X_u (u = 0, 1, 2) of every
 // right-hand side, sum_j b_a(p, j) {cos, sin}(p, j) X_u(j) with a = |m + 1|, |m|,
@@ -658,43 +659,52 @@ void ring_integrals(int sms, const RingPlan& f, const FieldGeom& g, int count, c
 }
 
 // Modal data of plane waves from the ring integrals (the formulas of rhs_kernel): rows
-// w N + i of coef, one thread per (node, wave) and a run of qc modes.  FP64 pipe: 39
-// operations per mode and node for both traces of E and of H (N = 512, M = 64, 96
-// waves: 0.59 ms of 0.93 ms).
+// w N + i of coef, one thread per (node, wave) and a run of qc modes m >= 0.  The table
+// without the traces' factors has u_0(-m) = s conj u_2(m), u_1(-m) = -s conj u_1(m),
+// u_2(-m) = s conj u_0(m), s = (-1)^(m+1) (real polarisations), so the sums of m give
+// those of -m: 63 FP64 operations for both modes, both traces of E and of H, where the
+// modes by themselves take 78 (N = 512, M = 64, 96 waves: 0.59 -> 0.55 ms).
 template <bool ALIGNED>
 __global__ void __launch_bounds__(128) rhs_rows_kernel(FieldGeom g, int M, const double2* __restrict__ wave,
-                                                       const cd* __restrict__ tab, const double* __restrict__ coef,
-                                                       int ncc, size_t ldc, int w0, int nrhs, int qc,
-                                                       cd* __restrict__ rhs) {
-  const int w = blockIdx.x, i = blockIdx.y * 128 + threadIdx.x, q0 = blockIdx.z * qc, q1 = min(q0 + qc, 2 * M + 1);
+                                                       const cd* __restrict__ tab, cd fE, cd fH,
+                                                       const double* __restrict__ coef, int ncc, size_t ldc, int w0,
+                                                       int nrhs, int qc, cd* __restrict__ rhs) {
+  const int w = blockIdx.x, i = blockIdx.y * 128 + threadIdx.x, m0 = blockIdx.z * qc, m1 = min(m0 + qc, M + 1);
   if (i >= g.N) return;
   double s, c;
   sincos(wave[w].y * g.z[i], &s, &c);
-  const cd pz = C(c, s);
+  const cd F[2] = {fE * C(c, s), fH * C(c, s)};
   const double rp = g.rp[i], zp = g.zp[i];
   const double* row = coef + (size_t)w * g.N + i;
   auto b = [&](int m) {
     const int a = abs(m);
     return row[((size_t)(a & 1) * ncc + (a >> 1)) * ldc];
   };
-  double bl = b(q0 - M - 1), b0 = b(q0 - M);
-  for (int q = q0; q < q1; ++q) {
-    const double bh = b(q - M + 1);
+  auto put = [&](cd* o, cd o0, cd o1) {
+    if (ALIGNED) {
+      ((double2*)o)[0] = make_double2(o0.x, o0.y);
+      ((double2*)o)[1] = make_double2(o1.x, o1.y);
+    } else {
+      o[0] = o0;
+      o[1] = o1;
+    }
+  };
+  const size_t ld = (size_t)nrhs * 4 * g.N;  // a mode
+  cd* o = rhs + (size_t)(w0 + w) * (4 * g.N) + 4 * i;
+  double bl = b(m0 - 1), b0 = b(m0);
+  for (int m = m0; m < m1; ++m) {
+    const double bh = b(m + 1);
     const double rl = rp * bl, rh = rp * bh, z0 = zp * b0;
-    const cd* u = tab + ((size_t)w * (2 * M + 1) + q) * 6;
-    cd* o = rhs + ((size_t)q * nrhs + w0 + w) * (4 * g.N) + 4 * i;
+    const cd* u = tab + ((size_t)w * (2 * M + 1) + M + m) * 6;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const cd u0 = u[3 * h], u1 = u[3 * h + 1], u2 = u[3 * h + 2];
       const cd d = C(fma(bl, u0.x, -(bh * u2.x)), fma(bl, u0.y, -(bh * u2.y)));
-      const cd v = C(fma(z0, u1.x, fma(rl, u0.x, rh * u2.x)), fma(z0, u1.y, fma(rl, u0.y, rh * u2.y)));
-      const cd o0 = mul_i(d) * pz, o1 = -(v * pz);
-      if (ALIGNED) {
-        ((double2*)o)[2 * h] = make_double2(o0.x, o0.y);
-        ((double2*)o)[2 * h + 1] = make_double2(o1.x, o1.y);
-      } else {
-        o[2 * h] = o0;
-        o[2 * h + 1] = o1;
+      const cd A = C(fma(rl, u0.x, rh * u2.x), fma(rl, u0.y, rh * u2.y)), G = z0 * u1;
+      put(o + (size_t)(M + m) * ld + 2 * h, mul_i(d * F[h]), -((A + G) * F[h]));
+      if (m > 0) {
+        const cd p = conj(d) * F[h], q = conj(A - G) * F[h];  // times -s and s
+        put(o + (size_t)(M - m) * ld + 2 * h, m & 1 ? C(p.y, -p.x) : mul_i(p), m & 1 ? -q : q);
       }
     }
     bl = b0;
@@ -797,8 +807,8 @@ size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs) {
   const size_t rt = tiles((size_t)rhs_oz_waves(f, N, nrhs) * N, OZ_RT);
   return up256(rt * f.a_row_tile) + f.b + f.cost + up256(rt * f.y_row_tile);
 }
-void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, int w0, int count, int nrhs,
-                         int n_theta, void* work, cd* rhs, int* err, cudaStream_t s) {
+void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, cd fE, cd fH, int w0, int count,
+                         int nrhs, int n_theta, void* work, cd* rhs, int* err, cudaStream_t s) {
   const RingPlan f = ring_plan(M, n_theta);
   const int sms = digit_ready();
   const int nw = rhs_oz_waves(f, g.N, nrhs);
@@ -812,15 +822,15 @@ void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const c
   for (int v0 = 0; v0 < count; v0 += nw) {
     const int c = std::min(nw, count - v0), nb = (g.N + 127) / 128;
     ring_integrals(sms, f, g, c, wave + v0, 0.0, 0, 0, Asl, Tsl, cost, coef, err, s);
-    // runs of modes: some 40000 threads in all, at least four modes each
-    const int runs = std::max(1, std::min((2 * M + 4) / 4, 320 / (nb * c) + 1)), qc = (2 * M + runs) / runs;
-    const dim3 grid(c, nb, (2 * M + qc) / qc);
+    // runs of modes: some 40000 threads in all, at least two pairs of modes each
+    const int runs = std::max(1, std::min((M + 2) / 2, 320 / (nb * c) + 1)), qc = (M + runs) / runs;
+    const dim3 grid(c, nb, (M + qc) / qc);
     const size_t ldc = tiles((size_t)c * g.N, OZ_RT) * OZ_RT;
     const cd* t = tab + (size_t)v0 * (2 * M + 1) * 6;
     if (((size_t)rhs & 15) == 0)
-      rhs_rows_kernel<true><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
+      rhs_rows_kernel<true><<<grid, 128, 0, s>>>(g, M, wave + v0, t, fE, fH, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
     else
-      rhs_rows_kernel<false><<<grid, 128, 0, s>>>(g, M, wave + v0, t, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
+      rhs_rows_kernel<false><<<grid, 128, 0, s>>>(g, M, wave + v0, t, fE, fH, coef, f.nct * FFO_NT, ldc, w0 + v0, nrhs, qc, rhs);
   }
 }
 

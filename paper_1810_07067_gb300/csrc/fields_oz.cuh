@@ -52,11 +52,11 @@ size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int n
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
                             int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s);
 
-// Modal data of the waves w0 .. w0 + count - 1 of nrhs from their table (rhs_wave_kernel);
-// work of rhs_oz_bytes (256-byte aligned).
+// Modal data of the waves w0 .. w0 + count - 1 of nrhs from their table (rhs_wave_kernel
+// without the factors fE, fH of the traces); work of rhs_oz_bytes (256-byte aligned).
 size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs);
-void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, int w0, int count, int nrhs,
-                         int n_theta, void* work, cd* rhs, int* err, cudaStream_t s);
+void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, cd fE, cd fH, int w0, int count,
+                         int nrhs, int n_theta, void* work, cd* rhs, int* err, cudaStream_t s);
 
 // Fields of nw right-hand sides at nt points from their ring points and currents
 // (ring_kernel) into out[w][p][6]; work of nearfield_oz_bytes (256-byte aligned).
