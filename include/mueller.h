@@ -189,7 +189,8 @@ int mueller_assemble(const mueller_curve* curve, const mueller_media* media, int
  * matrices until ||b' - A'y||_inf <= refine_tol (||A'||_inf ||y||_inf + ||b'||_inf)
  * for every mode and right-hand side (the normwise backward errors are
  * returned); MUELLER_ENOCONV with the last iterate if refine_max_iter steps
- * do not reach it. */
+ * do not reach it; MUELLER_ETIMEOUT if a bounded device-side wait of the
+ * residual or of the complex64 solve (nrhs > 4) gave up. */
 int mueller_solve(mueller_ctx* ctx, const mueller_c128* rhs_dev, int nrhs, mueller_c128* x_dev,
                   double* backward_err, void* stream);
 
@@ -198,7 +199,12 @@ int mueller_solve(mueller_ctx* ctx, const mueller_c128* rhs_dev, int nrhs, muell
  * (pols = unit e, orthogonal to d).  Rows are the Fourier coefficients
  * (1/2pi) int f e^{-i m theta} of the tangential traces n x E and n x H, scaled
  * by i omega eps0 and i omega mu0 (eq. mullerrep) or i omega mu0 and
- * i omega eps0 (eq. dualmullrep).  rhs_dev: [2M+1][nrhs][4N]. */
+ * i omega eps0 (eq. dualmullrep).  rhs_dev: [2M+1][nrhs][4N].
+ * With many waves the ring integrals are exact-digit products on the tensor
+ * cores, in a workspace allocated for the call (at most about 0.8 GB for
+ * bodies of a few thousand nodes; on the FP64 pipe where it cannot be had);
+ * MUELLER_ETIMEOUT if a bounded device-side wait of them gave up (rhs_dev is
+ * then unusable). */
 int mueller_rhs_planewave(mueller_ctx* ctx, const double* dirs, const double* pols, int nrhs,
                           mueller_c128* rhs_dev, void* stream);
 
@@ -218,7 +224,12 @@ int mueller_rhs_fields(mueller_ctx* ctx, const mueller_c128* EH_dev, int nrhs, i
  * the far field is a sum over m of e^{i m phi} times a per-mode vector
  * (Section 4's separation of variables applied to eq. farfieldform), then
  * rotated to Cartesian components.  x_dev: currents [2M+1][nrhs][4N];
- * E_dev: device [nrhs][n_polar][n_azim][3]. */
+ * E_dev: device [nrhs][n_polar][n_azim][3].  All but small grids run as
+ * exact-digit products on the tensor cores, in a workspace allocated for the
+ * call (operand digits in passes of 512 MB; on the FP64 pipe where it cannot
+ * be had); MUELLER_ETIMEOUT if a bounded device-side wait of them gave up
+ * (E_dev is then unusable).  A side with an infinite or NaN current has NaN
+ * in its field and leaves the other sides alone. */
 int mueller_far_field_grid(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs, int n_polar, int n_azim,
                            mueller_c128* E_dev, void* stream);
 
@@ -233,7 +244,11 @@ int mueller_far_field_grid(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs
  * 40 r_max / d_min) points (at most 8192), d_min the closest target-to-node
  * distance.  A target on a node ring is rejected (MUELLER_EINVAL).  x_dev:
  * currents [2M+1][nrhs][4N]; targets: host [ntargets][3]; out_dev: device
- * [nrhs][ntargets][6] complex, (E, H) in Cartesian components. */
+ * [nrhs][ntargets][6] complex, (E, H) in Cartesian components.  With many
+ * (target, ring point) pairs the kernels' products with the currents are
+ * exact-digit products on the tensor cores, in a workspace allocated for the
+ * call (on the FP64 pipe where it cannot be had); MUELLER_ETIMEOUT if a
+ * bounded device-side wait of them gave up (out_dev is then unusable). */
 int mueller_eval(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs, const double* targets, int ntargets,
                  int region, mueller_c128* out_dev, void* stream);
 
@@ -287,7 +302,12 @@ int mueller_modal_kernels_noalloc(const double* pairs_dev, long long npairs, mue
 
 /* Batched LU of `batch` column-major n x n complex matrices in place
  * (stride n*n); piv_dev [batch][n] (0-based LAPACK-style interchanges),
- * info_dev [batch] (0 or first zero-pivot column + 1). */
+ * info_dev [batch] (0 or first zero-pivot column + 1).  The updates are
+ * exact-digit products on the tensor cores (FP64 accuracy, relative to the
+ * largest |l| |u| of an entry's row and column), in a workspace allocated for
+ * the call (at most 4 GB, or one matrix's); they run on the FP64 pipe where it
+ * cannot be had.  Returns MUELLER_ETIMEOUT if a bounded device-side wait gave
+ * up (the factors are then unusable).  Synchronises `stream`. */
 int mueller_lu_batched(mueller_c128* A_dev, int n, int batch, int* piv_dev, int* info_dev, void* stream);
 
 /* The same factorisation in complex64, as used by the mixed-precision path

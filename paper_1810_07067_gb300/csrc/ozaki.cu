@@ -14,11 +14,11 @@
 // drained: the levels joined in 64-bit integers, converted on the integer pipe and
 // added in FP64 once per value (a conversion and a multiply-add per level on the
 // FP64 pipe took longer than the products: N = 512, M = 64, 192 vectors per mode,
-// 24.7 -> 15.0 ms a residual).  The complex product takes two MMAs per digit
-// pair: the B operand stacks the digits of Re y over those of Im y (2 jt
-// rows), so Re a [Re y | Im y] + Im a [-Im y | Re y] lands in [Re | Im] of the
-// accumulator; the y slices are stored as [-Im, Re, Im] per digit, and the
-// two B operands start at Re and at -Im.
+// 24.7 -> 15.0 ms a residual).  The complex product takes two MMAs: the B operand
+// stacks the digits of Re y over those of Im y (2 jt rows), so Re a [Re y | Im y] +
+// Im a [-Im y | Re y] lands in [Re | Im] of the accumulator; the y slices are stored as
+// [Re, Im] digit by digit and again as [-Im, Re], so that one MMA takes a digit of a
+// times as many digits of y as 256 columns hold.
 // Operand tiles are stored in global memory in the shared-memory layout of the
 // MMA (no-swizzle K-major core matrices), so each 16-wide k-tile is a single
 // bulk asynchronous copy (TMA).  The residual kernel is warp-specialised: a
