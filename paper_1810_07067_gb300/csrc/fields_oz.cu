@@ -103,56 +103,43 @@ __global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int nrt, co
 }
 
 // Columns of mode q and right-hand side w0 + w: X_0 = r' J1 + i J2, X_1 = z' J1,
-// X_2 = r' J1 - i J2 (and of M), for a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w).
+// X_2 = r' J1 - i J2 (and of M), for a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w, X).
 __global__ void __launch_bounds__(64) ffo_cols_kernel(FieldGeom g, int M, const cd* __restrict__ x, int nrhs, int w0,
                                                       int nw, int nct, __nv_bfloat16* __restrict__ Bsl,
                                                       double* __restrict__ cscale) {
-  __shared__ unsigned red[6][2];
-  const int q = blockIdx.x, w = blockIdx.y, m = q - M, N = g.N, nkt = N / OZ_KT, tid = threadIdx.x;
-  const cd* xv = x + ((size_t)q * nrhs + w0 + w) * 4 * N;
-  auto value = [&](int j, int h, int u) {
-    const cd v1 = xv[4 * j + 2 * h];
+  __shared__ unsigned red[2];
+  const int q = blockIdx.x, w = blockIdx.y, h = blockIdx.z / 3, u = blockIdx.z % 3;
+  const int s = q - M + 1 - u, a = abs(s), N = g.N, nkt = N / OZ_KT, tid = threadIdx.x;
+  const cd* xv = x + ((size_t)q * nrhs + w0 + w) * 4 * N + 2 * h;
+  auto value = [&](int j) {
+    const cd v1 = xv[4 * j];
     if (u == 1) return g.zp[j] * v1;
-    const cd r1 = g.rp[j] * v1, v2 = mul_i(xv[4 * j + 2 * h + 1]);
+    const cd r1 = g.rp[j] * v1, v2 = mul_i(xv[4 * j + 1]);
     return u == 0 ? r1 + v2 : r1 - v2;
   };
-  unsigned ex[6];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) ex[c] = 0u;
-  for (int j = tid; j < N; j += 64)
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const cd v = value(j, c / 3, c % 3);
-      ex[c] = max(ex[c], max(exp_field(v.x), exp_field(v.y)));
-    }
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    ex[c] = __reduce_max_sync(0xffffffffu, ex[c]);
-    if ((tid & 31) == 0) red[c][tid >> 5] = ex[c];
+  unsigned ex = 0u;
+  for (int j = tid; j < N; j += 64) {
+    const cd v = value(j);
+    ex = max(ex, max(exp_field(v.x), exp_field(v.y)));
   }
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  if ((tid & 31) == 0) red[tid >> 5] = ex;
   __syncthreads();
-#pragma unroll 1
-  for (int c = 0; c < 6; ++c) {
-    const int h = c / 3, u = c % 3, s = m + 1 - u, a = abs(s);
-    const unsigned e = max(red[c][0], red[c][1]);
-    const int col = ((u * 2 + (s < 0)) * nw + w) * 4 + 2 * h, ct = col / FFO_NT, cc = col % FFO_NT;
-    if (tid == 0) {
-      cscale[((size_t)a * nct) * FFO_NT + col] = scale_of(e);
-      cscale[((size_t)a * nct) * FFO_NT + col + 1] = scale_of(e);
-    }
-    __nv_bfloat16* base = Bsl + ((size_t)a * nct + ct) * nkt * FFO_BBLOCK;
-    for (int j = 8 * tid; j < N; j += 8 * 64) {
-      double re[8], im[8];
+  const unsigned e = max(red[0], red[1]);
+  const int col = ((u * 2 + (s < 0)) * nw + w) * 4 + 2 * h, ct = col / FFO_NT, cc = col % FFO_NT;
+  if (tid < 2) cscale[((size_t)a * nct) * FFO_NT + col + tid] = scale_of(e);
+  __nv_bfloat16* base = Bsl + ((size_t)a * nct + ct) * nkt * FFO_BBLOCK;
+  for (int j = 8 * tid; j < N; j += 8 * 64) {
+    double re[8], im[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const cd v = value(j + i, h, u);
-        re[i] = v.x;
-        im[i] = v.y;
-      }
-      __nv_bfloat16* d = base + (size_t)(j / OZ_KT) * FFO_BBLOCK;
-      put_digits(d + core_off(cc, j % OZ_KT), FFO_BTILE, re, scale_exp(e));
-      put_digits(d + core_off(cc + 1, j % OZ_KT), FFO_BTILE, im, scale_exp(e));
+    for (int i = 0; i < 8; ++i) {
+      const cd v = value(j + i);
+      re[i] = v.x;
+      im[i] = v.y;
     }
+    __nv_bfloat16* d = base + (size_t)(j / OZ_KT) * FFO_BBLOCK;
+    put_digits(d + core_off(cc, j % OZ_KT), FFO_BTILE, re, scale_exp(e));
+    put_digits(d + core_off(cc + 1, j % OZ_KT), FFO_BTILE, im, scale_exp(e));
   }
 }
 
@@ -321,22 +308,25 @@ __global__ void __launch_bounds__(128) ffo_vector_kernel(int M, double k0, doubl
 // (even and odd m) of the samples' digits with one table of weighted cosines.
 
 // Digits of the table, column c of parity par for m = 2 c + par <= M + 1, and
-// cost[t] = cos theta_t.  One CTA per (column, parity).
-__global__ void __launch_bounds__(32) ring_table_kernel(int M, int n, int nkt, int nct, int E,
-                                                        __nv_bfloat16* __restrict__ Bsl, double* __restrict__ cost) {
-  const int c = blockIdx.x, par = blockIdx.y, m = 2 * c + par, Q = n / 4 + 1;
+// cost[t] = cos theta_t.  One CTA per (column, parity); a value per thread, whose cosine
+// is a long chain of FP64 operations, then 8 values' digits per thread (M = 64, 65
+// samples: 20 -> 6 us against 8 values per thread).
+__global__ void __launch_bounds__(128) ring_table_kernel(int M, int n, int nkt, int nct, int E,
+                                                         __nv_bfloat16* __restrict__ Bsl, double* __restrict__ cost) {
+  __shared__ __align__(16) double v[128];
+  const int c = blockIdx.x, par = blockIdx.y, m = 2 * c + par, Q = n / 4 + 1, K = nkt * OZ_KT, tid = threadIdx.x;
   if (c == 0 && par == 0)
-    for (int t = threadIdx.x; t < nkt * OZ_KT; t += 32) cost[t] = t < Q ? cospi(2.0 * t / n) : 0.0;
+    for (int t = tid; t < K; t += 128) cost[t] = t < Q ? cospi(2.0 * t / n) : 0.0;
   if (m > M + 1) return;
   __nv_bfloat16* base = Bsl + ((size_t)par * nct + c / FFO_NT) * nkt * FFO_BBLOCK;
-  for (int t0 = 8 * threadIdx.x; t0 < nkt * OZ_KT; t0 += 8 * 32) {
-    double v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int t = t0 + i;
-      v[i] = t < Q ? (t == 0 || t == Q - 1 ? 2.0 : 4.0) / n * cospi(2.0 * (int)((long long)m * t % n) / n) : 0.0;
-    }
-    put_digits(base + (size_t)(t0 / OZ_KT) * FFO_BBLOCK + core_off(c % FFO_NT, t0 % OZ_KT), FFO_BTILE, v, E);
+  for (int t0 = 0; t0 < K; t0 += 128) {
+    const int t = t0 + tid;
+    v[tid] = t < Q ? (t == 0 || t == Q - 1 ? 2.0 : 4.0) / n * cospi(2.0 * (int)((long long)m * t % n) / n) : 0.0;
+    __syncthreads();
+    const int k = t0 + 8 * tid;
+    if (tid < 16 && k < K)
+      put_digits(base + (size_t)(k / OZ_KT) * FFO_BBLOCK + core_off(c % FFO_NT, k % OZ_KT), FFO_BTILE, v + 8 * tid, E);
+    __syncthreads();
   }
 }
 
@@ -416,19 +406,21 @@ __global__ void __launch_bounds__(128) synth_rows_kernel(int M, int n_polar, con
   if (tid < 12) rscale[(size_t)(tid / 6) * nrt * OZ_RT + 6ll * wp + tid % 6] = scale_of(ex[tid]);
 }
 
-// cos and sin of m phi_s, column s = 0..n_azim / 2.  One CTA per (column, index).
-__global__ void __launch_bounds__(32) synth_table_kernel(int M, int n, int nkt, int nct, __nv_bfloat16* __restrict__ Bsl) {
-  const int s = blockIdx.x, b = blockIdx.y;
+// cos and sin of m phi_s, column s = 0..n_azim / 2.  One CTA per (column, index), a value
+// per thread.
+__global__ void __launch_bounds__(128) synth_table_kernel(int M, int n, int nkt, int nct, __nv_bfloat16* __restrict__ Bsl) {
+  __shared__ __align__(16) double v[128];
+  const int s = blockIdx.x, b = blockIdx.y, K = nkt * OZ_KT, tid = threadIdx.x;
   __nv_bfloat16* base = Bsl + ((size_t)b * nct + s / FFO_NT) * nkt * FFO_BBLOCK;
-  for (int m0 = 8 * threadIdx.x; m0 < nkt * OZ_KT; m0 += 8 * 32) {
-    double v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int m = m0 + i;
-      const double x = 2.0 * (int)((long long)m * s % n) / n;
-      v[i] = m > M ? 0.0 : b ? sinpi(x) : cospi(x);
-    }
-    put_digits(base + (size_t)(m0 / OZ_KT) * FFO_BBLOCK + core_off(s % FFO_NT, m0 % OZ_KT), FFO_BTILE, v, 1);
+  for (int m0 = 0; m0 < K; m0 += 128) {
+    const int m = m0 + tid;
+    const double x = 2.0 * (int)((long long)m * s % n) / n;
+    v[tid] = m > M ? 0.0 : b ? sinpi(x) : cospi(x);
+    __syncthreads();
+    const int k = m0 + 8 * tid;
+    if (tid < 16 && k < K)
+      put_digits(base + (size_t)(k / OZ_KT) * FFO_BBLOCK + core_off(s % FFO_NT, k % OZ_KT), FFO_BTILE, v + 8 * tid, 1);
+    __syncthreads();
   }
 }
 
@@ -649,7 +641,7 @@ RingPlan ring_plan(int M, int n) {
   return f;
 }
 void ring_table(const RingPlan& f, int M, int n, __nv_bfloat16* Bsl, double* cost, cudaStream_t s) {
-  ring_table_kernel<<<dim3(f.nct * FFO_NT, 2), 32, 0, s>>>(M, n, f.nkt, f.nct, f.E, Bsl, cost);
+  ring_table_kernel<<<dim3(f.nct * FFO_NT, 2), 128, 0, s>>>(M, n, f.nkt, f.nct, f.E, Bsl, cost);
 }
 void ring_integrals(int sms, const RingPlan& f, const FieldGeom& g, int count, const double2* scale, double k0, int p0, int n_polar,
                     __nv_bfloat16* Asl, const __nv_bfloat16* Bsl, const double* cost, double* Y, int* err, cudaStream_t s) {
@@ -781,13 +773,13 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
                                                  tiles((size_t)np * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
     for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
       const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles(24 * nw, FFO_NT);
-      ffo_cols_kernel<<<dim3(2 * M + 1, nw), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
+      ffo_cols_kernel<<<dim3(2 * M + 1, nw, 6), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
       digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
       ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
           M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
     }
   }
-  synth_table_kernel<<<dim3(n_azim / 2 + 1, 2), 32, 0, s>>>(M, n_azim, f.snkt, f.snct, Bsl);
+  synth_table_kernel<<<dim3(n_azim / 2 + 1, 2), 128, 0, s>>>(M, n_azim, f.snkt, f.snct, Bsl);
   for (int w0 = 0; w0 < nrhs; w0 += f.snw) {
     const int nw = std::min(f.snw, nrhs - w0), nrt = (int)tiles((size_t)6 * nw * n_polar, OZ_RT);
     synth_rows_kernel<<<dim3(n_polar, nw), 128, 12 * (f.snkt * OZ_KT * 8 + 4), s>>>(
