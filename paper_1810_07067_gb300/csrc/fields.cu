@@ -190,7 +190,6 @@ __global__ void __launch_bounds__(128) rhs_wave_kernel(int M, double k0, cd hf, 
 // One CTA per (RHS_R nodes, wave): samples of the nodes' ring phases, their
 // coefficients b_m, then two rows (E or H) per (mode, node) and thread.
 #define RHS_R 8
-#define RHS_WAVES 1024
 __global__ void __launch_bounds__(256) rhs_kernel(FieldGeom g, int M, const double2* __restrict__ wave,
                                                   const cd* __restrict__ tab, const double* __restrict__ cost,
                                                   int w0, int nrhs, int n, cd* __restrict__ rhs) {
@@ -272,12 +271,17 @@ size_t rhs_planewave_scratch_doubles(int M, int nrhs, int n_theta) {
 #define RHS_FMA_MIN 4e7
 size_t rhs_planewave_work_bytes(int N, int M, int nrhs, int n_theta) {
   const double fma = (double)N * nrhs * (M + 2.0) * (n_theta / 4);
-  return fma >= RHS_FMA_MIN ? rhs_oz_bytes(N, M, n_theta, nrhs < RHS_WAVES ? nrhs : RHS_WAVES) : 0;
+  return fma >= RHS_FMA_MIN ? rhs_plan(N, M, n_theta, nrhs).bytes : 0;
 }
 
-void launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd mu0, cd sE, cd sH,
+bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd mu0, cd sE, cd sH,
                           const double* dirs_dev, const double* pols_dev, int nrhs, int n_theta, double* scratch,
-                          void* work, cd* rhs, int* err, cudaStream_t s) {
+                          void* work, size_t work_bytes, cd* rhs, int* err, cudaStream_t s) {
+  RhsPlan plan{};
+  if (work) {
+    plan = rhs_plan(g.N, M, n_theta, nrhs);
+    if (plan.bytes > work_bytes) return false;
+  }
   const int Q = n_theta / 4 + 1;
   const int smem_w = (M + 2) * (int)sizeof(cd);
   const int smem = (n_theta + 2 * RHS_R * Q + RHS_R * (M + 4)) * (int)sizeof(double);
@@ -293,9 +297,10 @@ void launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd
     const cd one = C(1.0);  // the tensor-core form applies the traces' factors itself
     rhs_wave_kernel<<<c, 128, smem_w, s>>>(M, k0, work ? one : hf, work ? one : sE, work ? one : sH,
                                            dirs_dev + 3 * (size_t)w0, pols_dev + 3 * (size_t)w0, n_theta, tab, wave, cost);
-    if (work) launch_rhs_products(g, M, wave, tab, sE, sH * hf, w0, c, nrhs, n_theta, work, rhs, err, s);
+    if (work) launch_rhs_products(g, M, wave, tab, sE, sH * hf, w0, c, nrhs, n_theta, plan, work, rhs, err, s);
     else rhs_kernel<<<dim3(g.N / RHS_R, c), 256, smem, s>>>(g, M, wave, tab, cost, w0, nrhs, n_theta, rhs);
   }
+  return true;
 }
 
 // Currents on the node rings: cur[w][i][t][a] = sum_m x[m][w][4i+a] e^{i m theta_t}

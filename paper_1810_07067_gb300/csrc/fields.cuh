@@ -10,12 +10,13 @@ struct FieldGeom {
 // Modal plane-wave data: rhs[q][w][4N], q = m + M (k0 real, n_theta a multiple
 // of 4); scratch of rhs_planewave_scratch_doubles values, 16-byte aligned, and work
 // of rhs_planewave_work_bytes (256-byte aligned; null: the ring integrals run on the
-// FP64 pipe); err (device int) is set if a bounded wait gives up.
+// FP64 pipe); err (device int) is set if a bounded wait gives up.  False, with nothing
+// launched, when work_bytes do not hold the layout.
 size_t rhs_planewave_scratch_doubles(int M, int nrhs, int n_theta);
 size_t rhs_planewave_work_bytes(int N, int M, int nrhs, int n_theta);
-void launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd mu0, cd sE, cd sH,
+bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd mu0, cd sE, cd sH,
                           const double* dirs_dev, const double* pols_dev, int nrhs, int n_theta, double* scratch,
-                          void* work, cd* rhs, int* err, cudaStream_t s);
+                          void* work, size_t work_bytes, cd* rhs, int* err, cudaStream_t s);
 
 // Far field E[rhs][dir][3] from currents x[q][rhs][4N]; ring work buffer
 // cur[rhs][N][n_theta][4].

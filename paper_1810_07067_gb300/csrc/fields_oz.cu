@@ -23,21 +23,16 @@
 #include <cmath>
 #include "digits.cuh"
 #include "fields_oz.cuh"
+#include "fields_plan.cuh"
 #include "ozaki.cuh"
 #include "smem.cuh"
 #include "tc.cuh"
 
 namespace {
 
-#define FFO_ATILE (OZ_RT * OZ_KT)
-#define FFO_ABLOCK (OZ_S * FFO_ATILE)       // bf16 elements per (row tile, k-tile)
-#define FFO_NT 32                           // columns of a tile
-#define FFO_BTILE (FFO_NT * OZ_KT)
-#define FFO_BBLOCK (OZ_S * FFO_BTILE)       // per (column tile, k-tile)
 #define FFO_STAGE ((FFO_ABLOCK + FFO_BBLOCK) * 2)
 #define FFO_NST 4
 #define FFO_SET (OZ_S * FFO_NT)             // tensor-memory columns of one accumulator set
-#define FFO_BYTES ((size_t)512 << 20)       // digits of either operand held at a time
 
 // exponent field of the largest |v| seen -> E with |v| / 2^E < 1/2; all zero: 2^E = 2^-1020
 __device__ __forceinline__ int scale_exp(unsigned ex) { return (int)max(ex, 1u) - 1021; }
@@ -619,27 +614,6 @@ void digit_gemm(int sms, const __nv_bfloat16* Asl, const double* rscale, const _
       Asl, rscale, Bsl, cscale, sc, nkt, nrt, nct, ntiles, Y, err);
 }
 
-size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
-size_t tiles(size_t v, size_t t) { return (v + t - 1) / t; }
-
-// Ring integrals of rows k N + i, k < count.
-struct RingPlan {
-  int nkt, nct, E;
-  size_t a_row_tile, b, cost, y_row_tile;  // bytes, per 128 rows (a, y) or in all
-};
-RingPlan ring_plan(int M, int n) {
-  RingPlan f{};
-  f.nkt = (int)tiles(n / 4 + 1, OZ_KT);
-  f.nct = (int)tiles(M / 2 + 1 + (M & 1), FFO_NT);  // m = 0, 2, ... (1, 3, ...) up to M + 1
-  int e = 0;
-  frexp(4.0 / n, &e);
-  f.E = e + 1;
-  f.a_row_tile = (size_t)2 * f.nkt * FFO_ABLOCK * 2;
-  f.b = up256((size_t)2 * f.nct * f.nkt * FFO_BBLOCK * 2);
-  f.cost = up256((size_t)f.nkt * OZ_KT * 8);
-  f.y_row_tile = (size_t)2 * f.nct * FFO_NT * OZ_RT * 8;
-  return f;
-}
 void ring_table(const RingPlan& f, int M, int n, __nv_bfloat16* Bsl, double* cost, cudaStream_t s) {
   ring_table_kernel<<<dim3(f.nct * FFO_NT, 2), 128, 0, s>>>(M, n, f.nkt, f.nct, f.E, Bsl, cost);
 }
@@ -790,26 +764,15 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
   }
 }
 
-// Waves of a pass: as many as keep the samples' digits within FFO_BYTES, at least one.
-static int rhs_oz_waves(const RingPlan& f, int N, int nrhs) {
-  return (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / f.a_row_tile * OZ_RT / N));
-}
-size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs) {
-  const RingPlan f = ring_plan(M, n_theta);
-  const size_t rt = tiles((size_t)rhs_oz_waves(f, N, nrhs) * N, OZ_RT);
-  return up256(rt * f.a_row_tile) + f.b + f.cost + up256(rt * f.y_row_tile);
-}
 void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, cd fE, cd fH, int w0, int count,
-                         int nrhs, int n_theta, void* work, cd* rhs, int* err, cudaStream_t s) {
-  const RingPlan f = ring_plan(M, n_theta);
+                         int nrhs, int n_theta, const RhsPlan& plan, void* work, cd* rhs, int* err, cudaStream_t s) {
+  const RingPlan& f = plan.ring;
   const int sms = digit_ready();
-  const int nw = rhs_oz_waves(f, g.N, nrhs);
-  const size_t rt = tiles((size_t)nw * g.N, OZ_RT);
-  char* p = (char*)work;
-  auto* Asl = (__nv_bfloat16*)p;
-  auto* Tsl = (__nv_bfloat16*)(p += up256(rt * f.a_row_tile));
-  auto* cost = (double*)(p += f.b);
-  auto* coef = (double*)(p += f.cost);
+  const int nw = plan.waves;
+  auto* Asl = (__nv_bfloat16*)((char*)work + plan.a);
+  auto* Tsl = (__nv_bfloat16*)((char*)work + plan.table);
+  auto* cost = (double*)((char*)work + plan.cost);
+  auto* coef = (double*)((char*)work + plan.coef);
   ring_table(f, M, n_theta, Tsl, cost, s);
   for (int v0 = 0; v0 < count; v0 += nw) {
     const int c = std::min(nw, count - v0), nb = (g.N + 127) / 128;

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include "cplx.cuh"
 #include "fields.cuh"
+#include "fields_plan.cuh"
 
 // F of mode m (index q) at polar angle p and, when it is another one, at its mirror
 // n_polar - 1 - p, from the sums A (cosine of the phase) and B (sine): u = 0, 1, 2
@@ -52,11 +53,11 @@ size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int n
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
                             int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s);
 
-// Modal data of the waves w0 .. w0 + count - 1 of nrhs from their table (rhs_wave_kernel
-// without the factors fE, fH of the traces); work of rhs_oz_bytes (256-byte aligned).
-size_t rhs_oz_bytes(int N, int M, int n_theta, int nrhs);
+// Modal data of the waves w0 .. w0 + count - 1 (count <= RHS_WAVES) of nrhs from their
+// table (rhs_wave_kernel without the factors fE, fH of the traces); work of plan.bytes
+// (256-byte aligned), plan the rhs_plan of the same nrhs.
 void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, cd fE, cd fH, int w0, int count,
-                         int nrhs, int n_theta, void* work, cd* rhs, int* err, cudaStream_t s);
+                         int nrhs, int n_theta, const RhsPlan& plan, void* work, cd* rhs, int* err, cudaStream_t s);
 
 // Fields of nw right-hand sides at nt points from their ring points and currents
 // (ring_kernel) into out[w][p][6]; work of nearfield_oz_bytes (256-byte aligned).

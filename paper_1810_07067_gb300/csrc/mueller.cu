@@ -1354,8 +1354,9 @@ extern "C" int mueller_rhs_planewave(mueller_ctx* c, const double* dirs, const d
     work = nullptr;
   }
   if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  launch_rhs_planewave(g, c->S.M, c->S.k0.x, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, nth, scratch, work,
-                       (cd*)rhs_dev, err, s);
+  if (!launch_rhs_planewave(g, c->S.M, c->S.k0.x, c->S.omega, c->S.mu0, c->S.sE, c->S.sH, dd, dp, nrhs, nth, scratch,
+                            work, bytes, (cd*)rhs_dev, err, s))
+    return fail(MUELLER_EINVAL, "workspace of the ring integrals too small");
   CK(cudaGetLastError());
   int herr = 0;
   if (work) CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));

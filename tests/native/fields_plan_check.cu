@@ -1,0 +1,20 @@
+// Host-side driver of the workspace plans (csrc/fields_plan.cuh, compiled for the
+// CPU).  Reads one plan's arguments per line from stdin and prints its fields.
+#include <cstdio>
+#include <cstring>
+#include "../../paper_1810_07067_gb300/csrc/fields_plan.cuh"
+
+int main() {
+  char op[8];
+  while (scanf("%7s", op) == 1) {
+    if (!strcmp(op, "rhs")) {
+      int N, M, n, nrhs;
+      if (scanf("%d %d %d %d", &N, &M, &n, &nrhs) != 4) return 1;
+      const RhsPlan f = rhs_plan(N, M, n, nrhs);
+      printf("%d %d %d %zu %zu %zu %zu %zu\n", f.ring.nkt, f.ring.nct, f.waves, f.a, f.table, f.cost, f.coef, f.bytes);
+    } else {
+      return 1;
+    }
+  }
+  return 0;
+}

@@ -1,0 +1,54 @@
+"""Workspace plans of the tensor-core field products (csrc/fields_plan.cuh, compiled for
+the CPU): what the kernels of every pass write, counted here from their tiles, ends
+inside the block that the plan asks for."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+pytestmark = pytest.mark.skipif(shutil.which("nvcc") is None, reason="nvcc not found")
+MB = 1 << 20
+
+
+def _up(a, b):
+    return -(-a // b)
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("plan") / "fields_plan_check")
+    subprocess.run(["nvcc", "-O2", "-std=c++17", "-o", exe, os.path.join(HERE, "native", "fields_plan_check.cu")],
+                   check=True, capture_output=True, timeout=300)
+
+    def run(op, cases):
+        lines = "".join(op + " " + " ".join(str(v) for v in c) + "\n" for c in cases)
+        out = subprocess.run([exe], input=lines, capture_output=True, text=True, timeout=300)
+        assert out.returncode == 0, out.stderr
+        rows = [[int(v) for v in line.split()] for line in out.stdout.strip().split("\n")]
+        assert len(rows) == len(cases)
+        return rows
+
+    return run
+
+
+def test_plane_wave_passes_stay_inside(plan):
+    """Bodies of 16 to 4096 nodes, 1 to 65535 waves; launches take at most 1024 of them."""
+    rng = np.random.default_rng(11)
+    cases = [(64, 10, 96, 2200), (128, 32, 144, 1500), (160, 20, 112, 2000), (256, 32, 144, 1500), (128, 64, 208, 1100)]
+    for N in (16, 32, 64, 128, 256, 512, 1024, 4096):
+        for nrhs in (1, 2, 1023, 1024, 1025, 2048, 65535):
+            M = int(rng.integers(0, 560))
+            cases.append((N, M, (2 * M + 64 + int(rng.integers(0, 400)) + 15) // 16 * 16, nrhs))
+    for (N, M, n, nrhs), (nkt, nct, waves, a, table, cost, coef, nbytes) in zip(cases, plan("rhs", cases)):
+        assert nkt == _up(n // 4 + 1, 16) and nct * 32 > (M + 1) // 2
+        assert 1 <= waves <= min(nrhs, 1024)
+        rows = _up(waves * N, 128) * 128                     # of the fullest pass
+        assert a == 0 and a + 2 * nkt * rows * 16 * 8 * 2 <= table          # two parities, 8 digits of 2 bytes
+        assert table + 2 * nkt * nct * 32 * 16 * 8 * 2 <= cost
+        assert cost + nkt * 16 * 8 <= coef
+        assert coef + 2 * nct * 32 * rows * 8 <= nbytes
+        assert waves == 1 or 2 * nkt * rows * 256 <= 512 * MB
+        assert all(v % 256 == 0 for v in (table, cost, coef))
