@@ -8,13 +8,13 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
-#include <list>
 #include <map>
 #include <mutex>
 #include <tuple>
 #include <vector>
 
 #include "mueller.h"
+#include "devcache.cuh"
 #include "green.cuh"
 #include "lu.cuh"
 #include "fields.cuh"
@@ -325,157 +325,53 @@ static void setup_support(Setup& S) {
 }
 
 // ---------------------------------------------------------------- device staging
-// Process-wide cache of freed device blocks, per device.  A build, a solve or a
-// field evaluation takes tens of buffers, and a cudaMalloc, a cudaFree or the
-// mapping of several GB costs tens of microseconds to milliseconds each (the
-// N = 64 sphere: 1.5 of 7.5 ms); released blocks are handed out again for
-// requests of the same rounded size.  Blocks of at least 64 MiB are rounded up to
-// 2 MiB and kept up to a cap (32 GiB by default, mueller_cache_limit); smaller ones
-// are rounded up to a quarter of their power of two and kept up to 256 MiB (none
-// when the cap is 0); beyond its cap a kind gives up what was released longest ago.  Releasing synchronizes the device first, once per group of
-// buffers, as cudaFree does for each, so no kernel of any stream still uses a
-// block when it is reused.  When an allocation fails the cache is emptied and the
-// allocation retried; mueller_cache_trim empties it too.
-namespace devcache {
-constexpr size_t kMinBlock = (size_t)64 << 20, kRound = (size_t)2 << 20, kSmallCap = (size_t)256 << 20;
-struct Block {
-  int dev;
-  size_t bytes;
-  void* p;
+struct CudaBlocks {
+  using Error = cudaError_t;
+  static constexpr Error ok = cudaSuccess;
+  struct Guard {  // frees and device-wide waits would end another thread's capture
+    std::lock_guard<std::mutex> lk{lu_capture_mutex()};
+  };
+  static int device() {
+    int d = 0;
+    cudaGetDevice(&d);
+    return d;
+  }
+  static void use(int d) { cudaSetDevice(d); }
+  static Error alloc(void** p, size_t bytes) { return cudaMalloc(p, bytes); }
+  static void free(void* p) { cudaFree(p); }
+  static void sync() { cudaDeviceSynchronize(); }
+  static void clear_error() { cudaGetLastError(); }
 };
-// big (0) and small (1) blocks, least recently released first
-std::mutex mu;
-std::list<Block> blocks[2];
-size_t held[2] = {0, 0}, cap = (size_t)32 << 30;
+static DeviceCache<CudaBlocks> devcache;
 
-inline size_t rounded(size_t b) {
-  if (b >= kMinBlock) return (b + kRound - 1) / kRound * kRound;
-  if (b <= 512) return 512;
-  size_t q = 128;  // a quarter of the largest power of two up to b
-  while (q * 8 <= b) q *= 2;
-  return (b + q - 1) / q * q;
-}
+extern "C" void mueller_cache_trim(void) { devcache.trim(); }
 
-// Takes blocks off the front until at most `most` bytes of the kind are held (mu held).
-void take_over(int kind, size_t most, std::vector<Block>& out) {
-  while (held[kind] > most) {
-    out.push_back(blocks[kind].front());
-    held[kind] -= out.back().bytes;
-    blocks[kind].pop_front();
-  }
-}
+extern "C" size_t mueller_cache_limit(size_t bytes) { return devcache.limit(bytes); }
 
-void free_blocks(const std::vector<Block>& v) {
-  int cur = 0;
-  cudaGetDevice(&cur);
-  for (const Block& b : v) {
-    if (b.dev != cur) cudaSetDevice(b.dev);
-    cudaFree(b.p);
-    if (b.dev != cur) cudaSetDevice(cur);
-  }
-}
-
-void shrink(size_t most_big, size_t most_small) {
-  std::lock_guard<std::mutex> capture(lu_capture_mutex());
-  std::vector<Block> out;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    take_over(0, most_big, out);
-    take_over(1, most_small, out);
-  }
-  free_blocks(out);
-}
-
-void trim() { shrink(0, 0); }
-
-size_t bytes_held() {
-  std::lock_guard<std::mutex> lk(mu);
-  return held[0] + held[1];
-}
-
-cudaError_t alloc(void** p, size_t bytes) {
-  const size_t req = rounded(bytes);
-  const int kind = req >= kMinBlock ? 0 : 1;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    for (auto it = blocks[kind].rbegin(); it != blocks[kind].rend(); ++it)
-      if (it->bytes == req && it->dev == dev) {
-        *p = it->p;
-        held[kind] -= req;
-        blocks[kind].erase(std::next(it).base());
-        return cudaSuccess;
-      }
-  }
-  cudaError_t e = cudaMalloc(p, req);
-  if (e != cudaSuccess && bytes_held() > 0) {
-    cudaGetLastError();
-    trim();
-    e = cudaMalloc(p, req);
-  }
-  return e;
-}
-
-// Gives back buffers (pointer, requested bytes) of the current device; blocks
-// beyond the caps leave, the least recently released first.
-void release(const std::pair<void*, size_t>* bufs, size_t count) {
-  if (count == 0) return;
-  std::lock_guard<std::mutex> capture(lu_capture_mutex());
-  int dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceSynchronize();
-  std::vector<Block> out;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    for (size_t k = 0; k < count; ++k) {
-      const size_t req = rounded(bufs[k].second);
-      const int kind = req >= kMinBlock ? 0 : 1;
-      blocks[kind].push_back(Block{dev, req, bufs[k].first});
-      held[kind] += req;
-    }
-    take_over(0, cap, out);
-    take_over(1, cap > 0 ? kSmallCap : 0, out);
-  }
-  free_blocks(out);
-}
-}  // namespace devcache
-
-extern "C" void mueller_cache_trim(void) { devcache::trim(); }
-
-extern "C" size_t mueller_cache_limit(size_t bytes) {
-  size_t old;
-  {
-    std::lock_guard<std::mutex> lk(devcache::mu);
-    old = devcache::cap;
-    devcache::cap = bytes;
-  }
-  devcache::shrink(bytes, bytes > 0 ? devcache::kSmallCap : 0);
-  return old;
-}
-
-extern "C" size_t mueller_cache_bytes(void) { return devcache::bytes_held(); }
+extern "C" size_t mueller_cache_bytes(void) { return devcache.bytes_held(); }
 
 struct DevBuf {
-  std::vector<std::pair<void*, size_t>> ptrs;
-  ~DevBuf() { devcache::release(ptrs.data(), ptrs.size()); }
+  std::vector<DevBlock> blocks;
+  ~DevBuf() { devcache.release(blocks.data(), blocks.size()); }
   template <class T>
   cudaError_t alloc(T** p, size_t count) {
-    const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-    cudaError_t e = devcache::alloc((void**)p, bytes);
-    if (e == cudaSuccess) ptrs.push_back({*p, bytes});
+    DevBlock b;
+    cudaError_t e = devcache.alloc(&b, std::max<size_t>(count, 1) * sizeof(T));
+    if (e != cudaSuccess) return e;
+    *p = (T*)b.p;
+    blocks.push_back(b);
     return e;
   }
   size_t size_of(const void* p) const {
-    for (const auto& e : ptrs)
-      if (e.first == p) return e.second;
+    for (const auto& b : blocks)
+      if (b.p == p) return b.bytes;
     return 0;
   }
   void release(void* p) {  // give one buffer back before the others
-    for (size_t k = 0; k < ptrs.size(); ++k)
-      if (ptrs[k].first == p) {
-        devcache::release(&ptrs[k], 1);
-        ptrs.erase(ptrs.begin() + k);
+    for (size_t k = 0; k < blocks.size(); ++k)
+      if (blocks[k].p == p) {
+        devcache.release(&blocks[k], 1);
+        blocks.erase(blocks.begin() + k);
         return;
       }
   }
@@ -962,7 +858,7 @@ static int build_prepare(const mueller_curve* curve, const mueller_media* media,
   c->bytes = (size_t)(M + 1) * n * n * (sizeof(cd) + (mixed ? sizeof(cf) : 0)) + slice_bytes;
   size_t freeb = 0, totb = 0;
   cudaMemGetInfo(&freeb, &totb);
-  freeb += devcache::bytes_held();  // cached blocks are returned when an allocation needs the room
+  freeb += devcache.bytes_held();  // cached blocks are returned when an allocation needs the room
   if (c->bytes + ((size_t)1 << 30) > freeb) { delete c; return fail(MUELLER_ENOMEM, "factors exceed free device memory"); }
   if (c->keep.alloc(&c->A, (size_t)(M + 1) * n * n) != cudaSuccess ||
       c->keep.alloc(&c->piv, (size_t)(M + 1) * n) != cudaSuccess || c->keep.alloc(&c->info, M + 1) != cudaSuccess ||
