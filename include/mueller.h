@@ -245,9 +245,10 @@ int mueller_far_field_grid(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs
  * distance.  A target on a node ring is rejected (MUELLER_EINVAL).  x_dev:
  * currents [2M+1][nrhs][4N]; targets: host [ntargets][3]; out_dev: device
  * [nrhs][ntargets][6] complex, (E, H) in Cartesian components.  With many
- * (target, ring point) pairs the kernels' products with the currents are
- * exact-digit products on the tensor cores, in a workspace allocated for the
- * call (on the FP64 pipe where it cannot be had); MUELLER_ETIMEOUT if a
+ * (target, ring point) pairs and more than a few targets the kernels' products
+ * with the currents are exact-digit products on the tensor cores, in a
+ * workspace allocated for the call (at most about 2.2 GB, in passes; on the
+ * FP64 pipe where it cannot be had); MUELLER_ETIMEOUT if a
  * bounded device-side wait of them gave up (out_dev is then unusable). */
 int mueller_eval(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs, const double* targets, int ntargets,
                  int region, mueller_c128* out_dev, void* stream);

@@ -555,27 +555,42 @@ size_t near_field_part(long long total, int nt, int nrhs) {
   return (size_t)nt * 12 * std::max(group * near_field_splits(total, nt, group), last * near_field_splits(total, nt, last));
 }
 
-// Fewer (point, ring point) pairs than this stay on the FP64 pipe, whose kernel needs
-// no digits: N = 128, M = 16, 10 points, one side (1.5e5) 0.17 ms there and 0.23 ms on
-// the tensor cores, 50 points (8e5) 0.41 and 0.39 ms; N = 320, M = 32, 100 points (5e6)
-// one side 1.83 and 1.57 ms, two 2.74 and 1.61 ms, eight 10.6 and 2.5 ms.
+// Fewer (point, ring point) pairs than NF_PAIRS_MIN stay on the FP64 pipe, whose kernel
+// needs no digits: N = 128, M = 16, 10 points, one side (1.5e5) 0.17 ms there and 0.23 ms
+// on the tensor cores, 50 points (8e5) 0.41 and 0.39 ms; N = 320, M = 32, 100 points (5e6)
+// one side 1.83 and 1.55 ms, two 2.74 and 1.56 ms, eight 10.6 and 2.5 ms.
+// So do points that fill too little of their row tiles of 128 (18 rows a point), whose
+// digits are copied and multiplied whole, for the sides that share the tiles:
+// nf_fills_rows.  N = 576, M = 64, targets 0.02 from the surface (2.8e6 ring points), one
+// side: one point 2.7 ms there and 4.2 ms on the tensor cores, four 4.2 and 5.1, seven 6.7
+// and 5.9, eight (two tiles) 6.3 and 7.1, thirty 21 and 18; two sides, one 4.6 and 6.2,
+// four 6.9 and 7.0; eight sides, one 16.7 and 20.3, two 20.0 and 20.6, four 27 and 21.
 #define NF_PAIRS_MIN 7e5
+static bool nf_fills_rows(int nt, int nrhs) {
+  const double row_tiles = (double)tiles((size_t)NF_ROWS * nt, OZ_RT);
+  return nt * (20.0 + 7.0 * nrhs) >= OZ_RT * row_tiles;
+}
 size_t near_field_work_bytes(long long total, int nt, int nrhs) {
   const int group = near_field_group(total, nrhs);
-  return (double)total * nt >= NF_PAIRS_MIN ? nearfield_oz_bytes(total, nt, group) : 0;
+  return (double)total * nt >= NF_PAIRS_MIN && nf_fills_rows(nt, group) ? nf_plan(total, nt, group).bytes : 0;
 }
 
-void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
-                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, void* work, cd* out, int* err,
-                       cudaStream_t s) {
+bool launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
+                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, void* work, size_t work_bytes,
+                       cd* out, int* err, cudaStream_t s) {
   const long long total = (long long)g.N * n_theta;
   const int group = near_field_group(total, nrhs);
+  NfPlan plan{};
+  if (work) {
+    plan = nf_plan(total, nt, group);
+    if (plan.bytes > work_bytes) return false;
+  }
   for (int w0 = 0; w0 < nrhs; w0 += group) {
     const int wc = std::min(group, nrhs - w0), splits = near_field_splits(total, nt, wc);
     const long long per = (total + splits - 1) / splits;
     launch_ring<true>(g, M, x, w0, wc, nrhs, n_theta, cur, (double4*)pts, s);
     if (work) {
-      launch_nearfield_products(total, (const double4*)pts, cur, X_dev, nt, wc, k, cJ, cM, dM, dJ, work,
+      launch_nearfield_products(total, (const double4*)pts, cur, X_dev, nt, wc, k, cJ, cM, dM, dJ, plan, work,
                                 out + (size_t)w0 * nt * 6, err, s);
       continue;
     }
@@ -588,6 +603,7 @@ void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const d
     nearfield_join_kernel<<<(unsigned)((items + 127) / 128), 128, 0, s>>>(items, splits, part, cJ, cM, dM, dJ,
                                                                           out + (size_t)w0 * nt * 6);
   }
+  return true;
 }
 
 // ---------------------------------------------------------------------------

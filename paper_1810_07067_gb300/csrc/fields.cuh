@@ -32,13 +32,14 @@ void launch_rhs_samples(const FieldGeom& g, int M, cd sE, cd sH, const cd* EH, i
 // [N][n_theta][4] (32-byte aligned), and either work of near_field_work_bytes
 // (256-byte aligned; err, a device int, is set if a bounded wait gives up) or part of
 // near_field_part values (work null: FP64 pipe); k and the four constants are the
-// region's.  total = N n_theta, a multiple of 16.
+// region's.  total = N n_theta, a multiple of 16.  False, with nothing launched, when
+// work_bytes do not hold the layout.
 int near_field_group(long long total, int nrhs);
 size_t near_field_work_bytes(long long total, int nt, int nrhs);
 size_t near_field_part(long long total, int nt, int nrhs);
-void launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
-                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, void* work, cd* out, int* err,
-                       cudaStream_t s);
+bool launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
+                       cd k, cd cJ, cd cM, cd dM, cd dJ, cd* cur, double* pts, cd* part, void* work, size_t work_bytes,
+                       cd* out, int* err, cudaStream_t s);
 
 // Far field on the grid theta_p = (p + 1/2) pi / n_polar, phi_s = 2 pi s / n_azim:
 // E[rhs][p][s][3] (k0 real, n_alpha a multiple of 4); F [rhs][n_polar][2M+1][3] and

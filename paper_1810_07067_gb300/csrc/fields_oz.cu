@@ -455,13 +455,12 @@ __global__ void __launch_bounds__(128) synth_join_kernel(int n_polar, int n_azim
 // FP64 work (about 100 operations) and bound the call, their products with the
 // currents (104 operations per right-hand side in nearfield_kernel) do not: N = 320,
 // M = 32, 2 sides, 100 points 2.74 -> 1.61 ms, of which kernels 0.87 and products 0.34.
-#define NF_KC 512
-#define NF_ROWS 18
 #define NF_LD (NF_KC + 2)
 
-// One CTA per (index, point): the rows of NF_KC ring points through shared memory.
+// One CTA per (index a0 + blockIdx.x, point p0 + blockIdx.y): the rows of NF_KC ring
+// points through shared memory.
 __global__ void __launch_bounds__(128) nf_rows_kernel(long long total, const double4* __restrict__ pts,
-                                                      const double* __restrict__ X, int p0, cd k, int nrt,
+                                                      const double* __restrict__ X, int a0, int p0, cd k, int nrt,
                                                       __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
   extern __shared__ __align__(16) double sv[];  // [NF_ROWS][NF_LD], then the rows' largest exponents
   unsigned* ex = (unsigned*)(sv + NF_ROWS * NF_LD);
@@ -477,7 +476,7 @@ __global__ void __launch_bounds__(128) nf_rows_kernel(long long total, const dou
 #pragma unroll 1
   for (int u = 0; u < NF_KC / 128; ++u) {
     const int col = tid + 128 * u;
-    const long long it = (long long)a * NF_KC + col;
+    const long long it = (long long)(a0 + a) * NF_KC + col;
     cd T[9];
     if (it < total) {
       const double4 y = pts[it];
@@ -525,14 +524,15 @@ __global__ void __launch_bounds__(128) nf_rows_kernel(long long total, const dou
   if (tid < NF_ROWS) rscale[(size_t)a * nrt * OZ_RT + r0 + tid] = scale_of(ex[tid]);
 }
 
-// Columns of one right-hand side's currents cur[w][it][J 3, M 3].  One CTA per (index, w).
-__global__ void __launch_bounds__(64) nf_cols_kernel(long long total, const cd* __restrict__ cur, int nct,
+// Columns of one right-hand side's currents cur[w0 + w][it][J 3, M 3].  One CTA per
+// (index a0 + blockIdx.x, w).
+__global__ void __launch_bounds__(64) nf_cols_kernel(long long total, const cd* __restrict__ cur, int a0, int w0, int nct,
                                                      __nv_bfloat16* __restrict__ Bsl, double* __restrict__ cscale) {
   __shared__ unsigned red[12][2];
   const int a = blockIdx.x, w = blockIdx.y, tid = threadIdx.x;
-  const long long it0 = (long long)a * NF_KC + 8 * tid;  // total is a multiple of 16
+  const long long it0 = (long long)(a0 + a) * NF_KC + 8 * tid;  // total is a multiple of 16
   const bool in = it0 < total;
-  const cd* src = cur + ((size_t)w * total + it0) * 6;
+  const cd* src = cur + ((size_t)(w0 + w) * total + it0) * 6;
   unsigned mx[12];
 #pragma unroll
   for (int c = 0; c < 12; ++c) mx[c] = 0u;
@@ -564,12 +564,12 @@ __global__ void __launch_bounds__(64) nf_cols_kernel(long long total, const cd* 
   }
 }
 
-// Ysum[column][row] = the sum of the indices' Y.
-__global__ void __launch_bounds__(128) nf_sum_kernel(int na, long long count, const double* __restrict__ Y,
+// Ysum[column][row] = the sum of the indices' Y (add: to what a pass before left there).
+__global__ void __launch_bounds__(128) nf_sum_kernel(int na, long long count, bool add, const double* __restrict__ Y,
                                                      double* __restrict__ Ysum) {
   const long long e = (long long)blockIdx.x * 128 + threadIdx.x;
   if (e >= count) return;
-  double acc = 0.0;
+  double acc = add ? Ysum[e] : 0.0;
 #pragma unroll 8
   for (int a = 0; a < na; ++a) acc += Y[(size_t)a * count + e];
   Ysum[e] = acc;
@@ -789,52 +789,44 @@ void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const c
   }
 }
 
-// Points of a pass: as many as keep the rows' digits within FFO_BYTES, at least one
-// tile of rows.
-struct NfPlan {
-  int na, np, nrt, nct;
-  size_t a, r, b, c, y, sum;
-};
-static NfPlan nf_plan(long long total, int nt, int nw) {
-  NfPlan f{};
-  f.na = (int)((total + NF_KC - 1) / NF_KC);
-  const size_t tile = (size_t)f.na * (NF_KC / OZ_KT) * FFO_ABLOCK * 2;
-  f.nrt = (int)std::max<size_t>(1, std::min<size_t>(tiles((size_t)NF_ROWS * nt, OZ_RT), FFO_BYTES / tile));
-  f.np = std::min(nt, f.nrt * OZ_RT / NF_ROWS);
-  f.np = (int)tiles(nt, tiles(nt, f.np));  // equal passes
-  f.nrt = (int)tiles((size_t)NF_ROWS * f.np, OZ_RT);
-  f.nct = (int)tiles((size_t)12 * nw, FFO_NT);
-  f.a = up256(f.nrt * tile);
-  f.r = up256((size_t)f.na * f.nrt * OZ_RT * 8);
-  f.b = up256((size_t)f.na * f.nct * (NF_KC / OZ_KT) * FFO_BBLOCK * 2);
-  f.c = up256((size_t)f.na * f.nct * FFO_NT * 8);
-  f.sum = up256((size_t)f.nct * FFO_NT * f.nrt * OZ_RT * 8);
-  f.y = (size_t)f.na * f.sum;
-  return f;
-}
-size_t nearfield_oz_bytes(long long total, int nt, int nw) {
-  const NfPlan f = nf_plan(total, nt, nw);
-  return f.a + f.r + f.b + f.c + f.y + f.sum;
-}
-void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nw, cd k,
-                               cd cJ, cd cM, cd dM, cd dJ, void* work, cd* out, int* err, cudaStream_t s) {
-  const NfPlan f = nf_plan(total, nt, nw);
+void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nrhs,
+                               cd k, cd cJ, cd cM, cd dM, cd dJ, const NfPlan& f, void* work, cd* out, int* err,
+                               cudaStream_t s) {
   const int sms = digit_ready();
   char* p = (char*)work;
-  auto* Asl = (__nv_bfloat16*)p;
-  auto* rscale = (double*)(p += f.a);
-  auto* Bsl = (__nv_bfloat16*)(p += f.r);
-  auto* cscale = (double*)(p += f.b);
-  auto* Y = (double*)(p += f.c);
-  auto* Ysum = (double*)(p += f.y);
-  nf_cols_kernel<<<dim3(f.na, nw), 64, 0, s>>>(total, cur, f.nct, Bsl, cscale);
-  for (int p0 = 0; p0 < nt; p0 += f.np) {
-    const int np = std::min(f.np, nt - p0), nrt = (int)tiles((size_t)NF_ROWS * np, OZ_RT);
-    nf_rows_kernel<<<dim3(f.na, np), 128, NF_ROWS * (NF_LD * 8 + 4), s>>>(total, pts, X, p0, k, nrt, Asl, rscale);
-    digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, NF_KC / OZ_KT, nrt, f.nct, f.na, Y, err, s);
-    const long long count = (long long)f.nct * FFO_NT * nrt * OZ_RT, items = (long long)nw * np * 6;
-    nf_sum_kernel<<<(unsigned)((count + 127) / 128), 128, 0, s>>>(f.na, count, Y, Ysum);
-    nf_join_kernel<<<(unsigned)((items + 127) / 128), 128, 0, s>>>(np, p0, nt, nw, (size_t)nrt * OZ_RT, Ysum, cJ, cM, dM,
-                                                                  dJ, out);
-  }
+  auto* Asl = (__nv_bfloat16*)(p + f.a);
+  auto* rscale = (double*)(p + f.r);
+  auto* Bsl = (__nv_bfloat16*)(p + f.b);
+  auto* cscale = (double*)(p + f.c);
+  auto* Y = (double*)(p + f.y);
+  auto* Ysum = (double*)(p + f.sum);
+  const int vs = f.groups * f.nw, qs = f.passes * f.np;
+  for (int v0 = 0; v0 < nrhs; v0 += vs)
+    for (int q0 = 0; q0 < nt; q0 += qs) {
+      const int v1 = std::min(nrhs, v0 + vs), q1 = std::min(nt, q0 + qs);
+      const bool kept = v1 - v0 <= f.nw;  // one product's columns: their digits serve every point
+      auto sums = [&](int p0, int w0) { return Ysum + ((size_t)((p0 - q0) / f.np) * f.groups + (w0 - v0) / f.nw) * f.sum_group; };
+      for (int a0 = 0; a0 < f.na; a0 += f.nap) {
+        const int na = std::min(f.nap, f.na - a0);
+        for (int p0 = q0; p0 < q1; p0 += f.np) {
+          const int np = std::min(f.np, q1 - p0), nrt = (int)tiles((size_t)NF_ROWS * np, OZ_RT);
+          nf_rows_kernel<<<dim3(na, np), 128, NF_ROWS * (NF_LD * 8 + 4), s>>>(total, pts, X, a0, p0, k, nrt, Asl, rscale);
+          for (int w0 = v0; w0 < v1; w0 += f.nw) {
+            const int nw = std::min(f.nw, v1 - w0), nct = (int)tiles((size_t)12 * nw, FFO_NT);
+            if (!kept || p0 == q0) nf_cols_kernel<<<dim3(na, nw), 64, 0, s>>>(total, cur, a0, w0, nct, Bsl, cscale);
+            digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, NF_KC / OZ_KT, nrt, nct, na, Y, err, s);
+            const long long count = (long long)nct * FFO_NT * nrt * OZ_RT;
+            nf_sum_kernel<<<(unsigned)((count + 127) / 128), 128, 0, s>>>(na, count, a0 > 0, Y, sums(p0, w0));
+          }
+        }
+      }
+      for (int p0 = q0; p0 < q1; p0 += f.np)
+        for (int w0 = v0; w0 < v1; w0 += f.nw) {
+          const int np = std::min(f.np, q1 - p0), nw = std::min(f.nw, v1 - w0);
+          const long long items = (long long)nw * np * 6;
+          nf_join_kernel<<<(unsigned)((items + 127) / 128), 128, 0, s>>>(
+              np, p0, nt, nw, tiles((size_t)NF_ROWS * np, OZ_RT) * OZ_RT, sums(p0, w0), cJ, cM, dM, dJ,
+              out + (size_t)w0 * nt * 6);
+        }
+    }
 }

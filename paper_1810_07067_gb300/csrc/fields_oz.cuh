@@ -59,8 +59,9 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
 void launch_rhs_products(const FieldGeom& g, int M, const double2* wave, const cd* tab, cd fE, cd fH, int w0, int count,
                          int nrhs, int n_theta, const RhsPlan& plan, void* work, cd* rhs, int* err, cudaStream_t s);
 
-// Fields of nw right-hand sides at nt points from their ring points and currents
-// (ring_kernel) into out[w][p][6]; work of nearfield_oz_bytes (256-byte aligned).
-size_t nearfield_oz_bytes(long long total, int nt, int nw);
-void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nw, cd k,
-                               cd cJ, cd cM, cd dM, cd dJ, void* work, cd* out, int* err, cudaStream_t s);
+// Fields of nrhs right-hand sides at nt points from their ring points and currents
+// (ring_kernel) into out[w][p][6]; work of plan.bytes (256-byte aligned), plan the
+// nf_plan of the same points and at least as many sides.
+void launch_nearfield_products(long long total, const double4* pts, const cd* cur, const double* X, int nt, int nrhs,
+                               cd k, cd cJ, cd cM, cd dM, cd dJ, const NfPlan& plan, void* work, cd* out, int* err,
+                               cudaStream_t s);

@@ -58,3 +58,48 @@ inline RhsPlan rhs_plan(int N, int M, int n_theta, int nrhs) {
   f.bytes = f.coef + up256(rt * f.ring.y_row_tile);
   return f;
 }
+
+// Fields at points.  The ring points are cut into indices of NF_KC; the rows' digits
+// (points), the columns' digits (sides) and the indices' sums are each held for as
+// many indices, points and sides at a time as FFO_BYTES takes: all the indices when
+// one row tile's digits of all of them fit, else passes over them whose sums add up
+// (the sums of all points are kept meanwhile, so that the columns are cut once a pass).
+// (A point close to the surface has 8192 azimuths on refined panels, 4e6 ring points:
+// 8 GB of digits for one row tile.)
+#define NF_KC 512
+#define NF_ROWS 18
+struct NfPlan {
+  int na, nap;             // indices in all, of a ring pass
+  int np, nrt;             // points of a pass and their row tiles
+  int nw, nct;             // sides of a product and their column tiles
+  int groups, passes;      // products of sides and passes of points whose sums are held together
+  size_t a, r, b, c, y, sum;  // offsets of the parts
+  size_t sum_group;        // values of one product's sums, [pass][group]
+  size_t bytes;
+};
+inline NfPlan nf_plan(long long total, int nt, int nrhs) {
+  NfPlan f{};
+  const size_t ta = (size_t)(NF_KC / OZ_KT) * FFO_ABLOCK * 2, tb = (size_t)(NF_KC / OZ_KT) * FFO_BBLOCK * 2;
+  const size_t ty = (size_t)FFO_NT * OZ_RT * 8;  // an index's digits of a row tile, a column tile, its sums of both
+  const size_t most = FFO_BYTES / ta;            // (index, row tile) pairs held
+  f.na = (int)tiles((size_t)total, NF_KC);
+  const size_t all = tiles((size_t)NF_ROWS * nt, OZ_RT);
+  f.nrt = (int)std::min(all, (size_t)f.na <= most ? most / f.na : (size_t)4);
+  f.np = std::min(nt, f.nrt * OZ_RT / NF_ROWS);
+  f.np = (int)tiles(nt, tiles(nt, f.np));  // equal passes
+  f.nrt = (int)tiles((size_t)NF_ROWS * f.np, OZ_RT);
+  f.nap = (int)tiles(f.na, tiles(f.na, std::max<size_t>(1, most / f.nrt)));
+  const size_t ct = std::min(FFO_BYTES / (f.nap * tb), FFO_BYTES / (f.nap * (size_t)f.nrt * ty));
+  f.nw = (int)std::min<size_t>(nrhs, std::max<size_t>(1, ct * FFO_NT / 12));
+  f.nct = (int)tiles((size_t)12 * f.nw, FFO_NT);
+  f.sum_group = (size_t)f.nct * FFO_NT * f.nrt * OZ_RT;
+  f.groups = (int)std::min(tiles(nrhs, f.nw), std::max<size_t>(1, FFO_BYTES / (f.sum_group * 8)));
+  f.passes = (int)std::min(tiles(nt, f.np), std::max<size_t>(1, FFO_BYTES / (f.groups * f.sum_group * 8)));
+  f.r = f.a + up256((size_t)f.nap * f.nrt * ta);
+  f.b = f.r + up256((size_t)f.nap * f.nrt * OZ_RT * 8);
+  f.c = f.b + up256((size_t)f.nap * f.nct * tb);
+  f.y = f.c + up256((size_t)f.nap * f.nct * FFO_NT * 8);
+  f.sum = f.y + up256((size_t)f.nap * f.sum_group * 8);
+  f.bytes = f.sum + up256(f.passes * f.groups * f.sum_group * 8);
+  return f;
+}

@@ -1362,7 +1362,13 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
       tmp.alloc(&pts, (size_t)nring * 4) != cudaSuccess ||
       tmp.alloc(&xs, (size_t)nvec * 4 * nsub) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "evaluation buffers");
-  unsigned char* work = nullptr;  // without it the sums run on the FP64 pipe
+  CK(tmp.upload(&X, vx, s));
+  CK(tmp.upload(&dgr, gr, s)); CK(tmp.upload(&dgz, gz, s)); CK(tmp.upload(&dgrp, grp, s));
+  CK(tmp.upload(&dgzp, gzp, s)); CK(tmp.upload(&dgw, gw, s)); CK(tmp.upload(&dLm, Lm, s));
+  CK(tmp.upload(&dn0, node0, s));
+  // last, so that it takes no room from the buffers that both forms need; without it
+  // the sums run on the FP64 pipe
+  unsigned char* work = nullptr;
   int* err = nullptr;
   const size_t bytes = near_field_work_bytes(nring, ntargets, nrhs);
   if (bytes && (tmp.alloc(&err, 1) != cudaSuccess || tmp.alloc(&work, bytes) != cudaSuccess)) {
@@ -1372,14 +1378,11 @@ extern "C" int mueller_eval(mueller_ctx* c, const mueller_c128* x_dev, int nrhs,
   if (!work && tmp.alloc(&part, near_field_part(nring, ntargets, nrhs)) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "evaluation buffers");
   if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  CK(tmp.upload(&X, vx, s));
-  CK(tmp.upload(&dgr, gr, s)); CK(tmp.upload(&dgz, gz, s)); CK(tmp.upload(&dgrp, grp, s));
-  CK(tmp.upload(&dgzp, gzp, s)); CK(tmp.upload(&dgw, gw, s)); CK(tmp.upload(&dLm, Lm, s));
-  CK(tmp.upload(&dn0, node0, s));
   launch_interp_currents((const cd*)x_dev, 4 * S.N, nsub, dn0, dLm, nvec, xs, s);
   FieldGeom g{dgr, dgz, dgrp, dgzp, dgw, nsub};
-  launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, pts, part, work, (cd*)out_dev,
-                    err, s);
+  if (!launch_near_field(g, S.M, xs, nrhs, X, ntargets, nth, k, cJ, cM, dM, dJ, cur, pts, part, work, bytes,
+                         (cd*)out_dev, err, s))
+    return fail(MUELLER_EINVAL, "workspace of the field evaluation too small");
   CK(cudaGetLastError());
   int herr = 0;
   if (work) CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -12,6 +12,13 @@ int main() {
       if (scanf("%d %d %d %d", &N, &M, &n, &nrhs) != 4) return 1;
       const RhsPlan f = rhs_plan(N, M, n, nrhs);
       printf("%d %d %d %zu %zu %zu %zu %zu\n", f.ring.nkt, f.ring.nct, f.waves, f.a, f.table, f.cost, f.coef, f.bytes);
+    } else if (!strcmp(op, "nf")) {
+      long long total;
+      int nt, nrhs;
+      if (scanf("%lld %d %d", &total, &nt, &nrhs) != 3) return 1;
+      const NfPlan f = nf_plan(total, nt, nrhs);
+      printf("%d %d %d %d %d %d %d %d %zu %zu %zu %zu %zu %zu %zu %zu\n", f.na, f.nap, f.np, f.nrt, f.nw, f.nct, f.groups, f.passes, f.a,
+             f.r, f.b, f.c, f.y, f.sum, f.sum_group, f.bytes);
     } else {
       return 1;
     }

@@ -52,3 +52,26 @@ def test_plane_wave_passes_stay_inside(plan):
         assert coef + 2 * nct * 32 * rows * 8 <= nbytes
         assert waves == 1 or 2 * nkt * rows * 256 <= 512 * MB
         assert all(v % 256 == 0 for v in (table, cost, coef))
+
+
+def test_field_passes_stay_inside_and_bounded(plan):
+    """From 16 ring points to those of 4096 sub-nodes at 8192 azimuths, 1 to 1e5 points, up
+    to 65535 sides: every pass inside its parts, no part above 512 MB."""
+    rng = np.random.default_rng(12)
+    cases = [(t, nt, w) for t in (16, 512, 528, 46080, 262144, 262160, 1024 * 8192, 4096 * 8192)
+             for nt in (1, 7, 8, 100, 100000) for w in (1, 2, 10, 11, 100, 65535)]
+    cases += [(16 * int(rng.integers(1, 1 << 20)), int(rng.integers(1, 3000)), int(rng.integers(1, 3000)))
+              for _ in range(200)]
+    for (total, nt, nrhs), row in zip(cases, plan("nf", cases)):
+        na, nap, npt, nrt, nw, nct, groups, passes, a, r, b, c, y, s, group, nbytes = row
+        assert na == _up(total, 512) and 1 <= nap <= na and 1 <= npt <= nt and 1 <= nw <= nrhs and groups >= 1 and passes >= 1
+        assert 18 * npt <= 128 * nrt and 12 * nw <= 32 * nct
+        rows, cols = 128 * nrt, 32 * nct                     # of the fullest product, 8 digits of 2 bytes each
+        assert a == 0 and a + nap * rows * 512 * 8 * 2 <= r and r + nap * rows * 8 <= b
+        assert b + nap * cols * 512 * 8 * 2 <= c and c + nap * cols * 8 <= y
+        assert y + nap * cols * rows * 8 <= s
+        assert group >= cols * rows and s + ((passes * groups - 1) * group + cols * rows) * 8 <= nbytes
+        assert max(r, c - b, s - y, nbytes - s) <= 512 * MB + 256 and nbytes <= 2200 * 10 ** 6
+        assert all(v % 256 == 0 for v in (r, b, c, y, s))
+        if na <= 512 and 18 * nt <= 128 * (512 // na):
+            assert nap == na and npt == nt                   # nothing is cut that fits whole
