@@ -228,7 +228,9 @@ int mueller_rhs_fields(mueller_ctx* ctx, const mueller_c128* EH_dev, int nrhs, i
  * exact-digit products on the tensor cores, in a workspace allocated for the
  * call (operand digits in passes of 512 MB; on the FP64 pipe where it cannot
  * be had); MUELLER_ETIMEOUT if a bounded device-side wait of them gave up
- * (E_dev is then unusable).  A side with an infinite or NaN current has NaN
+ * (E_dev is then unusable).  The products are FP64-accurate relative to the
+ * largest weighted current of a side and mode.  A side with an infinite or NaN
+ * current has NaN
  * in its field and leaves the other sides alone. */
 int mueller_far_field_grid(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs, int n_polar, int n_azim,
                            mueller_c128* E_dev, void* stream);
@@ -248,8 +250,10 @@ int mueller_far_field_grid(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs
  * (target, ring point) pairs and more than a few targets the kernels' products
  * with the currents are exact-digit products on the tensor cores, in a
  * workspace allocated for the call (at most about 2.2 GB, in passes; on the
- * FP64 pipe where it cannot be had); MUELLER_ETIMEOUT if a
- * bounded device-side wait of them gave up (out_dev is then unusable). */
+ * FP64 pipe where it cannot be had), FP64-accurate relative to the largest
+ * kernel times the largest current among 512 neighbouring ring points;
+ * MUELLER_ETIMEOUT if a bounded device-side wait of them gave up (out_dev is
+ * then unusable). */
 int mueller_eval(mueller_ctx* ctx, const mueller_c128* x_dev, int nrhs, const double* targets, int ntargets,
                  int region, mueller_c128* out_dev, void* stream);
 

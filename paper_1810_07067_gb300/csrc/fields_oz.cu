@@ -8,8 +8,19 @@
 // shifted mode, right-hand side, J or M, Re or Im), the nodes along k. Both operands
 // are cut into 8 exact digits of 7 bits (a scale per row and per column), the digit
 // products accumulate exactly in tensor memory 256 nodes at a time, the 8 levels
-// are joined in 64-bit integers and the chunks added in FP64: rounding below that
-// of FP64 sums of the same terms.
+// are joined in 64-bit integers and the chunks added in FP64.
+//
+// A sum of K terms is off by at most some K 2^-56 max_k |a_k| max_k |b_k| (measured:
+// its square root), where an FP64 sum is off by about 2^-53 sum_k |a_k b_k|: less for
+// operands of even size, more where the largest entries of row and column do not meet.
+// So the nodes' weights, which fall to 1e-9 of the largest toward the axis, go with the
+// currents and not with the rows: rows are then at most 1, b_a itself is only known to
+// a few 2^-53 of that, and currents near the axis alone keep their digits (weights in
+// the rows left errors of 1e-11 of such a field, now 3e-14 and less). Ring samples and cosines are of even
+// size. The kernels of a point are not when it is close to the surface: a sum is then
+// off by 2^-56 of the largest kernel times the largest current among NF_KC ring points.
+// Measured against 80-bit sums from 0.02 of the radius on, currents on the far side
+// among them: at most 1.5 times the FP64 pipe's error.
 //
 // The ring integrals b_a before and the sums over the modes after are contractions
 // with cosine tables and go the same way.
@@ -98,18 +109,20 @@ __global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int nrt, co
 }
 
 // Columns of mode q and right-hand side w0 + w: X_0 = r' J1 + i J2, X_1 = z' J1,
-// X_2 = r' J1 - i J2 (and of M), for a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w, X).
-__global__ void __launch_bounds__(64) ffo_cols_kernel(FieldGeom g, int M, const cd* __restrict__ x, int nrhs, int w0,
-                                                      int nw, int nct, __nv_bfloat16* __restrict__ Bsl,
+// X_2 = r' J1 - i J2 (and of M), times the nodes' weights (wt of ffo_phase_kernel), for
+// a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w, X).
+__global__ void __launch_bounds__(64) ffo_cols_kernel(int N, int M, const double* __restrict__ wt,
+                                                      const cd* __restrict__ x, int nrhs, int w0, int nw, int nct,
+                                                      __nv_bfloat16* __restrict__ Bsl,
                                                       double* __restrict__ cscale) {
   __shared__ unsigned red[2];
   const int q = blockIdx.x, w = blockIdx.y, h = blockIdx.z / 3, u = blockIdx.z % 3;
-  const int s = q - M + 1 - u, a = abs(s), N = g.N, nkt = N / OZ_KT, tid = threadIdx.x;
+  const int s = q - M + 1 - u, a = abs(s), nkt = N / OZ_KT, tid = threadIdx.x;
   const cd* xv = x + ((size_t)q * nrhs + w0 + w) * 4 * N + 2 * h;
   auto value = [&](int j) {
     const cd v1 = xv[4 * j];
-    if (u == 1) return g.zp[j] * v1;
-    const cd r1 = g.rp[j] * v1, v2 = mul_i(xv[4 * j + 1]);
+    if (u == 1) return wt[2 * N + j] * v1;
+    const cd r1 = wt[N + j] * v1, v2 = wt[j] * mul_i(xv[4 * j + 1]);
     return u == 0 ? r1 + v2 : r1 - v2;
   };
   unsigned ex = 0u;
@@ -350,14 +363,21 @@ __global__ void __launch_bounds__(128) ring_samples_kernel(const double* __restr
   for (int par = 0; par < 2; ++par) put_digits(Asl + (size_t)par * nrt * nkt * FFO_ABLOCK + o, FFO_ATILE, v[par], 1);
 }
 
-// Phases 2 pi w_j r_j e^{-i k0 z_j cos theta_p} of the angles 0..P2 - 1.
-__global__ void __launch_bounds__(128) ffo_phase_kernel(FieldGeom g, double k0, int n_polar, double2* __restrict__ phase) {
+// Phases e^{-i k0 z_j cos theta_p} of the angles 0..P2 - 1, and wt = the weights
+// 2 pi w_j r_j, the same times r' and times z'.
+__global__ void __launch_bounds__(128) ffo_phase_kernel(FieldGeom g, double k0, int n_polar, double2* __restrict__ phase,
+                                                        double* __restrict__ wt) {
   const int p = blockIdx.x, j = blockIdx.y * 128 + threadIdx.x;
   if (j >= g.N) return;
   double s, c;
   sincos(k0 * (g.z[j] * cospi((p + 0.5) / n_polar)), &s, &c);
-  const double wr = 6.283185307179586 * g.w[j] * g.r[j];
-  phase[(size_t)p * g.N + j] = make_double2(wr * c, -wr * s);
+  phase[(size_t)p * g.N + j] = make_double2(c, -s);
+  if (p == 0) {
+    const double wr = 6.283185307179586 * g.w[j] * g.r[j];
+    wt[j] = wr;
+    wt[g.N + j] = wr * g.rp[j];
+    wt[2 * g.N + j] = wr * g.zp[j];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -705,7 +725,7 @@ FfoPlan ffo_plan(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
   const size_t sy = (size_t)2 * f.snct * FFO_NT * 6 * n_polar * 8;
   f.snw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / std::max(sa, sy)));
   const size_t srt = tiles((size_t)6 * f.snw * n_polar, OZ_RT), rrt = tiles((size_t)f.np * N, OZ_RT);
-  f.phase = up256((size_t)f.P2 * N * 16);
+  f.phase = up256((size_t)N * (f.P2 * 16 + 24));  // and the weights
   f.a = up256(std::max({f.nrt * ta, rrt * f.ring.a_row_tile, srt * 2 * f.snkt * FFO_ABLOCK * 2}));
   f.r = up256(std::max((size_t)f.na * f.nrt, 2 * srt) * OZ_RT * 8);
   f.b = up256(std::max(f.nct * tb, (size_t)2 * f.snct * f.snkt * FFO_BBLOCK * 2));
@@ -730,6 +750,7 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
   const int sms = digit_ready();
   char* p = (char*)work;
   auto* phase = (double2*)p;
+  auto* wt = (double*)(phase + (size_t)f.P2 * g.N);
   auto* Asl = (__nv_bfloat16*)(p += f.phase);
   auto* rscale = (double*)(p += f.a);
   auto* Bsl = (__nv_bfloat16*)(p += f.r);
@@ -738,7 +759,7 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
   auto* Tsl = (__nv_bfloat16*)(p += f.y);
   auto* cost = (double*)(p += f.tb);
   auto* coef = (double*)(p += f.cost);
-  ffo_phase_kernel<<<dim3(f.P2, (g.N + 127) / 128), 128, 0, s>>>(g, k0, n_polar, phase);
+  ffo_phase_kernel<<<dim3(f.P2, (g.N + 127) / 128), 128, 0, s>>>(g, k0, n_polar, phase, wt);
   ring_table(f.ring, M, n_alpha, Tsl, cost, s);
   for (int p0 = 0; p0 < f.P2; p0 += f.np) {
     const int np = std::min(f.np, f.P2 - p0), nrt = (int)tiles(2 * np, OZ_RT);
@@ -747,7 +768,7 @@ void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, 
                                                  tiles((size_t)np * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
     for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
       const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles(24 * nw, FFO_NT);
-      ffo_cols_kernel<<<dim3(2 * M + 1, nw, 6), 64, 0, s>>>(g, M, x, nrhs, w0, nw, nct, Bsl, cscale);
+      ffo_cols_kernel<<<dim3(2 * M + 1, nw, 6), 64, 0, s>>>(g.N, M, wt, x, nrhs, w0, nw, nct, Bsl, cscale);
       digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
       ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
           M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
