@@ -271,7 +271,7 @@ size_t rhs_planewave_scratch_doubles(int M, int nrhs, int n_theta) {
 #define RHS_FMA_MIN 4e7
 size_t rhs_planewave_work_bytes(int N, int M, int nrhs, int n_theta) {
   const double fma = (double)N * nrhs * (M + 2.0) * (n_theta / 4);
-  return fma >= RHS_FMA_MIN ? rhs_plan(N, M, n_theta, nrhs).bytes : 0;
+  return fma >= RHS_FMA_MIN ? rhs_plan(N, M, n_theta, nrhs, pass_bytes()).bytes : 0;
 }
 
 bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd mu0, cd sE, cd sH,
@@ -279,7 +279,7 @@ bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd
                           void* work, size_t work_bytes, cd* rhs, int* err, cudaStream_t s) {
   RhsPlan plan{};
   if (work) {
-    plan = rhs_plan(g.N, M, n_theta, nrhs);
+    plan = rhs_plan(g.N, M, n_theta, nrhs, pass_bytes());
     if (plan.bytes > work_bytes) return false;
   }
   const int Q = n_theta / 4 + 1;
@@ -572,7 +572,7 @@ static bool nf_fills_rows(int nt, int nrhs) {
 }
 size_t near_field_work_bytes(long long total, int nt, int nrhs) {
   const int group = near_field_group(total, nrhs);
-  return (double)total * nt >= NF_PAIRS_MIN && nf_fills_rows(nt, group) ? nf_plan(total, nt, group).bytes : 0;
+  return (double)total * nt >= NF_PAIRS_MIN && nf_fills_rows(nt, group) ? nf_plan(total, nt, group, pass_bytes()).bytes : 0;
 }
 
 bool launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const double* X_dev, int nt, int n_theta,
@@ -582,7 +582,7 @@ bool launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const d
   const int group = near_field_group(total, nrhs);
   NfPlan plan{};
   if (work) {
-    plan = nf_plan(total, nt, group);
+    plan = nf_plan(total, nt, group, pass_bytes());
     if (plan.bytes > work_bytes) return false;
   }
   for (int w0 = 0; w0 < nrhs; w0 += group) {
@@ -810,19 +810,21 @@ static void launch_ffgrid_mode(const FieldGeom& g, int M, double k0, double omeg
 #define FFO_MIN 2e7
 size_t far_field_grid_work_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
   const double fma = 24.0 * ((n_polar + 1) / 2) * N * (2.0 * M + 1.0) * nrhs;
-  return fma >= FFO_MIN ? ffgrid_oz_bytes(N, M, n_polar, n_azim, n_alpha, nrhs) : 0;
+  return fma >= FFO_MIN ? ffo_plan(N, M, n_polar, n_azim, n_alpha, nrhs, pass_bytes()).bytes : 0;
 }
 
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar) {
   return (size_t)((n_polar + 1) / 2) * N * (M + 4);  // M + 2 coefficients and the complex phase
 }
 
-void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
-                           cudaStream_t s) {
+bool launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
+                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, size_t work_bytes, cd* F, cd* E,
+                           int* err, cudaStream_t s) {
   if (work) {
-    launch_ffgrid_products(g, M, k0, omega, eps0, x, nrhs, n_polar, n_azim, n_alpha, work, F, E, err, s);
-    return;
+    const FfoPlan plan = ffo_plan(g.N, M, n_polar, n_azim, n_alpha, nrhs, pass_bytes());
+    if (plan.bytes > work_bytes) return false;
+    launch_ffgrid_products(g, M, k0, omega, eps0, x, nrhs, n_polar, n_azim, n_alpha, plan, work, F, E, err, s);
+    return true;
   }
   const int P2 = (n_polar + 1) / 2, Q = n_alpha / 4 + 1;
   double2* phase = (double2*)coef;                 // 16-byte aligned at the block's start
@@ -839,6 +841,7 @@ void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, c
   const int smem3 = (6 * (M + 1) + n_azim) * (int)sizeof(cd);
   smem_optin(ffgrid_synth_kernel);
   ffgrid_synth_kernel<<<dim3(n_polar, nrhs), 128, smem3, s>>>(M, n_polar, n_azim, F, nrhs, E);
+  return true;
 }
 
 // Currents at refined nodes: xs[v][4s + a] = sum_k Lm[s][k] x[v][4 (node0[s] + k) + a]

@@ -45,12 +45,12 @@ bool launch_near_field(const FieldGeom& g, int M, const cd* x, int nrhs, const d
 // E[rhs][p][s][3] (k0 real, n_alpha a multiple of 4); F [rhs][n_polar][2M+1][3] and
 // either work of far_field_grid_work_bytes (256-byte aligned; err, a device int, is
 // set if a bounded wait gives up) or coef of far_field_grid_coef_doubles values (work
-// null: FP64 pipe).
+// null: FP64 pipe).  False, with nothing launched, when work_bytes do not hold the layout.
 size_t far_field_grid_coef_doubles(int N, int M, int n_polar);
 size_t far_field_grid_work_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs);
-void launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, cd* F, cd* E, int* err,
-                           cudaStream_t s);
+bool launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
+                           int n_polar, int n_azim, int n_alpha, double* coef, void* work, size_t work_bytes, cd* F, cd* E,
+                           int* err, cudaStream_t s);
 
 // Currents x[v][n] at the nodes -> xs[v][4 nsub] at refined nodes (rows Lm[nsub][16]
 // of the panel interpolants, node0 = first node of each sub-node's panel).

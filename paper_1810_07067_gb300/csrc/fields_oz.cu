@@ -66,14 +66,16 @@ __device__ __forceinline__ void put_digits(__nv_bfloat16* dst, int stride, const
   for (int q = 0; q < OZ_S; ++q) *(uint4*)(dst + (size_t)q * stride) = *(const uint4*)pc[q];
 }
 
-// Rows 2 pp + t (t = 0 cos, 1 sin) of index a for the angles p0 + pp: one CTA per (pp, a).
-// coef: b_a of row pp N + j at [a & 1][a / 2][row], ldc rows to a column, ncc columns.
-__global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int nrt, const double* __restrict__ coef, int ncc,
-                                                      size_t ldc, const double2* __restrict__ phase,
+// Rows 2 pp + t (t = 0 cos, 1 sin) of index a0 + a for the angles p0 + pp: one CTA per
+// (pp - b0, a).  coef: b_{a0 + a} of row (pp - b0) N + j at [index & 1][index / 2][row],
+// ldc rows to a column, ncc columns.
+__global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int b0, int a0, int nrt,
+                                                      const double* __restrict__ coef, int ncc, size_t ldc,
+                                                      const double2* __restrict__ phase,
                                                       __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
   __shared__ unsigned red[2][2];
-  const int pp = blockIdx.x, a = blockIdx.y, tid = threadIdx.x, nkt = N / OZ_KT;
-  const double* b = coef + ((size_t)(a & 1) * ncc + (a >> 1)) * ldc + (size_t)pp * N;
+  const int pp = b0 + blockIdx.x, a = blockIdx.y, tid = threadIdx.x, nkt = N / OZ_KT;
+  const double* b = coef + ((size_t)((a0 + a) & 1) * ncc + ((a0 + a) >> 1)) * ldc + (size_t)blockIdx.x * N;
   const double2* ph = phase + (size_t)(p0 + pp) * N;
   unsigned ex[2] = {0u, 0u};
   for (int j = tid; j < N; j += 64) {
@@ -110,14 +112,15 @@ __global__ void __launch_bounds__(64) ffo_rows_kernel(int N, int p0, int nrt, co
 
 // Columns of mode q and right-hand side w0 + w: X_0 = r' J1 + i J2, X_1 = z' J1,
 // X_2 = r' J1 - i J2 (and of M), times the nodes' weights (wt of ffo_phase_kernel), for
-// a = |m + 1|, |m|, |m - 1|.  One CTA per (q, w, X).
+// a = |m + 1|, |m|, |m - 1| where that is one of a0 .. a0 + na - 1.  One CTA per (q, w, X).
 __global__ void __launch_bounds__(64) ffo_cols_kernel(int N, int M, const double* __restrict__ wt,
-                                                      const cd* __restrict__ x, int nrhs, int w0, int nw, int nct,
-                                                      __nv_bfloat16* __restrict__ Bsl,
+                                                      const cd* __restrict__ x, int nrhs, int w0, int nw, int a0,
+                                                      int na, int nct, __nv_bfloat16* __restrict__ Bsl,
                                                       double* __restrict__ cscale) {
   __shared__ unsigned red[2];
   const int q = blockIdx.x, w = blockIdx.y, h = blockIdx.z / 3, u = blockIdx.z % 3;
-  const int s = q - M + 1 - u, a = abs(s), nkt = N / OZ_KT, tid = threadIdx.x;
+  const int s = q - M + 1 - u, a = abs(s) - a0, nkt = N / OZ_KT, tid = threadIdx.x;
+  if (a < 0 || a >= na) return;
   const cd* xv = x + ((size_t)q * nrhs + w0 + w) * 4 * N + 2 * h;
   auto value = [&](int j) {
     const cd v1 = xv[4 * j];
@@ -384,12 +387,12 @@ __global__ void __launch_bounds__(128) ffo_phase_kernel(FieldGeom g, double k0, 
 // Azimuths of the grid: rows (rhs, polar angle, component, Re or Im) of F_m + F_-m
 // (index 0, with cos m phi_s) and i (F_m - F_-m) (index 1, with sin), the modes along k.
 
-// One CTA per (polar angle, rhs): its 6 rows of both indices.
-__global__ void __launch_bounds__(128) synth_rows_kernel(int M, int n_polar, const cd* __restrict__ F, int nkt, int nrt,
+// One CTA per (rhs, polar angle) pair: its 6 rows of both indices.
+__global__ void __launch_bounds__(128) synth_rows_kernel(int M, const cd* __restrict__ F, int nkt, int nrt,
                                                          __nv_bfloat16* __restrict__ Asl, double* __restrict__ rscale) {
   extern __shared__ __align__(16) double sv[];  // [12][nkt 16], then the rows' largest exponents
   unsigned* ex = (unsigned*)(sv + 12 * nkt * OZ_KT);
-  const int K = nkt * OZ_KT, wp = blockIdx.y * n_polar + blockIdx.x, tid = threadIdx.x;
+  const int K = nkt * OZ_KT, wp = blockIdx.x, tid = threadIdx.x;
   const cd* src = F + (size_t)wp * (2 * M + 1) * 3;
   if (tid < 12) ex[tid] = 0u;
   __syncthreads();
@@ -440,9 +443,9 @@ __global__ void __launch_bounds__(128) synth_table_kernel(int M, int n, int nkt,
 }
 
 // Both azimuths s and n - s of a sum, turned into Cartesian components.
-__global__ void __launch_bounds__(128) synth_join_kernel(int n_polar, int n_azim, const double* __restrict__ Y, size_t ldy,
+__global__ void __launch_bounds__(128) synth_join_kernel(int n_azim, const double* __restrict__ Y, size_t ldy,
                                                          int nct, cd* __restrict__ E) {
-  const int s = blockIdx.y * 128 + threadIdx.x, wp = blockIdx.z * n_polar + blockIdx.x;
+  const int s = blockIdx.y * 128 + threadIdx.x, wp = blockIdx.x;
   if (s > n_azim / 2) return;
   cd a[3], b[3];
 #pragma unroll
@@ -698,90 +701,57 @@ __global__ void __launch_bounds__(128) rhs_rows_kernel(FieldGeom g, int M, const
   }
 }
 
-// Angles and right-hand sides of a pass: as many as keep any operand's digits
-// within FFO_BYTES, at least one row tile of angles and one side.
-struct FfoPlan {
-  int P2, na, nkt, np, nw, nrt, nct;  // np angles and nw sides of a full pass
-  RingPlan ring;
-  int snkt, snct, snw;                // azimuths: k-tiles, column tiles, sides of a pass
-  size_t phase, a, r, b, c, y, tb, cost, coef;  // bytes of the parts
-};
-FfoPlan ffo_plan(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
-  FfoPlan f{};
-  f.P2 = (n_polar + 1) / 2;
-  f.na = M + 2;
-  f.nkt = N / OZ_KT;
-  f.ring = ring_plan(M, n_alpha);
-  const size_t ta = (size_t)f.na * f.nkt * FFO_ABLOCK * 2, tb = (size_t)f.na * f.nkt * FFO_BBLOCK * 2;
-  const size_t tr = f.ring.a_row_tile * tiles((size_t)OZ_RT / 2 * N, OZ_RT);  // samples of one row tile of angles
-  f.nrt = (int)std::max<size_t>(1, std::min<size_t>(tiles(2 * f.P2, OZ_RT), FFO_BYTES / std::max(ta, tr)));
-  f.np = std::min(f.P2, f.nrt * OZ_RT / 2);
-  const size_t ty = (size_t)f.na * FFO_NT * f.nrt * OZ_RT * 8;  // sums of a column tile
-  f.nw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / std::max(tb, ty) * FFO_NT / 24));
-  f.nct = (int)tiles(24 * f.nw, FFO_NT);
-  f.snkt = (int)tiles(M + 1, OZ_KT);
-  f.snct = (int)tiles(n_azim / 2 + 1, FFO_NT);
-  const size_t sa = (size_t)2 * f.snkt * FFO_ABLOCK * 2 * tiles((size_t)6 * n_polar, OZ_RT);  // one side's rows, about
-  const size_t sy = (size_t)2 * f.snct * FFO_NT * 6 * n_polar * 8;
-  f.snw = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FFO_BYTES / std::max(sa, sy)));
-  const size_t srt = tiles((size_t)6 * f.snw * n_polar, OZ_RT), rrt = tiles((size_t)f.np * N, OZ_RT);
-  f.phase = up256((size_t)N * (f.P2 * 16 + 24));  // and the weights
-  f.a = up256(std::max({f.nrt * ta, rrt * f.ring.a_row_tile, srt * 2 * f.snkt * FFO_ABLOCK * 2}));
-  f.r = up256(std::max((size_t)f.na * f.nrt, 2 * srt) * OZ_RT * 8);
-  f.b = up256(std::max(f.nct * tb, (size_t)2 * f.snct * f.snkt * FFO_BBLOCK * 2));
-  f.c = up256((size_t)f.na * f.nct * FFO_NT * 8);
-  f.y = up256(std::max((size_t)f.na * f.nct * FFO_NT * f.nrt, (size_t)2 * f.snct * FFO_NT * srt) * OZ_RT * 8);
-  f.tb = f.ring.b;
-  f.cost = f.ring.cost;
-  f.coef = up256(rrt * f.ring.y_row_tile);
-  return f;
-}
-
 }  // namespace
 
-size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs) {
-  const FfoPlan f = ffo_plan(N, M, n_polar, n_azim, n_alpha, nrhs);
-  return f.phase + f.a + f.r + f.b + f.c + f.y + f.tb + f.cost + f.coef;
-}
-
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                            int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s) {
-  const FfoPlan f = ffo_plan(g.N, M, n_polar, n_azim, n_alpha, nrhs);
+                            int n_polar, int n_azim, int n_alpha, const FfoPlan& f, void* work, cd* F, cd* E, int* err,
+                            cudaStream_t s) {
   const int sms = digit_ready();
   char* p = (char*)work;
-  auto* phase = (double2*)p;
+  auto* phase = (double2*)(p + f.phase);
   auto* wt = (double*)(phase + (size_t)f.P2 * g.N);
-  auto* Asl = (__nv_bfloat16*)(p += f.phase);
-  auto* rscale = (double*)(p += f.a);
-  auto* Bsl = (__nv_bfloat16*)(p += f.r);
-  auto* cscale = (double*)(p += f.b);
-  auto* Y = (double*)(p += f.c);
-  auto* Tsl = (__nv_bfloat16*)(p += f.y);
-  auto* cost = (double*)(p += f.tb);
-  auto* coef = (double*)(p += f.cost);
+  auto* Asl = (__nv_bfloat16*)(p + f.a);
+  auto* rscale = (double*)(p + f.r);
+  auto* Bsl = (__nv_bfloat16*)(p + f.b);
+  auto* cscale = (double*)(p + f.c);
+  auto* Y = (double*)(p + f.y);
+  auto* Tsl = (__nv_bfloat16*)(p + f.table);
+  auto* cost = (double*)(p + f.cost);
+  auto coef = [&](int b0) { return (double*)(p + f.coef + b0 / f.nps * f.coef_block); };  // of the block at angle b0
   ffo_phase_kernel<<<dim3(f.P2, (g.N + 127) / 128), 128, 0, s>>>(g, k0, n_polar, phase, wt);
   ring_table(f.ring, M, n_alpha, Tsl, cost, s);
   for (int p0 = 0; p0 < f.P2; p0 += f.np) {
-    const int np = std::min(f.np, f.P2 - p0), nrt = (int)tiles(2 * np, OZ_RT);
-    ring_integrals(sms, f.ring, g, np, nullptr, k0, p0, n_polar, Asl, Tsl, cost, coef, err, s);
-    ffo_rows_kernel<<<dim3(np, f.na), 64, 0, s>>>(g.N, p0, nrt, coef, f.ring.nct * FFO_NT,
-                                                 tiles((size_t)np * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
+    const int np = std::min(f.np, f.P2 - p0), nrt = (int)tiles((size_t)2 * np, OZ_RT);
+    for (int b0 = 0; b0 < np; b0 += f.nps)
+      ring_integrals(sms, f.ring, g, std::min(f.nps, np - b0), nullptr, k0, p0 + b0, n_polar, Asl, Tsl, cost, coef(b0),
+                     err, s);
     for (int w0 = 0; w0 < nrhs; w0 += f.nw) {
-      const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles(24 * nw, FFO_NT);
-      ffo_cols_kernel<<<dim3(2 * M + 1, nw, 6), 64, 0, s>>>(g.N, M, wt, x, nrhs, w0, nw, nct, Bsl, cscale);
-      digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, f.na, Y, err, s);
+      const int nw = std::min(f.nw, nrhs - w0), nct = (int)tiles((size_t)24 * nw, FFO_NT);
+      for (int a0 = 0; a0 < f.na; a0 += f.nap) {
+        const int na = std::min(f.nap, f.na - a0);
+        if (w0 == 0 || f.nap < f.na)  // else the rows' digits are still there
+          for (int b0 = 0; b0 < np; b0 += f.nps) {
+            const int nb = std::min(f.nps, np - b0);
+            ffo_rows_kernel<<<dim3(nb, na), 64, 0, s>>>(g.N, p0, b0, a0, nrt, coef(b0), f.ring.nct * FFO_NT,
+                                                        tiles((size_t)nb * g.N, OZ_RT) * OZ_RT, phase, Asl, rscale);
+          }
+        ffo_cols_kernel<<<dim3(2 * M + 1, nw, 6), 64, 0, s>>>(g.N, M, wt, x, nrhs, w0, nw, a0, na, nct, Bsl, cscale);
+        digit_gemm(sms, Asl, rscale, Bsl, cscale, 1.0, f.nkt, nrt, nct, na, Y + (size_t)a0 * nct * FFO_NT * nrt * OZ_RT,
+                   err, s);
+      }
       ffo_vector_kernel<<<dim3((np + 127) / 128, 2 * M + 1, std::min(nw, 64)), 128, 0, s>>>(
           M, k0, omega, eps0, n_polar, f.P2, p0, np, nrt, nct, w0, nw, Y, F);
     }
   }
   synth_table_kernel<<<dim3(n_azim / 2 + 1, 2), 128, 0, s>>>(M, n_azim, f.snkt, f.snct, Bsl);
-  for (int w0 = 0; w0 < nrhs; w0 += f.snw) {
-    const int nw = std::min(f.snw, nrhs - w0), nrt = (int)tiles((size_t)6 * nw * n_polar, OZ_RT);
-    synth_rows_kernel<<<dim3(n_polar, nw), 128, 12 * (f.snkt * OZ_KT * 8 + 4), s>>>(
-        M, n_polar, F + (size_t)w0 * n_polar * (2 * M + 1) * 3, f.snkt, nrt, Asl, rscale);
+  const long long pairs = (long long)nrhs * n_polar;
+  for (long long q0 = 0; q0 < pairs; q0 += f.swp) {
+    const int nq = (int)std::min<long long>(f.swp, pairs - q0), nrt = (int)tiles((size_t)6 * nq, OZ_RT);
+    synth_rows_kernel<<<nq, 128, 12 * (f.snkt * OZ_KT * 8 + 4), s>>>(M, F + (size_t)q0 * (2 * M + 1) * 3, f.snkt, nrt,
+                                                                     Asl, rscale);
     digit_gemm(sms, Asl, rscale, Bsl, nullptr, 2.0, f.snkt, nrt, f.snct, 2, Y, err, s);
-    synth_join_kernel<<<dim3(n_polar, (n_azim / 2 + 128) / 128, nw), 128, 0, s>>>(
-        n_polar, n_azim, Y, (size_t)nrt * OZ_RT, f.snct, E + (size_t)w0 * n_polar * n_azim * 3);
+    synth_join_kernel<<<dim3(nq, (n_azim / 2 + 128) / 128), 128, 0, s>>>(n_azim, Y, (size_t)nrt * OZ_RT, f.snct,
+                                                                         E + (size_t)q0 * n_azim * 3);
   }
 }
 

@@ -46,12 +46,12 @@ __device__ __forceinline__ void ffgrid_vector(const cd* A, const cd* B, int m, i
   }
 }
 
-// Workspace of launch_ffgrid_products in bytes (256-byte aligned), and the whole grid
-// by products on the tensor cores: ring integrals, sums over the nodes (into F), sums
-// over the modes (into E); err (device int) is set if a bounded wait gives up.
-size_t ffgrid_oz_bytes(int N, int M, int n_polar, int n_azim, int n_alpha, int nrhs);
+// The whole grid by products on the tensor cores: ring integrals, sums over the nodes
+// (into F), sums over the modes (into E); work of plan.bytes (256-byte aligned), plan the
+// ffo_plan of the same arguments; err (device int) is set if a bounded wait gives up.
 void launch_ffgrid_products(const FieldGeom& g, int M, double k0, double omega, cd eps0, const cd* x, int nrhs,
-                            int n_polar, int n_azim, int n_alpha, void* work, cd* F, cd* E, int* err, cudaStream_t s);
+                            int n_polar, int n_azim, int n_alpha, const FfoPlan& plan, void* work, cd* F, cd* E, int* err,
+                            cudaStream_t s);
 
 // Modal data of the waves w0 .. w0 + count - 1 (count <= RHS_WAVES) of nrhs from their
 // table (rhs_wave_kernel without the factors fE, fH of the traces); work of plan.bytes

@@ -1433,8 +1433,9 @@ extern "C" int mueller_far_field_grid(mueller_ctx* c, const mueller_c128* x_dev,
   if (!work && tmp.alloc(&coef, far_field_grid_coef_doubles(c->S.N, M, n_polar)) != cudaSuccess)
     return fail(MUELLER_ENOMEM, "far-field grid buffers");
   if (work) CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-  launch_far_field_grid(g, M, c->S.k0.x, c->S.omega, c->S.eps0, (const cd*)x_dev, nrhs, n_polar, n_azim, nth, coef,
-                        work, F, (cd*)E_dev, err, s);
+  if (!launch_far_field_grid(g, M, c->S.k0.x, c->S.omega, c->S.eps0, (const cd*)x_dev, nrhs, n_polar, n_azim, nth, coef,
+                             work, bytes, F, (cd*)E_dev, err, s))
+    return fail(MUELLER_EINVAL, "workspace of the far-field grid too small");
   CK(cudaGetLastError());
   int herr = 0;
   if (work) CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
