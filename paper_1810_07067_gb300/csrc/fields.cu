@@ -661,30 +661,31 @@ __global__ void __launch_bounds__(256) ffgrid_coef_kernel(FieldGeom g, int M, do
 // whole grid, N = 512, M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex
 // coefficients per angle and the phase formed per mode and side; 0.94 ms on the
 // tensor cores, which take all but small grids).  One CTA per
-// (mode, 16 polar angles, WT right-hand sides); a thread owns one (angle, side)
-// and every JS-th node; the nodes pass through shared memory FFM_JC at a time.
-#define FFM_PT 16
-#define FFM_JC 16
-template <int WT>
+// (mode, PT polar angles, WT right-hand sides); a thread owns one (angle, side)
+// and every JS-th node; the nodes pass through shared memory JC at a time.
+// PT is 16, and 2 for at most four angles, whose 16-angle tiles would be idle lanes that
+// the FP64 pipe issues all the same: N = 128, M = 16, 8 sides, one direction 126 -> 24 us.
+template <int PT, int WT>
 __global__ void __launch_bounds__(128) ffgrid_mode_kernel(FieldGeom g, int M, double k0, double omega, cd eps0,
                                                           int n_polar, int P2, const double* __restrict__ coef,
                                                           const double2* __restrict__ phase,
                                                           const cd* __restrict__ x, int nrhs, cd* __restrict__ F) {
-  constexpr int JS = 128 / (FFM_PT * WT);
-  __shared__ double2 sb[3][FFM_JC][FFM_PT + 1];  // b_{m+1}, b_m, b_{m-1} times the phase's (cos, sin)
-  __shared__ cd sX[FFM_JC][WT][6];
-  __shared__ cd red[JS > 1 ? 128 : 1];
-  const int q = blockIdx.y, m = q - M, p0 = blockIdx.x * FFM_PT, w0 = blockIdx.z * WT;
-  const int tid = threadIdx.x, pl = tid % FFM_PT, wl = (tid / FFM_PT) % WT, js = tid / (FFM_PT * WT);
+  constexpr int JS = 128 / (PT * WT), JC = JS > 16 ? JS : 16;
+  __shared__ double2 sb[3][JC][PT + 1];  // b_{m+1}, b_m, b_{m-1} times the phase's (cos, sin)
+  __shared__ cd sX[JC][WT][6];
+  __shared__ cd red[PT == 16 ? (JS > 1 ? 128 : 1) : 12 * 4 * PT * WT];
+  const int q = blockIdx.y, m = q - M, p0 = blockIdx.x * PT, w0 = blockIdx.z * WT;
+  const int tid = threadIdx.x, pl = tid % PT, wl = (tid / PT) % WT, js = tid / (PT * WT);
   const int n = 4 * g.N;
   const int mi[3] = {abs(m + 1), abs(m), abs(m - 1)};
   cd A[6], B[6];
 #pragma unroll
   for (int u = 0; u < 6; ++u) { A[u] = C(0.0); B[u] = C(0.0); }
-  for (int j0 = 0; j0 < g.N; j0 += FFM_JC) {  // N is a multiple of 16
-    for (int it = tid; it < FFM_JC * FFM_PT; it += 128) {
-      const int jj = it % FFM_JC, pp = it / FFM_JC;
-      if (p0 + pp < P2) {
+  for (int j0 = 0; j0 < g.N; j0 += JC) {  // N is a multiple of 16
+    const int nj = JC == 16 ? JC : min(JC, g.N - j0);
+    for (int it = tid; it < JC * PT; it += 128) {
+      const int jj = it % JC, pp = it / JC;
+      if (p0 + pp < P2 && jj < nj) {
         const size_t o = (size_t)(p0 + pp) * g.N + j0 + jj;
         const double2 ph = phase[o];
 #pragma unroll
@@ -694,8 +695,9 @@ __global__ void __launch_bounds__(128) ffgrid_mode_kernel(FieldGeom g, int M, do
         }
       }
     }
-    for (int it = tid; it < FFM_JC * WT * 2; it += 128) {
-      const int h = it & 1, jj = (it >> 1) % FFM_JC, w = (it >> 1) / FFM_JC, j = j0 + jj;
+    for (int it = tid; it < JC * WT * 2; it += 128) {
+      const int h = it & 1, jj = (it >> 1) % JC, w = (it >> 1) / JC, j = j0 + jj;
+      if (jj >= nj) continue;
       cd v1 = C(0.0), v2 = C(0.0);
       if (w0 + w < nrhs) {
         const cd* xv = x + ((size_t)q * nrhs + w0 + w) * n + 4 * j + 2 * h;
@@ -710,7 +712,7 @@ __global__ void __launch_bounds__(128) ffgrid_mode_kernel(FieldGeom g, int M, do
     __syncthreads();
     if (p0 + pl < P2) {
 #pragma unroll 2
-      for (int jj = js; jj < FFM_JC; jj += JS) {
+      for (int jj = js; jj < nj; jj += JS) {
 #pragma unroll
         for (int u = 0; u < 6; ++u) {
           const double2 b = sb[u % 3][jj][pl];
@@ -722,13 +724,34 @@ __global__ void __launch_bounds__(128) ffgrid_mode_kernel(FieldGeom g, int M, do
     }
     __syncthreads();
   }
-  if (JS > 1) {
+  if constexpr (PT < 16) {  // the nodes' parts of a warp, then of the four warps
+    constexpr int L = PT * WT;
+    const int lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int v = 0; v < 12; ++v) {
+      cd t = v < 6 ? A[v % 6] : B[v % 6];
+#pragma unroll
+      for (int o = L; o < 32; o <<= 1) {
+        t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+        t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+      }
+      if (lane < L) red[(v * 4 + wid) * L + lane] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 12; ++v) {
+      const cd* x4 = red + v * 4 * L + lane % L;
+      const cd t = (x4[0] + x4[L]) + (x4[2 * L] + x4[3 * L]);
+      if (v < 6) A[v % 6] = t;
+      else B[v % 6] = t;
+    }
+  } else if (JS > 1) {
     for (int v = 0; v < 12; ++v) {
       red[tid] = v < 6 ? A[v % 6] : B[v % 6];
       __syncthreads();
       cd t = C(0.0);
 #pragma unroll
-      for (int k = 0; k < JS; ++k) t += red[k * FFM_PT * WT + tid % (FFM_PT * WT)];
+      for (int k = 0; k < JS; ++k) t += red[k * PT * WT + tid % (PT * WT)];
 #pragma unroll
       for (int u = 0; u < 6; ++u) {
         if (v == u) A[u] = t;
@@ -793,11 +816,11 @@ __global__ void __launch_bounds__(128) ffgrid_synth_kernel(int M, int n_polar, i
   }
 }
 
-template <int WT>
+template <int PT, int WT>
 static void launch_ffgrid_mode(const FieldGeom& g, int M, double k0, double omega, cd eps0, int n_polar, int P2,
                                const double* coef, const double2* phase, const cd* x, int nrhs, cd* F,
                                cudaStream_t s) {
-  ffgrid_mode_kernel<WT><<<dim3((P2 + FFM_PT - 1) / FFM_PT, 2 * M + 1, (nrhs + WT - 1) / WT), 128, 0, s>>>(
+  ffgrid_mode_kernel<PT, WT><<<dim3((P2 + PT - 1) / PT, 2 * M + 1, (nrhs + WT - 1) / WT), 128, 0, s>>>(
       g, M, k0, omega, eps0, n_polar, P2, coef, phase, x, nrhs, F);
 }
 
@@ -833,11 +856,20 @@ bool launch_far_field_grid(const FieldGeom& g, int M, double k0, double omega, c
   smem_optin(ffgrid_coef_kernel);
   ffgrid_coef_kernel<<<dim3(P2, (g.N + FFC_R - 1) / FFC_R), 256, smem1, s>>>(g, M, k0, n_polar, n_alpha, b, phase);
   // right-hand sides per CTA: the smallest of 1, 2, 4, 8 that holds them (the
-  // angles' coefficients are read once per group)
-  if (nrhs <= 1) launch_ffgrid_mode<1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
-  else if (nrhs <= 2) launch_ffgrid_mode<2>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
-  else if (nrhs <= 4) launch_ffgrid_mode<4>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
-  else launch_ffgrid_mode<8>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  // angles' coefficients are read once per group); with few angles fewer, as long as
+  // there are SMs for the CTAs (one direction, 8 sides a CTA, 4, 2, 1: N = 128, M = 16,
+  // 8 sides 38, 26, 21, 24 us; N = 512, M = 64, 4 sides 110, 65, 58, 78 us)
+  int wt = nrhs <= 1 ? 1 : nrhs <= 2 ? 2 : nrhs <= 4 ? 4 : 8;
+  if (P2 <= 4) {
+    while (wt > 1 && (long long)((P2 + 1) / 2) * (2 * M + 1) * ((nrhs + wt - 1) / wt) < 152) wt /= 2;
+    if (wt == 1) launch_ffgrid_mode<2, 1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+    else if (wt == 2) launch_ffgrid_mode<2, 2>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+    else if (wt == 4) launch_ffgrid_mode<2, 4>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+    else launch_ffgrid_mode<2, 8>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  } else if (wt == 1) launch_ffgrid_mode<16, 1>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  else if (wt == 2) launch_ffgrid_mode<16, 2>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  else if (wt == 4) launch_ffgrid_mode<16, 4>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
+  else launch_ffgrid_mode<16, 8>(g, M, k0, omega, eps0, n_polar, P2, b, phase, x, nrhs, F, s);
   const int smem3 = (6 * (M + 1) + n_azim) * (int)sizeof(cd);
   smem_optin(ffgrid_synth_kernel);
   ffgrid_synth_kernel<<<dim3(n_polar, nrhs), 128, smem3, s>>>(M, n_polar, n_azim, F, nrhs, E);
