@@ -129,8 +129,21 @@ __device__ __forceinline__ dd dd_add(dd a, dd b) {
 }
 __device__ __forceinline__ dd dd_neg(dd a) { return dd{-a.h, -a.l}; }
 
+__device__ __forceinline__ dd dd_shfl(dd a, int lane) {
+  return dd{__shfl_sync(0xffffffffu, a.h, lane), __shfl_sync(0xffffffffu, a.l, lane)};
+}
+struct ddc { dd x, y; };  // complex
+__device__ __forceinline__ ddc ddc_mul(ddc a, ddc b) {
+  return ddc{dd_add(dd_mul(a.x, b.x), dd_neg(dd_mul(a.y, b.y))), dd_add(dd_mul(a.x, b.y), dd_mul(a.y, b.x))};
+}
+__device__ __forceinline__ ddc ddc_shfl(ddc a, int lane) { return ddc{dd_shfl(a.x, lane), dd_shfl(a.y, lane)}; }
+
 // The table of the waves w0..w0 + gridDim.x - 1 (one CTA each), wave[w] =
-// (k0 d_rho, k0 d_z), and (first CTA) cost[n_theta] = cos(2 pi t / n_theta).
+// (k0 d_rho, k0 d_z), and (first CTA) cost[n_theta] = cos(2 pi t / n_theta).  A chain of
+// FP64 operations: warp 0 alone forms the powers of z = e^{-i phi_d}, z^1 .. z^32 by
+// doubling (lane l holds z^{l + 1}; five products), then 32 more with each product, while
+// the other warps form the cosines (every warp the direction, a binary power per mode:
+// M = 16 20.8 us, now 14).
 __global__ void __launch_bounds__(128) rhs_wave_kernel(int M, double k0, cd hf, cd sE, cd sH,
                                                        const double* __restrict__ dirs,
                                                        const double* __restrict__ pols, int n_theta,
@@ -141,32 +154,37 @@ __global__ void __launch_bounds__(128) rhs_wave_kernel(int M, double k0, cd hf, 
   const int w = blockIdx.x;
   const double* d = dirs + 3 * w;
   const double* e = pols + 3 * w;
-  if (w == 0)
-    for (int t = threadIdx.x; t < n_theta; t += blockDim.x) cost[t] = cospi(2.0 * t / n_theta);
-  const dd s2 = dd_add(dd_prod(d[0], d[0]), dd_prod(d[1], d[1]));
-  dd zr{1.0, 0.0}, zi{0.0, 0.0};  // e^{-i phi_d}
-  double drho = 0.0;
-  if (s2.h > 1e-280) {
-    const double r0 = rsqrt(s2.h);
-    const dd t = dd_mul(s2, dd_prod(r0, r0));
-    const dd r = dd_norm(r0, 0.5 * r0 * ((1.0 - t.h) - t.l));
-    zr = dd_mul(dd{d[0], 0.0}, r);
-    zi = dd_neg(dd_mul(dd{d[1], 0.0}, r));
-    drho = s2.h * r.h + (s2.h * r.l + s2.l * r.h);
-  }
-  if (threadIdx.x == 0) wave[w] = make_double2(k0 * drho, k0 * d[2]);
-  for (int m = threadIdx.x; m < M + 2; m += blockDim.x) {
-    dd pr{1.0, 0.0}, pi{0.0, 0.0}, br = zr, bi = zi;
-    for (int b = m; b; b >>= 1) {
-      if (b & 1) {
-        const dd nr = dd_add(dd_mul(pr, br), dd_neg(dd_mul(pi, bi))), ni = dd_add(dd_mul(pr, bi), dd_mul(pi, br));
-        pr = nr; pi = ni;
-      }
-      const dd nr = dd_add(dd_mul(br, br), dd_neg(dd_mul(bi, bi))), h = dd_mul(br, bi);
-      br = nr;
-      bi = dd{2.0 * h.h, 2.0 * h.l};
+  if (threadIdx.x >= 32) {
+    if (w == 0)
+      for (int t = threadIdx.x - 32; t < n_theta; t += 96) cost[t] = cospi(2.0 * t / n_theta);
+  } else {
+    const int lane = threadIdx.x;
+    const dd s2 = dd_add(dd_prod(d[0], d[0]), dd_prod(d[1], d[1]));
+    ddc z{dd{1.0, 0.0}, dd{0.0, 0.0}};
+    double drho = 0.0;
+    if (s2.h > 1e-280) {
+      const double r0 = rsqrt(s2.h);
+      const dd t = dd_mul(s2, dd_prod(r0, r0));
+      const dd r = dd_norm(r0, 0.5 * r0 * ((1.0 - t.h) - t.l));
+      z.x = dd_mul(dd{d[0], 0.0}, r);
+      z.y = dd_neg(dd_mul(dd{d[1], 0.0}, r));
+      drho = s2.h * r.h + (s2.h * r.l + s2.l * r.h);
     }
-    em[m] = C(pr.h, pi.h);
+    if (lane == 0) {
+      wave[w] = make_double2(k0 * drho, k0 * d[2]);
+      em[0] = C(1.0);
+    }
+    ddc p = z;
+#pragma unroll
+    for (int n = 1; n < 32; n <<= 1) {  // lanes 0..n - 1 hold z^1 .. z^n
+      const ddc q = ddc_mul(ddc_shfl(p, n - 1), ddc_shfl(p, lane & (n - 1)));
+      if (lane >= n) p = q;
+    }
+    const ddc z32 = ddc_shfl(p, 31);
+    for (int m0 = 1; m0 < M + 2; m0 += 32) {
+      if (m0 > 1) p = ddc_mul(p, z32);
+      if (m0 + lane < M + 2) em[m0 + lane] = C(p.x.h, p.y.h);
+    }
   }
   __syncthreads();
   const double hv[3] = {d[1] * e[2] - d[2] * e[1], d[2] * e[0] - d[0] * e[2], d[0] * e[1] - d[1] * e[0]};
@@ -187,41 +205,43 @@ __global__ void __launch_bounds__(128) rhs_wave_kernel(int M, double k0, cd hf, 
   }
 }
 
-// One CTA per (RHS_R nodes, wave): samples of the nodes' ring phases, their
-// coefficients b_m, then two rows (E or H) per (mode, node) and thread.
-#define RHS_R 8
+// One CTA per (R nodes, wave): samples of the nodes' ring phases, their
+// coefficients b_m, then two rows (E or H) per (mode, node) and thread.  An SM's FP64 pipe
+// issues a warp's operation in 19 clocks, so a call that leaves SMs without a CTA takes
+// fewer nodes a CTA: N = 128, M = 16, one wave, 8 nodes 11 us, 2 nodes 7 us.
+template <int R>
 __global__ void __launch_bounds__(256) rhs_kernel(FieldGeom g, int M, const double2* __restrict__ wave,
                                                   const cd* __restrict__ tab, const double* __restrict__ cost,
                                                   int w0, int nrhs, int n, cd* __restrict__ rhs) {
   extern __shared__ __align__(16) char smem[];
   const int Q = n / 4 + 1;
   double* ct = (double*)smem;           // [n], n a multiple of 4
-  double* smp = ct + n;                 // [2][RHS_R][Q]
-  double* b = smp + 2 * RHS_R * Q;      // [M + 2][RHS_R]
-  double2* phz = (double2*)(b + RHS_R * (M + 2));  // [RHS_R] e^{i k0 z d_z}
-  const int i0 = blockIdx.x * RHS_R, w = blockIdx.y;
+  double* smp = ct + n;                 // [2][R][Q]
+  double* b = smp + 2 * R * Q;      // [M + 2][R]
+  double2* phz = (double2*)(b + R * (M + 2));  // [R] e^{i k0 z d_z}
+  const int i0 = blockIdx.x * R, w = blockIdx.y;
   const double2 wv = wave[w];
   for (int t = threadIdx.x; t < n; t += blockDim.x) ct[t] = cost[t];
-  if (threadIdx.x < RHS_R) {
+  if (threadIdx.x < R) {
     double s, c;
     sincos(wv.y * g.z[i0 + threadIdx.x], &s, &c);
     phz[threadIdx.x] = make_double2(c, s);
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < RHS_R * Q; it += blockDim.x) {
+  for (int it = threadIdx.x; it < R * Q; it += blockDim.x) {
     const int row = it / Q, t = it - row * Q;
-    ring_even_sample(smp, RHS_R, Q, row, t, wv.x * g.r[i0 + row], ct, n);
+    ring_even_sample(smp, R, Q, row, t, wv.x * g.r[i0 + row], ct, n);
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < RHS_R * (M + 2); it += blockDim.x)
-    b[it] = ring_even_coef(smp, RHS_R, Q, it % RHS_R, it / RHS_R, ct, n);
+  for (int it = threadIdx.x; it < R * (M + 2); it += blockDim.x)
+    b[it] = ring_even_coef(smp, R, Q, it % R, it / R, ct, n);
   __syncthreads();
   const cd* tw = tab + (size_t)w * (2 * M + 1) * 6;
-  for (int it = threadIdx.x; it < 2 * RHS_R * (2 * M + 1); it += blockDim.x) {
-    const int h = it & 1, row = (it >> 1) % RHS_R, q = (it >> 1) / RHS_R, m = q - M, i = i0 + row;
+  for (int it = threadIdx.x; it < 2 * R * (2 * M + 1); it += blockDim.x) {
+    const int h = it & 1, row = (it >> 1) % R, q = (it >> 1) / R, m = q - M, i = i0 + row;
     const cd* u = tw + (size_t)q * 6 + 3 * h;
-    const cd al = b[abs(m - 1) * RHS_R + row] * u[0], be = b[abs(m + 1) * RHS_R + row] * u[2];
-    const cd D = b[abs(m) * RHS_R + row] * u[1];
+    const cd al = b[abs(m - 1) * R + row] * u[0], be = b[abs(m + 1) * R + row] * u[2];
+    const cd D = b[abs(m) * R + row] * u[1];
     cd* o = rhs + ((size_t)q * nrhs + w0 + w) * (4 * g.N) + 4 * i + 2 * h;
     const cd pz = C(phz[row].x, phz[row].y);
     o[0] = mul_i(al - be) * pz;
@@ -284,10 +304,11 @@ bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd
   }
   const int Q = n_theta / 4 + 1;
   const int smem_w = (M + 2) * (int)sizeof(cd);
-  const int smem = (n_theta + 2 * RHS_R * Q + RHS_R * (M + 4)) * (int)sizeof(double);
-  smem_optin(rhs_wave_kernel);
-  smem_optin(rhs_kernel);
+  if (smem_w > 48 * 1024) smem_optin(rhs_wave_kernel);
   const int nw = nrhs < RHS_WAVES ? nrhs : RHS_WAVES;
+  const int R = (long long)(g.N / 8) * nw < 152 ? 2 : 8;  // nodes of a CTA: N is a multiple of 16
+  const int smem = (n_theta + 2 * R * Q + R * (M + 4)) * (int)sizeof(double);
+  if (smem > 48 * 1024) R == 2 ? smem_optin(rhs_kernel<2>) : smem_optin(rhs_kernel<8>);
   cd* tab = (cd*)scratch;
   double2* wave = (double2*)(tab + (size_t)nw * (2 * M + 1) * 6);
   double* cost = (double*)(wave + nw);
@@ -298,7 +319,8 @@ bool launch_rhs_planewave(const FieldGeom& g, int M, double k0, double omega, cd
     rhs_wave_kernel<<<c, 128, smem_w, s>>>(M, k0, work ? one : hf, work ? one : sE, work ? one : sH,
                                            dirs_dev + 3 * (size_t)w0, pols_dev + 3 * (size_t)w0, n_theta, tab, wave, cost);
     if (work) launch_rhs_products(g, M, wave, tab, sE, sH * hf, w0, c, nrhs, n_theta, plan, work, rhs, err, s);
-    else rhs_kernel<<<dim3(g.N / RHS_R, c), 256, smem, s>>>(g, M, wave, tab, cost, w0, nrhs, n_theta, rhs);
+    else if (R == 2) rhs_kernel<2><<<dim3(g.N / 2, c), 256, smem, s>>>(g, M, wave, tab, cost, w0, nrhs, n_theta, rhs);
+    else rhs_kernel<8><<<dim3(g.N / 8, c), 256, smem, s>>>(g, M, wave, tab, cost, w0, nrhs, n_theta, rhs);
   }
   return true;
 }
