@@ -617,14 +617,26 @@ void launch_solve(const TF* LU, int n, int M, const int* perm, const double* sw,
   launch_sweep<TF, VT, false, PHYS>(a, s);
 }
 
-int cf_group(int nrhs) { return 2 * nrhs <= 4 ? 4 : 2 * nrhs <= 8 ? 8 : 2 * nrhs <= 16 ? 16 : 2 * nrhs <= 32 ? 32 : 64; }
+// Vectors per group, complex64: the smallest of 4, 8, 16, 32, 64 that holds a mode's 2 nrhs
+// vectors, but 16 up to 1600 and 32 up to 4200 vectors in all modes: a block step waits
+// for one warp's part of the triangle, whose chain grows with the vectors of a group, and
+// only with many vectors is it bound by the bytes that wider groups save.  Whole solves
+// with groups of 16, 32, 64, ms: N = 256: M = 0, 40 sides 2.4, 2.9, 4.2; M = 20, 40 sides
+// (1640 vectors) 5.4, 5.7, 7.1; N = 512, M = 20: 40 sides 14.8, 14.6, 16.7; 100 (4100) 32.2,
+// 29.1, 29.9.
+int cf_group(int M, int nrhs) {
+  const long long vectors = (2LL * M + 1) * nrhs;
+  const int most = vectors <= 1600 ? 16 : vectors <= 4200 ? 32 : 64;
+  const int fit = 2 * nrhs <= 4 ? 4 : 2 * nrhs <= 8 ? 8 : 2 * nrhs <= 16 ? 16 : 2 * nrhs <= 32 ? 32 : 64;
+  return std::min(fit, most);
+}
 int cd_group(int nrhs) { return 2 * nrhs <= 4 ? 4 : 8; }
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
 
 size_t lu_solve_scratch_bytes(int n, int M, int nrhs, bool c64) {
-  const int vt = c64 ? cf_group(nrhs) : cd_group(nrhs);
+  const int vt = c64 ? cf_group(M, nrhs) : cd_group(nrhs);
   const size_t groups = (2 * (size_t)nrhs + vt - 1) / vt;
   const size_t block = (size_t)SB * vt * (!c64 ? sizeof(cd) : vt <= 8 ? sizeof(cf) : 9 * sizeof(__nv_bfloat16));
   return up256((size_t)(M + 1) * n * 4) + 2 * (size_t)(M + 1) * groups * block;
@@ -638,9 +650,8 @@ void lu_solve_prepare(const int* piv, int n, int M, void* scratch, cudaStream_t 
   perm_kernel<<<M + 1, 1024, n * sizeof(int), s>>>(piv, n, (int*)scratch);
 }
 
-// Vectors per group: the smallest of 4, 8, 16, 32, 64 that holds a mode's 2 nrhs
-// vectors (complex128: 4 or 8; more would only lengthen the triangle, the FP64
-// pipe being the bound).
+// Vectors per group, complex128: 4 or 8; more would only lengthen the triangle, the FP64
+// pipe being the bound.
 void lu_solve_modes(const cd* LU, int n, int M, const double* sw, const cd* rhs, cd* x, int nrhs, void* scratch,
                     cudaStream_t s) {
   const int* perm = (const int*)scratch;
@@ -653,7 +664,7 @@ void lu_correction_solve_c64(const cf* LU, int n, int M, const cd* r, cd* d, int
                              cudaStream_t s) {
   const int* perm = (const int*)scratch;
   void* xb = (char*)scratch + up256((size_t)(M + 1) * n * 4);
-  switch (cf_group(nrhs)) {
+  switch (cf_group(M, nrhs)) {
     case 4: launch_solve<cf, 4, false>(LU, n, M, perm, nullptr, r, d, nrhs, xb, s); break;
     case 8: launch_solve<cf, 8, false>(LU, n, M, perm, nullptr, r, d, nrhs, xb, s); break;
     case 16: launch_tc_solve<16>(LU, n, M, perm, r, d, nrhs, xb, err, s); break;
