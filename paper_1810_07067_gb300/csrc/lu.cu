@@ -1,10 +1,15 @@
-// Batched complex128 LU (right-looking, blocked by LU_NB columns) and solves.
+// Batched LU with partial pivoting, complex128 and complex64, of matrices of one or of
+// several orders (right-looking; one table entry a matrix, largest first).
 //
-// Per block column: (1) the panel is factored by one CTA per matrix with a
-// warp-shuffle argmax for the pivot (largest |a|^2, lowest row on ties);
-// (2) its row interchanges are applied to the other columns; (3) the block
-// row of U is formed by a unit-lower triangular solve; (4) the trailing matrix
-// is updated by a complex FP64 GEMM, batched over all matrices.
+// Two levels: panels of LU_NB columns inside outer blocks of LU_OB.  A panel is factored
+// by a cluster of CTAs per matrix, its rows in shared memory (complex128,
+// panel_cluster_kernel) or in registers (complex64, panel_reg_kernel); panel_kernel, one CTA
+// in global memory, takes what no cluster holds.  Its interchanges and rows of U go to
+// the rest of the outer block, which is updated; the block's interchanges, rows of U and
+// one update of rank LU_OB then go to the columns right of it.  Updates are products on the
+// tensor cores: exact digits for complex128 (lu_oz.cu), BF16 pieces for complex64 (R3
+// below; its strips run on the CUDA cores).  Complex128 without a workspace updates the
+// whole trailing matrix after every panel on the FP64 pipe.  Triangular solves: solve.cu.
 #include <algorithm>
 #include <array>
 #include <cstdio>
@@ -351,7 +356,8 @@ static int sm_count() {
 // clusters stay within a group of SMs, so a batch that fills the device takes whole
 // waves, and the sizes that are no power of two often need one wave less (65
 // matrices of order 1280: 3 waves of 32 clusters of eight, 2 of 40 of seven;
-// 48.4 -> 47.7 ms; 9 of order 1250 with eight CTAs instead of two: 15.2 -> 13.7 ms).  Smaller matrices of a ragged batch own fewer rows of the same slices.
+// 48.4 -> 47.7 ms; 9 of order 1250 with eight CTAs instead of two: 15.2 -> 13.7 ms).
+// Smaller matrices of a ragged batch own fewer rows of the same slices.
 // Returns false (nothing launched) when none fits or no such cluster can be
 // resident; the caller then uses panel_kernel.
 template <class T>
@@ -689,37 +695,31 @@ __global__ void __launch_bounds__(256) swap_kernel(const LuMat* __restrict__ mat
 }
 
 // ---------------------------------------------------------------- U12 = L11^{-1} A12
-// Columns (mode): 0 all right of the panel; 1 those right of the panel
-// inside its LU_OB block; 2 those right of the block.
-template <class T>
-__global__ void trsm_kernel(const LuMat* __restrict__ mats, int k0, int K0, int mode) {
+// Complex128 without a workspace: all columns right of the panel, one thread a column.
+__global__ void trsm_kernel(const LuMat* __restrict__ mats, int k0) {
   const LuMat mat = mats[blockIdx.y];
   const int n = mat.n;
   if (k0 + LU_NB >= n) return;  // no columns right of the panel (or the panel is the last)
-  const int nbk = LU_NB;
-  const int bend = min(K0 + LU_OB, n);
-  const int clo = mode == 2 ? bend : k0 + nbk, chi = mode == 1 ? bend : n;
-  T* M = (T*)mat.A;
-  __shared__ T L[LU_NB][LU_NB + 1];
-  for (int t = threadIdx.x; t < nbk * nbk; t += blockDim.x) {
-    int r = t % nbk, cc = t / nbk;
+  cd* M = (cd*)mat.A;
+  __shared__ cd L[LU_NB][LU_NB + 1];
+  for (int t = threadIdx.x; t < LU_NB * LU_NB; t += blockDim.x) {
+    const int r = t % LU_NB, cc = t / LU_NB;
     L[r][cc] = M[(size_t)(k0 + cc) * n + k0 + r];
   }
   __syncthreads();
-  const int c = clo + blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= chi) return;
-  T* col = M + (size_t)c * n + k0;
-  T x[LU_NB];
+  const int c = k0 + LU_NB + blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  cd* col = M + (size_t)c * n + k0;
+  cd x[LU_NB];
 #pragma unroll
-  for (int r = 0; r < LU_NB; ++r) x[r] = (r < nbk) ? col[r] : czero<T>();
+  for (int r = 0; r < LU_NB; ++r) x[r] = col[r];
 #pragma unroll
   for (int k = 0; k < LU_NB; ++k) {
 #pragma unroll
     for (int r = k + 1; r < LU_NB; ++r) x[r] = x[r] - L[r][k] * x[k];
   }
 #pragma unroll
-  for (int r = 0; r < LU_NB; ++r)
-    if (r < nbk) col[r] = x[r];
+  for (int r = 0; r < LU_NB; ++r) col[r] = x[r];
 }
 
 // The same for complex64, one thread a column: the rows of 128 columns pass through
@@ -758,37 +758,37 @@ __global__ void __launch_bounds__(128) trsm_c64_kernel(const LuMat* __restrict__
 }
 
 // ---------------------------------------------------------------- trailing update
+// Complex128 without a workspace, on the FP64 pipe:
 // C[i0.., j0..] -= A[i0.., k0..k0+nbk) * A[k0..k0+nbk), j0..], 64x64 tiles,
 // 256 threads, each 4x4 outputs: rows tx + 16a, columns ty + 16b.
 #define GT 64
-template <class T>
 __global__ void __launch_bounds__(256) gemm_update_kernel(const LuMat* __restrict__ mats, int k0) {
   const LuMat mat = mats[blockIdx.z];
   const int n = mat.n;
   const int nbk = LU_NB;
   const int start = k0 + nbk;
   if ((int)blockIdx.x * GT >= n - start || (int)blockIdx.y * GT >= n - start) return;
-  T* M = (T*)mat.A;
+  cd* M = (cd*)mat.A;
   const int i0 = start + blockIdx.x * GT, j0 = start + blockIdx.y * GT;
-  __shared__ T As[LU_NB][GT];
-  __shared__ T Bs[LU_NB][GT];
+  __shared__ cd As[LU_NB][GT];
+  __shared__ cd Bs[LU_NB][GT];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int t = tid; t < nbk * GT; t += 256) {
     int r = t % GT, kk = t / GT;
     int gi = i0 + r;
-    As[kk][r] = (gi < n) ? M[(size_t)(k0 + kk) * n + gi] : czero<T>();
+    As[kk][r] = (gi < n) ? M[(size_t)(k0 + kk) * n + gi] : C(0.0);
     int kb = t % nbk, cj = t / nbk;  // B element (row k0+kb, column j0+cj)
     int gj = j0 + cj;
-    Bs[kb][cj] = (gj < n) ? M[(size_t)gj * n + k0 + kb] : czero<T>();
+    Bs[kb][cj] = (gj < n) ? M[(size_t)gj * n + k0 + kb] : C(0.0);
   }
   __syncthreads();
-  T acc[4][4];
+  cd acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = czero<T>();
+    for (int c = 0; c < 4; ++c) acc[a][c] = C(0.0);
   for (int kk = 0; kk < nbk; ++kk) {
-    T av[4], bv[4];
+    cd av[4], bv[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) av[a] = As[kk][tx + 16 * a];
 #pragma unroll
@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(256) gemm_update_kernel(const LuMat* __restric
     for (int a = 0; a < 4; ++a) {
       int gi = i0 + tx + 16 * a;
       if (gi < n) {
-        T* d = M + (size_t)gj * n + gi;
+        cd* d = M + (size_t)gj * n + gi;
         *d = *d - acc[a][c];
       }
     }
@@ -1430,7 +1430,7 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
       if (rest > 0) {
         if constexpr (c64) trsm_c64_kernel<<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
         else if (two_level) luz_panel_rows(d, K0, k0, rest, active, ls);
-        else trsm_kernel<T><<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0, K0, mode);
+        else trsm_kernel<<<dim3((rest + 127) / 128, active), 128, 0, ls>>>(d, k0);
         ++launches;
       }
       return rest;
@@ -1486,7 +1486,7 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
         const int rest = panel_step(k0, 0, 0);
         if (rest <= 0) continue;
         const int t = (rest + GT - 1) / GT;
-        timed_launch([&] { gemm_update_kernel<T><<<dim3(t, t, active), 256, 0, ls>>>(d, k0); });
+        timed_launch([&] { gemm_update_kernel<<<dim3(t, t, active), 256, 0, ls>>>(d, k0); });
         ++launches;
         count_update(k0, LU_NB);
       }

@@ -936,8 +936,11 @@ static int build_finish(mueller_ctx* c, const LuTiming& lt, double ms_lu, int wa
 }
 
 // Workspace of a complex128 factorization: what all matrices need, up to `most`
-// bytes, else what the largest needs, else none (the FP64 pipe).
+// bytes, else what the largest needs, else none (the FP64 pipe).  "lu_pool_one" and
+// "lu_pool_none" in MUELLER_FAULT_INJECT: as if no more could be had.
 static LuPool lu_z_pool(DevBuf& buf, const std::vector<int>& n, size_t most) {
+  if (fault_injected("lu_pool_none")) return LuPool{};
+  if (fault_injected("lu_pool_one")) most = 0;
   for (size_t cap : {most, (size_t)0}) {
     LuPool pool;
     pool.bytes = lu_z_pool_bytes(n.data(), (int)n.size(), cap);
