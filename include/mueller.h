@@ -308,8 +308,9 @@ int mueller_modal_kernels_noalloc(const double* pairs_dev, long long npairs, mue
 /* Batched LU of `batch` column-major n x n complex matrices in place
  * (stride n*n); piv_dev [batch][n] (0-based LAPACK-style interchanges),
  * info_dev [batch] (0 or first zero-pivot column + 1).  The updates are
- * exact-digit products on the tensor cores (FP64 accuracy, relative to the
- * largest |l| |u| of an entry's row and column), in a workspace allocated for
+ * exact-digit products on the tensor cores (FP64 accuracy relative to the
+ * largest entry of each column of A, as partial pivoting has it; where the
+ * digits would keep less, on the FP64 pipe), in a workspace allocated for
  * the call (at most 4 GB, or one matrix's); they run on the FP64 pipe where it
  * cannot be had.  Returns MUELLER_ETIMEOUT if a bounded device-side wait gave
  * up (the factors are then unusable).  Synchronises `stream`. */

@@ -1437,6 +1437,11 @@ static cudaError_t lu_factor_impl(const LuMat* items, int count, cudaStream_t s,
     };
     if (two_level) {
       // LU_NB panels inside LU_OB blocks, one rank-LU_OB tensor-core update per block
+      if constexpr (!c64)
+        if (nmax > LU_NB) {
+          luz_begin(d, nmax, active, ls);
+          ++launches;
+        }
       for (int K0 = 0; K0 < nmax; K0 += LU_OB) {
         for (int p = 0; p < LU_OB_CHUNKS; ++p) {
           const int k0 = K0 + p * LU_NB;

@@ -7,7 +7,16 @@
 // whose rows differ by many orders (rows near the axis carry m^2 / r^2) keep
 // their small rows this way: the error of an entry is a few 2^-56 of
 // max_k |l_ik| d_k max_k |u_kj| / d_k per term, where scaling L and U alone would
-// leave that of the product of their unrelated maxima.  Eight balanced 7-bit
+// leave that of the product of their unrelated maxima.  That is FP64 accuracy as
+// partial pivoting has it, relative to the largest entry of the column of A, wherever
+// max_k |l_ik| d_k and max_k |u_kj| / d_k meet near one k.  They need not: rows of U that
+// reach into unlike columns have unlike d_k, and a product of small terms then gets the
+// error of a large one that is not there (sparse or weakly coupled matrices, columns or
+// blocks scaled by 1e8: residuals of 1e-4 of the column).  So a tile whose row and
+// column bounds multiply to more than 2^Z_SAFE times a column's largest entry of A is formed
+// on the FP64 pipe instead, by the warps that would have drained it.  Gaussian matrices of
+// order 64 to 3000 stay at 2^6 and below, those of bodies (sphere, cylinder, cone, torus,
+// random, droplet; contrast up to 100) at 2^6 and mostly below 1.  Eight balanced 7-bit
 // digits a value, |v| / scale < 1 (the first digit up to 128: the dropped levels
 // s + t > 7 are the largest error, and a tighter scale divides them by 4); the
 // products of levels s + t <= 7 are exact FP32 integers (at most K 2 (l + 3) 64^2
@@ -50,14 +59,18 @@
 #define Z_DRAIN 16                              // drain warps of the product
 #define Z_THREADS (32 * (Z_DRAIN + 2))
 #define Z_NAN (1 << 28)                         // exponent that marks a row or column with Inf or NaN
+#define Z_NONE (-(1 << 24))                     // of a row or column of zeros
+#define Z_SAFE 8                                // largest exponent of a tile's bound over its columns' entries of A
 
 // Workspace of a matrix: digits of up to ceil(n/128) row tiles and ceil(n/32)
-// column tiles, their scale exponents, and the high words of the largest
-// magnitude in each row of U12.
+// column tiles, their scale exponents, the high words of the largest
+// magnitude in each row of U12, the exponents of the largest entry of each column of A,
+// and the largest of a tile's scale exponents (those of columns of U less the column's).
 struct ZWork {
   __nv_bfloat16 *Ad, *Bd;
   int *rowE, *colE;
   unsigned* dmax;  // [ZB]
+  int *colA, *rowT, *colT;
 };
 __host__ __device__ inline size_t z_up(size_t b) { return (b + 255) & ~(size_t)255; }
 __host__ __device__ inline int z_tiles(int n, int t) { return (n + t - 1) / t; }
@@ -67,10 +80,12 @@ __host__ __device__ inline size_t z_bytes(int n, ZWork* w, unsigned char* base) 
   auto take = [&](size_t b) { const size_t p = o; o += z_up(b); return p; };
   const size_t oa = take(nr * ZKT * ZA_BLOCK * 2), ob = take(nc * ZKT * ZB_BLOCK * 2);
   const size_t orr = take(nr * ZR * 4), oc = take(nc * ZC * 4), od = take(ZB * 4);
+  const size_t oca = take((size_t)n * 4), ort = take(nr * 4), oct = take(nc * 4);
   if (w) {
     w->Ad = (__nv_bfloat16*)(base + oa); w->Bd = (__nv_bfloat16*)(base + ob);
     w->rowE = (int*)(base + orr); w->colE = (int*)(base + oc);
     w->dmax = (unsigned*)(base + od);
+    w->colA = (int*)(base + oca); w->rowT = (int*)(base + ort); w->colT = (int*)(base + oct);
   }
   return o;
 }
@@ -105,6 +120,25 @@ __device__ __forceinline__ unsigned z_high(cd v) {
 __device__ __forceinline__ int z_grade(unsigned high) {
   const int x = (int)(high >> 20);
   return (x == 0 || x >= 0x7FF) ? 0 : x - 1023;
+}
+
+// exponent of a vector's scale as the tile's bound takes it, less that of its column of A
+__device__ __forceinline__ int z_bound_exp(unsigned long long g, int E, int column) {
+  return g == 0 ? Z_NONE : E >= Z_NAN ? Z_NAN : E - column;
+}
+
+// Exponents of the columns of A (0 for zero columns and those with Inf or NaN): a warp a
+// column, eight columns a CTA.
+__global__ void __launch_bounds__(256) z_columns_kernel(const LuMat* __restrict__ mats) {
+  const LuMat mat = mats[blockIdx.y];
+  const int n = mat.n, c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= n) return;
+  const cd* col = (const cd*)mat.A + (size_t)c * n;
+  unsigned mx = 0;
+#pragma unroll 8
+  for (int r = lane; r < n; r += 32) mx = max(mx, z_high(col[r]));
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) z_work(mat).colA[c] = z_grade(mx);
 }
 
 // ---------------------------------------------------------------- slicing
@@ -145,7 +179,7 @@ __global__ void __launch_bounds__(ZSL_THREADS) z_slice_rows_kernel(const LuMat* 
   const cd* M = (const cd*)mat.A;
   __shared__ unsigned long long smx[4][ZR];
   __shared__ unsigned sD[K];
-  __shared__ int sE[K];
+  __shared__ int sE[K], sT[ZR / 32];
   if (clear && blockIdx.x == 0 && threadIdx.x < ZB) w.dmax[threadIdx.x] = 0;
   z_grades(M, n, k0, K, g0, g1, dsel >= 0 ? w.dmax + dsel : nullptr, sD, sE);
   const int r = threadIdx.x % ZR, part = threadIdx.x / ZR, i = i0 + r;
@@ -164,7 +198,13 @@ __global__ void __launch_bounds__(ZSL_THREADS) z_slice_rows_kernel(const LuMat* 
   __syncthreads();
   g = max(max(smx[0][r], smx[1][r]), max(smx[2][r], smx[3][r]));
   const int E = z_scale_exp(g);
-  if (part == 0) w.rowE[blockIdx.x * ZR + r] = E;
+  if (part == 0) {
+    w.rowE[blockIdx.x * ZR + r] = E;
+    const int t = __reduce_max_sync(0xffffffffu, z_bound_exp(g, E, FROM_U && i < n ? w.colA[i] : 0));
+    if ((r & 31) == 0) sT[r >> 5] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) w.rowT[blockIdx.x] = max(max(sT[0], sT[1]), max(sT[2], sT[3]));
   const int sh = E >= Z_NAN ? -8192 : 56 - E;
   for (int kg = part * KP; kg < (part + 1) * KP; kg += 8) {
     int dr[8][OZ_S], di[8][OZ_S];
@@ -201,7 +241,8 @@ __global__ void __launch_bounds__(256) z_slice_cols_kernel(const LuMat* __restri
   const ZWork w = z_work(mat);
   const cd* M = (const cd*)mat.A;
   __shared__ unsigned sD[K];
-  __shared__ int sE[K];
+  __shared__ int sE[K], sT;
+  if (threadIdx.x == 0) sT = Z_NONE;
   z_grades(M, n, k0, K, g0, g1, dsel >= 0 ? w.dmax + dsel : nullptr, sD, sE);
   constexpr int G = K / 8;  // threads per vector
   const int sg = FROM_L ? 1 : -1;
@@ -217,7 +258,10 @@ __global__ void __launch_bounds__(256) z_slice_cols_kernel(const LuMat* __restri
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
     const int E = z_scale_exp(g);
-    if (kg == 0) w.colE[blockIdx.x * ZC + jj] = E;
+    if (kg == 0) {
+      w.colE[blockIdx.x * ZC + jj] = E;
+      atomicMax(&sT, z_bound_exp(g, E, !FROM_L && j < v1 ? w.colA[j] : 0));
+    }
     const int sh = E >= Z_NAN ? -8192 : 56 - E;
     int dr[8][OZ_S], di[8][OZ_S];
 #pragma unroll
@@ -241,6 +285,8 @@ __global__ void __launch_bounds__(256) z_slice_cols_kernel(const LuMat* __restri
       *(uint4*)(blk + (2 * OZ_S + 2 * s + 1) * ZB_TILE) = *(const uint4*)re;
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) w.colT[blockIdx.x] = sT;
 }
 
 // Rows k0..k0+LU_NB of U in the columns [c0, ccap): unit-lower triangular solve,
@@ -296,8 +342,31 @@ __global__ void __launch_bounds__(128) z_trsm_kernel(const LuMat* __restrict__ m
 // Every wait is bounded: a role that gives up sets the CTA's failure flag (and
 // *err), the others stop at their next wait, and before the CTA exits the
 // copies in flight land and the MMAs complete.
+// Tiles that the digits would not keep (Z_SAFE) are no work for copies and MMAs; the drain
+// warps form them from L and U (inner rows k0 ..) in FP64.
+
+// Row i of such a tile, its columns j0 .. j0 + nc - 1.
 template <bool SWAP>
-__global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __restrict__ mats, int r0, int c0,
+__device__ __noinline__ void z_tile_fp64(cd* M, int n, int k0, int K, int i, int j0, int nc) {
+  cd acc[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] = C(0.0);
+  for (int k = k0; k < k0 + K; ++k) {
+    const cd a = SWAP ? M[(size_t)i * n + k] : M[(size_t)k * n + i];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (c < nc) acc[c] = fma(a, SWAP ? M[(size_t)k * n + j0 + c] : M[(size_t)(j0 + c) * n + k], acc[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    if (c < nc) {
+      cd* o = SWAP ? M + (size_t)i * n + j0 + c : M + (size_t)(j0 + c) * n + i;
+      *o = *o - acc[c];
+    }
+}
+
+template <bool SWAP>
+__global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __restrict__ mats, int k0, int r0, int c0,
                                                                  int ccap, int nkt, int nrt, int nct, int count,
                                                                  int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -315,6 +384,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
     const int n = mats[z].n;
     return r0 + x * ZR < n && c0 + y * ZC < min(n, ccap);
   };
+  auto kept = [](const ZWork& w, int x, int y) { return w.rowT[x] + w.colT[y] <= Z_SAFE; };
   if (warp == 0) tc::tmem_alloc(&tmem_base, 512);
   if (tid == 32) {
     s_fail = 0;
@@ -335,6 +405,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
         int z, x, y;
         if (!tile_of(t, z, x, y)) continue;
         const ZWork w = z_work(mats[z]);
+        if (!kept(w, x, y)) continue;
         const __nv_bfloat16* As = w.Ad + (size_t)x * ZKT * ZA_BLOCK;
         const __nv_bfloat16* Bs = w.Bd + (size_t)y * ZKT * ZB_BLOCK;
         for (int kt = 0; kt < nkt; ++kt, ++q) {
@@ -353,7 +424,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
       int q = 0, k = 0;
       for (long long t = blockIdx.x; t < total && !*fail; t += gridDim.x) {
         int z, x, y;
-        if (!tile_of(t, z, x, y)) continue;
+        if (!tile_of(t, z, x, y) || !kept(z_work(mats[z]), x, y)) continue;
         for (int kt = 0; kt < nkt && !*fail; ++kt, ++q) {
           const int st = q % Z_NST;
           if (!tc::mbar_wait(&full[st], (q / Z_NST) & 1)) { *fail = 1; break; }
@@ -395,6 +466,10 @@ __global__ void __launch_bounds__(Z_THREADS, 1) z_product_kernel(const LuMat* __
       const int nc = i < n ? min(8, min(n, ccap) - c0 - jt) : 0;  // columns of this thread's row
       cd* M = SWAP ? (cd*)mat.A + (size_t)i * n + c0 + jt : (cd*)mat.A + (size_t)(c0 + jt) * n + i;
       const size_t sc = SWAP ? 1 : n;
+      if (!kept(w, x, y)) {
+        if (nc > 0) z_tile_fp64<SWAP>((cd*)mat.A, n, k0, nkt * ZK, i, c0 + jt, nc);
+        continue;
+      }
       const int Er = w.rowE[x * ZR + (warp & 3) * 32 + lane] - 54;
       if (!tc::mbar_wait(&tfull[0], k & 1)) { *fail = 1; break; }
       tc::fence_after();
@@ -471,12 +546,16 @@ static int z_sms() {
 }
 
 template <bool SWAP>
-static void z_product(const LuMat* d, int r0, int rows, int c0, int ccap, int cols, int K, int count, int* err,
+static void z_product(const LuMat* d, int k0, int r0, int rows, int c0, int ccap, int cols, int K, int count, int* err,
                       cudaStream_t s) {
   const int nrt = z_tiles(rows, ZR), nct = z_tiles(cols, ZC);
   cudaFuncSetAttribute(z_product_kernel<SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_NST * Z_STAGE);
   const int grid = (int)std::min<long long>((long long)nrt * nct * count, z_sms());
-  z_product_kernel<SWAP><<<grid, Z_THREADS, Z_NST * Z_STAGE, s>>>(d, r0, c0, ccap, K / ZK, nrt, nct, count, err);
+  z_product_kernel<SWAP><<<grid, Z_THREADS, Z_NST * Z_STAGE, s>>>(d, k0, r0, c0, ccap, K / ZK, nrt, nct, count, err);
+}
+
+void luz_begin(const LuMat* d, int nmax, int count, cudaStream_t s) {
+  z_columns_kernel<<<dim3(z_tiles(nmax, 8), count), 256, 0, s>>>(d);
 }
 
 void luz_panel_rows(const LuMat* d, int K0, int k0, int cols, int count, cudaStream_t s) {
@@ -488,7 +567,7 @@ int luz_panel_update(const LuMat* d, int K0, int k0, int nmax, int count, int* e
   z_slice_rows_kernel<LU_NB, false><<<dim3(z_tiles(rows, ZR), count), ZSL_THREADS, 0, s>>>(d, r0, k0, r0, ccap, -1,
                                                                                            k0 == K0);
   z_slice_cols_kernel<LU_NB, false><<<dim3(z_tiles(cols, ZC), count), 256, 0, s>>>(d, r0, ccap, k0, r0, ccap, -1);
-  z_product<false>(d, r0, rows, r0, ccap, cols, LU_NB, count, err, s);
+  z_product<false>(d, k0, r0, rows, r0, ccap, cols, LU_NB, count, err, s);
   return 3;
 }
 
@@ -503,11 +582,11 @@ int luz_block_update(const LuMat* d, int K0, int nmax, int count, int* err, cuda
     z_slice_rows_kernel<LU_NB, true><<<dim3(z_tiles(rest, ZR), count), ZSL_THREADS, 0, s>>>(d, r0, k0, r0, cap,
                                                                                             k0 - K0, 0);
     z_slice_cols_kernel<LU_NB, true><<<dim3(z_tiles(brows, ZC), count), 256, 0, s>>>(d, v0, r0, k0, r0, cap, k0 - K0);
-    z_product<true>(d, r0, rest, v0, r0, brows, LU_NB, count, err, s);
+    z_product<true>(d, k0, r0, rest, v0, r0, brows, LU_NB, count, err, s);
     launches += 3;
   }
   z_slice_rows_kernel<ZB, false><<<dim3(z_tiles(rest, ZR), count), ZSL_THREADS, 0, s>>>(d, r0, K0, r0, cap, 0, 0);
   z_slice_cols_kernel<ZB, false><<<dim3(z_tiles(rest, ZC), count), 256, 0, s>>>(d, r0, cap, K0, r0, cap, 0);
-  z_product<false>(d, r0, rest, r0, cap, rest, ZB, count, err, s);
+  z_product<false>(d, K0, r0, rest, r0, cap, rest, ZB, count, err, s);
   return launches + 3;
 }

@@ -8,6 +8,8 @@
 // Workspace bytes of one n x n matrix (LuMat::ws, 256-byte aligned).
 size_t luz_matrix_bytes(int n);
 
+// Before the first panel: the exponents of the matrices' columns.
+void luz_begin(const LuMat* d, int nmax, int count, cudaStream_t s);
 // Rows k0..k0+LU_NB of U in the `cols` columns of the block right of the panel.
 void luz_panel_rows(const LuMat* d, int K0, int k0, int cols, int count, cudaStream_t s);
 // C = A[k0+LU_NB.., k0+LU_NB..min(K0+ZB, n)) -= L U of the panel at column k0 of the
