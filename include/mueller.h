@@ -356,8 +356,10 @@ size_t mueller_footprint_bytes(int N, int M);
  * for requests of the same rounded size, so repeated calls skip the driver's
  * allocation and release: buffers of at least 64 MiB (rounded up to 2 MiB) up to
  * a cap, smaller ones (rounded up to a quarter of their power of two) up to 256
- * MiB in all, the least recently released given up first.  A release synchronizes the device first (as cudaFree does).  When
- * an allocation fails, the cache is emptied and the allocation retried.
+ * MiB in all, the least recently released given up first.  A block stays with the
+ * device it was allocated on, whichever is current when it comes back.  A release
+ * synchronizes that device first (as cudaFree does).  When an allocation fails, the
+ * cache is emptied and the allocation retried.
  * mueller_cache_limit sets the cap (default 32 GiB; 0 disables caching) and
  * returns the previous one; mueller_cache_trim returns every cached block to
  * the driver; mueller_cache_bytes reports the bytes held.  Callers that budget

@@ -4,8 +4,6 @@
 #include "fields.cuh"
 #include "fields_oz.cuh"
 
-// One CTA per (node, wave): samples of the tangential traces on the node's
-// ring at n_theta azimuths, then their Fourier coefficients for m = -M..M.
 // Fourier coefficients (1/n_theta) sum_t s_t e^{-i m theta_t} of the four ring
 // traces smp[n_theta][4] (twiddles tw[t] = e^{-2 pi i t/n_theta}), scaled by
 // sE (rows 0, 1) and sH (rows 2, 3).  With n_theta = 2^L q (L <= 4), L
@@ -110,8 +108,8 @@ __device__ __forceinline__ double ring_even_coef(const double* smp, int R, int Q
 // complex transforms of its sampled traces, and everything that depends on
 // the wave alone sits in a table tab[w][q][6]: the factors of b_{m-1}, b_m,
 // b_{m+1} for E and for H.
-// FP64 pipe: N = 512, M = 64, 96 waves: 1.09 ms (7.91 ms with the four sampled
-// traces transformed ring by ring; 0.90 ms with the ring integrals of many waves on
+// FP64 pipe: N = 512, M = 64, 96 waves: 1.08 ms (7.91 ms with the four sampled
+// traces transformed ring by ring; 0.88 ms with the ring integrals of many waves on
 // the tensor cores).
 
 // double-double helpers (error-free transforms) for the wave's rotation e^{-i m phi_d}:
@@ -285,9 +283,9 @@ size_t rhs_planewave_scratch_doubles(int M, int nrhs, int n_theta) {
 // N is a multiple of 16.  Waves pass RHS_WAVES at a time, so the table stays
 // below 1 KiB x (2M + 1) x 96 bytes whatever the number of waves.
 // Ring integrals of fewer multiply-adds than this stay on the FP64 pipe with the rest
-// of the data (one launch instead of four): N = 512, M = 64: 8 waves (1.3e7) 0.17 ms
+// of the data (two launches instead of five): N = 512, M = 64: 8 waves (1.3e7) 0.17 ms
 // there and 0.20 ms on the tensor cores, 32 waves (5e7) 0.43 and 0.40 ms, 96 waves
-// (1.6e8) 1.08 and 0.90 ms; N = 128, M = 16, 200 waves (1e7) 0.29 and 0.31 ms.
+// (1.6e8) 1.08 and 0.88 ms; N = 128, M = 16, 200 waves (1e7) 0.29 and 0.31 ms.
 #define RHS_FMA_MIN 4e7
 size_t rhs_planewave_work_bytes(int N, int M, int nrhs, int n_theta) {
   const double fma = (double)N * nrhs * (M + 2.0) * (n_theta / 4);
@@ -681,7 +679,7 @@ __global__ void __launch_bounds__(256) ffgrid_coef_kernel(FieldGeom g, int M, do
 // so the two mirrored angles are A + iB and A - iB: 4 multiply-adds per term
 // for both.  FP64 pipe: 24 multiply-adds per node, mode, angle pair and side; the
 // whole grid, N = 512, M = 64, 8 sides, 180 x 360: 3.93 ms (49.2 ms with complex
-// coefficients per angle and the phase formed per mode and side; 0.94 ms on the
+// coefficients per angle and the phase formed per mode and side; 0.81 ms on the
 // tensor cores, which take all but small grids).  One CTA per
 // (mode, PT polar angles, WT right-hand sides); a thread owns one (angle, side)
 // and every JS-th node; the nodes pass through shared memory JC at a time.

@@ -136,7 +136,7 @@ void launch_support_post(const BuildArgs& a, const int* list, int q0, int count,
 // far pairs with the transform on the tensor cores: bins by grid size
 // (g.nl / 8), a pair list sorted by bin and place, then per bin and chunk the samples'
 // digit rows, ozaki_real_gemm with the bin's cos(2 pi m j / nl), and the
-// blocks (the same modes, zeros and tail queue as far_kernel)
+// blocks (the same modes and zeros as far_kernel)
 int far_tiles(int N);  // tile_hist holds nbins * far_tiles(N) integers, start nbins + 1
 void launch_far_bins(const BuildArgs& a, int nbins, unsigned short* tag, int* tile_hist, int* start,
                      cudaStream_t s);

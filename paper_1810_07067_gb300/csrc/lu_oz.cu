@@ -27,11 +27,12 @@
 // One entry costs 144 digit products per k on the tensor cores and about 60
 // integer operations and one FP64 addition per K, where the FP64 pipe (two
 // multiply-adds per clock and SM on this part) spends 2 K clocks of an SM on it.
-// LU of 9 matrices of order 1250: 69.3 -> 13.1 ms; the cylinder's 65 matrices of order
+// LU of 9 matrices of order 1250: 69.3 -> 13.2 ms; the cylinder's 65 matrices of order
 // 1280: updates 298 -> 12 ms (17 ms with an MMA per pair of digits, which is bound by
 // reading the tiles of L again and again: the digits of U lie behind one another, so
-// one MMA takes a digit of L times up to four of U into as many levels).  Residuals of random factors 1.4e-15 (1.9e-15 on the
-// FP64 pipe), of diagonally dominant ones 1.7e-16 (1.9e-16).
+// one MMA takes a digit of L times up to four of U into as many levels).  Residuals of
+// random factors 1.4e-15 (1.9e-15 on the FP64 pipe), of diagonally dominant ones 1.7e-16
+// (1.9e-16).
 //
 // The block row U12 = L11^{-1} A12 of a 128-column block: four FP64 triangular
 // solves of 32 rows, the rows below updated by products with the tile roles

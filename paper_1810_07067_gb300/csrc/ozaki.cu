@@ -14,7 +14,7 @@
 // drained: the levels joined in 64-bit integers, converted on the integer pipe and
 // added in FP64 once per value (a conversion and a multiply-add per level on the
 // FP64 pipe took longer than the products: N = 512, M = 64, 192 vectors per mode,
-// 24.7 -> 15.0 ms a residual).  The complex product takes two MMAs: the B operand
+// 24.7 -> 15.0 ms a residual, 11.7 with the wide MMAs below).  The complex product takes two MMAs: the B operand
 // stacks the digits of Re y over those of Im y (2 jt rows), so Re a [Re y | Im y] +
 // Im a [-Im y | Re y] lands in [Re | Im] of the accumulator; the y slices are stored as
 // [Re, Im] digit by digit and again as [-Im, Re], so that one MMA takes a digit of a

@@ -114,6 +114,9 @@ HD KPow kpow(cd k) {
   return p;
 }
 
+// The entire functions that the nine kernels are made of, one wavenumber at a time.  The
+// samples take them from SampleFun below; these are the reference that the tests hold
+// against 60 digits (and so are ellipk_c and carlson_rd, of which ellipke took the place).
 HD Ent entire(const SeriesTables& T, const KPow& kp, double su) {
   cd x = kp.k * su;
   cd h = 0.5 * x;
